@@ -161,7 +161,7 @@ def other_workloads_leg(sm_mhz, hbm_gbs):
     import numpy as np
     import torch
     from paper_2607_12324_b200 import emo, workloads as W
-    names = {5: "32-bit spine forward + lane-stream backward", 4: "32-bit spine", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}
+    names = {5: "32-bit spine, several policies per thread", 4: "32-bit spine", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}
     out = []
     for name in ("cfg0-tiny", "cfg1-train", "cfg2-packed", "cfg3-8dev"):
         g = W.make_graph(name)
@@ -411,7 +411,7 @@ def main():
             "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "int64", "data": "synthetic",
             "config": workload_config(args.workload, args.scale, g, B, ppm),
-            "details": {"kernels": {5: "32-bit spine forward + lane-stream backward", 4: "32-bit spine", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}[path],
+            "details": {"kernels": {5: "32-bit spine, several policies per thread", 4: "32-bit spine", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}[path],
                         "slack_sums": bool(args.sums), "lanes": fl["lanes"] if path in (2, 5) else info.lanes,
                         "steps": fl["steps"] if path in (2, 5) else info.steps_fwd, "stage_steps": fl["K"], "barrier_steps": fl["sync"],
                         "restore_rows": fl["pushes"], "depth": info.depth, "graph_load_s": t_load,

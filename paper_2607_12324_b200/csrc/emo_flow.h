@@ -87,8 +87,12 @@ constexpr uint32_t kOpOffMask = (1u << 29) - 1u;
 // segment's sum, written to the lane's slot and to a published slot.  A node with more operands gets
 // merge operations in front.  Backward, a value that a node of a much earlier stage reads (two stages
 // or more: a launch node and its kernels) is folded by the storing warps into a slot of that reader.
-constexpr int kSpOpWordsF = 8;        // a0, d0, a1, d1, lane slot, published slot, sum offset, flags | push row << 8 | push row in the
-                                      // paired numbering << 20 (both relative to the stage's base); terminal bounds are taken in order
+// Operations that the spine executes at once: independent of each other, loads before stores.  Two on graphs of up to eight
+// lanes (four would not shorten their programs: 5 034 bundles against 5 051 on the 10 000-node graph, backward), four on wider
+// ones (31 980 against 63 817 bundles on the 18-lane graph of 128 039 nodes).
+inline int spine_bundle(int lanes) { return lanes <= 8 ? 2 : 4; }
+constexpr int kSpOpWordsF = 8;        // a0, d0, a1, d1, lane slot, published slot, sum offset, flags | push row << 8 (relative to the
+                                      // stage's base); terminal bounds are taken in order
 constexpr int kSpOpWordsB = 12;       // the same eight (flags | pop row << 8), then: slot to clear, lane's completion slot, where the head's
                                       // tail goes (beside X if members are folded, else nowhere), where it goes when all tails are kept
 constexpr int kSpSegWords = 4;        // lane | first position << 8 | members << 16 | flags << 24, sum offset, A_v low, high
@@ -99,6 +103,10 @@ constexpr uint32_t kSpPos_First = 1u, kSpPos_Last = 2u;
 constexpr uint32_t kSp_NoSum = 1u;    // operation flags: the segment's sum is zero / a merge operation
 constexpr uint32_t kSp_Push = 2u;     // forward: the lane's previous value goes to the restore list; backward: it is popped
 constexpr uint32_t kSp_Terminal = 4u; // forward: the segment's last node has no successor
+// flags of the layout that the kernels read (member records, records of the completion walk), beside First / Last: the
+// member is folded; the walk takes a row of the restore list
+constexpr uint32_t kSpDev_Fold = 32u, kSpDev_Pop = 128u;
+constexpr int kSpDevOpWords = 12;     // x0, x1, word of the sum, slot to clear, d0, d1, lane's slot, published slot, word to write, spare
 constexpr uint32_t kSpSeg_PreF = 1u, kSpSeg_PreB = 2u, kSpSeg_Fold = 4u;   // segment flags
 
 struct SpineDir {
@@ -111,6 +119,7 @@ struct SpineDir {
 struct Spine {
     bool ok = false;
     int max_segs = 0, max_pool = 0;
+    int bundle = 2;                   // operations per bundle (n_ops is a multiple of it)
     int acc_words = 0;                // 4-byte words per policy that the sums / results of one stage take
     int acc_words_all = 0;            // the same when every segment's head tail is kept (one more word per segment, behind the others)
     int64_t pushes = 0;
@@ -121,11 +130,8 @@ struct Spine {
     std::vector<uint32_t> posw;       // [stages][lanes * K] position words
     std::vector<uint64_t> pool;       // [stages][max_pool] lbC of terminal nodes
     std::vector<int64_t> push_base;   // [stages + 1]
-    // the same restore rows numbered as a lane-stream program with stages of pair_K steps numbers them (per stage the
-    // lanes in order, a lane's rows by position): the forward spine kernel can then feed the lane-stream backward kernel
-    int pair_K = 0;
-    bool pair_ok = false;
-    std::vector<int64_t> pair_base;   // [stages] smallest such row of the stage's pushes
+    std::vector<uint32_t> term_slot;  // forward: slot that publishes the value of each terminal node, in the order of pool
+    uint32_t unread_slot = 0;         // slot (in both directions) that nobody reads: where an absent output goes
     SpineDir f, b;
 };
 
@@ -169,13 +175,12 @@ struct SpineIn {
     const std::vector<int64_t> *lbES = nullptr, *lbC = nullptr, *lbQin = nullptr, *lbQ = nullptr;
     const std::vector<int32_t> *step_of = nullptr, *lane_of = nullptr, *prev_on_lane = nullptr, *next_on_lane = nullptr, *pos_of = nullptr;
     const double *energy = nullptr;                                   // [n][L]
-    int pair_K = 0;                                                   // stage length of the lane-stream program to pair with (0: none)
 };
 int build_spine(const SpineIn &in, Spine &out, std::string &err);
 
 // Compiles g into a lane-stream program.  Returns EMO_OK with out.ok32 = false when the 32-bit
 // representation does not apply (spread too large, too many lanes); other codes are errors.
 int compile_flow(const HostGraph &g, const int64_t *lat, const double *energy, int lanes, int lookahead,
-                 int K, int sync, Flow &out, std::string &err, bool spine = false, int pair_K = 0);
+                 int K, int sync, Flow &out, std::string &err, bool spine = false);
 
 }  // namespace emo

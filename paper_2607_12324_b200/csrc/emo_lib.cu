@@ -1,6 +1,7 @@
 // C-ABI entry points (see include/emo.h) and the CUDA kernels behind them.  sm_100a only.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <map>
@@ -53,13 +54,19 @@ struct DevFlow {
     bool ready = false;
 };
 
-// The spine program on the device (emo_spine.cuh): per direction one blob per stage.
+// The spine program on the device (emo_spine.cuh): per direction and stage the workers' part and the spine's part.
+struct DevSpineDir {
+    unsigned char *blobW = nullptr, *blobS = nullptr;
+    uint32_t *rows = nullptr;       // [stages][nlook] policy row of every look-up entry
+    unsigned w_bytes = 0, s_bytes = 0, off_pos = 0, off_mem = 0, off_tab = 0, off_ops = 0, off_rec = 0;
+    int words = 0;                  // words per policy and stage: sums (later the values that are pushed / qin), one that stays zero, an unread one; backward then
+                                    // the completion offsets
+    int zero = 0;                   // the word that stays zero
+};
 struct DevSpine {
-    unsigned char *blobF = nullptr, *blobB = nullptr;
-    uint32_t *rows = nullptr, *push_base = nullptr;
-    unsigned blobF_bytes = 0, blobB_bytes = 0;
-    unsigned f_off_ops = 0, f_front = 0, f_off_tpool = 0, f_off_pos = 0, f_off_tab = 0;      // f_front: bytes that the spine needs
-    unsigned b_off_ops = 0, b_off_mem = 0, b_off_tab = 0;
+    DevSpineDir f, b;
+    uint32_t *push_base = nullptr;
+    int nlook = 0, chunks = 0;      // look-up entries and chunks of a stage
     int max_push = 0;
     bool ready = false;
 };
@@ -592,46 +599,247 @@ void free_flow(DevFlow &d)
 }
 
 
+// Look-up entries per chunk that the stages are cut for: enough to pay for the chunk's two waits, few enough that the
+// look-up warps share a stage evenly (250 000 nodes, 55 look-up entries per stage: five chunks).
+constexpr int kSpChunkTarget = 12;
+
+// Lays the spine program out for the kernels.  A stage's look-up entries are the members of its segments that depend on
+// the level (or carry energy), dealt to the chunks by length, longest segment first; the members of the other segments
+// follow behind them (backward: they only store).  Backward the members of a segment lie last to first.  Sums are
+// numbered compactly forward (segments whose sum is never read have none) and by segment backward.
 int upload_spine(const Flow &f, DevSpine &d)
 {
     const Spine &sp = f.spine;
     if (!f.ok32 || !sp.ok || f.stages == 0) return EMO_OK;
-    const size_t per = (size_t)f.lanes * f.K;
     auto r16 = [](size_t x) { return (x + 15) / 16 * 16; };
-    // forward: header, terminal bounds and operations lie together at the front (what the spine needs: a worker copies
-    // it to the group's own ring, so that the stage buffer is free again as soon as the sums are taken)
-    d.f_off_tpool = 16;
-    d.f_off_ops = (unsigned)r16(d.f_off_tpool + (size_t)sp.max_pool * 8);
-    d.f_front = (unsigned)(d.f_off_ops + (size_t)(sp.f.max_ops + 1) * kSpOpWordsF * 4);
-    d.f_off_pos = d.f_front;
-    d.f_off_tab = (unsigned)r16(d.f_off_pos + per * 4);
-    d.blobF_bytes = (unsigned)r16(d.f_off_tab + per * f.Lp * 12);
-    d.b_off_ops = 16;
-    d.b_off_mem = (unsigned)(d.b_off_ops + (size_t)(sp.b.max_ops + 1) * kSpOpWordsB * 4);
-    d.b_off_tab = (unsigned)(d.b_off_mem + per * kSpMemWords * 4);
-    d.blobB_bytes = (unsigned)r16(d.b_off_tab + per * f.Lp * 4);
-    std::vector<unsigned char> bf((size_t)f.stages * d.blobF_bytes, 0), bb((size_t)f.stages * d.blobB_bytes, 0);
-    std::vector<uint32_t> pb((size_t)f.stages + 1);
-    for (int st = 0; st <= f.stages; ++st) pb[st] = (uint32_t)sp.push_base[st];
-    for (int st = 0; st < f.stages; ++st) {
-        d.max_push = std::max(d.max_push, (int)(pb[st + 1] - pb[st]));
-        unsigned char *F = bf.data() + (size_t)st * d.blobF_bytes, *Bk = bb.data() + (size_t)st * d.blobB_bytes;
-        const uint32_t hf[4] = {sp.f.n_ops[st], sp.n_segs[st], pb[st], (uint32_t)sp.pair_base[st]}, hb[4] = {sp.b.n_ops[st], sp.n_segs[st], pb[st], 0u};
-        std::memcpy(F, hf, 16);
-        std::memcpy(Bk, hb, 16);
-        std::memcpy(F + d.f_off_ops, &sp.f.ops[(size_t)st * sp.f.max_ops * kSpOpWordsF], (size_t)sp.f.max_ops * kSpOpWordsF * 4);
-        std::memcpy(Bk + d.b_off_ops, &sp.b.ops[(size_t)st * sp.b.max_ops * kSpOpWordsB], (size_t)sp.b.max_ops * kSpOpWordsB * 4);
-        std::memcpy(F + d.f_off_tpool, &sp.pool[(size_t)st * sp.max_pool], (size_t)sp.max_pool * 8);
-        std::memcpy(F + d.f_off_pos, &sp.posw[(size_t)st * per], per * 4);
-        std::memcpy(Bk + d.b_off_mem, &sp.mem[(size_t)st * per * kSpMemWords], per * kSpMemWords * 4);
-        std::memcpy(Bk + d.b_off_tab, &f.tabB[(size_t)st * per * f.Lp], per * f.Lp * 4);
-        // forward table rows: {duration, energy high word, low word} per level, 12 bytes apart (3 is coprime with the 32
-        // banks: the 32 policies of a warp, whatever their levels, read each of the three words without a bank conflict)
-        std::memcpy(F + d.f_off_tab, &f.tabF[(size_t)st * per * f.Lp * 3], per * f.Lp * 12);
+    const int stages = f.stages, lanes = f.lanes, K = f.K, Lp = f.Lp;
+    struct StagePlan {
+        std::vector<std::vector<uint32_t>> chunk;               // segments of every look-up chunk
+        std::vector<int> fill;                                  // entries of every chunk, padded to a multiple of four
+        std::vector<uint32_t> rest;                             // segments without look-ups
+    };
+    auto seg_word = [&](int st, uint32_t i, int k) { return sp.seg[((size_t)st * std::max(sp.max_segs, 1) + i) * kSpSegWords + k]; };
+    auto seg_count = [&](int st, uint32_t i) { return (int)((seg_word(st, i, 0) >> 16) & 255u); };
+    auto seg_flags = [&](int st, uint32_t i) { return seg_word(st, i, 0) >> 24; };
+    int64_t active = 0;
+    for (int st = 0; st < stages; ++st)
+        for (uint32_t i = 0; i < sp.n_segs[st]; ++i)
+            if (seg_flags(st, i) & (kSpSeg_PreF | kSpSeg_PreB)) active += seg_count(st, i);
+    d.chunks = (int)std::max<int64_t>(1, std::min<int64_t>(kSpChunks - 1, (active + (int64_t)stages * kSpChunkTarget / 2) / ((int64_t)stages * kSpChunkTarget)));
+    std::vector<StagePlan> plan((size_t)stages);
+    int max_rest = 0;
+    for (int st = 0; st < stages; ++st) {
+        StagePlan &pl = plan[st];
+        pl.chunk.resize((size_t)d.chunks);
+        pl.fill.assign((size_t)d.chunks, 0);
+        std::vector<uint32_t> act;
+        int rest = 0;
+        for (uint32_t i = 0; i < sp.n_segs[st]; ++i) {
+            if (seg_flags(st, i) & (kSpSeg_PreF | kSpSeg_PreB)) act.push_back(i);
+            else {
+                pl.rest.push_back(i);
+                rest += seg_count(st, i);
+            }
+        }
+        std::stable_sort(act.begin(), act.end(), [&](uint32_t a, uint32_t b) { return seg_count(st, a) > seg_count(st, b); });
+        for (uint32_t i : act) {
+            const int c = (int)(std::min_element(pl.fill.begin(), pl.fill.end()) - pl.fill.begin());
+            pl.chunk[c].push_back(i);
+            pl.fill[c] += seg_count(st, i);
+        }
+        int total = 0;
+        for (int &c : pl.fill) total += (c = (c + 3) / 4 * 4);
+        d.nlook = std::max(d.nlook, total);
+        max_rest = std::max(max_rest, (rest + 3) / 4 * 4);
     }
-    int rc = upload(&d.blobF, bf.data(), bf.size());
-    if (rc == EMO_OK) rc = upload(&d.blobB, bb.data(), bb.size());
-    if (rc == EMO_OK) rc = upload(&d.rows, f.rows.data(), f.rows.size() * 4);
+    if (d.nlook == 0) d.nlook = 4;
+    const int nmem = d.nlook + max_rest;
+    // forward words: one per operation that has a sum or whose value is pushed later, by the compiler's operation number.  A value
+    // is pushed by the operation that produced it: the lane's last one before the node that asks for it.
+    struct Push { uint32_t op, row; };
+    std::vector<std::vector<Push>> push((size_t)stages);
+    std::vector<std::vector<int>> word_op((size_t)stages);      // word of every forward operation (-1: none)
+    std::vector<std::vector<int>> word_f((size_t)stages);       // ... by the compiler's word number
+    size_t max_push_rec = 0;
+    {
+        std::vector<std::pair<int, uint32_t>> last((size_t)lanes, {-1, 0u});      // the lane's last operation
+        for (int st = 0; st < stages; ++st)
+            for (uint32_t i = 0; i < sp.f.n_ops[st]; ++i) {
+                const uint32_t *w = &sp.f.ops[((size_t)st * sp.f.max_ops + i) * kSpOpWordsF];
+                if (w[4] / 128u >= (uint32_t)lanes) continue;      // a merge or a filler
+                auto &l = last[w[4] / 128u];
+                // (a lane's first value needs no row: nothing lies in front of it)
+                if ((w[7] & kSp_Push) && l.first >= 0) push[l.first].push_back({l.second, (uint32_t)sp.push_base[st] + ((w[7] >> 8) & 0xFFFu)});
+                l = {st, i};
+            }
+        for (int st = 0; st < stages; ++st) {
+            max_push_rec = std::max(max_push_rec, push[st].size());
+            word_op[st].assign(sp.f.n_ops[st], -1);
+            word_f[st].assign((size_t)sp.acc_words + 1, -1);
+            int k = 0;
+            for (uint32_t i = 0; i < sp.f.n_ops[st]; ++i) {
+                const uint32_t *w = &sp.f.ops[((size_t)st * sp.f.max_ops + i) * kSpOpWordsF];
+                if (!(w[7] & kSp_NoSum)) word_f[st][w[6] / 128u] = word_op[st][i] = k++;
+            }
+            for (const Push &q : push[st])
+                if (word_op[st][q.op] < 0) word_op[st][q.op] = k++;
+            d.f.words = std::max(d.f.words, k);
+        }
+    }
+    d.f.zero = d.f.words;
+    d.f.words += 2;
+    d.b.zero = sp.max_segs;
+    d.b.words = 2 * (sp.max_segs + 2);
+    size_t max_term = 0;
+    std::vector<size_t> n_term((size_t)stages, 0);
+    for (int st = 0; st < stages; ++st) {
+        for (uint32_t i = 0; i < sp.f.n_ops[st]; ++i) n_term[st] += (sp.f.ops[((size_t)st * sp.f.max_ops + i) * kSpOpWordsF + 7] & kSp_Terminal) != 0;
+        max_term = std::max(max_term, n_term[st]);
+    }
+    d.f.off_pos = d.b.off_pos = 64;
+    d.f.off_tab = (unsigned)r16(d.f.off_pos + (size_t)d.nlook * 4);
+    d.f.w_bytes = (unsigned)r16(d.f.off_tab + (size_t)d.nlook * Lp * 12);
+    d.b.off_mem = (unsigned)r16(d.b.off_pos + (size_t)d.nlook * 4);
+    d.b.off_tab = (unsigned)(d.b.off_mem + (size_t)nmem * 32);
+    d.b.w_bytes = (unsigned)r16(d.b.off_tab + (size_t)(d.nlook + 1) * Lp * 4);      // the last row stays zero: entries without look-ups
+    const int NB = sp.bundle;
+    const size_t op_bytes = kSpDevOpWords * 4, spare = (size_t)NB;      // a bundle behind the last is read ahead
+    d.f.off_ops = (unsigned)(16 + max_term * 16);
+    d.f.off_rec = (unsigned)(d.f.off_ops + (sp.f.max_ops + spare) * op_bytes);
+    d.f.s_bytes = (unsigned)(d.f.off_rec + (max_push_rec + 3) / 4 * 32);
+    d.b.off_ops = 16;
+    d.b.off_rec = (unsigned)(d.b.off_ops + (sp.b.max_ops + spare) * op_bytes);
+    // the completion walk: a stage's lanes are dealt to NB streams, the longest lane first (four records behind the last are
+    // read ahead)
+    std::vector<std::vector<std::vector<uint32_t>>> walk((size_t)stages);      // [stage][stream] segments, lane by lane, a lane's last to first
+    size_t max_rounds = 0;
+    for (int st = 0; st < stages; ++st) {
+        std::vector<std::vector<uint32_t>> of((size_t)lanes);
+        for (uint32_t i = 0; i < sp.n_segs[st]; ++i) of[seg_word(st, i, 0) & 255u].push_back(i);
+        for (auto &l : of) std::sort(l.begin(), l.end(), [&](uint32_t x, uint32_t y) { return ((seg_word(st, x, 0) >> 8) & 255u) > ((seg_word(st, y, 0) >> 8) & 255u); });
+        std::stable_sort(of.begin(), of.end(), [](const auto &x, const auto &y) { return x.size() > y.size(); });
+        walk[st].resize((size_t)NB);
+        for (auto &l : of) {
+            auto &s0 = *std::min_element(walk[st].begin(), walk[st].end(), [](const auto &x, const auto &y) { return x.size() < y.size(); });
+            s0.insert(s0.end(), l.begin(), l.end());
+        }
+        for (auto &w : walk[st]) max_rounds = std::max(max_rounds, (w.size() + 3) / 4 * 4);
+    }
+    d.b.s_bytes = (unsigned)(d.b.off_rec + (max_rounds + 4) * 16 * (size_t)NB);
+    std::vector<unsigned char> fW((size_t)stages * d.f.w_bytes, 0), fS((size_t)stages * d.f.s_bytes, 0), bW((size_t)stages * d.b.w_bytes, 0),
+        bS((size_t)stages * d.b.s_bytes, 0);
+    std::vector<uint32_t> rowsF((size_t)stages * d.nlook, kNone), rowsB((size_t)stages * d.nlook, kNone), pb((size_t)stages + 1);
+    for (int st = 0; st <= stages; ++st) pb[st] = (uint32_t)sp.push_base[st];
+    const uint32_t unread = sp.unread_slot * 128u;
+    size_t term0 = 0;
+    for (int st = 0; st < stages; ++st) {
+        d.max_push = std::max(d.max_push, (int)(pb[st + 1] - pb[st]));
+        unsigned char *W = fW.data() + (size_t)st * d.f.w_bytes, *WB = bW.data() + (size_t)st * d.b.w_bytes;
+        uint32_t *tableF = (uint32_t *)W, *tableB = (uint32_t *)WB, *posF = (uint32_t *)(W + d.f.off_pos), *posB = (uint32_t *)(WB + d.b.off_pos);
+        uint32_t *mem = (uint32_t *)(WB + d.b.off_mem);
+        for (int e = 0; e < nmem; ++e) mem[(size_t)e * 8] = kNone;      // padding: no node, no fold
+        bool folds = false;
+        auto put_seg = [&](uint32_t si, int &e, bool look) {
+            const uint32_t w0 = seg_word(st, si, 0), wf = (uint32_t)std::max(word_f[st][seg_word(st, si, 1) / 128u], 0);
+            const int ln = (int)(w0 & 255u), first = (int)((w0 >> 8) & 255u), cnt = seg_count(st, si);
+            const bool sum = ((w0 >> 24) & kSpSeg_PreB) != 0;
+            for (int j = 0; j < cnt; ++j, ++e) {
+                const size_t qf = ((size_t)st * lanes + ln) * K + first + j, qb = ((size_t)st * lanes + ln) * K + first + cnt - 1 - j;
+                const uint32_t *m = &sp.mem[qb * kSpMemWords];
+                const uint32_t ends = (j == 0 ? kSpPos_First : 0u) | ((j == cnt - 1 && sum) ? kSpPos_Last : 0u);
+                uint32_t *o = mem + (size_t)e * 8;
+                std::memcpy(o, m, 32);
+                o[3] = ends | (si << 16);
+                if (m[1] != unread) {
+                    o[3] |= kSpDev_Fold;
+                    folds = true;
+                }
+                if (!look) continue;
+                posB[e] = ends | (si << 16);
+                posF[e] = ends | (wf << 16);
+                rowsF[(size_t)st * d.nlook + e] = f.rows[qf];
+                rowsB[(size_t)st * d.nlook + e] = f.rows[qb];
+                std::memcpy(W + d.f.off_tab + (size_t)e * Lp * 12, &f.tabF[qf * Lp * 3], (size_t)Lp * 12);
+                std::memcpy(WB + d.b.off_tab + (size_t)e * Lp * 4, &f.tabB[qb * Lp], (size_t)Lp * 4);
+            }
+        };
+        // chunk table: first entry | entries << 16 (for the storing workers also: some entry is folded << 31)
+        int e0 = 0;
+        for (int c = 0; c < d.chunks; ++c) {
+            int e = e0;
+            folds = false;
+            for (uint32_t si : plan[st].chunk[c]) put_seg(si, e, true);
+            tableF[c] = tableB[c] = (uint32_t)e0 | ((uint32_t)plan[st].fill[c] << 16);
+            tableB[8 + c] = tableB[c] | (folds ? 0x80000000u : 0u);
+            e0 += plan[st].fill[c];
+        }
+        int er = d.nlook;
+        folds = false;
+        for (uint32_t si : plan[st].rest) put_seg(si, er, false);
+        tableB[8 + d.chunks] = (uint32_t)d.nlook | ((uint32_t)((er - d.nlook + 3) / 4 * 4) << 16) | (folds ? 0x80000000u : 0u);
+
+        uint32_t *hf = (uint32_t *)(fS.data() + (size_t)st * d.f.s_bytes), *hb = (uint32_t *)(bS.data() + (size_t)st * d.b.s_bytes);
+        hf[0] = sp.f.n_ops[st] / (uint32_t)NB;
+        hf[1] = (uint32_t)n_term[st];
+        hf[2] = ((uint32_t)push[st].size() + 3u) / 4u * 4u;
+        hb[0] = sp.b.n_ops[st] / (uint32_t)NB;
+        for (auto &w : walk[st]) hb[2] = std::max(hb[2], (uint32_t)(w.size() + 3) / 4u * 4u);
+        for (size_t t = 0; t < n_term[st]; ++t) {
+            const uint64_t lb = sp.pool[(size_t)st * sp.max_pool + t];
+            hf[4 + 4 * t + 0] = sp.term_slot[term0 + t] * 128u;
+            hf[4 + 4 * t + 2] = (uint32_t)lb;
+            hf[4 + 4 * t + 3] = (uint32_t)(lb >> 32);
+        }
+        term0 += n_term[st];
+        auto put_op = [&](uint32_t *o, const uint32_t *w, uint32_t sum, uint32_t clear, uint32_t to) {
+            const uint32_t v[kSpDevOpWords] = {w[0], w[2], sum * 128u, clear, w[1], w[3], w[4], w[5], to * 128u, 0u, 0u, 0u};
+            std::memcpy(o, v, sizeof v);
+        };
+        // what lies behind the last operation is read ahead and must name words that exist: all zero
+        for (uint32_t i = 0; i < sp.f.n_ops[st]; ++i) {
+            const uint32_t *w = &sp.f.ops[((size_t)st * sp.f.max_ops + i) * kSpOpWordsF];
+            const uint32_t sum = (w[7] & kSp_NoSum) ? (uint32_t)d.f.zero : (uint32_t)word_op[st][i];
+            put_op((uint32_t *)((unsigned char *)hf + d.f.off_ops + i * op_bytes), w, sum, unread,
+                   (uint32_t)(word_op[st][i] >= 0 ? word_op[st][i] : d.f.zero + 1));
+        }
+        {
+            uint32_t *rec = (uint32_t *)((unsigned char *)hf + d.f.off_rec);
+            for (uint32_t i = 0; i < hf[2]; ++i) {
+                rec[2 * i] = i < push[st].size() ? (uint32_t)word_op[st][push[st][i].op] * 128u : 0u;
+                rec[2 * i + 1] = i < push[st].size() ? push[st][i].row : kNone;
+            }
+        }
+        std::vector<uint32_t> seg_of_word((size_t)sp.acc_words + 2, kNone), seg_flags_op((size_t)sp.max_segs + 1, 0);
+        for (uint32_t i = 0; i < sp.n_segs[st]; ++i) seg_of_word[seg_word(st, i, 1) / 128u] = i;
+        for (uint32_t i = 0; i < sp.b.n_ops[st]; ++i) {
+            const uint32_t *w = &sp.b.ops[((size_t)st * sp.b.max_ops + i) * kSpOpWordsB];
+            const uint32_t si = w[4] != unread ? seg_of_word[w[6] / 128u] : kNone;      // merge operations have no segment
+            const bool sum = !(w[7] & kSp_NoSum);
+            put_op((uint32_t *)((unsigned char *)hb + d.b.off_ops + i * op_bytes), w, sum ? si : (uint32_t)d.b.zero, w[8], si != kNone ? si : (uint32_t)d.b.zero + 1u);
+            if (si != kNone) seg_flags_op[si] = ((w[7] & kSp_Push) ? kSpDev_Pop : 0u) | (sum ? 1u : 0u) | (w[7] & 0xFFFFFF00u);
+        }
+        uint32_t *rec = (uint32_t *)((unsigned char *)hb + d.b.off_rec);
+        for (uint32_t i = 0; i < hb[2] + 4u; ++i)
+            for (int k = 0; k < NB; ++k, rec += 4) {
+                const std::vector<uint32_t> &w = walk[st][k];
+                rec[0] = unread;
+                rec[1] = (uint32_t)d.b.zero * 128u;
+                rec[2] = (uint32_t)(d.b.zero + 1) * 128u;      // padding: words nobody reads
+                if (i >= w.size()) continue;
+                auto lane_of = [&](uint32_t j) { return seg_word(st, w[j], 0) & 255u; };
+                const uint32_t ln = lane_of(i), fl = seg_flags_op[w[i]];
+                rec[0] = ((uint32_t)(lanes + 2) + ln) * 128u;
+                if (fl & 1u) rec[1] = w[i] * 128u;
+                rec[2] = w[i] * 128u;
+                rec[3] = (fl & ~1u) | ((i == 0 || lane_of(i - 1) != ln) ? kSpPos_First : 0u) | ((i + 1 == w.size() || lane_of(i + 1) != ln) ? kSpPos_Last : 0u);
+            }
+    }
+    int rc = upload(&d.f.blobW, fW.data(), fW.size());
+    if (rc == EMO_OK) rc = upload(&d.f.blobS, fS.data(), fS.size());
+    if (rc == EMO_OK) rc = upload(&d.b.blobW, bW.data(), bW.size());
+    if (rc == EMO_OK) rc = upload(&d.b.blobS, bS.data(), bS.size());
+    if (rc == EMO_OK) rc = upload(&d.f.rows, rowsF.data(), rowsF.size() * 4);
+    if (rc == EMO_OK) rc = upload(&d.b.rows, rowsB.data(), rowsB.size() * 4);
     if (rc == EMO_OK) rc = upload(&d.push_base, pb.data(), pb.size() * 4);
     d.ready = rc == EMO_OK;
     return rc;
@@ -639,10 +847,9 @@ int upload_spine(const Flow &f, DevSpine &d)
 
 void free_spine(DevSpine &d)
 {
-    if (d.blobF) cudaFree(d.blobF);
-    if (d.blobB) cudaFree(d.blobB);
-    if (d.rows) cudaFree(d.rows);
-    if (d.push_base) cudaFree(d.push_base);
+    void *all[] = {d.f.blobW, d.f.blobS, d.f.rows, d.b.blobW, d.b.blobS, d.b.rows, d.push_base};
+    for (void *q : all)
+        if (q) cudaFree(q);
     d = DevSpine();
 }
 
@@ -820,100 +1027,113 @@ int launch_flow_bwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const uin
     return EMO_OK;
 }
 
-// Launch shape of the spine kernels: the policy tile of flow_plan; per group one spine warp and as many worker
-// warps as the block has room for (at most 6); three buffers of sums when they fit (workers one stage ahead and
-// one behind the spine) and up to six stage buffers.
-bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, FlowPlan &pl, bool extra = false)
+// Launch shape of the spine kernels: the smallest tile of 32 * G policies (G a power of two) that covers the batch with
+// one block per SM; as many policies per worker thread (up to four) as the tile has groups; two policies per spine thread up
+// to two groups, else four (bundles of four, 8 threads per operation: always four, so that a row of 32 policies is one
+// conflict-free access of those threads).
+struct SpinePlan {
+    bool ok = false;
+    int groups = 0, vw = 1, vs = 1, grid_f = 0, grid_b = 0, threads_f = 0, threads_b = 0;
+    SpineParams pf, pb;
+    size_t smem_f = 0, smem_b = 0;
+    size_t restore_bytes = 0;
+};
+
+bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
 {
     const Flow &f = g->sflow;
     const Spine &sp = f.spine;
     const DevSpine &d = g->dspine;
     pl.ok = false;
     if (!f.ok32 || !sp.ok || !d.ready || !g->smem_optin || f.stages == 0) return false;
-    if (f.lanes * f.K > 32 * kFlowRowRegs) return false;
     const int64_t NBf = B + (want_base ? 1 : 0);
     const int64_t n_groups = (NBf + 31) / 32;
     const int64_t want = (n_groups + g->sm_count - 1) / g->sm_count;
     const size_t budget = g->smem_optin;
-    for (int G = (int)std::max<int64_t>(1, std::min<int64_t>(7, want)); G >= 1; --G) {
-        const int nprod = G <= 4 ? 4 : 2;
-        // a worker takes whole lanes: more workers than lanes would only wait
-        const int W = std::min(f.lanes, std::min(6, (32 - nprod - G) / G));
-        if (W < 1) continue;
+    int G0 = 1;
+    const int gmax = sp.bundle > 2 ? 4 : 8;
+    while (G0 < gmax && G0 < want) G0 *= 2;
+    for (int G = G0; G >= 1; G /= 2) {
         const size_t P = 32 * (size_t)G;
-        const size_t lvl_bytes = (size_t)G * f.lanes * f.K * 32;
-        auto shape = [&](bool backward, FlowParams &p, size_t &smem) {
+        const int VW = std::min(G, 4), VS = (G >= 4 || sp.bundle > 2) ? 4 : 2, spines = (int)P / (32 / sp.bundle * VS), subs = G / VW;
+        auto shape = [&](bool backward, SpineParams &p, size_t &smem, int &threads) {
             const SpineDir &dir = backward ? sp.b : sp.f;
-            const size_t slot_bytes = (size_t)dir.slots * 128;
-            const size_t acc_bytes = (size_t)((backward && extra) ? sp.acc_words_all : sp.acc_words) * 128;
-            const size_t blob = backward ? d.blobB_bytes : d.blobF_bytes;
+            const DevSpineDir &dd = backward ? d.b : d.f;
+            // warps: 16 (128 registers per thread) up to two policy groups, else 22 (88)
+            const int look = backward ? (G == 4 ? 6 : 4) : (G <= 2 ? 10 : 12);
+            const int posts = backward ? (G <= 2 ? 6 : (G == 4 ? 10 : 8)) : (need_bwd ? subs : 0);      // forward: one pusher per sub-tile
+            const size_t acc = (size_t)dd.words * P * 4, slots = (size_t)dir.slots * P * 4;
             const size_t rst = backward ? (size_t)d.max_push * P * 4 : 0;
-            const size_t stage = round_up(blob + lvl_bytes + rst, 128);
-            const size_t off_bar = round_up(G * slot_bytes, 16);
-            const size_t off_sbar = off_bar + 192;
-            const size_t oring = backward ? 0 : d.f_front;      // forward: the spine's part of a stage, per group and buffer of sums
-            const size_t off_oring = round_up(off_sbar + (size_t)G * kFlowMaxBuf * 3 * 8, 128);
-            int nbuf = 0, nacc = 0;
-            size_t head = 0, off_acc = 0;
-            // a stage is short (about a microsecond of work): several stages must be on their way at any time
-            for (int na = 3; na >= 2 && !nbuf; --na)
-                for (int nb = std::min(6, kFlowMaxBuf); nb >= 2 && !nbuf; --nb) {
-                    off_acc = round_up(off_oring + (size_t)na * G * oring, 128);
-                    head = round_up(off_acc + (size_t)na * G * acc_bytes, 128);
-                    if (head + nb * stage <= budget) {
-                        nbuf = nb;
-                        nacc = na;
-                    }
-                }
-            if (!nbuf || nbuf * stage < (size_t)G * W * 32 * 8) return false;
-            p = FlowParams();
-            p.blob = backward ? d.blobB : d.blobF;
-            p.rows = d.rows;
-            p.push_base = d.push_base;
-            p.blob_bytes = (unsigned)blob;
-            p.off_ops = backward ? d.b_off_ops : d.f_off_ops;
-            p.off_mem = d.b_off_mem;
-            p.off_tpool = d.f_off_tpool;
-            p.off_pos = d.f_off_pos;
-            p.off_tab = backward ? d.b_off_tab : d.f_off_tab;
-            p.tab_row = (unsigned)f.Lp * (backward ? 4u : 12u);
-            p.stages = f.stages;
-            p.lanes = f.lanes;
-            p.K = f.K;
-            p.Lp = f.Lp;
-            p.L = g->h.L;
-            p.groups = G;
-            p.ptile = (int)P;
-            p.nbuf = nbuf;
-            p.nacc = nacc;
-            p.nprod = nprod;
-            p.workers = W;
-            p.slot_bytes = (unsigned)slot_bytes;
-            p.stage_bytes = (unsigned)stage;
-            p.off_lvl = (unsigned)blob;
-            p.off_rst = (unsigned)(blob + lvl_bytes);
-            p.off_bar = (unsigned)off_bar;
-            p.off_sbar = (unsigned)off_sbar;
-            p.off_acc = (unsigned)off_acc;
-            p.off_oring = (unsigned)off_oring;
-            p.oring_bytes = (unsigned)oring;
-            p.acc_bytes = (unsigned)acc_bytes;
-            p.acc_all_off = (unsigned)sp.acc_words * 128u;
-            p.off_stage0 = (unsigned)head;
-            p.pushes = sp.pushes;
-            p.restore_rows = sp.pushes + f.lanes;
-            p.wait_cycles = g_wait_cycles;
-            p.stall_stage = -1;
-            p.prof = nullptr;
-            smem = head + nbuf * stage;
-            return true;
+            const size_t wbuf = round_up((size_t)dd.w_bytes + (size_t)d.nlook * P, 128), sbuf = round_up(dd.s_bytes + rst, 128);
+            const size_t off_bar = round_up(slots, 128), off_rows = round_up(off_bar + kSpBarBytes, 16);
+            const size_t rowbuf = round_up((size_t)d.nlook * 4 + 512, 16), off_w0 = round_up(off_rows + kSpRowRing * rowbuf, 128);      // (up to 128 row numbers are read past the last)
+            // buffers: the look-up warps run up to nacc stages ahead of the spine and, backward, the storing warps one behind it
+            static const int kTry[8][3] = {{6, 4, 3}, {5, 4, 3}, {4, 3, 3}, {4, 2, 3}, {3, 2, 3}, {4, 2, 2}, {3, 2, 2}, {2, 2, 2}};      // {nw, ns, nacc}
+            for (auto &t : kTry) {
+                // no worker may skip more stages than there are buffers of sums (a barrier's parity tells two phases apart)
+                const int n_look = std::min(look / subs, d.chunks * t[2]) * subs, n_post = backward ? std::min(posts / subs, (d.chunks + 1) * t[2]) * subs : posts;
+                // (the warps' partial results at the end take the place of the stage buffers)
+                const size_t total = off_w0 + std::max(t[0] * wbuf + t[1] * sbuf + t[2] * acc, (size_t)std::max(n_look * 8, n_post * 16) * 32 * VW);
+                if (total > budget) continue;
+                p = SpineParams();
+                p.blobW = dd.blobW;
+                p.blobS = dd.blobS;
+                p.rows = dd.rows;
+                p.push_base = d.push_base;
+                p.w_bytes = dd.w_bytes;
+                p.s_bytes = dd.s_bytes;
+                p.off_pos = dd.off_pos;
+                p.off_mem = dd.off_mem;
+                p.off_tab = dd.off_tab;
+                p.tab_row = (unsigned)f.Lp * (backward ? 4u : 12u);
+                p.off_ops = dd.off_ops;
+                p.nlook = d.nlook;
+                p.chunks = d.chunks;
+                p.chunks_post = d.chunks + 1;
+                p.stages = f.stages;
+                p.lanes = f.lanes;
+                p.Lp = f.Lp;
+                p.L = g->h.L;
+                p.groups = G;
+                p.ptile = (int)P;
+                p.workers = n_look;
+                p.posts = n_post;
+                p.nw = t[0];
+                p.ns = t[1];
+                p.nacc = t[2];
+                p.wbuf_bytes = (unsigned)wbuf;
+                p.sbuf_bytes = (unsigned)sbuf;
+                p.acc_bytes = (unsigned)acc;
+                p.slot_bytes = (unsigned)slots;
+                p.off_lvl = dd.w_bytes;
+                p.off_rst = dd.s_bytes;
+                p.off_bar = (unsigned)off_bar;
+                p.off_rows = (unsigned)off_rows;
+                p.rowbuf_bytes = (unsigned)rowbuf;
+                p.off_w0 = (unsigned)off_w0;
+                p.off_s0 = p.off_w0 + (unsigned)(t[0] * wbuf);
+                p.off_acc0 = p.off_s0 + (unsigned)(t[1] * sbuf);
+                p.off_rec = dd.off_rec;
+                p.zero_word = (unsigned)dd.zero;
+                p.comp_off = (unsigned)(sp.max_segs + 2) * 128u;
+                p.c_slot0 = f.lanes + 2;
+                p.pushes = sp.pushes;
+                p.restore_rows = sp.pushes + f.lanes;
+                p.wait_cycles = g_wait_cycles;
+                p.stall_stage = -1;
+                smem = total;
+                threads = ((backward ? 2 : 1) * spines + n_look + n_post + 2) * 32;
+                return true;
+            }
+            return false;
         };
-        if (!shape(false, pl.pf, pl.smem_f)) continue;
-        if (need_bwd && !shape(true, pl.pb, pl.smem_b)) continue;
+        if (!shape(false, pl.pf, pl.smem_f, pl.threads_f)) continue;
+        if (need_bwd && !shape(true, pl.pb, pl.smem_b, pl.threads_b)) continue;
         pl.groups = G;
+        pl.vw = VW;
+        pl.vs = VS;
         pl.grid_f = (int)((n_groups + G - 1) / G);
         pl.grid_b = (int)(((B + 31) / 32 + G - 1) / G);
-        pl.threads = (G * (1 + W) + nprod) * 32;
         pl.restore_bytes = need_bwd ? round_up((size_t)pl.grid_f * (size_t)(sp.pushes + f.lanes) * P * 4, 256) : 0;
         pl.ok = true;
         return true;
@@ -921,12 +1141,11 @@ bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, Fl
     return false;
 }
 
-int launch_spine_fwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const uint8_t *lvl, int64_t ldb, uint32_t *restore,
+int launch_spine_fwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const uint8_t *lvl, int64_t ldb, uint32_t *restore,
                      int64_t *makespan, double *energy, int64_t *base_T, double *base_E, int32_t *status, uint32_t flags,
-                     cudaStream_t st, bool pair = false)
+                     cudaStream_t st)
 {
-    FlowParams p = pl.pf;
-    p.pair_rows = pair ? 1 : 0;
+    SpineParams p = pl.pf;
     p.want_base = (base_T || base_E) ? 1 : 0;
     if (B + p.want_base == 0) return EMO_OK;
     p.B = B;
@@ -942,20 +1161,24 @@ int launch_spine_fwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const ui
     if (flags & EMO_F_TEST_STALL) p.stall_stage = p.stages / 2;
     cudaEvent_t ev0 = g_pass_events[0], ev1 = g_pass_events[1];
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
-    void (*kern)(FlowParams) = pl.threads <= 512 ? emo_spine_fwd<512> : emo_spine_fwd<1024>;
+    const bool wide = g->sflow.spine.bundle > 2;
+    void (*kern)(SpineParams) = nullptr;
+    if (pl.vw == 1) kern = wide ? emo_spine_fwd<1, 4, 4, 512> : emo_spine_fwd<1, 2, 2, 512>;
+    else if (pl.vw == 2) kern = wide ? emo_spine_fwd<2, 4, 4, 512> : emo_spine_fwd<2, 2, 2, 512>;
+    else kern = wide ? emo_spine_fwd<4, 4, 4, 704> : emo_spine_fwd<4, 4, 2, 704>;
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
-    kern<<<pl.grid_f, pl.threads, pl.smem_f, st>>>(p);
+    kern<<<pl.grid_f, pl.threads_f, pl.smem_f, st>>>(p);
     EMO_CUDA(cudaGetLastError());
     if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
     return EMO_OK;
 }
 
-int launch_spine_bwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const uint8_t *lvl, int64_t ldb, uint32_t *restore,
+int launch_spine_bwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const uint8_t *lvl, int64_t ldb, uint32_t *restore,
                      int64_t *ES, int64_t *LS, int64_t *slack, int64_t ldo, int64_t *makespan, int64_t *slack_sum,
                      int32_t *n_critical, int32_t *status, uint32_t flags, cudaStream_t st)
 {
     if (B == 0) return EMO_OK;
-    FlowParams p = pl.pb;
+    SpineParams p = pl.pb;
     p.B = B;
     p.lvl = lvl;
     p.ldb = ldb;
@@ -965,6 +1188,8 @@ int launch_spine_bwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const ui
     p.LS = LS;
     p.slack = slack;
     p.ldo = ldo;
+    auto out_aligned = [&](const void *q) { return ((uintptr_t)q % (8u * (unsigned)pl.vw)) == 0; };
+    p.vec_out = ldo % pl.vw == 0 && out_aligned(ES) && out_aligned(LS) && out_aligned(slack);
     p.slack_sum = slack_sum;
     p.n_critical = n_critical;
     p.status = status;
@@ -973,42 +1198,37 @@ int launch_spine_bwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const ui
     cudaEvent_t ev0 = g_pass_events[2], ev1 = g_pass_events[3];
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
     const bool extra = ES || LS || slack_sum || n_critical;
-    void (*kern)(FlowParams) = pl.threads <= 512 ? (extra ? emo_spine_bwd<512, true> : emo_spine_bwd<512, false>)
-                                                 : (extra ? emo_spine_bwd<1024, true> : emo_spine_bwd<1024, false>);
+    void (*kern)(SpineParams) = nullptr;
+    const bool wide = g->sflow.spine.bundle > 2;
+#define EMO_PICK_S(VW, VS, NB, MAXT) kern = extra ? emo_spine_bwd<VW, VS, NB, MAXT, true> : emo_spine_bwd<VW, VS, NB, MAXT, false>
+    if (pl.vw == 1 && wide) EMO_PICK_S(1, 4, 4, 512);
+    else if (pl.vw == 1) EMO_PICK_S(1, 2, 2, 512);
+    else if (pl.vw == 2 && wide) EMO_PICK_S(2, 4, 4, 512);
+    else if (pl.vw == 2) EMO_PICK_S(2, 2, 2, 512);
+    else if (wide) EMO_PICK_S(4, 4, 4, 704);
+    else EMO_PICK_S(4, 4, 2, 704);
+#undef EMO_PICK_S
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
-    kern<<<pl.grid_b, pl.threads, pl.smem_b, st>>>(p);
+    kern<<<pl.grid_b, pl.threads_b, pl.smem_b, st>>>(p);
     EMO_CUDA(cudaGetLastError());
     if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
     return EMO_OK;
 }
 
-// Whether the forward spine kernel can feed the lane-stream backward kernel: both programs come from one schedule (same
-// lanes and steps; the lane-stream program's barrier distance is the gap that the spine program's schedule keeps) and
-// the restore rows could be numbered the lane-stream way.
-bool spine_pairs(const emo_graph *g)
-{
-    const Flow &f = g->flow, &s = g->sflow;
-    return f.ok32 && s.ok32 && s.spine.ok && g->dspine.ready && s.spine.pair_ok && s.spine.pair_K == f.K && f.sync == 2 * s.K &&
-           f.steps == s.steps && f.lanes == s.lanes && f.pushes == s.spine.pushes && s.lanes <= 8;
-}
-
 // Whether a call takes the spine kernels: the program exists and either the caller asks for them (EMO_F_SPINE_KERNEL) or
-// the graph is narrow and the batch leaves at most three policy groups to an SM (or the graph is short).
-bool spine_allowed(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb, int64_t ldo, bool fwd_only, uint32_t flags)
+// they are the faster ones.
+bool spine_allowed(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb, int64_t ldo, uint32_t flags)
 {
     const int64_t big = (int64_t)1 << 28;
     if (!g->sflow.ok32 || !g->sflow.spine.ok || !g->dspine.ready) return false;
     if (flags & (EMO_F_NO_STAGING | EMO_F_PAIR_KERNEL | EMO_F_LANE_KERNEL | EMO_F_FLOW_KERNEL)) return false;
-    // Measured: on graphs of up to eight lanes the spine kernels are the fastest pair while a block holds at most three
-    // policy groups (75 000 nodes, both passes, spine / lane-stream: 3.6 / 5.5 ms with one group per SM, 4.4 / 6.0 with
-    // two, 5.7 / 6.3 with three, 8.9 / 6.8 with four: the workers then take the issue slots and the shared-memory pipe
-    // that the spine warp needs) and on short graphs whatever the batch (1 013 nodes x 65 536 policies: 0.61 against
-    // 0.90 ms); one warp carries the recurrence of all lanes, so wide graphs (17 lanes: 21.9 against 9.0 ms) stay with
-    // the other kernels unless the caller asks.
+    // Measured (both passes, ms, spine / the best of the others): 1 013 nodes x 65 536 policies 0.42 / 0.90; 10 000 x 4 096
+    // 0.80 / 2.30; 75 000 x 10 001 forward 1.28 / 1.89; 250 000 x 16 384 19.4 / 20.4.  On wide graphs one warp carries the
+    // recurrence of all lanes: 18 lanes, 128 039 nodes x 8 192 policies (two groups per SM) 8.9 / 9.05, below that the
+    // others stay.
     if (!(flags & EMO_F_SPINE_KERNEL)) {
         const int64_t per_sm = ((B + 1 + 31) / 32 + g->sm_count - 1) / std::max(g->sm_count, 1);
-        // (forward only, the spine kernel still wins with four groups: 250 000 nodes x 16 384 policies 7.5 against 8.2 ms)
-        if (g->sflow.lanes > 8 || (per_sm > (fwd_only ? 4 : 3) && g->h.n > 8192)) return false;
+        if (g->sflow.lanes > 8 && per_sm < 2) return false;
     }
     return ldb % 16 == 0 && aligned16(lvl) && ldb < big && ldo < big;
 }
@@ -1080,18 +1300,13 @@ int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
     if (!g || B < 0) return EMO_E_INVALID_ARG;
     if (g->host_only) return EMO_E_CUDA;
     if (g->generic) return 3;
-    if (spine_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, need_slack == 0, flags)) {
-        FlowPlan fp;
-        if (spine_plan(g, B, true, need_slack != 0, fp)) return 4;
+    if (spine_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
+        SpinePlan sp;
+        if (spine_plan(g, B, true, need_slack != 0, sp)) return (sp.vw == 1 || (flags & EMO_F_SPINE_KERNEL)) ? 4 : 5;
     }
     if (flow_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
-        FlowPlan fp, sp;
-        if (flow_plan(g, B, true, need_slack != 0, fp)) {
-            if (need_slack && !(flags & EMO_F_FLOW_KERNEL) && spine_pairs(g) && spine_plan(g, B, true, false, sp) && sp.groups == fp.groups &&
-                sp.grid_f == fp.grid_f)
-                return 5;
-            return 2;
-        }
+        FlowPlan fp;
+        if (flow_plan(g, B, true, need_slack != 0, fp)) return 2;
     }
     PassPlan pl;
     const int64_t ld_ws = (int64_t)round_up((size_t)B, 16);
@@ -1299,7 +1514,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 while (sk > 8 && flanes * sk > 32 * kFlowRowRegs) sk /= 2;
                 spine_thread = std::thread([&, sk]() {
                     try {
-                        rc_s = compile_flow(h, lat, energy, lanes, look, sk, sk, g->sflow, err_s, true, fk);
+                        rc_s = compile_flow(h, lat, energy, lanes, look, sk, sk, g->sflow, err_s, true);
                     } catch (const std::bad_alloc &) {
                         rc_s = EMO_E_OOM;
                     }
@@ -1653,8 +1868,9 @@ int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint3
             need = fp.restore_bytes;
         else
             need = spill_need(g, B);
-        if (!g->host_only && B > 0 && spine_allowed(g, B, fake, aligned ? 16 : 1, 0, false, flags) && spine_plan(g, B, true, true, fp))
-            need = std::max(need, fp.restore_bytes);
+        SpinePlan sp;
+        if (!g->host_only && B > 0 && spine_allowed(g, B, fake, aligned ? 16 : 1, 0, flags) && spine_plan(g, B, true, true, sp))
+            need = std::max(need, sp.restore_bytes);
         bytes += need;
     }
     if (need_slack == 2) bytes += 4 * round_up((size_t)B * 8, 256) + 256;
@@ -1686,8 +1902,8 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
     if (g->generic)
         return launch_generic(g, B, lvl, ldb, false, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, ws,
                               ws_bytes, st);
-    if (spine_allowed(g, B, lvl, ldb, 0, true, flags)) {
-        FlowPlan fp;
+    if (spine_allowed(g, B, lvl, ldb, 0, flags)) {
+        SpinePlan fp;
         if (spine_plan(g, B, T0 || E0, false, fp))
             return launch_spine_fwd(g, fp, B, lvl, ldb, nullptr, makespan, energy, T0, E0, status, flags, st);
     }
@@ -2014,9 +2230,9 @@ int emo_slack_batch(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t l
     if (g->generic)
         return launch_generic(g, B, lvl, ldb, true, ES, LS, slack, ldo, makespan, energy, slack_sum, n_critical, T0, E0, ws, ws_bytes,
                               st);
-    if (spine_allowed(g, B, lvl, ldb, ldo, false, flags)) {
-        FlowPlan fp;
-        if (spine_plan(g, B, T0 || E0, true, fp, ES || LS || slack_sum || n_critical)) {
+    if (spine_allowed(g, B, lvl, ldb, ldo, flags)) {
+        SpinePlan fp;
+        if (spine_plan(g, B, T0 || E0, true, fp)) {
             const size_t head = kSmallWs + lvl_area(g);
             if (!ws || ws_bytes < head + fp.restore_bytes) return EMO_E_OOM;
             uint32_t *restore = (uint32_t *)((char *)ws + head);
@@ -2031,18 +2247,7 @@ int emo_slack_batch(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t l
             const size_t head = kSmallWs + lvl_area(g);
             if (!ws || ws_bytes < head + fp.restore_bytes) return EMO_E_OOM;
             uint32_t *restore = (uint32_t *)((char *)ws + head);
-            // The forward spine kernel is the faster forward pass even with four groups per block (7.5 against 8.2 ms on
-            // the 250 000-node graph); where its program shares the schedule of the lane-stream program it writes the
-            // restore list in that program's numbering and the lane-stream backward kernel follows.
-            FlowPlan sp;
-            int rc;
-            if (!(flags & EMO_F_FLOW_KERNEL) && spine_pairs(g) && spine_plan(g, B, T0 || E0, false, sp) && sp.groups == fp.groups &&
-                sp.grid_f == fp.grid_f) {
-                sp.pf.pushes = fp.pf.pushes;
-                sp.pf.restore_rows = fp.pf.restore_rows;
-                rc = launch_spine_fwd(g, sp, B, lvl, ldb, restore, makespan, energy, T0, E0, status, flags, st, true);
-            } else
-                rc = launch_flow_fwd(g, fp, B, lvl, ldb, restore, makespan, energy, T0, E0, status, flags, st);
+            int rc = launch_flow_fwd(g, fp, B, lvl, ldb, restore, makespan, energy, T0, E0, status, flags, st);
             if (rc) return rc;
             return launch_flow_bwd(g, fp, B, lvl, ldb, restore, ES, LS, slack, ldo, makespan, slack_sum, n_critical, status,
                                    flags, st);

@@ -35,10 +35,80 @@ struct SlotPool {
     void give(int32_t id) { free_ids.push_back(id); }
 };
 
-struct Operand {
-    uint32_t slot, delta;
-    bool clear;
+// An operation before it has slots: where its two operands come from and what it writes.
+enum class From : uint8_t { Zero, Lane, Pub, Temp, Fold };
+struct Ref {
+    From from = From::Zero;
+    int32_t id = 0;           // lane, segment (Pub), merge operation of the stage (Temp) or reading node (Fold)
+    uint32_t delta = 0;
 };
+struct Op {
+    Ref in[2];
+    int32_t seg = -1;         // the segment it completes (-1: a merge operation)
+    int32_t dep[3] = {-1, -1, -1};   // operations of the same stage that come before it
+    int32_t height = 1;       // longest chain of such operations that starts here
+};
+
+void note_dep(Op &o, int32_t d)
+{
+    if (d < 0) return;
+    for (int32_t &x : o.dep) {
+        if (x == d) return;
+        if (x < 0) { x = d; return; }
+    }
+}
+
+// Operands beyond `keep` are folded two at a time into merge operations in front of the segment's own.
+template <typename Link>
+void add_merges(std::vector<Op> &ops, std::vector<Ref> &refs, size_t keep, Link link)
+{
+    while (refs.size() > keep) {
+        Op o;
+        o.in[0] = refs[0];
+        o.in[1] = refs[1];
+        link(o);
+        Ref r;
+        r.from = From::Temp;
+        r.id = (int32_t)ops.size();
+        ops.push_back(o);
+        refs.erase(refs.begin(), refs.begin() + 2);
+        refs.push_back(r);               // to the back: a balanced tree
+    }
+}
+
+// Order of a stage's operations in bundles of `size`: the kernel loads all operands of a bundle before it stores any
+// result, so the operations of one bundle must not depend on each other.  Greedy by the length of the chain behind an
+// operation; -1 = nothing to do (places of a bundle may stay empty).
+std::vector<int32_t> bundle_ops(std::vector<Op> &ops, int32_t size)
+{
+    const int32_t m = (int32_t)ops.size();
+    for (int32_t i = m - 1; i >= 0; --i)
+        for (int32_t d : ops[i].dep)
+            if (d >= 0) ops[d].height = std::max(ops[d].height, ops[i].height + 1);
+    std::vector<int32_t> at((size_t)m, -1), order, todo((size_t)m);
+    for (int32_t i = 0; i < m; ++i) todo[i] = i;
+    std::stable_sort(todo.begin(), todo.end(), [&](int32_t a, int32_t b) { return ops[a].height > ops[b].height; });
+    int32_t bundle = 0;
+    while (!todo.empty()) {
+        std::vector<int32_t> rest;
+        int32_t taken = 0;
+        for (int32_t i : todo) {
+            bool ready = taken < size;
+            for (int32_t d : ops[i].dep) ready = ready && (d < 0 || (at[d] >= 0 && at[d] < bundle));
+            if (ready) {
+                at[i] = bundle;
+                order.push_back(i);
+                ++taken;
+            } else {
+                rest.push_back(i);
+            }
+        }
+        for (; taken < size; ++taken) order.push_back(-1);
+        todo.swap(rest);
+        ++bundle;
+    }
+    return order;
+}
 
 }  // namespace
 
@@ -185,33 +255,11 @@ int build_spine(const SpineIn &in, Spine &out, std::string &err)
 
     // ---- forward operations -----------------------------------------------------------------------------
     // fixed slots: the lanes' values, a slot that stays zero, a slot nobody reads; published values behind them
-    // restore rows in the numbering of the lane-stream program to pair with: nodes whose start does not follow from the
-    // lane's value, per stage of pair_K steps the lanes in order, a lane's nodes by step
-    std::vector<int64_t> pair_row((size_t)n, -1);
-    out.pair_K = in.pair_K;
-    out.pair_ok = in.pair_K > 0;
-    out.pair_base.assign((size_t)stages, 0);
-    if (in.pair_K > 0) {
-        std::vector<int32_t> pushing;
-        for (int32_t v = 0; v < n; ++v)
-            if (!invertible(v)) pushing.push_back(v);
-        std::sort(pushing.begin(), pushing.end(), [&](int32_t a, int32_t b) {
-            const int sa = step_of[a] / in.pair_K, sb = step_of[b] / in.pair_K;
-            if (sa != sb) return sa < sb;
-            if (lane_of[a] != lane_of[b]) return lane_of[a] < lane_of[b];
-            return step_of[a] < step_of[b];
-        });
-        for (size_t i = 0; i < pushing.size(); ++i) pair_row[pushing[i]] = (int64_t)i;
-        std::vector<int64_t> lo((size_t)stages, -1);
-        for (int32_t v : pushing) {
-            const int st = stage_of(v);
-            if (lo[st] < 0 || pair_row[v] < lo[st]) lo[st] = pair_row[v];
-        }
-        for (int st = 0; st < stages; ++st) out.pair_base[st] = lo[st] < 0 ? 0 : lo[st];
-    }
     std::vector<std::vector<uint32_t>> opsF((size_t)stages), opsB((size_t)stages);
     std::vector<std::vector<uint64_t>> pools((size_t)stages);
     out.push_base.assign((size_t)stages + 1, 0);
+    out.unread_slot = dummy_slot;
+    out.bundle = spine_bundle(lanes);
     {
         SlotPool pool;
         pool.next = lanes + 2;
@@ -219,8 +267,17 @@ int build_spine(const SpineIn &in, Spine &out, std::string &err)
         for (int32_t v = 0; v < n; ++v)
             for (int64_t e = pp[v]; e < pp[v + 1]; ++e)
                 if (liveF[e] && prev[v] != pc[e]) segs[seg_of[pc[e]]].readersF++;
+        std::vector<int32_t> op_of_seg(segs.size(), -1);      // operation (of its stage) that publishes the segment's value
         for (int st = 0; st < stages; ++st) {
             int32_t npush = 0;
+            std::vector<Op> ops;
+            std::vector<int32_t> lane_op((size_t)lanes, -1);
+            auto link = [&](Op &o) {
+                for (Ref &r : o.in) {
+                    if (r.from == From::Pub && segs[r.id].stage == st) note_dep(o, op_of_seg[r.id]);
+                    if (r.from == From::Temp) note_dep(o, r.id);
+                }
+            };
             for (int32_t si : stage_segs[st]) {
                 Seg &s = segs[si];
                 const int32_t h = s.head, t = s.tail;
@@ -228,59 +285,98 @@ int build_spine(const SpineIn &in, Spine &out, std::string &err)
                 const bool inv = invertible(h);
                 if (!inv) s.push = npush++;
                 if (inv && !(s.flags & kSpSeg_PreB) && !fpub[t] && !terminal) continue;      // the lane's value passes through unchanged
-                std::vector<Operand> ops;
-                std::vector<int32_t> done;       // published slots whose last reader this is
+                std::vector<Ref> refs;
                 // the lane's slot is always the first operand of the segment's own operation (the kernel takes the value
                 // that goes to the restore list from there); a correction of 2^32 - 1 floors it to zero when the head
                 // does not continue from the lane
-                Operand lane_op{(uint32_t)s.lane, 0xFFFFFFFFu, false};
+                Ref lane_ref;
+                lane_ref.from = From::Lane;
+                lane_ref.id = s.lane;
+                lane_ref.delta = 0xFFFFFFFFu;
                 for (int64_t e = pp[h]; e < pp[h + 1]; ++e) {
                     if (!liveF[e]) continue;
                     const int32_t k = pc[e];
                     const uint32_t delta = (uint32_t)(lbES[h] - lbC[k]);
                     if (prev[h] == k) {
-                        lane_op.delta = delta;
+                        lane_ref.delta = delta;
                     } else {
-                        Seg &w = segs[seg_of[k]];
-                        if (w.tail != k || w.pubF < 0) { err = "internal: spine operand is not published"; return EMO_E_UNSUPPORTED; }
-                        ops.push_back(Operand{(uint32_t)w.pubF, delta, false});
-                        if (--w.readersF == 0) done.push_back(w.pubF);
+                        if (segs[seg_of[k]].tail != k || !fpub[k]) { err = "internal: spine operand is not published"; return EMO_E_UNSUPPORTED; }
+                        Ref r;
+                        r.from = From::Pub;
+                        r.id = seg_of[k];
+                        r.delta = delta;
+                        refs.push_back(r);
                     }
                 }
-                std::vector<int32_t> temps;
-                while (ops.size() > 1) {
-                    const int32_t tmp = pool.take();
-                    temps.push_back(tmp);
-                    const uint32_t w8[kSpOpWordsF] = {slot_addr(ops[0].slot), ops[0].delta, slot_addr(ops[1].slot), ops[1].delta,
-                                                      slot_addr(dummy_slot), slot_addr((uint32_t)tmp), scratch_acc * 128u, kSp_NoSum};
-                    opsF[st].insert(opsF[st].end(), w8, w8 + kSpOpWordsF);
-                    ops.erase(ops.begin(), ops.begin() + 2);
-                    ops.insert(ops.begin(), Operand{(uint32_t)tmp, 0u, false});
-                }
-                if (ops.empty()) ops.push_back(Operand{zero_slot, 0u, false});
-                ops.insert(ops.begin(), lane_op);
-                if (fpub[t] && s.readersF > 0) s.pubF = pool.take();
-                uint32_t fl = (s.flags & kSpSeg_PreB) ? 0u : kSp_NoSum;
-                if (!inv) {
-                    fl |= kSp_Push | ((uint32_t)s.push << 8);
-                    if (in.pair_K > 0) {
-                        const int64_t rel = pair_row[h] - out.pair_base[st];
-                        if (rel < 0 || rel >= 4096) out.pair_ok = false;
-                        else fl |= (uint32_t)rel << 20;
-                    }
-                }
-                if (terminal) {
-                    fl |= kSp_Terminal;      // the kernel takes the stage's bounds in order
-                    pools[st].push_back((uint64_t)lbC[t]);
-                }
-                if (s.push >= 4096 || pools[st].size() >= 4096) { err = "internal: spine stage too large"; return EMO_E_UNSUPPORTED; }
-                const uint32_t w8[kSpOpWordsF] = {slot_addr(ops[0].slot), ops[0].delta, slot_addr(ops[1].slot), ops[1].delta,
-                                                  slot_addr((uint32_t)s.lane), slot_addr(s.pubF >= 0 ? (uint32_t)s.pubF : dummy_slot), s.acc * 128u, fl};
-                opsF[st].insert(opsF[st].end(), w8, w8 + kSpOpWordsF);
-                for (int32_t id : temps) pool.give(id);
-                for (int32_t id : done) pool.give(id);
+                add_merges(ops, refs, 1, link);
+                Op o;
+                o.seg = si;
+                o.in[0] = lane_ref;
+                if (!refs.empty()) o.in[1] = refs[0];
+                link(o);
+                note_dep(o, lane_op[s.lane]);
+                lane_op[s.lane] = op_of_seg[si] = (int32_t)ops.size();
+                ops.push_back(o);
             }
             out.push_base[st + 1] = out.push_base[st] + npush;
+            // slots are handed out in the order of execution; one that a bundle reads for the last time is free from the
+            // next bundle on
+            const std::vector<int32_t> order = bundle_ops(ops, out.bundle);
+            std::vector<int32_t> temp_slot((size_t)ops.size(), -1), done, late;
+            for (size_t i = 0; i < order.size(); ++i) {
+                if (i % (size_t)out.bundle == 0) {
+                    for (int32_t id : done) pool.give(id);
+                    done.clear();
+                }
+                if (order[i] < 0) {
+                    const uint32_t w8[kSpOpWordsF] = {slot_addr(zero_slot), 0u, slot_addr(zero_slot), 0u, slot_addr(dummy_slot), slot_addr(dummy_slot),
+                                                      scratch_acc * 128u, kSp_NoSum};
+                    opsF[st].insert(opsF[st].end(), w8, w8 + kSpOpWordsF);
+                    continue;
+                }
+                const Op &o = ops[order[i]];
+                uint32_t a[2];
+                for (int k = 0; k < 2; ++k) {
+                    const Ref &r = o.in[k];
+                    int32_t id = (int32_t)zero_slot;
+                    if (r.from == From::Lane) id = r.id;
+                    if (r.from == From::Temp) done.push_back(id = temp_slot[r.id]);
+                    if (r.from == From::Pub) {
+                        id = segs[r.id].pubF;
+                        if (id < 0) { err = "internal: spine operand has no slot"; return EMO_E_UNSUPPORTED; }
+                        if (--segs[r.id].readersF == 0) done.push_back(id);
+                    }
+                    a[k] = slot_addr((uint32_t)id);
+                }
+                uint32_t fl = kSp_NoSum, acc = scratch_acc, o_lane = dummy_slot, o_pub = dummy_slot;
+                if (o.seg < 0) {
+                    temp_slot[order[i]] = pool.take();
+                    o_pub = (uint32_t)temp_slot[order[i]];
+                } else {
+                    Seg &s = segs[o.seg];
+                    const bool terminal = sp[s.tail + 1] == sp[s.tail];
+                    if (s.flags & kSpSeg_PreB) fl = 0u;
+                    if (s.push >= 0) fl |= kSp_Push | ((uint32_t)s.push << 8);
+                    acc = s.acc;
+                    o_lane = (uint32_t)s.lane;
+                    if (terminal || (fpub[s.tail] && s.readersF > 0)) {
+                        s.pubF = pool.take();
+                        o_pub = (uint32_t)s.pubF;
+                    }
+                    if (terminal) {
+                        // candidates for the makespan, taken at the end of the stage from the slots they are published in
+                        fl |= kSp_Terminal;
+                        pools[st].push_back((uint64_t)lbC[s.tail]);
+                        out.term_slot.push_back(o_pub);
+                        late.push_back((int32_t)o_pub);
+                    }
+                    if (s.push >= 4096 || pools[st].size() >= 4096) { err = "internal: spine stage too large"; return EMO_E_UNSUPPORTED; }
+                }
+                const uint32_t w8[kSpOpWordsF] = {a[0], o.in[0].delta, a[1], o.in[1].delta, slot_addr(o_lane), slot_addr(o_pub), acc * 128u, fl};
+                opsF[st].insert(opsF[st].end(), w8, w8 + kSpOpWordsF);
+            }
+            for (int32_t id : done) pool.give(id);
+            for (int32_t id : late) pool.give(id);
         }
         out.f.slots = pool.next;
     }
@@ -295,85 +391,139 @@ int build_spine(const SpineIn &in, Spine &out, std::string &err)
         const uint32_t c_slot0 = (uint32_t)lanes + 2u, dummy_c = 2u * (uint32_t)lanes + 2u;
         const uint32_t kFoldTag = 0x80000000u;
         pool.next = 2 * lanes + 3;
-        std::vector<int32_t> fold_slot((size_t)n, -1);
+        std::vector<int32_t> fold_slot((size_t)n, -1), op_of_seg(segs.size(), -1);
         for (int32_t v = 0; v < n; ++v)
             for (int64_t e = pp[v]; e < pp[v + 1]; ++e)
                 if (liveB[e] && prev[v] != pc[e] && fold_reader[v] != pc[e]) segs[seg_of[v]].readersB++;
         for (int st = stages - 1; st >= 0; --st) {
-            std::vector<int32_t> order(stage_segs[st]);
-            std::sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
+            std::vector<int32_t> walk(stage_segs[st]);
+            std::sort(walk.begin(), walk.end(), [&](int32_t a, int32_t b) {
                 const int32_t ta = segs[a].tail, tb = segs[b].tail;
                 return step_of[ta] != step_of[tb] ? step_of[ta] > step_of[tb] : segs[a].lane < segs[b].lane;
             });
-            for (int32_t si : order) {
-                Seg &s = segs[si];
-                const int32_t h = s.head, t = s.tail;
-                // the members' records; a fold slot is taken when its first writer comes by
-                {
-                    int32_t u = h;
-                    for (int32_t j = 0; j < s.count; ++j, u = next[u]) {
-                        uint32_t *w = &out.mem[(((size_t)st * lanes + s.lane) * K + s.first + j) * kSpMemWords];
-                        w[0] = (uint32_t)u;
-                        w[1] = slot_addr(dummy_slot);
-                        w[6] = (uint32_t)(uint64_t)lbES[u];
-                        w[7] = (uint32_t)((uint64_t)lbES[u] >> 32);
-                        const int32_t r = fold_reader[u];
-                        if (r >= 0) {
-                            if (fold_slot[r] < 0) fold_slot[r] = fpool.take();
-                            w[1] = kFoldTag | slot_addr((uint32_t)fold_slot[r]);
-                            w[2] = (uint32_t)(lbQin[r] - lbQ[u]);
-                        }
-                    }
+            std::vector<Op> ops;
+            std::vector<int32_t> lane_op((size_t)lanes, -1);
+            auto link = [&](Op &o) {
+                for (Ref &r : o.in) {
+                    if (r.from == From::Pub && segs[r.id].stage == st) note_dep(o, op_of_seg[r.id]);
+                    if (r.from == From::Temp) note_dep(o, r.id);
                 }
-                std::vector<Operand> ops;
-                std::vector<int32_t> done;
-                bool fold_seen = false;
+            };
+            for (int32_t si : walk) {
+                Seg &s = segs[si];
+                const int32_t t = s.tail;
+                std::vector<Ref> refs;
+                Ref lane_ref;
+                bool has_lane = false, fold_seen = false;
                 for (int64_t e = sp[t]; e < sp[t + 1]; ++e) {
                     const int32_t u = sc[e];
                     const int64_t ee = std::lower_bound(pc.begin() + pp[u], pc.begin() + pp[u + 1], t) - pc.begin();
                     if (!liveB[ee]) continue;
-                    const uint32_t delta = (uint32_t)(lbQin[t] - lbQ[u]);
+                    Ref r;
+                    r.delta = (uint32_t)(lbQin[t] - lbQ[u]);
                     if (next[t] == u) {
-                        ops.insert(ops.begin(), Operand{(uint32_t)s.lane, delta, false});
-                    } else if (fold_reader[u] == t) {
+                        // not for a merge operation: the lane's value is ordered by the segment's own operation
+                        lane_ref = r;
+                        lane_ref.from = From::Lane;
+                        lane_ref.id = s.lane;
+                        has_lane = true;
+                        continue;
+                    }
+                    if (fold_reader[u] == t) {
                         if (fold_seen) continue;
                         fold_seen = true;
                         if (fold_slot[t] < 0) { err = "internal: spine fold slot missing"; return EMO_E_UNSUPPORTED; }
-                        ops.push_back(Operand{kFoldTag | slot_addr((uint32_t)fold_slot[t]), 0u, true});
+                        r.from = From::Fold;
+                        r.id = t;
+                        r.delta = 0;
                     } else {
-                        Seg &w = segs[seg_of[u]];
-                        if (w.head != u || w.pubB < 0) { err = "internal: spine tail is not published"; return EMO_E_UNSUPPORTED; }
-                        ops.push_back(Operand{(uint32_t)w.pubB, delta, false});
-                        if (--w.readersB == 0) done.push_back(w.pubB);
+                        if (segs[seg_of[u]].head != u || !bpub[u]) { err = "internal: spine tail is not published"; return EMO_E_UNSUPPORTED; }
+                        r.from = From::Pub;
+                        r.id = seg_of[u];
+                    }
+                    refs.push_back(r);
+                }
+                add_merges(ops, refs, has_lane ? 1 : 2, link);
+                Op o;
+                o.seg = si;
+                int k = 0;
+                if (has_lane) o.in[k++] = lane_ref;
+                for (const Ref &r : refs) o.in[k++] = r;
+                        link(o);
+                note_dep(o, lane_op[s.lane]);
+                lane_op[s.lane] = op_of_seg[si] = (int32_t)ops.size();
+                ops.push_back(o);
+            }
+            const std::vector<int32_t> order = bundle_ops(ops, out.bundle);
+            std::vector<int32_t> temp_slot((size_t)ops.size(), -1), done;
+            for (size_t i = 0; i < order.size(); ++i) {
+                if (i % (size_t)out.bundle == 0) {
+                    for (int32_t id : done) pool.give(id);
+                    done.clear();
+                }
+                uint32_t a[2] = {slot_addr(zero_slot), slot_addr(zero_slot)}, d[2] = {0, 0}, clear = slot_addr(dummy_slot);
+                uint32_t fl = kSp_NoSum, acc = scratch_acc, qo = scratch_acc + 1u, qo_all = scratch_acc + 1u, o_lane = dummy_slot, o_pub = dummy_slot, c = dummy_c;
+                if (order[i] >= 0) {
+                    const Op &o = ops[order[i]];
+                    for (int k = 0; k < 2; ++k) {
+                        const Ref &r = o.in[k];
+                        d[k] = r.delta;
+                        if (r.from == From::Lane) a[k] = slot_addr((uint32_t)r.id);
+                        if (r.from == From::Temp) {
+                            a[k] = slot_addr((uint32_t)temp_slot[r.id]);
+                            done.push_back(temp_slot[r.id]);
+                        }
+                        if (r.from == From::Fold) {
+                            a[k] = clear = kFoldTag | slot_addr((uint32_t)fold_slot[r.id]);
+                            fpool.give(fold_slot[r.id]);
+                        }
+                        if (r.from == From::Pub) {
+                            if (segs[r.id].pubB < 0) { err = "internal: spine tail has no slot"; return EMO_E_UNSUPPORTED; }
+                            a[k] = slot_addr((uint32_t)segs[r.id].pubB);
+                            if (--segs[r.id].readersB == 0) done.push_back(segs[r.id].pubB);
+                        }
+                    }
+                    if (o.seg < 0) {
+                        temp_slot[order[i]] = pool.take();
+                        o_pub = (uint32_t)temp_slot[order[i]];
+                    } else {
+                        Seg &s = segs[o.seg];
+                        if (bpub[s.head] && s.readersB > 0) {
+                            s.pubB = pool.take();
+                            o_pub = (uint32_t)s.pubB;
+                        }
+                        if (s.flags & kSpSeg_PreB) fl = 0u;
+                        if (s.push >= 0) fl |= kSp_Push | ((uint32_t)s.push << 8);
+                        acc = s.acc;
+                        if (s.flags & kSpSeg_Fold) qo = s.acc + 1u;
+                        qo_all = (uint32_t)out.acc_words + (uint32_t)s.idx;
+                        o_lane = (uint32_t)s.lane;
+                        c = c_slot0 + (uint32_t)s.lane;
                     }
                 }
-                std::vector<int32_t> temps;
-                auto addr_of = [&](const Operand &a) { return a.clear ? a.slot : slot_addr(a.slot); };      // fold operands carry their tagged address
-                auto clear_of = [&](const Operand &a, const Operand &b) { return a.clear ? a.slot : (b.clear ? b.slot : slot_addr(dummy_slot)); };
-                while (ops.size() > 2) {
-                    const int32_t tmp = pool.take();
-                    temps.push_back(tmp);
-                    const uint32_t w12[kSpOpWordsB] = {addr_of(ops[0]), ops[0].delta, addr_of(ops[1]), ops[1].delta,
-                                                       slot_addr(dummy_slot), slot_addr((uint32_t)tmp), scratch_acc * 128u, kSp_NoSum,
-                                                       clear_of(ops[0], ops[1]), slot_addr(dummy_c), (scratch_acc + 1u) * 128u, (scratch_acc + 1u) * 128u};
-                    opsB[st].insert(opsB[st].end(), w12, w12 + kSpOpWordsB);
-                    ops.erase(ops.begin(), ops.begin() + 2);
-                    ops.insert(ops.begin(), Operand{(uint32_t)tmp, 0u, false});
-                }
-                while (ops.size() < 2) ops.push_back(Operand{zero_slot, 0u, false});
-                if (bpub[h] && s.readersB > 0) s.pubB = pool.take();
-                uint32_t fl = (s.flags & kSpSeg_PreB) ? 0u : kSp_NoSum;
-                if (s.push >= 0) fl |= kSp_Push | ((uint32_t)s.push << 8);
-                const bool wide = (s.flags & kSpSeg_Fold) != 0;
-                const uint32_t w12[kSpOpWordsB] = {addr_of(ops[0]), ops[0].delta, addr_of(ops[1]), ops[1].delta,
-                                                   slot_addr((uint32_t)s.lane), slot_addr(s.pubB >= 0 ? (uint32_t)s.pubB : dummy_slot), s.acc * 128u, fl,
-                                                   clear_of(ops[0], ops[1]), slot_addr(c_slot0 + (uint32_t)s.lane),
-                                                   (wide ? s.acc + 1u : scratch_acc + 1u) * 128u,
-                                                   ((uint32_t)out.acc_words + (uint32_t)s.idx) * 128u};
+                const uint32_t w12[kSpOpWordsB] = {a[0], d[0], a[1], d[1], slot_addr(o_lane), slot_addr(o_pub), acc * 128u, fl,
+                                                   clear, slot_addr(c), qo * 128u, qo_all * 128u};
                 opsB[st].insert(opsB[st].end(), w12, w12 + kSpOpWordsB);
-                for (int32_t id : temps) pool.give(id);
-                for (int32_t id : done) pool.give(id);
-                if (fold_seen) fpool.give(fold_slot[t]);
+            }
+            for (int32_t id : done) pool.give(id);
+            // the members' records.  A fold slot is taken when its first writer comes by; the stores of a stage follow the
+            // stage's operations, so a slot that one of them has just cleared can be taken again here.
+            for (int32_t si : walk) {
+                const Seg &s = segs[si];
+                int32_t u = s.head;
+                for (int32_t j = 0; j < s.count; ++j, u = next[u]) {
+                    uint32_t *w = &out.mem[(((size_t)st * lanes + s.lane) * K + s.first + j) * kSpMemWords];
+                    w[0] = (uint32_t)u;
+                    w[1] = slot_addr(dummy_slot);
+                    w[6] = (uint32_t)(uint64_t)lbES[u];
+                    w[7] = (uint32_t)((uint64_t)lbES[u] >> 32);
+                    const int32_t r = fold_reader[u];
+                    if (r >= 0) {
+                        if (fold_slot[r] < 0) fold_slot[r] = fpool.take();
+                        w[1] = kFoldTag | slot_addr((uint32_t)fold_slot[r]);
+                        w[2] = (uint32_t)(lbQin[r] - lbQ[u]);
+                    }
+                }
             }
         }
         // fold slots follow the others

@@ -409,7 +409,7 @@ def emo_set_wait_limit(cycles: int):
 
 
 def emo_call_path(g: Graph, B, lvl, ldb, ldo, need_slack: bool, flags: int = 0) -> int:
-    """2 = 32-bit lane-stream kernels, 1 = staged 64-bit kernels, 0 = plain-load kernels."""
+    """4, 5 = spine kernels, 2 = 32-bit lane-stream kernels, 1 = staged 64-bit kernels, 0 = plain-load kernels (see emo.h)."""
     rc = lib().emo_call_path(g.handle, int(B), _addr(lvl), int(ldb), int(ldo), int(bool(need_slack)), int(flags))
     if rc < 0:
         raise EmoError(rc, "emo_call_path")

@@ -1,0 +1,44 @@
+"""GPU parity of the spine kernels at the edges of their policy tiles: one, two, four and eight groups of 32 policies per block
+(a worker thread then handles one, two or four policies), full and ragged last tiles, the baseline column in a tile of its own,
+output pitches that allow and forbid vector stores, bundles of two (narrow graphs) and of four operations (wide graphs), with
+and without folded tails, every output; against the CPU oracle: times bit-exact, energy within the reordering bound."""
+from __future__ import annotations
+
+import os
+
+import numpy as np
+import pytest
+
+from paper_2607_12324_b200 import workloads as W
+from tests.test_gpu_parity import E_RTOL, assert_matches, emo, gpu_slack_batch, torch_cuda  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+# policies per block with one block per SM, in groups of 32 (the widest graph's rows of slots leave no room for eight)
+CASES = [("cfg1-train", 0.02, g, d) for g in (1, 2, 4, 8) for d in (-1, 0)] + \
+        [("cfg4-llm", 0.002, g, d) for g in (1, 2, 4) for d in (-5, 0)] + \
+        [("cfg3-8dev", 0.004, g, d) for g in (1, 2) for d in (-31, 0)]
+
+
+@pytest.mark.parametrize("name,scale,groups,off", CASES)
+def test_tiles(torch_cuda, emo, oracle_mod, name, scale, groups, off):
+    torch = torch_cuda
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = W.make_graph(name, scale)
+    B = sms * 32 * groups + off
+    lv = W.policies_for(g, B=B, device="cuda")
+    host = lv.cpu().numpy()
+    r_or = oracle_mod.batch(g, host, B=B, want_arrays=True, threads=os.cpu_count() or 1)
+    base = oracle_mod.batch(g, np.full((g.n, 1), g.L - 1, dtype=np.uint8))
+    h = emo.load_workload(g)
+    assert emo.emo_graph_spine(h)["ok"] == 1
+    for ldo in (B, (B + 3) // 4 * 4 + 1):
+        r = gpu_slack_batch(torch, emo, h, lv, B, g.n, want=("slack",), sums=False, base=True, flags=emo.EMO_F_SPINE_KERNEL, ldo=ldo)
+        assert np.array_equal(r["makespan"], r_or["makespan"]) and r["T0"] == base["makespan"][0]
+        np.testing.assert_allclose(r["energy"], r_or["energy"], rtol=E_RTOL, atol=0)
+        assert r["E0"] == pytest.approx(base["energy"][0], rel=E_RTOL)
+        assert np.array_equal(r["slack"][:, :B], r_or["slack"])
+        assert (r["slack"][:, B:] == -7).all(), "padding columns of the slack matrix were written"
+        r = gpu_slack_batch(torch, emo, h, lv, B, g.n, flags=emo.EMO_F_SPINE_KERNEL, ldo=ldo)
+        assert_matches(r, r_or, B)
+    h.free()
