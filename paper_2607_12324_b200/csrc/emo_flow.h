@@ -103,9 +103,9 @@ constexpr uint32_t kSpPos_First = 1u, kSpPos_Last = 2u;
 constexpr uint32_t kSp_NoSum = 1u;    // operation flags: the segment's sum is zero / a merge operation
 constexpr uint32_t kSp_Push = 2u;     // forward: the lane's previous value goes to the restore list; backward: it is popped
 constexpr uint32_t kSp_Terminal = 4u; // forward: the segment's last node has no successor
-// flags of the layout that the kernels read (member records, records of the completion walk), beside First / Last: the
-// member is folded; the walk takes a row of the restore list
-constexpr uint32_t kSpDev_Fold = 32u, kSpDev_Pop = 128u;
+// flag of the layout that the kernels read (records of the completion walk), beside First / Last: the walk takes a row of
+// the restore list
+constexpr uint32_t kSpDev_Pop = 128u;
 constexpr int kSpDevOpWords = 12;     // x0, x1, word of the sum, slot to clear, d0, d1, lane's slot, published slot, word to write, spare
 constexpr uint32_t kSpSeg_PreF = 1u, kSpSeg_PreB = 2u, kSpSeg_Fold = 4u;   // segment flags
 

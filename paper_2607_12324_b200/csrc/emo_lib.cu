@@ -58,7 +58,7 @@ struct DevFlow {
 struct DevSpineDir {
     unsigned char *blobW = nullptr, *blobS = nullptr;
     uint32_t *rows = nullptr;       // [stages][nlook] policy row of every look-up entry
-    unsigned w_bytes = 0, s_bytes = 0, off_pos = 0, off_mem = 0, off_tab = 0, off_ops = 0, off_rec = 0;
+    unsigned w_bytes = 0, s_bytes = 0, off_pos = 0, off_mem = 0, off_first = 0, off_tab = 0, off_ops = 0, off_rec = 0;
     int words = 0;                  // words per policy and stage: sums (later the values that are pushed / qin), one that stays zero, an unread one; backward then
                                     // the completion offsets
     int zero = 0;                   // the word that stays zero
@@ -696,11 +696,12 @@ int upload_spine(const Flow &f, DevSpine &d)
         for (uint32_t i = 0; i < sp.f.n_ops[st]; ++i) n_term[st] += (sp.f.ops[((size_t)st * sp.f.max_ops + i) * kSpOpWordsF + 7] & kSp_Terminal) != 0;
         max_term = std::max(max_term, n_term[st]);
     }
-    d.f.off_pos = d.b.off_pos = 64;
+    d.f.off_pos = d.b.off_pos = 8 * kSpChunks;
     d.f.off_tab = (unsigned)r16(d.f.off_pos + (size_t)d.nlook * 4);
     d.f.w_bytes = (unsigned)r16(d.f.off_tab + (size_t)d.nlook * Lp * 12);
     d.b.off_mem = (unsigned)r16(d.b.off_pos + (size_t)d.nlook * 4);
-    d.b.off_tab = (unsigned)(d.b.off_mem + (size_t)nmem * 32);
+    d.b.off_first = (unsigned)(d.b.off_mem + (size_t)nmem * 32);
+    d.b.off_tab = (unsigned)r16(d.b.off_first + (size_t)(nmem + 31) / 32 * 4);
     d.b.w_bytes = (unsigned)r16(d.b.off_tab + (size_t)(d.nlook + 1) * Lp * 4);      // the last row stays zero: entries without look-ups
     const int NB = sp.bundle;
     const size_t op_bytes = kSpDevOpWords * 4, spare = (size_t)NB;      // a bundle behind the last is read ahead
@@ -737,7 +738,11 @@ int upload_spine(const Flow &f, DevSpine &d)
         unsigned char *W = fW.data() + (size_t)st * d.f.w_bytes, *WB = bW.data() + (size_t)st * d.b.w_bytes;
         uint32_t *tableF = (uint32_t *)W, *tableB = (uint32_t *)WB, *posF = (uint32_t *)(W + d.f.off_pos), *posB = (uint32_t *)(WB + d.b.off_pos);
         uint32_t *mem = (uint32_t *)(WB + d.b.off_mem);
-        for (int e = 0; e < nmem; ++e) mem[(size_t)e * 8] = kNone;      // padding: no node, no fold
+        for (int e = 0; e < nmem; ++e) {      // padding: no node, folded into the slot nobody reads
+            mem[(size_t)e * 8] = kNone;
+            mem[(size_t)e * 8 + 1] = unread;
+        }
+        uint32_t *first_bits = (uint32_t *)(WB + d.b.off_first);
         bool folds = false;
         auto put_seg = [&](uint32_t si, int &e, bool look) {
             const uint32_t w0 = seg_word(st, si, 0), wf = (uint32_t)std::max(word_f[st][seg_word(st, si, 1) / 128u], 0);
@@ -750,10 +755,8 @@ int upload_spine(const Flow &f, DevSpine &d)
                 uint32_t *o = mem + (size_t)e * 8;
                 std::memcpy(o, m, 32);
                 o[3] = ends | (si << 16);
-                if (m[1] != unread) {
-                    o[3] |= kSpDev_Fold;
-                    folds = true;
-                }
+                folds = folds || m[1] != unread;
+                if (j == 0) first_bits[e / 32] |= 1u << (e % 32);
                 if (!look) continue;
                 posB[e] = ends | (si << 16);
                 posF[e] = ends | (wf << 16);
@@ -770,13 +773,13 @@ int upload_spine(const Flow &f, DevSpine &d)
             folds = false;
             for (uint32_t si : plan[st].chunk[c]) put_seg(si, e, true);
             tableF[c] = tableB[c] = (uint32_t)e0 | ((uint32_t)plan[st].fill[c] << 16);
-            tableB[8 + c] = tableB[c] | (folds ? 0x80000000u : 0u);
+            tableB[kSpChunks + c] = tableB[c] | (folds ? 0x80000000u : 0u);
             e0 += plan[st].fill[c];
         }
         int er = d.nlook;
         folds = false;
         for (uint32_t si : plan[st].rest) put_seg(si, er, false);
-        tableB[8 + d.chunks] = (uint32_t)d.nlook | ((uint32_t)((er - d.nlook + 3) / 4 * 4) << 16) | (folds ? 0x80000000u : 0u);
+        tableB[kSpChunks + d.chunks] = (uint32_t)d.nlook | ((uint32_t)((er - d.nlook + 3) / 4 * 4) << 16) | (folds ? 0x80000000u : 0u);
 
         uint32_t *hf = (uint32_t *)(fS.data() + (size_t)st * d.f.s_bytes), *hb = (uint32_t *)(bS.data() + (size_t)st * d.b.s_bytes);
         hf[0] = sp.f.n_ops[st] / (uint32_t)NB;
@@ -1059,9 +1062,13 @@ bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, Sp
         auto shape = [&](bool backward, SpineParams &p, size_t &smem, int &threads) {
             const SpineDir &dir = backward ? sp.b : sp.f;
             const DevSpineDir &dd = backward ? d.b : d.f;
-            // warps: 16 (128 registers per thread) up to two policy groups, else 22 (88)
-            const int look = backward ? (G == 4 ? 6 : 4) : (G <= 2 ? 10 : 12);
-            const int posts = backward ? (G <= 2 ? 6 : (G == 4 ? 10 : 8)) : (need_bwd ? subs : 0);      // forward: one pusher per sub-tile
+            // warps: 16 (128 registers per thread) up to two policy groups, else 20 (96).  What the spine (backward also the
+            // completion walk) and the producers leave goes to the workers, backward two fifths of it to the look-ups (250 000
+            // nodes x 16 384 policies: 5 look-up and 9 storing warps); multiples of the sub-tiles.
+            const int avail = (G <= 2 ? 16 : 20) - (backward ? 2 : 1) * spines - 2;
+            const int pushers = !backward && need_bwd ? subs : 0;
+            const int look = (backward ? std::max(avail * 2 / 5, subs) : std::min(avail - pushers, 12)) / subs * subs;
+            const int posts = backward ? (avail - look) / subs * subs : pushers;
             const size_t acc = (size_t)dd.words * P * 4, slots = (size_t)dir.slots * P * 4;
             const size_t rst = backward ? (size_t)d.max_push * P * 4 : 0;
             const size_t wbuf = round_up((size_t)dd.w_bytes + (size_t)d.nlook * P, 128), sbuf = round_up(dd.s_bytes + rst, 128);
@@ -1084,6 +1091,7 @@ bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, Sp
                 p.s_bytes = dd.s_bytes;
                 p.off_pos = dd.off_pos;
                 p.off_mem = dd.off_mem;
+                p.off_first = dd.off_first;
                 p.off_tab = dd.off_tab;
                 p.tab_row = (unsigned)f.Lp * (backward ? 4u : 12u);
                 p.off_ops = dd.off_ops;
@@ -1165,7 +1173,7 @@ int launch_spine_fwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const u
     void (*kern)(SpineParams) = nullptr;
     if (pl.vw == 1) kern = wide ? emo_spine_fwd<1, 4, 4, 512> : emo_spine_fwd<1, 2, 2, 512>;
     else if (pl.vw == 2) kern = wide ? emo_spine_fwd<2, 4, 4, 512> : emo_spine_fwd<2, 2, 2, 512>;
-    else kern = wide ? emo_spine_fwd<4, 4, 4, 704> : emo_spine_fwd<4, 4, 2, 704>;
+    else kern = wide ? emo_spine_fwd<4, 4, 4, 640> : emo_spine_fwd<4, 4, 2, 640>;
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
     kern<<<pl.grid_f, pl.threads_f, pl.smem_f, st>>>(p);
     EMO_CUDA(cudaGetLastError());
@@ -1205,8 +1213,8 @@ int launch_spine_bwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const u
     else if (pl.vw == 1) EMO_PICK_S(1, 2, 2, 512);
     else if (pl.vw == 2 && wide) EMO_PICK_S(2, 4, 4, 512);
     else if (pl.vw == 2) EMO_PICK_S(2, 2, 2, 512);
-    else if (wide) EMO_PICK_S(4, 4, 4, 704);
-    else EMO_PICK_S(4, 4, 2, 704);
+    else if (wide) EMO_PICK_S(4, 4, 4, 640);
+    else EMO_PICK_S(4, 4, 2, 640);
 #undef EMO_PICK_S
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
     kern<<<pl.grid_b, pl.threads_b, pl.smem_b, st>>>(p);
@@ -1222,10 +1230,10 @@ bool spine_allowed(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ld
     const int64_t big = (int64_t)1 << 28;
     if (!g->sflow.ok32 || !g->sflow.spine.ok || !g->dspine.ready) return false;
     if (flags & (EMO_F_NO_STAGING | EMO_F_PAIR_KERNEL | EMO_F_LANE_KERNEL | EMO_F_FLOW_KERNEL)) return false;
-    // Measured (both passes, ms, spine / the best of the others): 1 013 nodes x 65 536 policies 0.42 / 0.90; 10 000 x 4 096
-    // 0.80 / 2.30; 75 000 x 10 001 forward 1.28 / 1.89; 250 000 x 16 384 19.4 / 20.4.  On wide graphs one warp carries the
-    // recurrence of all lanes: 18 lanes, 128 039 nodes x 8 192 policies (two groups per SM) 8.9 / 9.05, below that the
-    // others stay.
+    // Measured (both passes, ms, spine / the best of the others): 1 013 nodes x 65 536 policies 0.36 / 0.90; 10 000 x 4 096
+    // 0.77 / 2.30; 75 000 x 10 001 forward 1.28 / 1.89; 250 000 x 16 384 15.0 / 20.4.  On wide graphs one warp carries the
+    // recurrence of all lanes: 18 lanes, 128 039 nodes x 8 192 policies (two groups per SM) 6.2 / 9.05; 51 000 x 333 to
+    // 4 500 (one group) 2.09 / 2.05 and 6 400 nodes 0.31 / 0.30, so there the others stay.
     if (!(flags & EMO_F_SPINE_KERNEL)) {
         const int64_t per_sm = ((B + 1 + 31) / 32 + g->sm_count - 1) / std::max(g->sm_count, 1);
         if (g->sflow.lanes > 8 && per_sm < 2) return false;
@@ -1510,7 +1518,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             std::thread spine_thread;
             if (want_spine) {
                 const int code = (int)((flags >> 30) & 3u);
-                int sk = code == 1 ? 8 : (code == 3 ? 32 : 16);
+                // Measured (forward + backward, ms): 18 lanes, 128 039 nodes x 8 192 policies 6.2 with 4 positions, 6.6 with 5
+                // and 8.9 with 8 (a stage of 8 leaves room for one buffer less); 4 lanes, 250 000 x 16 384 15.0 with
+                // 16, 17.2 with 12; 1 013 x 65 536 0.36 with 16, 0.48 with 20 and 0.43 with 8.
+                int sk = code == 1 ? 8 : (code == 3 ? 32 : (code == 2 || flanes <= 8 ? 16 : 4));
                 while (sk > 8 && flanes * sk > 32 * kFlowRowRegs) sk /= 2;
                 spine_thread = std::thread([&, sk]() {
                     try {

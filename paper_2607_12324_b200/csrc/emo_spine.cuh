@@ -36,18 +36,18 @@
 #include "emo_flow.cuh"
 
 constexpr int kSpRing = 8;               // most buffers of a ring
-constexpr int kSpChunks = 8;             // most chunks of a stage and kind
+constexpr int kSpChunks = 16;            // most chunks of a stage and kind (look-up, storing)
 constexpr int kSpRowRing = 4;            // stages whose row numbers are on their way or in use
 
 struct SpineParams {
-    const unsigned char *blobW;          // [stages][w_bytes] the workers' part: chunk table (64 bytes), position words, (backward) member
-                                         // records, table rows
+    const unsigned char *blobW;          // [stages][w_bytes] the workers' part: chunk table (4 * 2 * kSpChunks bytes), position words, (backward) member
+                                         // records, bits of the segments' first entries, table rows
     const unsigned char *blobS;          // [stages][s_bytes] the spine's part: header, (forward) terminal nodes, operations, records of the pushers or the
                                          // completion walk
     const uint32_t *rows;                // [stages][nlook] policy row of every look-up entry (kNone: none)
     const uint32_t *push_base;           // [stages + 1] first restore row of every stage
     unsigned w_bytes, s_bytes, off_pos, off_tab, tab_row, off_ops;
-    unsigned off_mem, off_rec;           // backward: members; forward: records of the pushers, backward: of the completion walk
+    unsigned off_mem, off_first, off_rec;      // backward: members, a bit per entry (first of its segment); forward: records of the pushers, backward: of the completion walk
     int nlook;                           // look-up entries that a stage has room for (entries behind them have none)
     int chunks, chunks_post;             // per stage: look-up chunks; backward: chunks of the storing workers
     int stages, lanes, Lp, L;
@@ -171,10 +171,6 @@ __device__ __forceinline__ void emo_stg_out_if(long long *base, unsigned row, un
     if constexpr (V == 4)
         asm volatile("{\n\t.reg .pred p;\n\t.reg .u64 a;\n\tsetp.ne.u32 p, %7, 0;\n\tmad.wide.u32 a, %1, %2, %0;\n\t@p st.global.v4.b64 [a], {%3, %4, %5, %6};\n\t}" ::"l"(base), "r"(row),
                      "r"(pitch_bytes), "l"(x[0]), "l"(x[1]), "l"(x[2]), "l"(x[3]), "r"(ok) : "memory");
-}
-__device__ __forceinline__ void emo_red_max_u32_if(unsigned a, unsigned v, unsigned ok)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.shared.max.u32 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"(ok) : "memory");
 }
 // 16-byte asynchronous copy of a piece of matrix row `row` (kNone: no copy)
 __device__ __forceinline__ void emo_cp_async16_row(unsigned dst, const uint8_t *base, unsigned row, unsigned pitch)
@@ -684,14 +680,24 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_fwd(SpineParams p)
 // before a stage waits for the stores of the stage two back (folded values are read at least two stages
 // after they are written).  EXTRA: also ES, LS, the slack sums and critical counts (ES_v = lbES_v + X - tail_v).
 // ---------------------------------------------------------------------------------------------------
-// The stores of one chunk: entries e0 .. e0 + n - 1 (n a multiple of four).  VEC: this thread's policies all exist and leave as
-// one store per node.  FOLD: some member is folded (or ES, LS are asked for), so the tails are needed and with them the
-// members' durations; otherwise a member costs two loads per policy, the subtraction and its store.
-template <int V, bool VEC, bool FOLD, bool EXTRA>
-__device__ __forceinline__ void emo_spine_stores(const SpineParams &p, const EmoLevels<V> &lev, unsigned wbuf, unsigned acc_t, unsigned slot_t, unsigned e0, unsigned n,
-                                                 bool looks, const long long (&T)[V], int64_t b, long long (&ssum)[V], int (&ncrit)[V])
+// Stores of this thread's V policies of one node.  VEC: they all exist and leave as one store.
+template <int V, bool VEC>
+__device__ __forceinline__ void emo_spine_put(const SpineParams &p, long long *base, unsigned row, unsigned ldo8, const long long (&x)[V], int64_t b, unsigned ok)
 {
-    constexpr int U = (V == 4 || EXTRA) ? 2 : 4;
+    if (VEC) {
+        emo_stg_out_if<V>(base, row, ldo8, x, ok);
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) emo_stg_s64_if(base + v, row, ldo8, x[v], ok & (unsigned)(b + v < p.B));
+    }
+}
+// The stores of one chunk, entries e0 .. e0 + n - 1 (n a multiple of four), everything taken for every member: without tails a
+// member costs two loads per policy, the subtraction and its store.  EXTRA: with the tails, for ES, LS and the sums.
+template <int V, bool VEC, bool EXTRA>
+__device__ __forceinline__ void emo_spine_flat(const SpineParams &p, const EmoLevels<V> &lev, unsigned wbuf, unsigned acc_t, unsigned slot_t, unsigned e0, unsigned n,
+                                               bool looks, const long long (&T)[V], int64_t b, long long (&ssum)[V], int (&ncrit)[V])
+{
+    constexpr int U = V == 4 ? (EXTRA ? 1 : 2) : (EXTRA ? 2 : 4);
     const unsigned P = (unsigned)p.ptile, P4 = P * 4u, G = (unsigned)p.groups, ldo8 = (unsigned)p.ldo * 8u, comp = p.comp_off * G;
     // entries without look-ups read the table row that stays zero
     const unsigned tab_row = looks ? p.tab_row : 0u, lvl_row = looks ? P : 0u;
@@ -699,14 +705,6 @@ __device__ __forceinline__ void emo_spine_stores(const SpineParams &p, const Emo
     long long *const es_t = (EXTRA && p.ES) ? reinterpret_cast<long long *>(p.ES) + b : nullptr;
     long long *const ls_t = (EXTRA && p.LS) ? reinterpret_cast<long long *>(p.LS) + b : nullptr;
     const unsigned sl_ok = sl_t != nullptr, es_ok = es_t != nullptr, ls_ok = ls_t != nullptr;
-    auto put = [&](long long *base, unsigned row, const long long (&x)[V], unsigned ok) {
-        if (VEC) {
-            emo_stg_out_if<V>(base, row, ldo8, x, ok);
-        } else {
-#pragma unroll
-            for (int v = 0; v < V; ++v) emo_stg_s64_if(base + v, row, ldo8, x[v], ok & (unsigned)(b + v < p.B));
-        }
-    };
     unsigned mem_a = wbuf + p.off_mem + e0 * 32u, lvl_a = wbuf + p.off_lvl + e0 * lvl_row, tab_a = wbuf + p.off_tab + (looks ? e0 : (unsigned)p.nlook) * p.tab_row;
     unsigned q[V], wn[U];
     uint4 mn[U], an[U];
@@ -715,7 +713,7 @@ __device__ __forceinline__ void emo_spine_stores(const SpineParams &p, const Emo
         for (int i = 0; i < U; ++i) {
             mn[i] = emo_lds128(mem_a + 32u * i);            // node, fold slot, fold correction, word << 16 | flags
             an[i] = emo_lds128(mem_a + 32u * i + 16u);      // A, lbES
-            if (FOLD) wn[i] = lev.load(lvl_a + (unsigned)i * lvl_row);
+            if (EXTRA) wn[i] = lev.load(lvl_a + (unsigned)i * lvl_row);
         }
         mem_a += 32u * U;
         lvl_a += lvl_row * U;
@@ -735,7 +733,7 @@ __device__ __forceinline__ void emo_spine_stores(const SpineParams &p, const Emo
             for (int v = 0; v < V; ++v) {
                 qn[i][v] = emo_lds_u32(at + 128u * v);
                 cn[i][v] = emo_lds_u32(at + comp + 128u * v);
-                if (FOLD) d[i][v] = emo_lds_u32(lev.template addr<4u>(wn[i], v, tab_a + (unsigned)i * tab_row));
+                if (EXTRA) d[i][v] = emo_lds_u32(lev.template addr<4u>(wn[i], v, tab_a + (unsigned)i * tab_row));
             }
         }
         fetch();                         // the next entries (past the last ones: read, not used)
@@ -743,7 +741,7 @@ __device__ __forceinline__ void emo_spine_stores(const SpineParams &p, const Emo
 #pragma unroll
         for (int i = 0; i < U; ++i) {
             const long long A = (long long)((unsigned long long)m2[i].x | ((unsigned long long)m2[i].y << 32));
-            const unsigned real = (unsigned)(m[i].x != emo::kNone);
+            const unsigned real = (unsigned)(m[i].x != emo::kNone), slot = slot_t + m[i].y * G;
             long long sl[V];
             unsigned X[V];
 #pragma unroll
@@ -751,29 +749,92 @@ __device__ __forceinline__ void emo_spine_stores(const SpineParams &p, const Emo
                 X[v] = qn[i][v] + cn[i][v];
                 sl[v] = (T[v] - A) - (long long)(unsigned long long)X[v];
             }
-            put(sl_t, m[i].x, sl, sl_ok & real);
-            if (FOLD) {
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    q[v] = ((m[i].w & emo::kSpPos_First) ? qn[i][v] : q[v]) + d[i][v];
-                    emo_red_max_u32_if(slot_t + m[i].y * G + 128u * v, emo_floor_sub(q[v], m[i].z), m[i].w & emo::kSpDev_Fold);
-                }
-            }
+            emo_spine_put<V, VEC>(p, sl_t, m[i].x, ldo8, sl, b, sl_ok & real);
             if (EXTRA) {
                 // ES_v = lbES_v + eo_v with eo_v = X - tail_v (X = eo + tail for every member)
                 const long long lb = (long long)((unsigned long long)m2[i].z | ((unsigned long long)m2[i].w << 32));
                 long long es[V], ls[V];
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
+                    q[v] = ((m[i].w & emo::kSpPos_First) ? qn[i][v] : q[v]) + d[i][v];
+                    emo_red_max_u32(slot + 128u * v, emo_floor_sub(q[v], m[i].z));
                     es[v] = lb + (long long)(unsigned long long)(X[v] - q[v]);
                     ls[v] = es[v] + sl[v];
                     ssum[v] += real ? sl[v] : 0;
                     ncrit[v] += (real && sl[v] == 0) ? 1 : 0;
                 }
-                put(es_t, m[i].x, es, es_ok & real);
-                put(ls_t, m[i].x, ls, ls_ok & real);
+                emo_spine_put<V, VEC>(p, es_t, m[i].x, ldo8, es, b, es_ok & real);
+                emo_spine_put<V, VEC>(p, ls_t, m[i].x, ldo8, ls, b, ls_ok & real);
             }
         }
+    }
+}
+// The same for slack alone where members are folded.  What is one number per segment is taken at its first member only: a bit per
+// entry, made uniform once for up to 32 entries, says where (a branch on a freshly loaded word costs 100 cycles and more;
+// taking everything for every member was 20 of the backward pass's 50 instructions per node and 32 policies).  Members that
+// are not folded name a slot nobody reads.
+template <int V, bool VEC>
+__device__ __forceinline__ void emo_spine_folds(const SpineParams &p, const EmoLevels<V> &lev, unsigned wbuf, unsigned acc_t, unsigned slot_t, unsigned e0, unsigned n,
+                                                bool looks, const long long (&T)[V], int64_t b)
+{
+    constexpr int U = V == 1 ? 4 : 2;
+    const unsigned P = (unsigned)p.ptile, P4 = P * 4u, G = (unsigned)p.groups, ldo8 = (unsigned)p.ldo * 8u, comp = p.comp_off * G;
+    const unsigned tab_row = looks ? p.tab_row : 0u, lvl_row = looks ? P : 0u;
+    long long *const sl_t = p.slack ? reinterpret_cast<long long *>(p.slack) + b : nullptr;
+    const unsigned sl_ok = sl_t != nullptr;
+    unsigned mem_a = wbuf + p.off_mem + e0 * 32u, lvl_a = wbuf + p.off_lvl + e0 * lvl_row, tab_a = wbuf + p.off_tab + (looks ? e0 : (unsigned)p.nlook) * p.tab_row;
+    unsigned q[V], wn[U], first = 0;
+    long long sl[V];
+    uint4 mn[U];
+    auto fetch = [&]() {
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            mn[i] = emo_lds128(mem_a + 32u * i);            // node, fold slot, fold correction, word << 16 | flags
+            wn[i] = lev.load(lvl_a + (unsigned)i * lvl_row);
+        }
+        lvl_a += lvl_row * U;
+    };
+    fetch();
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        q[v] = 0;
+        sl[v] = 0;
+    }
+    for (unsigned e = e0; e < e0 + n; e += U) {
+        if (e == e0 || (e & 31u) == 0u) first = emo_uniform(emo_lds_u32(wbuf + p.off_first + (e >> 5) * 4u)) >> (e & 31u);
+        const unsigned rec_a = mem_a;
+        uint4 m[U];
+        unsigned d[U][V];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            m[i] = mn[i];
+#pragma unroll
+            for (int v = 0; v < V; ++v) d[i][v] = emo_lds_u32(lev.template addr<4u>(wn[i], v, tab_a + (unsigned)i * tab_row));
+        }
+        mem_a += 32u * U;
+        tab_a += tab_row * U;
+        fetch();                         // the next entries (past the last ones: read, not used)
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            if (first & (1u << i)) {
+                const EmoVec<2> a = emo_ldv<2>(rec_a + 32u * i + 16u);
+                const unsigned at = acc_t + (m[i].w >> 16) * P4;
+                const long long A = (long long)((unsigned long long)a.v[0] | ((unsigned long long)a.v[1] << 32));
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    q[v] = emo_lds_u32(at + 128u * v);
+                    sl[v] = (T[v] - A) - (long long)(unsigned long long)(q[v] + emo_lds_u32(at + comp + 128u * v));
+                }
+            }
+            const unsigned slot = slot_t + m[i].y * G;
+            emo_spine_put<V, VEC>(p, sl_t, m[i].x, ldo8, sl, b, sl_ok & (unsigned)(m[i].x != emo::kNone));
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                q[v] += d[i][v];
+                emo_red_max_u32(slot + 128u * v, emo_floor_sub(q[v], m[i].z));
+            }
+        }
+        first >>= U;
     }
 }
 
@@ -843,7 +904,9 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_bwd(SpineParams p)
     } else if (role.comp) {
         // The completion offsets: per lane and stage the segments last to first.  co of a segment's last member is what the
         // segment behind it started from: that segment's co minus its sum, or a word of the restore list.  The lanes are dealt
-        // to NB streams, one for every part of the warp.
+        // to NB streams, one for every part of the warp; R records at a time (what the registers hold without spilling: with
+        // the shared memory in use there is hardly any L1, a spilled word comes back from L2).
+        constexpr int R = VS == 4 ? 2 : 4;
         const unsigned word = (unsigned)((role.idx * LP + (lane & (LP - 1))) * VS), P4 = (unsigned)P * 4u, G4 = (unsigned)G, comp = p.comp_off * G4;
         const unsigned slot_t = smem0 + word * 4u;
         for (int ln = 0; ln < p.lanes; ++ln) {
@@ -875,17 +938,14 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_bwd(SpineParams p)
             EmoVec<VS> co;
 #pragma unroll
             for (int v = 0; v < VS; ++v) co.v[v] = 0u;
-            uint4 rn[4];
+            for (unsigned i = 0; i < n; i += R) {
+                uint4 r[R];
+                EmoVec<VS> S[R], in[R], pop[R];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) rn[k] = emo_lds128(rec_a + 16u * NB * k);      // the lane's slot, word of the sum, word of the segment, flags
-            for (unsigned i = 0; i < n; i += 4u) {
-                uint4 r[4];
-                EmoVec<VS> S[4], in[4], pop[4];
+                for (int k = 0; k < R; ++k) r[k] = emo_lds128(rec_a + 16u * NB * k);      // the lane's slot, word of the sum, word of the segment, flags
+                rec_a += 16u * NB * R;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) r[k] = rn[k];
-                rec_a += 64u * NB;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < R; ++k) {
 #pragma unroll
                     for (int v = 0; v < VS; ++v) pop[k].v[v] = 0u;
                     S[k] = emo_ldv<VS>(acc_t + r[k].y * G4);
@@ -893,9 +953,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_bwd(SpineParams p)
                     emo_ldv_if<VS>(pop[k], rst_a + (r[k].w >> 8) * P4, r[k].w & emo::kSpDev_Pop);
                 }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) rn[k] = emo_lds128(rec_a + 16u * NB * k);      // (four spare records per stream follow the last)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < R; ++k) {
 #pragma unroll
                     for (int v = 0; v < VS; ++v) co.v[v] = (r[k].w & emo::kSpPos_First) ? in[k].v[v] : co.v[v];
                     emo_stv<VS>(acc_t + r[k].z * G4 + comp, co);
@@ -954,13 +1012,14 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_bwd(SpineParams p)
             const long long tw1 = EMO_SCLK();
             t_w += tw1 - tw0;
             const unsigned wbuf = smem0 + p.off_w0 + (unsigned)rw.idx * p.wbuf_bytes, acc_t = smem0 + p.off_acc0 + (unsigned)ra.idx * p.acc_bytes + col;
-            const unsigned ck = emo_uniform(emo_lds_u32(wbuf + 32u + 4u * (unsigned)chunk)), e0 = ck & 0xFFFFu, n = (ck >> 16) & 0x7FFFu;
-            if (EXTRA || (ck >> 31)) {
-                if (vec) emo_spine_stores<VW, true, true, EXTRA>(p, lev, wbuf, acc_t, smem0 + col, e0, n, chunk < p.chunks, T, b, ssum, ncrit);
-                else emo_spine_stores<VW, false, true, EXTRA>(p, lev, wbuf, acc_t, smem0 + col, e0, n, chunk < p.chunks, T, b, ssum, ncrit);
+            const unsigned ck = emo_uniform(emo_lds_u32(wbuf + 4u * (unsigned)(kSpChunks + chunk))), e0 = ck & 0xFFFFu, n = (ck >> 16) & 0x7FFFu;
+            const bool looks = chunk < p.chunks;
+            if (!EXTRA && (ck >> 31)) {
+                if (vec) emo_spine_folds<VW, true>(p, lev, wbuf, acc_t, smem0 + col, e0, n, looks, T, b);
+                else emo_spine_folds<VW, false>(p, lev, wbuf, acc_t, smem0 + col, e0, n, looks, T, b);
             } else {
-                if (vec) emo_spine_stores<VW, true, false, false>(p, lev, wbuf, acc_t, smem0 + col, e0, n, chunk < p.chunks, T, b, ssum, ncrit);
-                else emo_spine_stores<VW, false, false, false>(p, lev, wbuf, acc_t, smem0 + col, e0, n, chunk < p.chunks, T, b, ssum, ncrit);
+                if (vec) emo_spine_flat<VW, true, EXTRA>(p, lev, wbuf, acc_t, smem0 + col, e0, n, looks, T, b, ssum, ncrit);
+                else emo_spine_flat<VW, false, EXTRA>(p, lev, wbuf, acc_t, smem0 + col, e0, n, looks, T, b, ssum, ncrit);
             }
             __syncwarp();
             if (lane == 0) {
