@@ -460,59 +460,108 @@ __device__ __forceinline__ void emo_flow_fwd_run(unsigned la, unsigned ta0, unsi
     ea += g[0];
 }
 
-// What the forward kernel carries for time-interval policies beside its parameters.
+// What the forward kernel carries for time-interval policies beside its parameters.  Start times only grow along a lane, and an
+// interval holds hundreds of its entries, so a thread keeps the interval that its lane is in and the table entry of its level:
+// the look-ups of the following entries then depend on no start time, and the chain per entry is an addition and a comparison.
 struct FlowIntv {
     const long long *brk;        // change points in shared memory
     unsigned Fs;                 // the block's columns of F in shared memory (shared-window address of this thread's column): [rowsF * I][ptile]
-    int col;                     // this thread's column in the block
     int64_t b;                   // this thread's policy
     bool count;                  // this thread adds busy time (a live policy and a busy array)
-    unsigned key;                // busy time collected for (row, interval) = key, not yet added to memory
+    unsigned row;                // device of the interval at hand (the same for the whole warp; kNone: none yet)
+    unsigned at;                 // where its level lies in a table row (bytes)
+    long long iend;              // where it ends
+    unsigned key;                // (row, interval) whose busy time is collected, not yet added to memory
     unsigned long long sum;
 };
-// The level of an entry whose start offset is eo (Alg. 1: the interval that holds the start time), then its
-// table entry.  No branch on anything loaded here: a node outside every policy reads the last row and any
-// level (its table row holds one value), the interval index is a float guess with one exact correction (uniform
-// grid), and busy time is collected in a register while the (row, interval) stays the same.
+// End offsets below this value end inside the interval at hand (an entry of no policy: always).
+__device__ __forceinline__ unsigned emo_flow_intv_room(const FlowIntv &iv, const uint4 &meta)
+{
+    const long long r = iv.iend - ((long long)((unsigned long long)meta.x | ((unsigned long long)meta.y << 32)) + (long long)meta.w);
+    const unsigned c = r < 0 ? 0u : (r > 0xFFFFFFFFll ? 0xFFFFFFFFu : (unsigned)r);
+    return meta.z == emo::kNone ? 0xFFFFFFFFu : (meta.z == iv.row ? c : 0u);
+}
+__device__ __forceinline__ double emo_flow_intv_energy(unsigned ta, unsigned tok)
+{
+    return __hiloint2double((int)emo_tld_u32(ta + 4u, tok), (int)emo_tld_u32(ta + 8u, tok));
+}
+// An entry at start offset eo whose pack does not end inside the interval at hand: the interval that holds its start (Alg. 1) by
+// a float guess with one exact correction (uniform grid), its level, its table entry; then the interval that holds its end is
+// the one at hand.  Threads whose pack did end inside it arrive at the same values.
 __device__ __forceinline__ void emo_flow_intv_lookup(const FlowParams &p, FlowIntv &iv, const uint4 &meta, unsigned eo, unsigned ta0,
                                                      unsigned lmask, unsigned tok, unsigned &dd, double &e)
 {
+    if (meta.z == emo::kNone) {      // no policy: its table row holds one value
+        dd = emo_tld_u32(ta0 + iv.at, tok);
+        e = emo_flow_intv_energy(ta0 + iv.at, tok);
+        return;
+    }
     const long long start = (long long)((unsigned long long)meta.x | ((unsigned long long)meta.y << 32)) + (long long)eo;
-    const bool pack = meta.z != emo::kNone;
-    const unsigned rowc = min(meta.z, (unsigned)p.rowsF - 1u);
+    const unsigned row_key = meta.z * (unsigned)p.I;
     long long iend;
     const int i = emo_interval_index<true>(start, p.I, p.delta, p.inv_mean, iv.brk, iend);
-    const unsigned key = rowc * (unsigned)p.I + (unsigned)i;
-    const unsigned lv = emo_vld_u8(iv.Fs + key * (unsigned)p.ptile);
-    const unsigned ta = ta0 + (lv & lmask) * 12u;
-    dd = emo_tld_u32(ta, tok);
-    e = __hiloint2double((int)emo_tld_u32(ta + 4u, tok), (int)emo_tld_u32(ta + 8u, tok));
-    const long long dur = (long long)meta.w + (long long)dd;
-    const bool on = pack && iv.count;
-    if (on && key != iv.key) {      // rare: the lane moved on to another interval (or device)
-        if (iv.sum) atomicAdd(p.busy + (size_t)iv.key * p.ldw + iv.b, iv.sum);
-        iv.key = key;
+    unsigned at = (emo_vld_u8(iv.Fs + (row_key + (unsigned)i) * (unsigned)p.ptile) & lmask) * 12u;
+    dd = emo_tld_u32(ta0 + at, tok);
+    e = emo_flow_intv_energy(ta0 + at, tok);
+    const long long end = start + ((long long)meta.w + (long long)dd);
+    const bool inside = end < iend;
+    if (!inside || row_key + (unsigned)i != iv.key) {
+        if (iv.count && iv.sum) atomicAdd(p.busy + (size_t)iv.key * p.ldw + iv.b, iv.sum);
         iv.sum = 0;
+        iv.key = row_key + (unsigned)i;
     }
-    const bool single = start + dur <= iend;
-    iv.sum += (on && single) ? (unsigned long long)dur : 0ull;
-    if (on && !single) emo_interval_busy(p.busy, p.ldw, iv.b, rowc, p.I, i, iend, start, start + dur, iv.brk);      // rare
+    if (inside) {
+        iv.sum += (unsigned long long)(end - start);
+    } else {
+        if (iv.count) emo_interval_busy(p.busy, p.ldw, iv.b, meta.z, p.I, i, iend, start, end, iv.brk);
+        const int j = emo_interval_index<true>(end, p.I, p.delta, p.inv_mean, iv.brk, iend);
+        iv.key = row_key + (unsigned)j;
+        at = (emo_vld_u8(iv.Fs + iv.key * (unsigned)p.ptile) & lmask) * 12u;
+    }
+    iv.at = at;
+    iv.iend = iend;
+    iv.row = meta.z;
 }
-// A run of r plain entries: every start time depends on the entry before it, so the look-ups form one chain
-// and there is nothing to gain from one instantiation per length (which would only crowd the instruction
-// cache: the look-up is some sixty instructions); a loop, inlined so that the parameters and the lane's running
-// values stay in registers, with the next entry's constants requested one entry ahead.
-__device__ __forceinline__ void emo_flow_fwd_run_intv(const FlowParams &p, FlowIntv &iv, unsigned r, unsigned meta_a, unsigned ta0, unsigned tab_row,
-                                                   unsigned lmask, unsigned tok, unsigned &h, double &ea)
+// R plain entries from the interval at hand; nothing is changed when one of them leaves it in some thread.
+template <int R>
+__device__ __forceinline__ bool emo_flow_fwd_run_intv(FlowIntv &iv, unsigned meta_a, unsigned ta0, unsigned tab_row, unsigned tok, unsigned &h,
+                                                      double &ea)
 {
-    uint4 meta = emo_tld_128(meta_a, tok);
+    uint4 m[R];
+    unsigned d[R];
+    double e[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        m[i] = emo_tld_128(meta_a + 16u * i, tok);
+        d[i] = emo_tld_u32(ta0 + (unsigned)i * tab_row + iv.at, tok);
+        e[i] = emo_flow_intv_energy(ta0 + (unsigned)i * tab_row + iv.at, tok);
+    }
+    unsigned v = h;
+    bool out = false;
+    unsigned long long add = 0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        v += d[i];
+        out = out || v >= emo_flow_intv_room(iv, m[i]);
+        add += m[i].z != emo::kNone ? (unsigned long long)m[i].w + d[i] : 0ull;
+    }
+    if (__any_sync(0xFFFFFFFFu, out)) return false;
+    h = v;
+#pragma unroll
+    for (int i = 0; i < R; ++i) ea += e[i];
+    iv.sum += add;
+    return true;
+}
+// The same one by one, where the interval changes.
+__device__ __forceinline__ void emo_flow_fwd_run_intv_slow(const FlowParams &p, FlowIntv &iv, unsigned r, unsigned meta_a, unsigned ta0,
+                                                           unsigned tab_row, unsigned lmask, unsigned tok, unsigned &h, double &ea)
+{
 #pragma unroll 1
-    for (unsigned i = 0; i < r; ++i) {
-        const uint4 cur = meta;
-        meta = emo_tld_128(meta_a + 16u * min(i + 1u, r - 1u), tok);      // never past the run: the last entry's constants end the stage buffer
+    for (unsigned i = 0; i < r; ++i, meta_a += 16u, ta0 += tab_row) {
+        if (emo_flow_fwd_run_intv<1>(iv, meta_a, ta0, tab_row, tok, h, ea)) continue;
         unsigned dd;
         double e;
-        emo_flow_intv_lookup(p, iv, cur, h, ta0 + i * tab_row, lmask, tok, dd, e);
+        emo_flow_intv_lookup(p, iv, emo_tld_128(meta_a, tok), h, ta0, lmask, tok, dd, e);
         h += dd;
         ea += e;
     }
@@ -542,7 +591,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
     volatile int *abort_word = reinterpret_cast<volatile int *>(emo_smem + p.off_bar + 16 * kFlowMaxBuf);
     const unsigned stage0 = smem0 + p.off_stage0;
     emo_flow_init(p, smem0, emo_smem, n_cons);
-    FlowIntv iv{nullptr, 0u, col, b, act && p.busy != nullptr, 0u, 0ull};
+    FlowIntv iv{nullptr, 0u, b, act && p.busy != nullptr, emo::kNone, 0u, 0ll, 0u, 0ull};
     if (INTV) {
         long long *brk = reinterpret_cast<long long *>(emo_smem + p.off_brk);
         for (int i = threadIdx.x; i < p.I; i += blockDim.x) brk[i] = p.breaks[i];
@@ -632,8 +681,14 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                     unsigned dd = 0;
                     double ee = 0.0;
                     uint4 meta = make_uint4(0, 0, 0, 0);
+                    unsigned room = 0;
                     if (INTV) {
+                        // the level of the interval at hand, unless the entry does not follow the lane's last one in time
                         meta = emo_tld_128(meta_a, tok);
+                        dd = emo_tld_u32(tab_a + iv.at, tok);
+                        ee = emo_flow_intv_energy(tab_a + iv.at, tok);
+                        if (!(fl & emo::kF_HasReg)) iv.row = emo::kNone;
+                        room = emo_flow_intv_room(iv, meta);
                     } else {
                         const unsigned lb = emo_tld_u8(lvl_a, tok);
                         const unsigned ta = tab_a + (lb & lmask) * 12u;
@@ -662,7 +717,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                         dead = __any_sync(0xFFFFFFFFu, dead);
                         if (dead) continue;      // on to the group's next barrier
                         if (INTV) {
-                            term = (fl & emo::kF_Terminal) != 0u;      // its duration is not known yet
+                            term = (fl & emo::kF_Terminal) != 0u;      // its duration is not certain yet
                         } else if (fl & emo::kF_Terminal) {
                             // a node without successors: candidate for the makespan (its bound follows the operands in the pool)
                             const long long lbc = (long long)((unsigned long long)emo_tld_u32(pa, tok) | ((unsigned long long)emo_tld_u32(pa + 4u, tok) << 32));
@@ -671,8 +726,10 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                         }
                     }
                     v = max(v, emo_floor_sub(x0, r1.z));
-                    // time-interval policies: the level follows from the start time, which is known only now
-                    if (INTV) emo_flow_intv_lookup(p, iv, meta, v, tab_a, lmask, tok, dd, ee);
+                    if (INTV) {
+                        if (__any_sync(0xFFFFFFFFu, v + dd >= room)) emo_flow_intv_lookup(p, iv, meta, v, tab_a, lmask, tok, dd, ee);
+                        else iv.sum += meta.z != emo::kNone ? (unsigned long long)meta.w + dd : 0ull;
+                    }
                     if ((fl & emo::kF_Push) && push) {
                         *push = h;
                         push += ptile;
@@ -693,7 +750,18 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                 }
                 // the run: every entry continues from the lane's previous value
                 if (INTV) {
-                    if (r) emo_flow_fwd_run_intv(p, iv, (unsigned)r, meta_a, tab_a, tab_row, lmask, tok, h, ea);
+                    // up to four entries at a time (the run is at most eight)
+                    unsigned ma = meta_a, ta = tab_a;
+                    for (int left = r; left > 0; left -= 4, ma += 64u, ta += 4u * tab_row) {
+                        bool ok;
+                        switch (min(left, 4)) {
+                            case 1: ok = emo_flow_fwd_run_intv<1>(iv, ma, ta, tab_row, tok, h, ea); break;
+                            case 2: ok = emo_flow_fwd_run_intv<2>(iv, ma, ta, tab_row, tok, h, ea); break;
+                            case 3: ok = emo_flow_fwd_run_intv<3>(iv, ma, ta, tab_row, tok, h, ea); break;
+                            default: ok = emo_flow_fwd_run_intv<4>(iv, ma, ta, tab_row, tok, h, ea); break;
+                        }
+                        if (!ok) emo_flow_fwd_run_intv_slow(p, iv, (unsigned)min(left, 4), ma, ta, tab_row, lmask, tok, h, ea);
+                    }
                 } else {
                     switch (r) {
                         case 1: emo_flow_fwd_run<1>(lvl_a, tab_a, tab_row, lmask, tok, h, ea); break;

@@ -65,6 +65,7 @@ struct DevSpineDir {
 };
 struct DevSpine {
     DevSpineDir f, b;
+    unsigned char *mem = nullptr;   // the allocation that holds all of it
     uint32_t *push_base = nullptr;
     int nlook = 0, chunks = 0;      // look-up entries and chunks of a stage
     int max_push = 0;
@@ -727,15 +728,26 @@ int upload_spine(const Flow &f, DevSpine &d)
         for (auto &w : walk[st]) max_rounds = std::max(max_rounds, (w.size() + 3) / 4 * 4);
     }
     d.b.s_bytes = (unsigned)(d.b.off_rec + (max_rounds + 4) * 16 * (size_t)NB);
-    std::vector<unsigned char> fW((size_t)stages * d.f.w_bytes, 0), fS((size_t)stages * d.f.s_bytes, 0), bW((size_t)stages * d.b.w_bytes, 0),
-        bS((size_t)stages * d.b.s_bytes, 0);
-    std::vector<uint32_t> rowsF((size_t)stages * d.nlook, kNone), rowsB((size_t)stages * d.nlook, kNone), pb((size_t)stages + 1);
+    // all of it in one allocation and one copy (an allocation costs about a millisecond, more than a small graph's data)
+    size_t total = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = total;
+        total += round_up(bytes, 256);
+        return at;
+    };
+    const size_t row_bytes = (size_t)stages * d.nlook * 4;
+    const size_t at_fW = part((size_t)stages * d.f.w_bytes), at_fS = part((size_t)stages * d.f.s_bytes), at_bW = part((size_t)stages * d.b.w_bytes),
+                 at_bS = part((size_t)stages * d.b.s_bytes), at_rowsF = part(row_bytes), at_rowsB = part(row_bytes), at_pb = part(((size_t)stages + 1) * 4);
+    std::vector<unsigned char> host(total, 0);
+    uint32_t *rowsF = (uint32_t *)(host.data() + at_rowsF), *rowsB = (uint32_t *)(host.data() + at_rowsB), *pb = (uint32_t *)(host.data() + at_pb);
+    std::fill(rowsF, rowsF + row_bytes / 4, kNone);
+    std::fill(rowsB, rowsB + row_bytes / 4, kNone);
     for (int st = 0; st <= stages; ++st) pb[st] = (uint32_t)sp.push_base[st];
     const uint32_t unread = sp.unread_slot * 128u;
     size_t term0 = 0;
     for (int st = 0; st < stages; ++st) {
         d.max_push = std::max(d.max_push, (int)(pb[st + 1] - pb[st]));
-        unsigned char *W = fW.data() + (size_t)st * d.f.w_bytes, *WB = bW.data() + (size_t)st * d.b.w_bytes;
+        unsigned char *W = host.data() + at_fW + (size_t)st * d.f.w_bytes, *WB = host.data() + at_bW + (size_t)st * d.b.w_bytes;
         uint32_t *tableF = (uint32_t *)W, *tableB = (uint32_t *)WB, *posF = (uint32_t *)(W + d.f.off_pos), *posB = (uint32_t *)(WB + d.b.off_pos);
         uint32_t *mem = (uint32_t *)(WB + d.b.off_mem);
         for (int e = 0; e < nmem; ++e) {      // padding: no node, folded into the slot nobody reads
@@ -781,7 +793,7 @@ int upload_spine(const Flow &f, DevSpine &d)
         for (uint32_t si : plan[st].rest) put_seg(si, er, false);
         tableB[kSpChunks + d.chunks] = (uint32_t)d.nlook | ((uint32_t)((er - d.nlook + 3) / 4 * 4) << 16) | (folds ? 0x80000000u : 0u);
 
-        uint32_t *hf = (uint32_t *)(fS.data() + (size_t)st * d.f.s_bytes), *hb = (uint32_t *)(bS.data() + (size_t)st * d.b.s_bytes);
+        uint32_t *hf = (uint32_t *)(host.data() + at_fS + (size_t)st * d.f.s_bytes), *hb = (uint32_t *)(host.data() + at_bS + (size_t)st * d.b.s_bytes);
         hf[0] = sp.f.n_ops[st] / (uint32_t)NB;
         hf[1] = (uint32_t)n_term[st];
         hf[2] = ((uint32_t)push[st].size() + 3u) / 4u * 4u;
@@ -837,22 +849,22 @@ int upload_spine(const Flow &f, DevSpine &d)
                 rec[3] = (fl & ~1u) | ((i == 0 || lane_of(i - 1) != ln) ? kSpPos_First : 0u) | ((i + 1 == w.size() || lane_of(i + 1) != ln) ? kSpPos_Last : 0u);
             }
     }
-    int rc = upload(&d.f.blobW, fW.data(), fW.size());
-    if (rc == EMO_OK) rc = upload(&d.f.blobS, fS.data(), fS.size());
-    if (rc == EMO_OK) rc = upload(&d.b.blobW, bW.data(), bW.size());
-    if (rc == EMO_OK) rc = upload(&d.b.blobS, bS.data(), bS.size());
-    if (rc == EMO_OK) rc = upload(&d.f.rows, rowsF.data(), rowsF.size() * 4);
-    if (rc == EMO_OK) rc = upload(&d.b.rows, rowsB.data(), rowsB.size() * 4);
-    if (rc == EMO_OK) rc = upload(&d.push_base, pb.data(), pb.size() * 4);
-    d.ready = rc == EMO_OK;
-    return rc;
+    const int rc = upload(&d.mem, host.data(), total);
+    if (rc != EMO_OK) return rc;
+    d.f.blobW = d.mem + at_fW;
+    d.f.blobS = d.mem + at_fS;
+    d.b.blobW = d.mem + at_bW;
+    d.b.blobS = d.mem + at_bS;
+    d.f.rows = (uint32_t *)(d.mem + at_rowsF);
+    d.b.rows = (uint32_t *)(d.mem + at_rowsB);
+    d.push_base = (uint32_t *)(d.mem + at_pb);
+    d.ready = true;
+    return EMO_OK;
 }
 
 void free_spine(DevSpine &d)
 {
-    void *all[] = {d.f.blobW, d.f.blobS, d.f.rows, d.b.blobW, d.b.blobS, d.b.rows, d.push_base};
-    for (void *q : all)
-        if (q) cudaFree(q);
+    if (d.mem) cudaFree(d.mem);
     d = DevSpine();
 }
 
