@@ -67,7 +67,7 @@ struct FlowParams {
     const long long *breaks;             // device [I]
     unsigned long long *busy;            // [rowsF][I][ldw] or NULL
     int64_t ldw;
-    unsigned off_meta;                   // inside a stage: 16 bytes per entry {lbES_v (8), group, dmin_v}
+    unsigned off_meta;                   // inside a stage: 32 bytes per entry {lbES_v (8), group, dmin_v; check (16)}
     unsigned off_brk, off_Fs;            // inside the block's shared memory: change points, columns of F
 };
 
@@ -474,12 +474,12 @@ struct FlowIntv {
     unsigned key;                // (row, interval) whose busy time is collected, not yet added to memory
     unsigned long long sum;
 };
-// End offsets below this value end inside the interval at hand (an entry of no policy: always).
-__device__ __forceinline__ unsigned emo_flow_intv_room(const FlowIntv &iv, const uint4 &meta)
+// Whether a pack that ends at offset v (c: earliest end, device, shortest duration) does not end inside the interval at hand; an
+// entry of no policy never leaves it.
+__device__ __forceinline__ bool emo_flow_intv_leaves(const FlowIntv &iv, const uint4 &c, unsigned v)
 {
-    const long long r = iv.iend - ((long long)((unsigned long long)meta.x | ((unsigned long long)meta.y << 32)) + (long long)meta.w);
-    const unsigned c = r < 0 ? 0u : (r > 0xFFFFFFFFll ? 0xFFFFFFFFu : (unsigned)r);
-    return meta.z == emo::kNone ? 0xFFFFFFFFu : (meta.z == iv.row ? c : 0u);
+    const long long room = iv.iend - (long long)((unsigned long long)c.x | ((unsigned long long)c.y << 32));
+    return c.z != emo::kNone && (c.z != iv.row || (long long)v >= room);
 }
 __device__ __forceinline__ double emo_flow_intv_energy(unsigned ta, unsigned tok)
 {
@@ -522,34 +522,63 @@ __device__ __forceinline__ void emo_flow_intv_lookup(const FlowParams &p, FlowIn
     iv.iend = iend;
     iv.row = meta.z;
 }
-// R plain entries from the interval at hand; nothing is changed when one of them leaves it in some thread.
+// An entry with start offset eo, whose pack leaves the interval at hand in some thread: the common case, into the next interval and
+// no further, at one look-up of that interval's level; anything else goes the general way.
+__device__ __forceinline__ void emo_flow_intv_cross(const FlowParams &p, FlowIntv &iv, const uint4 &meta, unsigned eo, bool out, unsigned ta0,
+                                                    unsigned lmask, unsigned tok, unsigned &dd, double &e)
+{
+    const unsigned last = meta.z * (unsigned)p.I + (unsigned)p.I - 1u;
+    const bool known = meta.z == iv.row && iv.key < last;
+    const unsigned key = known ? iv.key + 1u : iv.key;
+    const unsigned at = (emo_vld_u8(iv.Fs + key * (unsigned)p.ptile) & lmask) * 12u;
+    const unsigned dd2 = emo_tld_u32(ta0 + at, tok);
+    const double e2 = emo_flow_intv_energy(ta0 + at, tok);
+    const long long start = (long long)((unsigned long long)meta.x | ((unsigned long long)meta.y << 32)) + (long long)eo;
+    const bool late = start >= iv.iend;      // begins there
+    const long long dur = (long long)meta.w + (long long)(late ? dd2 : dd), end = start + dur;
+    const long long iend = key < last ? iv.iend + p.delta : 0x7FFFFFFFFFFFFFFFll;
+    if (__all_sync(0xFFFFFFFFu, !out || (known && end < iend))) {
+        if (out) {
+            const unsigned long long sum = iv.sum + (late ? 0ull : (unsigned long long)(iv.iend - start));
+            if (iv.count && sum) atomicAdd(p.busy + (size_t)iv.key * p.ldw + iv.b, sum);
+            iv.sum = (unsigned long long)(late ? dur : end - iv.iend);
+            iv.key = key;
+            iv.at = at;
+            iv.iend = iend;
+            dd = late ? dd2 : dd;
+            e = late ? e2 : e;
+        } else {
+            iv.sum += (unsigned long long)dur;
+        }
+    } else {
+        emo_flow_intv_lookup(p, iv, meta, eo, ta0, lmask, tok, dd, e);
+    }
+}
+// A run of R plain entries from the interval at hand: it stays in it when its last pack does (run: that pack's earliest end and
+// device, the shortest durations of all packs; an entry of no policy adds nothing to either sum).  Nothing is changed when it does
+// not in some thread.  Energies are added one by one, as where the interval changes: equal policies have equal energies
+// whatever the warp's other policies do.
 template <int R>
-__device__ __forceinline__ bool emo_flow_fwd_run_intv(FlowIntv &iv, unsigned meta_a, unsigned ta0, unsigned tab_row, unsigned tok, unsigned &h,
+__device__ __forceinline__ bool emo_flow_fwd_run_intv(FlowIntv &iv, const uint4 &run, unsigned ta0, unsigned tab_row, unsigned tok, unsigned &h,
                                                       double &ea)
 {
-    uint4 m[R];
     unsigned d[R];
     double e[R];
+    ta0 += iv.at;
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-        m[i] = emo_tld_128(meta_a + 16u * i, tok);
-        d[i] = emo_tld_u32(ta0 + (unsigned)i * tab_row + iv.at, tok);
-        e[i] = emo_flow_intv_energy(ta0 + (unsigned)i * tab_row + iv.at, tok);
+        d[i] = emo_tld_u32(ta0 + (unsigned)i * tab_row, tok);
+        e[i] = emo_flow_intv_energy(ta0 + (unsigned)i * tab_row, tok);
     }
-    unsigned v = h;
-    bool out = false;
-    unsigned long long add = 0;
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-        v += d[i];
-        out = out || v >= emo_flow_intv_room(iv, m[i]);
-        add += m[i].z != emo::kNone ? (unsigned long long)m[i].w + d[i] : 0ull;
-    }
-    if (__any_sync(0xFFFFFFFFu, out)) return false;
-    h = v;
+    for (int w = 1; w < R; w *= 2)
+#pragma unroll
+        for (int i = 0; i + w < R; i += 2 * w) d[i] += d[i + w];
+    if (__any_sync(0xFFFFFFFFu, emo_flow_intv_leaves(iv, run, h + d[0]))) return false;
+    h += d[0];
 #pragma unroll
     for (int i = 0; i < R; ++i) ea += e[i];
-    iv.sum += add;
+    iv.sum += (unsigned long long)run.w + d[0];
     return true;
 }
 // The same one by one, where the interval changes.
@@ -557,11 +586,14 @@ __device__ __forceinline__ void emo_flow_fwd_run_intv_slow(const FlowParams &p, 
                                                            unsigned tab_row, unsigned lmask, unsigned tok, unsigned &h, double &ea)
 {
 #pragma unroll 1
-    for (unsigned i = 0; i < r; ++i, meta_a += 16u, ta0 += tab_row) {
-        if (emo_flow_fwd_run_intv<1>(iv, meta_a, ta0, tab_row, tok, h, ea)) continue;
-        unsigned dd;
-        double e;
-        emo_flow_intv_lookup(p, iv, emo_tld_128(meta_a, tok), h, ta0, lmask, tok, dd, e);
+    for (unsigned i = 0; i < r; ++i, meta_a += 32u, ta0 += tab_row) {
+        const uint4 meta = emo_tld_128(meta_a, tok);
+        unsigned dd = emo_tld_u32(ta0 + iv.at, tok);
+        double e = emo_flow_intv_energy(ta0 + iv.at, tok);
+        const long long end = (long long)((unsigned long long)meta.x | ((unsigned long long)meta.y << 32)) + (long long)meta.w + (long long)(h + dd);
+        const bool out = meta.z != emo::kNone && (meta.z != iv.row || end >= iv.iend);
+        if (__any_sync(0xFFFFFFFFu, out)) emo_flow_intv_cross(p, iv, meta, h, out, ta0, lmask, tok, dd, e);
+        else iv.sum += (unsigned long long)(meta.z != emo::kNone ? meta.w : 0u) + dd;
         h += dd;
         ea += e;
     }
@@ -648,7 +680,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
             unsigned tab_a = sta + p.off_tab + (unsigned)(chain * K) * tab_row;
             unsigned lvl_a = sta + p.off_lvl + ((unsigned)((group * lanes + chain) * K) << 5) + (unsigned)lane;
             const unsigned pool_a = sta + p.off_pool;
-            unsigned meta_a = sta + p.off_meta + (unsigned)(chain * K) * 16u;
+            unsigned meta_a = sta + p.off_meta + (unsigned)(chain * K) * 32u;
             uint32_t *push = rst_lane ? rst_lane + ((size_t)hd1.z + hd1.y) * ptile : nullptr;
             hd0.x = emo_uniform(hd0.x);
             const int nseg = (int)(hd0.x & 255u);
@@ -681,14 +713,12 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                     unsigned dd = 0;
                     double ee = 0.0;
                     uint4 meta = make_uint4(0, 0, 0, 0);
-                    unsigned room = 0;
                     if (INTV) {
-                        // the level of the interval at hand, unless the entry does not follow the lane's last one in time
-                        meta = emo_tld_128(meta_a, tok);
+                        // the level of the interval at hand
+                        meta = emo_tld_128(meta_a + 16u, tok);
                         dd = emo_tld_u32(tab_a + iv.at, tok);
                         ee = emo_flow_intv_energy(tab_a + iv.at, tok);
-                        if (!(fl & emo::kF_HasReg)) iv.row = emo::kNone;
-                        room = emo_flow_intv_room(iv, meta);
+                        if (!(fl & emo::kF_HasReg)) iv.row = emo::kNone;      // the entry does not follow the lane's last one in time
                     } else {
                         const unsigned lb = emo_tld_u8(lvl_a, tok);
                         const unsigned ta = tab_a + (lb & lmask) * 12u;
@@ -727,8 +757,9 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                     }
                     v = max(v, emo_floor_sub(x0, r1.z));
                     if (INTV) {
-                        if (__any_sync(0xFFFFFFFFu, v + dd >= room)) emo_flow_intv_lookup(p, iv, meta, v, tab_a, lmask, tok, dd, ee);
-                        else iv.sum += meta.z != emo::kNone ? (unsigned long long)meta.w + dd : 0ull;
+                        const bool out = emo_flow_intv_leaves(iv, meta, v + dd);
+                        if (__any_sync(0xFFFFFFFFu, out)) emo_flow_intv_cross(p, iv, emo_tld_128(meta_a, tok), v, out, tab_a, lmask, tok, dd, ee);
+                        else iv.sum += (unsigned long long)meta.w + dd;
                     }
                     if ((fl & emo::kF_Push) && push) {
                         *push = h;
@@ -743,25 +774,27 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                         acc = emo_max64(acc, lbc + (long long)v);
                     }
                     h = v;
-                    meta_a += 16u;
+                    meta_a += 32u;
                     rec_a += 32u;
                     tab_a += tab_row;
                     lvl_a += 32u;
                 }
                 // the run: every entry continues from the lane's previous value
                 if (INTV) {
-                    // up to four entries at a time (the run is at most eight)
-                    unsigned ma = meta_a, ta = tab_a;
-                    for (int left = r; left > 0; left -= 4, ma += 64u, ta += 4u * tab_row) {
-                        bool ok;
-                        switch (min(left, 4)) {
-                            case 1: ok = emo_flow_fwd_run_intv<1>(iv, ma, ta, tab_row, tok, h, ea); break;
-                            case 2: ok = emo_flow_fwd_run_intv<2>(iv, ma, ta, tab_row, tok, h, ea); break;
-                            case 3: ok = emo_flow_fwd_run_intv<3>(iv, ma, ta, tab_row, tok, h, ea); break;
-                            default: ok = emo_flow_fwd_run_intv<4>(iv, ma, ta, tab_row, tok, h, ea); break;
-                        }
-                        if (!ok) emo_flow_fwd_run_intv_slow(p, iv, (unsigned)min(left, 4), ma, ta, tab_row, lmask, tok, h, ea);
+                    const uint4 run = emo_tld_128(meta_a + 16u, tok);      // (an empty run's is not looked at; it lies inside the stage buffer)
+                    bool ok = true;
+                    switch (r) {
+                        case 1: ok = emo_flow_fwd_run_intv<1>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        case 2: ok = emo_flow_fwd_run_intv<2>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        case 3: ok = emo_flow_fwd_run_intv<3>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        case 4: ok = emo_flow_fwd_run_intv<4>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        case 5: ok = emo_flow_fwd_run_intv<5>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        case 6: ok = emo_flow_fwd_run_intv<6>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        case 7: ok = emo_flow_fwd_run_intv<7>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        case 8: ok = emo_flow_fwd_run_intv<8>(iv, run, tab_a, tab_row, tok, h, ea); break;
+                        default: break;
                     }
+                    if (!ok) emo_flow_fwd_run_intv_slow(p, iv, (unsigned)r, meta_a, tab_a, tab_row, lmask, tok, h, ea);
                 } else {
                     switch (r) {
                         case 1: emo_flow_fwd_run<1>(lvl_a, tab_a, tab_row, lmask, tok, h, ea); break;
@@ -775,7 +808,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                         default: break;
                     }
                 }
-                meta_a += (unsigned)r * 16u;
+                meta_a += (unsigned)r * 32u;
                 rec_a += (unsigned)r * 32u;
                 tab_a += (unsigned)r * tab_row;
                 lvl_a += (unsigned)r * 32u;

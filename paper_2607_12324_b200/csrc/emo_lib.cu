@@ -44,7 +44,7 @@ struct DevProgramLane {
 // The lane-stream program on the device: one blob per stage and direction (see emo_flow.cuh).
 struct DevFlow {
     unsigned char *blobF = nullptr, *blobB = nullptr;
-    unsigned char *blobFI = nullptr;      // the forward blob followed by 16 bytes per entry {lbES_v, group, dmin_v}: time-interval policies
+    unsigned char *blobFI = nullptr;      // the forward blob followed by 32 bytes per entry: time-interval policies
     uint32_t *rows = nullptr, *push_base = nullptr;
     unsigned blobF_bytes = 0, blobB_bytes = 0, blobFI_bytes = 0, f_off_meta = 0;
     unsigned off_seg = 0;
@@ -569,16 +569,41 @@ int upload_flow(const Flow &f, DevFlow &d, bool intervals)
     if (rc == EMO_OK) rc = upload(&d.blobB, bb.data(), bb.size());
     if (rc == EMO_OK && intervals) {
         d.f_off_meta = d.blobF_bytes;
-        d.blobFI_bytes = (unsigned)r16(d.f_off_meta + per * 16);
+        // per entry {lbES_v, group, dmin_v} and what tells whether the entry, or the run of plain entries that begins with it, ends inside
+        // an interval: {earliest end of its last pack, that pack's group, shortest durations of all packs}; a run over several
+        // groups (or 32 bits) names a group that no policy has and goes entry by entry.  One more entry is read behind the last.
+        d.blobFI_bytes = (unsigned)r16(d.f_off_meta + (per + 1) * 32);
         std::vector<unsigned char> bi((size_t)f.stages * d.blobFI_bytes, 0);
         for (int st = 0; st < f.stages; ++st) {
             unsigned char *dst = bi.data() + (size_t)st * d.blobFI_bytes;
             std::memcpy(dst, bf.data() + (size_t)st * d.blobF_bytes, d.blobF_bytes);
-            for (size_t e = 0; e < per; ++e) {
-                const size_t q = (size_t)st * per + e;
-                const int64_t lb = f.lbes[q];
-                const uint32_t w[4] = {(uint32_t)(uint64_t)lb, (uint32_t)((uint64_t)lb >> 32), f.grp[q], f.dmin[q]};
-                std::memcpy(dst + d.f_off_meta + e * 16, w, 16);
+            for (int ln = 0; ln < f.lanes; ++ln) {
+                size_t e = (size_t)ln * f.K;
+                auto check = [&](size_t first, size_t count) {
+                    uint32_t grp = kNone;
+                    uint64_t dsum = 0;
+                    int64_t end = 0;
+                    for (size_t j = first; j < first + count; ++j) {
+                        const size_t q = (size_t)st * per + j;
+                        const int64_t lb = f.lbes[q];
+                        const uint32_t w[4] = {(uint32_t)(uint64_t)lb, (uint32_t)((uint64_t)lb >> 32), f.grp[q], f.dmin[q]};
+                        std::memcpy(dst + d.f_off_meta + j * 32, w, 16);
+                        if (f.grp[q] == kNone) continue;
+                        grp = (grp == kNone || grp == f.grp[q]) ? f.grp[q] : kNone - 1u;
+                        end = lb + (int64_t)f.dmin[q];
+                        dsum += f.dmin[q];
+                    }
+                    if (dsum > 0xFFFFFFFFull) grp = kNone - 1u;
+                    const uint32_t w[4] = {(uint32_t)(uint64_t)end, (uint32_t)((uint64_t)end >> 32), grp, (uint32_t)dsum};
+                    std::memcpy(dst + d.f_off_meta + first * 32 + 16, w, 16);
+                };
+                const int nseg = (int)(f.hdr[((size_t)st * f.lanes + ln) * kHdrWords] & 255u);
+                for (int i = 0; i < nseg; ++i) {
+                    const uint32_t sg = f.f.seg[((size_t)st * f.lanes + ln) * kSegBytes + i];
+                    if (sg & kSegSpecial) check(e++, 1);
+                    if (sg & kSegRunMask) check(e, sg & kSegRunMask);
+                    e += sg & kSegRunMask;
+                }
             }
         }
         rc = upload(&d.blobFI, bi.data(), bi.size());
