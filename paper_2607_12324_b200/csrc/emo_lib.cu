@@ -2236,8 +2236,13 @@ int emo_pack_model(int32_t n_packs, int32_t n_metrics, int32_t m, int32_t L, con
     if (n_packs < 0 || n_metrics < 1 || m < 1 || m > kModelMaxM || L < 1) return EMO_E_INVALID_ARG;
     if (n_packs == 0) return EMO_OK;
     if (!Bmat || !feat || !Tb || !Eb || !x || !T_out || !E_out) return EMO_E_INVALID_ARG;
-    const size_t smem = ((size_t)m * m + (size_t)n_metrics * m + 2 * (size_t)m * L) * sizeof(double);
-    if (smem > 48 * 1024) return EMO_E_UNSUPPORTED;
+    const size_t smem = ((size_t)n_metrics * m + 2 * (size_t)m * L) * sizeof(double);
+    if (smem + (size_t)m * m * sizeof(double) > 48 * 1024) return EMO_E_UNSUPPORTED;
+    int dev = 0, sms = 0;
+    EMO_CUDA(cudaGetDevice(&dev));
+    EMO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // with its own arrays the kernel passes what a launch has without asking
+    if (smem > 40 * 1024) EMO_CUDA(cudaFuncSetAttribute(emo_pack_model_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ModelParams p;
     p.n_packs = n_packs;
     p.n = n_metrics;
@@ -2254,7 +2259,9 @@ int emo_pack_model(int32_t n_packs, int32_t n_metrics, int32_t m, int32_t L, con
     cudaStream_t st = (cudaStream_t)stream;
     cudaEvent_t ev0 = g_pass_events[0], ev1 = g_pass_events[1];
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
-    emo_pack_model_kernel<<<(unsigned)((n_packs + 127) / 128), 128, smem, st>>>(p);
+    const int per_block = kModelThreads / 16;
+    const int blocks = std::min((n_packs + per_block - 1) / per_block, 3 * std::max(sms, 1));
+    emo_pack_model_kernel<<<(unsigned)blocks, kModelThreads, smem, st>>>(p);
     EMO_CUDA(cudaGetLastError());
     if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
     return EMO_OK;

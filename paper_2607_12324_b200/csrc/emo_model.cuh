@@ -18,22 +18,41 @@ struct ModelParams {
     int32_t *status;
 };
 
-// One thread per pack.  The problem is tiny (m <= 16 unknowns) and every pack is independent; the Gram matrix
-// G = B^T B is the same for all packs and is built once per block in shared memory, so a pack costs B^T b, the
-// active-set iterations on (G, c) and the two weighted sums.
+// Half a warp per pack, lane i for unknown i (m <= 16).  The Gram matrix G = B^T B is the same for all packs; every block builds
+// it once in shared memory and then takes packs in turn.
 //
 // Active-set method of Lawson and Hanson on the normal equations: start from x = 0 with every variable held at
 // zero; move the variable with the largest positive gradient component w = c - G x into the free set; solve
-// the free set's equations G_PP z = c_P (Cholesky); while z has non-positive entries step from x towards z as
+// the free set's equations G_PP z = c_P; while z has non-positive entries step from x towards z as
 // far as feasibility allows and return the variables that reach zero to the held set; accept z; repeat until no
 // gradient component is positive.  Every accepted x lowers the objective, so the loop ends; it is also bounded
 // by 3 m outer and 3 m inner rounds (status -9 otherwise: never seen).
-__global__ void __launch_bounds__(128) emo_pack_model_kernel(ModelParams p)
+//
+// The equations are never solved anew: the lanes keep the rows of the dictionary
+//     basic_i = b_i - sum_j a_ij nonbasic_j        (x_i is basic where i is free, the residual r_i = (c - G x)_i where it is held)
+// in registers, and a variable that changes sides is one principal pivot, m fused multiply-adds per lane with the pivot's row
+// broadcast through shared memory.  b then holds z on the free set and w on the held one.  A dictionary of a symmetric matrix is
+// symmetric up to the sign between free and held, which gives every lane its entry of the pivot column from the pivot's row.
+// One step of iterative refinement against G at the end takes out what the pivots' roundings left (a_PP is the inverse of G_PP).
+//
+// Measured, 14 694 packs of 16 metrics, 12 unknowns and 32 levels: one thread per pack with a factorisation in local memory per
+// step 500 us (115 blocks of four warps, every operand through L1); this one 48 us; 200 000 packs 0.46 ms.
+constexpr int kModelThreads = 256, kModelRow = 18;      // scratch row of a pack: 16 entries and b, padded to keep two rows off each other's banks
+
+__device__ __forceinline__ double emo_model_half_max(double v)
 {
-    extern __shared__ double emo_model_smem[];
+#pragma unroll
+    for (int o = 8; o; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+
+__global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelParams p)
+{
+    extern __shared__ __align__(16) double emo_model_smem[];
+    __shared__ __align__(16) double G[kModelMaxM * kModelMaxM];
+    __shared__ __align__(16) double rows[kModelThreads / 16 * kModelRow];
     const int m = p.m, n = p.n, L = p.L;
-    double *G = emo_model_smem;                    // [m][m]
-    double *Bs = G + m * m;                        // [n][m]
+    double *Bs = emo_model_smem;                   // [n][m]
     double *Ts = Bs + n * m;                       // [m][L]
     double *Es = Ts + m * L;                       // [m][L]
     for (int i = threadIdx.x; i < n * m; i += blockDim.x) Bs[i] = p.B[i];
@@ -42,119 +61,132 @@ __global__ void __launch_bounds__(128) emo_pack_model_kernel(ModelParams p)
         Es[i] = p.Eb[i];
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < m * m; i += blockDim.x) {
-        const int a = i / m, b = i - a * m;
+    for (int i = threadIdx.x; i < kModelMaxM * kModelMaxM; i += blockDim.x) {
+        const int a = i / kModelMaxM, b = i % kModelMaxM;
         double s = 0.0;
-        for (int r = 0; r < n; ++r) s += Bs[r * m + a] * Bs[r * m + b];
+        if (a < m && b < m)
+            for (int r = 0; r < n; ++r) s += Bs[r * m + a] * Bs[r * m + b];
         G[i] = s;
     }
     __syncthreads();
-    const int pk = blockIdx.x * blockDim.x + threadIdx.x;
-    if (pk >= p.n_packs) return;
-
-    double c[kModelMaxM], x[kModelMaxM], z[kModelMaxM], Lc[kModelMaxM * kModelMaxM];
-    int idx[kModelMaxM];
-    unsigned free_set = 0;
-    double cmax = 0.0;
-    for (int i = 0; i < m; ++i) {
-        double s = 0.0;
-        for (int r = 0; r < n; ++r) s += Bs[r * m + i] * p.feat[(size_t)pk * n + r];
-        c[i] = s;
-        x[i] = 0.0;
-        cmax = fmax(cmax, fabs(s));
-    }
-    const double tol = 1e-13 * (cmax > 0.0 ? cmax : 1.0);
-    bool failed = false;
-    for (int outer = 0; outer < 3 * m; ++outer) {
-        // the held variable with the largest gradient component
-        int j = -1;
-        double wj = tol;
-        for (int i = 0; i < m; ++i) {
-            if (free_set & (1u << i)) continue;
-            double w = c[i];
-            for (int k = 0; k < m; ++k) w -= G[i * m + k] * x[k];
-            if (w > wj) {
-                wj = w;
-                j = i;
-            }
-        }
-        if (j < 0) break;
-        free_set |= 1u << j;
-        bool accepted = false;
-        for (int inner = 0; inner < 3 * m && !accepted; ++inner) {
+    constexpr unsigned kFull = 0xFFFFFFFFu;
+    const int me = threadIdx.x & 15, half = (threadIdx.x & 31) >> 4;
+    const int mc = min(me, m - 1);                 // lanes beyond the unknowns shadow the last one and are never chosen
+    double *row = rows + (threadIdx.x / 16) * kModelRow;
+    const unsigned stride = gridDim.x * (blockDim.x / 16), n_packs = (unsigned)p.n_packs;
+    // both halves of a warp go round together
+    for (unsigned base = (blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / 16; base < n_packs; base += stride) {
+        const bool live = base + (unsigned)half < n_packs;
+        const size_t pk = (size_t)(live ? base + half : base);
+        double c = 0.0;
+        for (int r = 0; r < n; ++r) c += Bs[r * m + mc] * p.feat[pk * n + r];
+        if (me >= m) c = 0.0;
+        const double cmax = emo_model_half_max(fabs(c));
+        const double tol = 1e-13 * (cmax > 0.0 ? cmax : 1.0);
+        double a[kModelMaxM], b = c, x = 0.0;
+#pragma unroll
+        for (int j = 0; j < kModelMaxM; ++j) a[j] = G[j * kModelMaxM + me];
+        bool is_free = false, done = !live, failed = false;
+        unsigned leaving = 0;                      // variables of this pack still to be returned to the held set
+        int outer = 0, inner = 0;
+        while (__any_sync(kFull, !done)) {
+            // the next pivot: a variable that leaves, else the held one with the largest gradient component, the first among equals
+            const double w = (!is_free && me < m && b > tol) ? b : 0.0;
+            const double best = emo_model_half_max(w);
+            const unsigned who = (__ballot_sync(kFull, w > 0.0 && w == best) >> (16 * half)) & 0xFFFFu;
+            const unsigned free_set = (__ballot_sync(kFull, is_free) >> (16 * half)) & 0xFFFFu;
             int k = 0;
-            for (int i = 0; i < m; ++i)
-                if (free_set & (1u << i)) idx[k++] = i;
-            // Cholesky of G_PP, then the two triangular solves
-            bool ok = true;
-            for (int a = 0; a < k && ok; ++a)
-                for (int b = 0; b <= a; ++b) {
-                    double s = G[idx[a] * m + idx[b]];
-                    for (int q = 0; q < b; ++q) s -= Lc[a * kModelMaxM + q] * Lc[b * kModelMaxM + q];
-                    if (a == b) {
-                        if (s <= 1e-14 * G[idx[a] * m + idx[a]]) { ok = false; break; }
-                        Lc[a * kModelMaxM + a] = sqrt(s);
-                    } else {
-                        Lc[a * kModelMaxM + b] = s / Lc[b * kModelMaxM + b];
-                    }
+            if (leaving) {
+                k = __ffs(leaving) - 1;
+                leaving &= leaving - 1u;
+            } else if (!done) {
+                if (who == 0u || outer == 3 * m) done = true;
+                else {
+                    k = __ffs(who) - 1;
+                    ++outer;
+                    inner = 0;
                 }
-            if (!ok) {
-                // the new column depends on the free ones: it cannot improve the fit, hold it again
-                free_set &= ~(1u << j);
-                accepted = true;
-                break;
             }
-            for (int a = 0; a < k; ++a) {
-                double s = c[idx[a]];
-                for (int q = 0; q < a; ++q) s -= Lc[a * kModelMaxM + q] * z[q];
-                z[a] = s / Lc[a * kModelMaxM + a];
+            const bool k_free = (free_set >> k) & 1u;
+            if (!done && me == k) {
+                double2 *o = reinterpret_cast<double2 *>(row);
+#pragma unroll
+                for (int j = 0; j < kModelMaxM; j += 2) o[j / 2] = make_double2(a[j], a[j + 1]);
+                row[kModelMaxM] = b;
             }
-            for (int a = k - 1; a >= 0; --a) {
-                double s = z[a];
-                for (int q = a + 1; q < k; ++q) s -= Lc[q * kModelMaxM + a] * z[q];
-                z[a] = s / Lc[a * kModelMaxM + a];
+            __syncwarp();
+            const double d = row[k];
+            double f = row[me];
+            // a column that depends on the free ones cannot improve the fit, and no other one has a larger component
+            if (!done && !k_free && d <= 1e-14 * G[k * (kModelMaxM + 1)]) done = true;
+            __syncwarp();
+            if (!done && me == k) row[k] = 1.0;
+            __syncwarp();
+            if (!done) {
+                const double inv = 1.0 / d;
+                f = me == k ? -inv : (is_free == k_free ? f * inv : -(f * inv));
+                const unsigned clear = me == k ? 0xFFFFu : 1u << k;
+                const double2 *o = reinterpret_cast<const double2 *>(row);
+#pragma unroll
+                for (int j = 0; j < kModelMaxM; j += 2) {
+                    const double2 q = o[j / 2];
+                    a[j] = ((clear >> j) & 1u ? 0.0 : a[j]) - f * q.x;
+                    a[j + 1] = ((clear >> (j + 1)) & 1u ? 0.0 : a[j + 1]) - f * q.y;
+                }
+                b = (me == k ? 0.0 : b) - f * row[kModelMaxM];
+                if (me == k) is_free = !is_free;
             }
+            __syncwarp();
             // feasible?  otherwise the longest step towards z that keeps x >= 0
+            const bool solved = !done && leaving == 0u, bad = solved && is_free && b <= 0.0;
             double alpha = 2.0;
-            for (int a = 0; a < k; ++a)
-                if (z[a] <= 0.0) {
-                    const double xa = x[idx[a]];
-                    alpha = fmin(alpha, xa / (xa - z[a]));
-                }
-            if (alpha > 1.0) {
-                for (int a = 0; a < k; ++a) x[idx[a]] = z[a];
-                accepted = true;
-            } else {
-                for (int a = 0; a < k; ++a) {
-                    const int i = idx[a];
-                    x[i] += alpha * (z[a] - x[i]);
-                    if (x[i] <= 0.0 || (z[a] <= 0.0 && x[i] <= 1e-300)) {
-                        x[i] = 0.0;
-                        free_set &= ~(1u << i);
-                    }
-                }
-                // the variable that set alpha is exactly at zero up to rounding: make sure it leaves
-                for (int a = 0; a < k; ++a) {
-                    const int i = idx[a];
-                    if ((free_set & (1u << i)) && z[a] <= 0.0 && x[i] <= 1e-15 * fabs(z[a])) {
-                        x[i] = 0.0;
-                        free_set &= ~(1u << i);
-                    }
-                }
+            if (__any_sync(kFull, bad)) alpha = -emo_model_half_max(bad ? -(x / (x - b)) : -2.0);
+            const bool step = solved && alpha <= 1.0;
+            if (solved && !step && is_free) x = b;
+            bool out = false;
+            if (step && is_free) {
+                const bool bound = bad && x / (x - b) == alpha;      // exactly at zero up to rounding: it leaves
+                x += alpha * (b - x);
+                out = bound || x <= 0.0 || (b <= 0.0 && (x <= 1e-300 || x <= 1e-15 * fabs(b)));
+                if (out) x = 0.0;
+            }
+            const unsigned outs = (__ballot_sync(kFull, out) >> (16 * half)) & 0xFFFFu;
+            if (step) {
+                leaving = outs;
+                if (++inner == 3 * m) failed = done = true;
             }
         }
-        if (!accepted) { failed = true; break; }
-    }
-    if (failed && p.status) atomicMin(p.status, -9);
-    for (int i = 0; i < m; ++i) p.x[(size_t)pk * m + i] = x[i];
-    // Eq. 7
-    for (int l = 0; l < L; ++l) {
-        double t = 0.0, e = 0.0;
-        for (int i = 0; i < m; ++i) {
-            t += x[i] * Ts[i * L + l];
-            e += x[i] * Es[i * L + l];
+        if (failed && live && me == 0 && p.status) atomicMin(p.status, -9);
+        row[me] = x;
+        __syncwarp();
+        double r = c;
+#pragma unroll
+        for (int j = 0; j < kModelMaxM; ++j) r -= G[j * kModelMaxM + me] * row[j];
+        __syncwarp();
+        row[me] = is_free ? r : 0.0;
+        __syncwarp();
+        if (is_free && !failed) {
+            double dx = 0.0;
+#pragma unroll
+            for (int j = 0; j < kModelMaxM; ++j) dx += a[j] * row[j];
+            x = fmax(x + dx, 0.0);
         }
-        p.T_out[(size_t)pk * L + l] = t;
-        p.E_out[(size_t)pk * L + l] = e;
+        __syncwarp();
+        row[me] = x;
+        __syncwarp();
+        if (live) {
+            if (me < m) p.x[pk * m + me] = x;
+            // Eq. 7
+            for (int l = me; l < L; l += 16) {
+                double t = 0.0, e = 0.0;
+                for (int i = 0; i < m; ++i) {
+                    t += row[i] * Ts[i * L + l];
+                    e += row[i] * Es[i * L + l];
+                }
+                p.T_out[pk * L + l] = t;
+                p.E_out[pk * L + l] = e;
+            }
+        }
+        __syncwarp();
     }
 }
