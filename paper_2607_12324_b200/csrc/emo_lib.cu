@@ -81,6 +81,8 @@ struct emo_graph {
     DevFlow dflow;
     Flow sflow;                      // the same graph compiled with short stages and its spine program (sflow.spine.ok: usable)
     DevSpine dspine;
+    Flow lflow;                      // ... and once more with longer stages, for calls of at most two policy groups per SM
+    DevSpine dlong;
     bool host_only = false;
     // graphs beyond the schedule compilers' limits (or loaded with EMO_F_GENERIC): evaluated by the generic kernels
     bool generic = false;
@@ -1079,11 +1081,9 @@ struct SpinePlan {
     size_t restore_bytes = 0;
 };
 
-bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+bool spine_plan_for(const emo_graph *g, const Flow &f, const DevSpine &d, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
 {
-    const Flow &f = g->sflow;
     const Spine &sp = f.spine;
-    const DevSpine &d = g->dspine;
     pl.ok = false;
     if (!f.ok32 || !sp.ok || !d.ready || !g->smem_optin || f.stages == 0) return false;
     const int64_t NBf = B + (want_base ? 1 : 0);
@@ -1186,6 +1186,17 @@ bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, Sp
     return false;
 }
 
+// Up to two policy groups per SM a block has shared memory to spare and its stages are bound by latency: the program with the
+// longer stages.  Measured (both passes, ms, long / short stages): 10 000 nodes x 4 096 policies 0.60 / 0.77, x 9 000 0.69 / 0.86;
+// 25 000 x 2 000 0.78 / 0.83, x 8 192 1.03 / 1.07; 1 013 x 4 096 0.085 / 0.096.  Above that the larger buffers cost tiles or stages in
+// flight: 1 013 x 65 536 0.50 / 0.36.  On wide graphs only up to one group: 18 lanes, 51 000 x 1 000 1.82 / 2.09, x 8 192 2.7 / 2.49.
+bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+{
+    const int64_t n_groups = (B + (want_base ? 1 : 0) + 31) / 32;
+    if (n_groups <= (g->lflow.lanes > 8 ? 1 : 2) * (int64_t)g->sm_count && spine_plan_for(g, g->lflow, g->dlong, B, want_base, need_bwd, pl)) return true;
+    return spine_plan_for(g, g->sflow, g->dspine, B, want_base, need_bwd, pl);
+}
+
 int launch_spine_fwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const uint8_t *lvl, int64_t ldb, uint32_t *restore,
                      int64_t *makespan, double *energy, int64_t *base_T, double *base_E, int32_t *status, uint32_t flags,
                      cudaStream_t st)
@@ -1270,10 +1281,11 @@ bool spine_allowed(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ld
     // Measured (both passes, ms, spine / the best of the others): 1 013 nodes x 65 536 policies 0.36 / 0.90; 10 000 x 4 096
     // 0.77 / 2.30; 75 000 x 10 001 forward 1.28 / 1.89; 250 000 x 16 384 15.0 / 20.4.  On wide graphs one warp carries the
     // recurrence of all lanes: 18 lanes, 128 039 nodes x 8 192 policies (two groups per SM) 6.2 / 9.05; 51 000 x 333 to
-    // 4 500 (one group) 2.09 / 2.05 and 6 400 nodes 0.31 / 0.30, so there the others stay.
+    // 4 500 (one group) 2.09 / 2.05 and 6 400 nodes 0.31 / 0.30 with stages of four positions, so there the others stay; with the
+    // program of longer stages 1.82 and 0.25.
     if (!(flags & EMO_F_SPINE_KERNEL)) {
         const int64_t per_sm = ((B + 1 + 31) / 32 + g->sm_count - 1) / std::max(g->sm_count, 1);
-        if (g->sflow.lanes > 8 && per_sm < 2) return false;
+        if (g->sflow.lanes > 8 && per_sm < 2 && !g->dlong.ready) return false;
     }
     return ldb % 16 == 0 && aligned16(lvl) && ldb < big && ldo < big;
 }
@@ -1550,9 +1562,16 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             // says otherwise; compiled on a thread of its own beside the lane-stream program (they share nothing but
             // their inputs)
             const bool want_spine = !(flags & EMO_F_INTERVALS);
-            int rc_s = EMO_OK;
-            std::string err_s;
-            std::thread spine_thread;
+            int rc_s = EMO_OK, rc_l = EMO_E_UNSUPPORTED;
+            std::string err_s, err_l;
+            std::thread spine_thread, long_thread;
+            auto compile_spine = [&](int k, Flow &out, int &rc_k, std::string &err_k) {
+                try {
+                    rc_k = compile_flow(h, lat, energy, lanes, look, k, k, out, err_k, true);
+                } catch (const std::bad_alloc &) {
+                    rc_k = EMO_E_OOM;
+                }
+            };
             if (want_spine) {
                 const int code = (int)((flags >> 30) & 3u);
                 // Measured (forward + backward, ms): 18 lanes, 128 039 nodes x 8 192 policies 6.2 with 4 positions, 6.6 with 5
@@ -1560,13 +1579,13 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 // 16, 17.2 with 12; 1 013 x 65 536 0.36 with 16, 0.48 with 20 and 0.43 with 8.
                 int sk = code == 1 ? 8 : (code == 3 ? 32 : (code == 2 || flanes <= 8 ? 16 : 4));
                 while (sk > 8 && flanes * sk > 32 * kFlowRowRegs) sk /= 2;
-                spine_thread = std::thread([&, sk]() {
-                    try {
-                        rc_s = compile_flow(h, lat, energy, lanes, look, sk, sk, g->sflow, err_s, true);
-                    } catch (const std::bad_alloc &) {
-                        rc_s = EMO_E_OOM;
-                    }
-                });
+                spine_thread = std::thread([&, sk]() { compile_spine(sk, g->sflow, rc_s, err_s); });
+                // the long stages: as many positions as keep a stage at about a hundred entries (25 000 nodes, 5 lanes x 2 000
+                // policies: 20 positions 0.78 ms, 16 0.83; 10 000, 3 lanes x 4 096: 32 0.60, 24 0.66; 51 000, 18 lanes x 1 000: 7 1.82,
+                // 6 1.90, 5 1.96)
+                const int lk = std::min(32, (flanes > 8 ? 126 : 100) / flanes);
+                if (code == 0 && lk > sk && !(flags & EMO_F_HOST_ONLY))
+                    long_thread = std::thread([&, lk]() { compile_spine(lk, g->lflow, rc_l, err_l); });
             }
             try {
                 rc = compile_flow(h, lat, energy, lanes, look, fk, fs, g->flow, err);
@@ -1574,11 +1593,13 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 rc = EMO_E_OOM;
             }
             if (spine_thread.joinable()) spine_thread.join();
+            if (long_thread.joinable()) long_thread.join();
             if (rc == EMO_E_UNSUPPORTED) {      // the 64-bit programs exist: they serve
                 g->flow = Flow();
                 rc = EMO_OK;
             }
             if (rc == EMO_OK && rc_s != EMO_OK && rc_s != EMO_E_UNSUPPORTED) rc = rc_s;
+            if (rc == EMO_OK && rc_l == EMO_E_OOM) rc = rc_l;
             if (rc != EMO_OK) { delete g; return rc; }
             if (!want_spine || rc_s != EMO_OK || !g->flow.ok32 || !g->sflow.spine.ok) g->sflow = Flow();
             else {
@@ -1586,6 +1607,17 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 g->sflow.f = FlowDir();
                 g->sflow.b = FlowDir();
             }
+            // (a tail is folded only over a distance of two stages: where long stages leave fewer folds the program has more
+            // operations, and the short one is faster: 25 000 nodes with 21 positions 59 000 operations, 1.7 ms, with 20 15 000, 0.78 ms)
+            auto operations = [](const Spine &s2) {
+                int64_t c = 0;
+                for (uint32_t k : s2.f.n_ops) c += k;
+                for (uint32_t k : s2.b.n_ops) c += k;
+                return c;
+            };
+            if (rc_l != EMO_OK || !g->sflow.spine.ok || !g->lflow.spine.ok || operations(g->lflow.spine) > operations(g->sflow.spine) * 5 / 4) g->lflow = Flow();
+            g->lflow.f = FlowDir();
+            g->lflow.b = FlowDir();
         }
         std::vector<int32_t> hop((size_t)std::max(n, 1), 0);
         int32_t depth = 0;
@@ -1660,6 +1692,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             }
         }
         if (rc == EMO_OK) rc = upload_spine(g->sflow, g->dspine);
+        if (rc == EMO_OK) rc = upload_spine(g->lflow, g->dlong);
         }
         } catch (const std::bad_alloc &) {
             rc = EMO_E_OOM;
@@ -1680,6 +1713,7 @@ int emo_graph_free(emo_graph *g)
         free_program_lane(g->lbwd);
         free_flow(g->dflow);
         free_spine(g->dspine);
+        free_spine(g->dlong);
         void *gen[] = {g->gen_row_ptr, g->gen_col, g->gen_srow_ptr, g->gen_scol, g->gen_group, g->gen_lat, g->gen_energy};
         for (void *q : gen)
             if (q) cudaFree(q);
@@ -1918,7 +1952,8 @@ int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint3
             need = spill_need(g, B);
         SpinePlan sp;
         if (!g->host_only && B > 0 && spine_allowed(g, B, fake, aligned ? 16 : 1, 0, flags) && spine_plan(g, B, true, true, sp))
-            need = std::max(need, sp.restore_bytes);
+            // (rows of the larger of the two programs: a smaller batch may take the other one)
+            need = std::max(need, sp.restore_bytes / (size_t)sp.pf.restore_rows * (size_t)std::max(sp.pf.restore_rows, g->lflow.spine.pushes + g->lflow.lanes) + 256);
         bytes += need;
     }
     if (need_slack == 2) bytes += 4 * round_up((size_t)B * 8, 256) + 256;
