@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                         }
                     }
                     v = max(v, emo_floor_sub(x0, r1.z));
-                    if (INTV) {
+                    if (INTV && meta.z != emo::kNone) {
                         const bool out = emo_flow_intv_leaves(iv, meta, v + dd);
                         if (__any_sync(0xFFFFFFFFu, out)) emo_flow_intv_cross(p, iv, emo_tld_128(meta_a, tok), v, out, tab_a, lmask, tok, dd, ee);
                         else iv.sum += (unsigned long long)meta.w + dd;

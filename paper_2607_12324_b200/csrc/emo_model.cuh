@@ -36,7 +36,8 @@ struct ModelParams {
 // One step of iterative refinement against G at the end takes out what the pivots' roundings left (a_PP is the inverse of G_PP).
 //
 // Measured, 14 694 packs of 16 metrics, 12 unknowns and 32 levels: one thread per pack with a factorisation in local memory per
-// step 500 us (115 blocks of four warps, every operand through L1); this one 48 us; 200 000 packs 0.46 ms.
+// step 500 us (115 blocks of four warps, every operand through L1); this one 48 us; 200 000 packs 0.42 ms (0.46 with a case for the pivot's row and
+// column in every update: the selects were a third of its instructions).
 constexpr int kModelThreads = 256, kModelRow = 18;      // scratch row of a pack: 16 entries and b, padded to keep two rows off each other's banks
 
 __device__ __forceinline__ double emo_model_half_max(double v)
@@ -50,6 +51,7 @@ __global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelP
 {
     extern __shared__ __align__(16) double emo_model_smem[];
     __shared__ __align__(16) double G[kModelMaxM * kModelMaxM];
+    __shared__ double unit[kModelMaxM];
     __shared__ __align__(16) double rows[kModelThreads / 16 * kModelRow];
     const int m = p.m, n = p.n, L = p.L;
     double *Bs = emo_model_smem;                   // [n][m]
@@ -69,8 +71,18 @@ __global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelP
         G[i] = s;
     }
     __syncthreads();
+    // every unknown in units of a power of two that brings its diagonal entry to [1/2, 2): exact, and no pivot of an entering
+    // variable is above 2
+    if (threadIdx.x < kModelMaxM) {
+        const double g = G[threadIdx.x * (kModelMaxM + 1)];
+        unit[threadIdx.x] = (g > 0.0 && g < 1e300) ? ldexp(1.0, -(ilogb(g) / 2)) : 1.0;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kModelMaxM * kModelMaxM; i += blockDim.x) G[i] *= unit[i / kModelMaxM] * unit[i % kModelMaxM];
+    __syncthreads();
     constexpr unsigned kFull = 0xFFFFFFFFu;
     const int me = threadIdx.x & 15, half = (threadIdx.x & 31) >> 4;
+    const double scale = unit[me], unscale = 1.0 / scale;
     const int mc = min(me, m - 1);                 // lanes beyond the unknowns shadow the last one and are never chosen
     double *row = rows + (threadIdx.x / 16) * kModelRow;
     const unsigned stride = gridDim.x * (blockDim.x / 16), n_packs = (unsigned)p.n_packs;
@@ -83,6 +95,7 @@ __global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelP
         if (me >= m) c = 0.0;
         const double cmax = emo_model_half_max(fabs(c));
         const double tol = 1e-13 * (cmax > 0.0 ? cmax : 1.0);
+        c *= scale;
         double a[kModelMaxM], b = c, x = 0.0;
 #pragma unroll
         for (int j = 0; j < kModelMaxM; ++j) a[j] = G[j * kModelMaxM + me];
@@ -91,7 +104,7 @@ __global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelP
         int outer = 0, inner = 0;
         while (__any_sync(kFull, !done)) {
             // the next pivot: a variable that leaves, else the held one with the largest gradient component, the first among equals
-            const double w = (!is_free && me < m && b > tol) ? b : 0.0;
+            const double grad = b * unscale, w = (!is_free && me < m && grad > tol) ? grad : 0.0;
             const double best = emo_model_half_max(w);
             const unsigned who = (__ballot_sync(kFull, w > 0.0 && w == best) >> (16 * half)) & 0xFFFFu;
             const unsigned free_set = (__ballot_sync(kFull, is_free) >> (16 * half)) & 0xFFFFu;
@@ -120,22 +133,40 @@ __global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelP
             // a column that depends on the free ones cannot improve the fit, and no other one has a larger component
             if (!done && !k_free && d <= 1e-14 * G[k * (kModelMaxM + 1)]) done = true;
             __syncwarp();
-            if (!done && me == k) row[k] = 1.0;
-            __syncwarp();
-            if (!done) {
-                const double inv = 1.0 / d;
-                f = me == k ? -inv : (is_free == k_free ? f * inv : -(f * inv));
-                const unsigned clear = me == k ? 0xFFFFu : 1u << k;
-                const double2 *o = reinterpret_cast<const double2 *>(row);
+            const bool go = !done;
+            const double inv = 1.0 / d;
+            const double2 *o = reinterpret_cast<const double2 *>(row);
+            if (!__any_sync(kFull, go && k_free)) {
+                // a variable enters: with d + 1 in the pivot's place every entry is one fused multiply-add, without a case for the
+                // pivot's row (a - (1 - inv) a = inv a) or column (f - f inv (d + 1) = -f inv); nothing cancels, d being at most 2
+                if (go && me == k) row[k] = d + 1.0;
+                __syncwarp();
+                if (go) {
+                    f = me == k ? 1.0 - inv : (is_free ? -(f * inv) : f * inv);
 #pragma unroll
-                for (int j = 0; j < kModelMaxM; j += 2) {
-                    const double2 q = o[j / 2];
-                    a[j] = ((clear >> j) & 1u ? 0.0 : a[j]) - f * q.x;
-                    a[j + 1] = ((clear >> (j + 1)) & 1u ? 0.0 : a[j + 1]) - f * q.y;
+                    for (int j = 0; j < kModelMaxM; j += 2) {
+                        const double2 q = o[j / 2];
+                        a[j] -= f * q.x;
+                        a[j + 1] -= f * q.y;
+                    }
+                    b -= f * row[kModelMaxM];
                 }
-                b = (me == k ? 0.0 : b) - f * row[kModelMaxM];
-                if (me == k) is_free = !is_free;
+            } else {
+                if (go && me == k) row[k] = 1.0;
+                __syncwarp();
+                if (go) {
+                    f = me == k ? -inv : (is_free == k_free ? f * inv : -(f * inv));
+                    const unsigned clear = me == k ? 0xFFFFu : 1u << k;
+#pragma unroll
+                    for (int j = 0; j < kModelMaxM; j += 2) {
+                        const double2 q = o[j / 2];
+                        a[j] = ((clear >> j) & 1u ? 0.0 : a[j]) - f * q.x;
+                        a[j + 1] = ((clear >> (j + 1)) & 1u ? 0.0 : a[j + 1]) - f * q.y;
+                    }
+                    b = (me == k ? 0.0 : b) - f * row[kModelMaxM];
+                }
             }
+            if (go && me == k) is_free = !is_free;
             __syncwarp();
             // feasible?  otherwise the longest step towards z that keeps x >= 0
             const bool solved = !done && leaving == 0u, bad = solved && is_free && b <= 0.0;
@@ -171,6 +202,7 @@ __global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelP
             for (int j = 0; j < kModelMaxM; ++j) dx += a[j] * row[j];
             x = fmax(x + dx, 0.0);
         }
+        x *= scale;
         __syncwarp();
         row[me] = x;
         __syncwarp();
