@@ -2378,7 +2378,8 @@ int emo_slack(const emo_graph *g, const uint8_t *lvl_one, int64_t *ES, int64_t *
     // per-node outputs are written at pitch 1 directly
     uint8_t *lv = (uint8_t *)ws + kSmallWs;
     const size_t rows = (size_t)std::max(g->h.rows, 1);
-    EMO_CUDA(cudaMemcpy2DAsync(lv, 16, lvl_one, 1, 1, rows, cudaMemcpyDeviceToDevice, st));
+    emo_spread_levels<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(lvl_one, lv, (int64_t)rows);
+    EMO_CUDA(cudaGetLastError());
     double *e = energy ? energy : (double *)((char *)ws + 1024);
     return emo_slack_batch(g, 1, lv, 16, ES, LS, slack, 1, makespan, e, nullptr, nullptr, nullptr, nullptr, ws, ws_bytes,
                            status, 0, stream);
