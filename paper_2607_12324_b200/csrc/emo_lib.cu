@@ -1663,6 +1663,19 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             g->host_lat = std::vector<int64_t>();
             g->host_energy = std::vector<double>();
         } else {
+        // the spine programs are laid out and copied beside the others (250 000 nodes: a quarter of a second each)
+        int rc_u[2] = {EMO_OK, EMO_OK};
+        auto upload_beside = [&](const Flow &f, DevSpine &d, int &rc_k) {
+            try {
+                rc_k = cudaSetDevice(dev) == cudaSuccess ? upload_spine(f, d) : EMO_E_CUDA;
+            } catch (const std::bad_alloc &) {
+                rc_k = EMO_E_OOM;
+            }
+        };
+        struct Joined {      // (joined whatever is thrown meanwhile)
+            std::thread t;
+            ~Joined() { if (t.joinable()) t.join(); }
+        } up_short{std::thread([&]() { upload_beside(g->sflow, g->dspine, rc_u[0]); })}, up_long{std::thread([&]() { upload_beside(g->lflow, g->dlong, rc_u[1]); })};
         rc = upload_program(g->fwd, g->dfwd);
         if (rc == EMO_OK) rc = upload_program(g->bwd, g->dbwd);
         if (rc == EMO_OK && g->fwd.lanes <= 32 - kProducerWarps && g->bwd.lanes <= 32 - kProducerWarps) {
@@ -1691,8 +1704,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 if (rc == EMO_OK) rc = upload_flow(g->flow, g->dflow, (flags & EMO_F_INTERVALS) != 0);
             }
         }
-        if (rc == EMO_OK) rc = upload_spine(g->sflow, g->dspine);
-        if (rc == EMO_OK) rc = upload_spine(g->lflow, g->dlong);
+        up_short.t.join();
+        up_long.t.join();
+        for (int k : rc_u)
+            if (rc == EMO_OK) rc = k;
         }
         } catch (const std::bad_alloc &) {
             rc = EMO_E_OOM;
