@@ -56,6 +56,11 @@ __host__ __device__ inline int64_t emo_budget(int64_t T0, int64_t ppm)
     return T0 + q * ppm + (r * ppm) / M;
 }
 
+// Kernels of one call that follow each other are launched ahead of their predecessor's end: its blocks allow that when they have
+// started, and what depends on its results waits here for all of it.
+__device__ __forceinline__ void emo_grid_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void emo_grid_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // One policy's levels, a byte per row, to rows of 16 bytes (the pitch that the pass kernels fetch); the other columns belong to no
 // policy.  A pitched copy moves such rows one by one: 250 000 rows 145 us, here 3.
 __global__ void emo_spread_levels(const uint8_t *in, uint8_t *out, int64_t rows)
@@ -276,6 +281,8 @@ __global__ void emo_select_stage1(int64_t B, const int64_t *makespan, const doub
                                   const int64_t *target_dev, int64_t delta_ppm, SelectPartial *part)
 {
     __shared__ SelectPartial sh[32];
+    emo_grid_allow_next();
+    emo_grid_wait_previous();
     if (target_dev) target = emo_budget(target_dev[0], delta_ppm);
     double e = 0.0;
     long long idx = -1;
@@ -293,6 +300,7 @@ __global__ void emo_select_stage2(int nparts, const SelectPartial *part, const i
                                   int64_t *out_index, int64_t *out_T, double *out_E)
 {
     __shared__ SelectPartial sh[32];
+    emo_grid_wait_previous();
     double e = 0.0;
     long long idx = -1;
     for (int i = threadIdx.x; i < nparts; i += blockDim.x) {

@@ -993,6 +993,24 @@ bool flow_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, Flo
     return false;
 }
 
+// Launches a kernel that may start before its predecessor in the stream ends (it waits for it where it needs it).  Measured:
+// 400 nodes x 64, forward, backward and selection, 41 us one after the other, 34 ahead.
+template <typename... A>
+cudaError_t launch_ahead(void (*kern)(A...), int grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, args...);
+}
+
 // The opt-in shared-memory size is set once per kernel (not per launch: concurrent callers with
 // different batch sizes would otherwise race on the attribute).
 template <typename K>
@@ -1265,8 +1283,7 @@ int launch_spine_bwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const u
     else EMO_PICK_S(4, 4, 2, 640);
 #undef EMO_PICK_S
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
-    kern<<<pl.grid_b, pl.threads_b, pl.smem_b, st>>>(p);
-    EMO_CUDA(cudaGetLastError());
+    EMO_CUDA(launch_ahead(kern, pl.grid_b, pl.threads_b, pl.smem_b, st, p));
     if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
     return EMO_OK;
 }
@@ -2422,10 +2439,8 @@ int emo_select(int64_t B, const int64_t *makespan, const double *energy, int64_t
     cudaStream_t st = (cudaStream_t)stream;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((B + 1023) / 1024, kSelectMaxBlocks));
     SelectPartial *part = (SelectPartial *)ws;
-    emo_select_stage1<<<blocks, 256, 0, st>>>(B, makespan, energy, target, target_dev, delta_ppm, part);
-    EMO_CUDA(cudaGetLastError());
-    emo_select_stage2<<<1, 256, 0, st>>>(blocks, part, makespan, out_index, out_T, out_E);
-    EMO_CUDA(cudaGetLastError());
+    EMO_CUDA(launch_ahead(emo_select_stage1, blocks, 256, 0, st, B, makespan, energy, target, target_dev, delta_ppm, part));
+    EMO_CUDA(launch_ahead(emo_select_stage2, 1, 256, 0, st, blocks, (const SelectPartial *)part, makespan, out_index, out_T, out_E));
     return EMO_OK;
 }
 
@@ -2459,10 +2474,8 @@ int emo_select_static(int64_t B, const int64_t *makespan, const double *energy, 
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((B + 1023) / 1024, kSelectMaxBlocks));
     // stage 1 overwrites the first `blocks` candidates and stage 2 reads exactly those, so nothing
     // left behind by an earlier call is ever read and nothing needs clearing
-    emo_select_stage1<<<blocks, 256, 0, st>>>(B, makespan, energy, target, target_dev, delta_ppm, part);
-    EMO_CUDA(cudaGetLastError());
-    emo_select_stage2<<<1, 256, 0, st>>>(blocks, part, makespan, out_index, out_T, out_E);
-    EMO_CUDA(cudaGetLastError());
+    EMO_CUDA(launch_ahead(emo_select_stage1, blocks, 256, 0, st, B, makespan, energy, target, target_dev, delta_ppm, part));
+    EMO_CUDA(launch_ahead(emo_select_stage2, 1, 256, 0, st, blocks, (const SelectPartial *)part, makespan, out_index, out_T, out_E));
     return EMO_OK;
 }
 

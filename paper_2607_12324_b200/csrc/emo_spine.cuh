@@ -285,6 +285,7 @@ __device__ __forceinline__ void emo_spine_produce(const SpineParams &p, unsigned
             rst_first = __ldg(p.push_base + st);
             rst_rows = __ldg(p.push_base + st + 1) - rst_first;
         }
+        if (BWD && which == 0 && c == nbuf) emo_grid_wait_previous();      // (no wait for other warps runs while these may not)
         const long long tw0 = EMO_SCLK();
         bool ok = c < nbuf || emo_spine_wait(emo_spine_bar(bar0, empty_k, s), ring.par ^ 1, abort_word, p.wait_cycles);
         ok = ok && (which != 0 || emo_spine_wait(emo_spine_bar(bar0, kBarRows, rrow.idx), rrow.par, abort_word, p.wait_cycles));
@@ -305,6 +306,7 @@ __device__ __forceinline__ void emo_spine_produce(const SpineParams &p, unsigned
             if (lane == 0) {
                 const unsigned dst = smem0 + p.off_s0 + (unsigned)s * p.sbuf_bytes, rst_bytes = rst_rows * P * 4u;
                 emo_mbar_expect_tx(full, p.s_bytes + rst_bytes);
+                if (BWD && c == 0) asm volatile("fence.proxy.async;" ::: "memory");      // the restore list was written by ordinary stores
                 emo_bulk_g2s(dst, p.blobS + (size_t)st * p.s_bytes, p.s_bytes, full);
                 if (BWD && rst_bytes)
                     emo_bulk_g2s(dst + p.off_rst, p.restore + ((size_t)blockIdx.x * p.restore_rows + rst_first) * P, rst_bytes, full);
@@ -543,6 +545,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_fwd(SpineParams p)
     const unsigned smem0 = emo_smem_addr(emo_smem), bar0 = smem0 + p.off_bar;
     volatile int *abort_word = reinterpret_cast<volatile int *>(emo_smem + p.off_bar + kBarKinds * kSpRing * 8);
     const long long limit = p.wait_cycles;
+    emo_grid_allow_next();               // the backward kernel's blocks may take SMs that are free
     emo_spine_init(p, emo_smem, bar0, spines, subs, false);
 
     long long T[VS];
@@ -851,7 +854,10 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_bwd(SpineParams p)
     const unsigned smem0 = emo_smem_addr(emo_smem), bar0 = smem0 + p.off_bar;
     volatile int *abort_word = reinterpret_cast<volatile int *>(emo_smem + p.off_bar + kBarKinds * kSpRing * 8);
     const long long limit = p.wait_cycles;
+    emo_grid_allow_next();
     emo_spine_init(p, emo_smem, bar0, spines, subs, true);
+    // everything but the first loads of level rows and tables waits for the forward kernel
+    if (!(role.prod && role.idx == 0)) emo_grid_wait_previous();
 
     bool failed = false;
     long long ssum[VW];
