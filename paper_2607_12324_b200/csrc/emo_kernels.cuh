@@ -65,6 +65,7 @@ __device__ __forceinline__ void emo_grid_wait_previous() { asm volatile("griddep
 // policy.  A pitched copy moves such rows one by one: 250 000 rows 145 us, here 3.
 __global__ void emo_spread_levels(const uint8_t *in, uint8_t *out, int64_t rows)
 {
+    emo_grid_allow_next();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < rows) out[i * 16] = in[i];
 }

@@ -631,11 +631,17 @@ void free_flow(DevFlow &d)
 // look-up warps share a stage evenly (250 000 nodes, 55 look-up entries per stage: five chunks).
 constexpr int kSpChunkTarget = 12;
 
+// The spine program as the device gets it: one allocation, one copy.
+struct SpineImage {
+    std::vector<unsigned char> host;
+    size_t at_fW = 0, at_fS = 0, at_bW = 0, at_bS = 0, at_rowsF = 0, at_rowsB = 0, at_pb = 0;
+};
+
 // Lays the spine program out for the kernels.  A stage's look-up entries are the members of its segments that depend on
 // the level (or carry energy), dealt to the chunks by length, longest segment first; the members of the other segments
 // follow behind them (backward: they only store).  Backward the members of a segment lie last to first.  Sums are
 // numbered compactly forward (segments whose sum is never read have none) and by segment backward.
-int upload_spine(const Flow &f, DevSpine &d)
+int lay_out_spine(const Flow &f, DevSpine &d, SpineImage &im)
 {
     const Spine &sp = f.spine;
     if (!f.ok32 || !sp.ok || f.stages == 0) return EMO_OK;
@@ -763,10 +769,16 @@ int upload_spine(const Flow &f, DevSpine &d)
         return at;
     };
     const size_t row_bytes = (size_t)stages * d.nlook * 4;
-    const size_t at_fW = part((size_t)stages * d.f.w_bytes), at_fS = part((size_t)stages * d.f.s_bytes), at_bW = part((size_t)stages * d.b.w_bytes),
-                 at_bS = part((size_t)stages * d.b.s_bytes), at_rowsF = part(row_bytes), at_rowsB = part(row_bytes), at_pb = part(((size_t)stages + 1) * 4);
-    std::vector<unsigned char> host(total, 0);
-    uint32_t *rowsF = (uint32_t *)(host.data() + at_rowsF), *rowsB = (uint32_t *)(host.data() + at_rowsB), *pb = (uint32_t *)(host.data() + at_pb);
+    im.at_fW = part((size_t)stages * d.f.w_bytes);
+    im.at_fS = part((size_t)stages * d.f.s_bytes);
+    im.at_bW = part((size_t)stages * d.b.w_bytes);
+    im.at_bS = part((size_t)stages * d.b.s_bytes);
+    im.at_rowsF = part(row_bytes);
+    im.at_rowsB = part(row_bytes);
+    im.at_pb = part(((size_t)stages + 1) * 4);
+    std::vector<unsigned char> &host = im.host;
+    host.assign(total, 0);
+    uint32_t *rowsF = (uint32_t *)(host.data() + im.at_rowsF), *rowsB = (uint32_t *)(host.data() + im.at_rowsB), *pb = (uint32_t *)(host.data() + im.at_pb);
     std::fill(rowsF, rowsF + row_bytes / 4, kNone);
     std::fill(rowsB, rowsB + row_bytes / 4, kNone);
     for (int st = 0; st <= stages; ++st) pb[st] = (uint32_t)sp.push_base[st];
@@ -774,7 +786,7 @@ int upload_spine(const Flow &f, DevSpine &d)
     size_t term0 = 0;
     for (int st = 0; st < stages; ++st) {
         d.max_push = std::max(d.max_push, (int)(pb[st + 1] - pb[st]));
-        unsigned char *W = host.data() + at_fW + (size_t)st * d.f.w_bytes, *WB = host.data() + at_bW + (size_t)st * d.b.w_bytes;
+        unsigned char *W = host.data() + im.at_fW + (size_t)st * d.f.w_bytes, *WB = host.data() + im.at_bW + (size_t)st * d.b.w_bytes;
         uint32_t *tableF = (uint32_t *)W, *tableB = (uint32_t *)WB, *posF = (uint32_t *)(W + d.f.off_pos), *posB = (uint32_t *)(WB + d.b.off_pos);
         uint32_t *mem = (uint32_t *)(WB + d.b.off_mem);
         for (int e = 0; e < nmem; ++e) {      // padding: no node, folded into the slot nobody reads
@@ -820,7 +832,7 @@ int upload_spine(const Flow &f, DevSpine &d)
         for (uint32_t si : plan[st].rest) put_seg(si, er, false);
         tableB[kSpChunks + d.chunks] = (uint32_t)d.nlook | ((uint32_t)((er - d.nlook + 3) / 4 * 4) << 16) | (folds ? 0x80000000u : 0u);
 
-        uint32_t *hf = (uint32_t *)(host.data() + at_fS + (size_t)st * d.f.s_bytes), *hb = (uint32_t *)(host.data() + at_bS + (size_t)st * d.b.s_bytes);
+        uint32_t *hf = (uint32_t *)(host.data() + im.at_fS + (size_t)st * d.f.s_bytes), *hb = (uint32_t *)(host.data() + im.at_bS + (size_t)st * d.b.s_bytes);
         hf[0] = sp.f.n_ops[st] / (uint32_t)NB;
         hf[1] = (uint32_t)n_term[st];
         hf[2] = ((uint32_t)push[st].size() + 3u) / 4u * 4u;
@@ -876,15 +888,21 @@ int upload_spine(const Flow &f, DevSpine &d)
                 rec[3] = (fl & ~1u) | ((i == 0 || lane_of(i - 1) != ln) ? kSpPos_First : 0u) | ((i + 1 == w.size() || lane_of(i + 1) != ln) ? kSpPos_Last : 0u);
             }
     }
-    const int rc = upload(&d.mem, host.data(), total);
+    return EMO_OK;
+}
+
+int upload_spine(const SpineImage &im, DevSpine &d)
+{
+    if (im.host.empty()) return EMO_OK;
+    const int rc = upload(&d.mem, im.host.data(), im.host.size());
     if (rc != EMO_OK) return rc;
-    d.f.blobW = d.mem + at_fW;
-    d.f.blobS = d.mem + at_fS;
-    d.b.blobW = d.mem + at_bW;
-    d.b.blobS = d.mem + at_bS;
-    d.f.rows = (uint32_t *)(d.mem + at_rowsF);
-    d.b.rows = (uint32_t *)(d.mem + at_rowsB);
-    d.push_base = (uint32_t *)(d.mem + at_pb);
+    d.f.blobW = d.mem + im.at_fW;
+    d.f.blobS = d.mem + im.at_fS;
+    d.b.blobW = d.mem + im.at_bW;
+    d.b.blobS = d.mem + im.at_bS;
+    d.f.rows = (uint32_t *)(d.mem + im.at_rowsF);
+    d.b.rows = (uint32_t *)(d.mem + im.at_rowsB);
+    d.push_base = (uint32_t *)(d.mem + im.at_pb);
     d.ready = true;
     return EMO_OK;
 }
@@ -994,7 +1012,7 @@ bool flow_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, Flo
 }
 
 // Launches a kernel that may start before its predecessor in the stream ends (it waits for it where it needs it).  Measured:
-// 400 nodes x 64, forward, backward and selection, 41 us one after the other, 34 ahead.
+// 400 nodes x 64, forward, backward and selection, 41 us one after the other, 31 ahead.
 template <typename... A>
 cudaError_t launch_ahead(void (*kern)(A...), int grid, int threads, size_t smem, cudaStream_t st, A... args)
 {
@@ -1241,8 +1259,7 @@ int launch_spine_fwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const u
     else if (pl.vw == 2) kern = wide ? emo_spine_fwd<2, 4, 4, 512> : emo_spine_fwd<2, 2, 2, 512>;
     else kern = wide ? emo_spine_fwd<4, 4, 4, 640> : emo_spine_fwd<4, 4, 2, 640>;
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
-    kern<<<pl.grid_f, pl.threads_f, pl.smem_f, st>>>(p);
-    EMO_CUDA(cudaGetLastError());
+    EMO_CUDA(launch_ahead(kern, pl.grid_f, pl.threads_f, pl.smem_f, st, p));
     if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
     return EMO_OK;
 }
@@ -1469,6 +1486,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
     const int64_t m = row_ptr[n];
     if (m > 0 && !col) return EMO_E_INVALID_ARG;
     int32_t max_span = 0;
+    SpineImage image_s, image_l;
     for (int32_t v = 0; v < n; ++v)
         for (int64_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
             if (col[e] < 0 || col[e] >= n) return EMO_E_INVALID_ARG;
@@ -1582,9 +1600,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             int rc_s = EMO_OK, rc_l = EMO_E_UNSUPPORTED;
             std::string err_s, err_l;
             std::thread spine_thread, long_thread;
-            auto compile_spine = [&](int k, Flow &out, int &rc_k, std::string &err_k) {
+            auto compile_spine = [&](int k, Flow &out, DevSpine &d, SpineImage &im, int &rc_k, std::string &err_k) {
                 try {
                     rc_k = compile_flow(h, lat, energy, lanes, look, k, k, out, err_k, true);
+                    if (rc_k == EMO_OK && !(flags & EMO_F_HOST_ONLY)) rc_k = lay_out_spine(out, d, im);
                 } catch (const std::bad_alloc &) {
                     rc_k = EMO_E_OOM;
                 }
@@ -1596,13 +1615,13 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 // 16, 17.2 with 12; 1 013 x 65 536 0.36 with 16, 0.48 with 20 and 0.43 with 8.
                 int sk = code == 1 ? 8 : (code == 3 ? 32 : (code == 2 || flanes <= 8 ? 16 : 4));
                 while (sk > 8 && flanes * sk > 32 * kFlowRowRegs) sk /= 2;
-                spine_thread = std::thread([&, sk]() { compile_spine(sk, g->sflow, rc_s, err_s); });
+                spine_thread = std::thread([&, sk]() { compile_spine(sk, g->sflow, g->dspine, image_s, rc_s, err_s); });
                 // the long stages: as many positions as keep a stage at about a hundred entries (25 000 nodes, 5 lanes x 2 000
                 // policies: 20 positions 0.78 ms, 16 0.83; 10 000, 3 lanes x 4 096: 32 0.60, 24 0.66; 51 000, 18 lanes x 1 000: 7 1.82,
                 // 6 1.90, 5 1.96)
                 const int lk = std::min(32, (flanes > 8 ? 126 : 100) / flanes);
                 if (code == 0 && lk > sk && !(flags & EMO_F_HOST_ONLY))
-                    long_thread = std::thread([&, lk]() { compile_spine(lk, g->lflow, rc_l, err_l); });
+                    long_thread = std::thread([&, lk]() { compile_spine(lk, g->lflow, g->dlong, image_l, rc_l, err_l); });
             }
             try {
                 rc = compile_flow(h, lat, energy, lanes, look, fk, fs, g->flow, err);
@@ -1680,19 +1699,6 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             g->host_lat = std::vector<int64_t>();
             g->host_energy = std::vector<double>();
         } else {
-        // the spine programs are laid out and copied beside the others (250 000 nodes: a quarter of a second each)
-        int rc_u[2] = {EMO_OK, EMO_OK};
-        auto upload_beside = [&](const Flow &f, DevSpine &d, int &rc_k) {
-            try {
-                rc_k = cudaSetDevice(dev) == cudaSuccess ? upload_spine(f, d) : EMO_E_CUDA;
-            } catch (const std::bad_alloc &) {
-                rc_k = EMO_E_OOM;
-            }
-        };
-        struct Joined {      // (joined whatever is thrown meanwhile)
-            std::thread t;
-            ~Joined() { if (t.joinable()) t.join(); }
-        } up_short{std::thread([&]() { upload_beside(g->sflow, g->dspine, rc_u[0]); })}, up_long{std::thread([&]() { upload_beside(g->lflow, g->dlong, rc_u[1]); })};
         rc = upload_program(g->fwd, g->dfwd);
         if (rc == EMO_OK) rc = upload_program(g->bwd, g->dbwd);
         if (rc == EMO_OK && g->fwd.lanes <= 32 - kProducerWarps && g->bwd.lanes <= 32 - kProducerWarps) {
@@ -1721,10 +1727,8 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 if (rc == EMO_OK) rc = upload_flow(g->flow, g->dflow, (flags & EMO_F_INTERVALS) != 0);
             }
         }
-        up_short.t.join();
-        up_long.t.join();
-        for (int k : rc_u)
-            if (rc == EMO_OK) rc = k;
+        if (rc == EMO_OK && g->sflow.spine.ok) rc = upload_spine(image_s, g->dspine);
+        if (rc == EMO_OK && g->lflow.spine.ok) rc = upload_spine(image_l, g->dlong);
         }
         } catch (const std::bad_alloc &) {
             rc = EMO_E_OOM;

@@ -547,6 +547,7 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_fwd(SpineParams p)
     const long long limit = p.wait_cycles;
     emo_grid_allow_next();               // the backward kernel's blocks may take SMs that are free
     emo_spine_init(p, emo_smem, bar0, spines, subs, false);
+    emo_grid_wait_previous();            // (who wrote the levels; nothing in memory was touched so far)
 
     long long T[VS];
     double ea[VW];
