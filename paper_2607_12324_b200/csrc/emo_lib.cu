@@ -2225,14 +2225,15 @@ int emo_search_dp(const emo_graph *g, int32_t I, const int64_t *breaks, const do
         std::vector<double> hE((size_t)max_batch);
         // Pred of a chunk of candidates (policy c = cand[c], the same levels for every device row)
         auto predict = [&](const std::vector<const uint8_t *> &cand, const std::vector<std::pair<int32_t, uint8_t>> &patch) -> int {
-            const int64_t nb = (int64_t)cand.size();
+            // (rows as long as this chunk: a round has hundreds of candidates, the workspace room for thousands)
+            const int64_t nb = (int64_t)cand.size(), ld = (int64_t)round_up((size_t)nb, 16);
             for (int r = 0; r < rows; ++r)
                 for (int32_t i = 0; i < I; ++i) {
-                    uint8_t *dst = &hF[((size_t)r * I + i) * ldb];
+                    uint8_t *dst = &hF[((size_t)r * I + i) * ld];
                     for (int64_t c = 0; c < nb; ++c) dst[c] = (patch[c].first == i) ? patch[c].second : cand[c][i];
                 }
-            if (cudaMemcpyAsync(dF, hF.data(), hF.size(), cudaMemcpyHostToDevice, st) != cudaSuccess) return EMO_E_CUDA;
-            int rc = emo_eval_intervals(g, nb, dF, ldb, I, breaks, p_idle, dT, dE, nullptr, iws, iws_bytes, nullptr, 0, stream);
+            if (cudaMemcpyAsync(dF, hF.data(), (size_t)rows * I * ld, cudaMemcpyHostToDevice, st) != cudaSuccess) return EMO_E_CUDA;
+            int rc = emo_eval_intervals(g, nb, dF, ld, I, breaks, p_idle, dT, dE, nullptr, iws, iws_bytes, nullptr, 0, stream);
             if (rc) return rc;
             if (cudaMemcpyAsync(hT.data(), dT, (size_t)nb * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) return EMO_E_CUDA;
             if (cudaMemcpyAsync(hE.data(), dE, (size_t)nb * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) return EMO_E_CUDA;
