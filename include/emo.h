@@ -524,6 +524,14 @@ int emo_graph_flow(const emo_graph *g, emo_flow_view *out);
  * slots, most segments of a stage, 4-byte words of sums per policy and stage, restore rows.  Host memory. */
 int emo_graph_spine(const emo_graph *g, int64_t out[12]);
 
+/* The launch of the spine kernels that B policies would get on a device of sm_count SMs with smem_bytes of shared memory per
+ * block: out[0] = 1 if there is one (else the rest is 0), 1 for the program with the longer stages, its lanes, steps per
+ * stage, stages and operations per bundle, the bundle and most threads of the kernels that are launched, policy groups of 32
+ * per block, policies per worker and per spine thread, threads per block (the larger of the two passes).  Host-only handles
+ * answer too; it launches nothing. */
+int emo_graph_spine_plan(const emo_graph *g, int64_t B, int need_slack, int want_base, int32_t sm_count, int64_t smem_bytes,
+                         int64_t out[12]);
+
 /* The spine program itself, as pointers into the handle's host memory (valid until emo_graph_free; for the host-side
  * tests of the compiler, which interpret it).  Arrays: n_ops_fwd / n_ops_bwd [stages]; ops_fwd [stages][max_ops_fwd][8]
  * = {operand slot 0, its correction, operand slot 1, its correction, the lane's slot, published slot, offset of the

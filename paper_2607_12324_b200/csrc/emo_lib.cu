@@ -69,7 +69,13 @@ struct DevSpine {
     uint32_t *push_base = nullptr;
     int nlook = 0, chunks = 0;      // look-up entries and chunks of a stage
     int max_push = 0;
-    bool ready = false;
+    bool ready = false;             // on the device (host-only handles: laid out)
+};
+
+// The spine program as the device gets it: one allocation, one copy.
+struct SpineImage {
+    std::vector<unsigned char> host;
+    size_t at_fW = 0, at_fS = 0, at_bW = 0, at_bS = 0, at_rowsF = 0, at_rowsB = 0, at_pb = 0;
 };
 
 struct emo_graph {
@@ -83,6 +89,7 @@ struct emo_graph {
     DevSpine dspine;
     Flow lflow;                      // ... and once more with longer stages, for calls of at most two policy groups per SM
     DevSpine dlong;
+    SpineImage simage, limage;       // both as laid out for the device (kept by host-only handles, else until they are copied)
     bool host_only = false;
     // graphs beyond the schedule compilers' limits (or loaded with EMO_F_GENERIC): evaluated by the generic kernels
     bool generic = false;
@@ -631,12 +638,6 @@ void free_flow(DevFlow &d)
 // look-up warps share a stage evenly (250 000 nodes, 55 look-up entries per stage: five chunks).
 constexpr int kSpChunkTarget = 12;
 
-// The spine program as the device gets it: one allocation, one copy.
-struct SpineImage {
-    std::vector<unsigned char> host;
-    size_t at_fW = 0, at_fS = 0, at_bW = 0, at_bS = 0, at_rowsF = 0, at_rowsB = 0, at_pb = 0;
-};
-
 // Lays the spine program out for the kernels.  A stage's look-up entries are the members of its segments that depend on
 // the level (or carry energy), dealt to the chunks by length, longest segment first; the members of the other segments
 // follow behind them (backward: they only store).  Backward the members of a segment lie last to first.  Sums are
@@ -1110,22 +1111,40 @@ int launch_flow_bwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const uin
 // to two groups, else four (bundles of four, 8 threads per operation: always four, so that a row of 32 policies is one
 // conflict-free access of those threads).
 struct SpinePlan {
-    bool ok = false;
+    bool ok = false, is_long = false;
     int groups = 0, vw = 1, vs = 1, grid_f = 0, grid_b = 0, threads_f = 0, threads_b = 0;
+    const struct SpineKernels *k = nullptr;
     SpineParams pf, pb;
     size_t smem_f = 0, smem_b = 0;
     size_t restore_bytes = 0;
 };
 
-bool spine_plan_for(const emo_graph *g, const Flow &f, const DevSpine &d, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+// The kernels of one shape.  The operations of a program come in bundles of its own size (the two programs of a graph are
+// scheduled apart, so their lanes and with them their bundles may differ): a plan names the kernels of its program's.
+struct SpineKernels {
+    int vw, vs, nb, max_threads;
+    void (*fwd)(SpineParams), (*bwd)(SpineParams), (*bwd_extra)(SpineParams);
+};
+template <int VW, int VS, int NB, int MAXT>
+constexpr SpineKernels spine_kernels() { return {VW, VS, NB, MAXT, emo_spine_fwd<VW, VS, NB, MAXT>, emo_spine_bwd<VW, VS, NB, MAXT, false>, emo_spine_bwd<VW, VS, NB, MAXT, true>}; }
+const SpineKernels kSpineKernels[] = {spine_kernels<1, 2, 2, 512>(), spine_kernels<2, 2, 2, 512>(), spine_kernels<4, 4, 2, 640>(),
+                                      spine_kernels<1, 4, 4, 512>(), spine_kernels<2, 4, 4, 512>(), spine_kernels<4, 4, 4, 640>()};
+
+// What a launch shape depends on beside the program and the batch.
+struct SpineChip {
+    int sm_count;
+    size_t smem;
+};
+
+bool spine_plan_for(const emo_graph *g, const SpineChip &chip, const Flow &f, const DevSpine &d, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
 {
     const Spine &sp = f.spine;
     pl.ok = false;
-    if (!f.ok32 || !sp.ok || !d.ready || !g->smem_optin || f.stages == 0) return false;
+    if (!f.ok32 || !sp.ok || !d.ready || !chip.smem || f.stages == 0) return false;
     const int64_t NBf = B + (want_base ? 1 : 0);
     const int64_t n_groups = (NBf + 31) / 32;
-    const int64_t want = (n_groups + g->sm_count - 1) / g->sm_count;
-    const size_t budget = g->smem_optin;
+    const int64_t want = (n_groups + chip.sm_count - 1) / chip.sm_count;
+    const size_t budget = chip.smem;
     int G0 = 1;
     const int gmax = sp.bundle > 2 ? 4 : 8;
     while (G0 < gmax && G0 < want) G0 *= 2;
@@ -1210,6 +1229,10 @@ bool spine_plan_for(const emo_graph *g, const Flow &f, const DevSpine &d, int64_
         };
         if (!shape(false, pl.pf, pl.smem_f, pl.threads_f)) continue;
         if (need_bwd && !shape(true, pl.pb, pl.smem_b, pl.threads_b)) continue;
+        pl.k = nullptr;
+        for (const SpineKernels &k : kSpineKernels)
+            if (k.vw == VW && k.vs == VS && k.nb == sp.bundle && pl.threads_f <= k.max_threads && (!need_bwd || pl.threads_b <= k.max_threads)) pl.k = &k;
+        if (!pl.k) continue;
         pl.groups = G;
         pl.vw = VW;
         pl.vs = VS;
@@ -1226,11 +1249,16 @@ bool spine_plan_for(const emo_graph *g, const Flow &f, const DevSpine &d, int64_
 // longer stages.  Measured (both passes, ms, long / short stages): 10 000 nodes x 4 096 policies 0.60 / 0.77, x 9 000 0.69 / 0.86;
 // 25 000 x 2 000 0.78 / 0.83, x 8 192 1.03 / 1.07; 1 013 x 4 096 0.085 / 0.096.  Above that the larger buffers cost tiles or stages in
 // flight: 1 013 x 65 536 0.50 / 0.36.  On wide graphs only up to one group: 18 lanes, 51 000 x 1 000 1.82 / 2.09, x 8 192 2.7 / 2.49.
-bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+bool spine_plan_on(const emo_graph *g, const SpineChip &chip, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
 {
     const int64_t n_groups = (B + (want_base ? 1 : 0) + 31) / 32;
-    if (n_groups <= (g->lflow.lanes > 8 ? 1 : 2) * (int64_t)g->sm_count && spine_plan_for(g, g->lflow, g->dlong, B, want_base, need_bwd, pl)) return true;
-    return spine_plan_for(g, g->sflow, g->dspine, B, want_base, need_bwd, pl);
+    pl.is_long = n_groups <= (g->lflow.lanes > 8 ? 1 : 2) * (int64_t)chip.sm_count && spine_plan_for(g, chip, g->lflow, g->dlong, B, want_base, need_bwd, pl);
+    return pl.is_long || spine_plan_for(g, chip, g->sflow, g->dspine, B, want_base, need_bwd, pl);
+}
+
+bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+{
+    return spine_plan_on(g, SpineChip{g->sm_count, g->smem_optin}, B, want_base, need_bwd, pl);
 }
 
 int launch_spine_fwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const uint8_t *lvl, int64_t ldb, uint32_t *restore,
@@ -1253,11 +1281,7 @@ int launch_spine_fwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const u
     if (flags & EMO_F_TEST_STALL) p.stall_stage = p.stages / 2;
     cudaEvent_t ev0 = g_pass_events[0], ev1 = g_pass_events[1];
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
-    const bool wide = g->sflow.spine.bundle > 2;
-    void (*kern)(SpineParams) = nullptr;
-    if (pl.vw == 1) kern = wide ? emo_spine_fwd<1, 4, 4, 512> : emo_spine_fwd<1, 2, 2, 512>;
-    else if (pl.vw == 2) kern = wide ? emo_spine_fwd<2, 4, 4, 512> : emo_spine_fwd<2, 2, 2, 512>;
-    else kern = wide ? emo_spine_fwd<4, 4, 4, 640> : emo_spine_fwd<4, 4, 2, 640>;
+    void (*kern)(SpineParams) = pl.k->fwd;
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
     EMO_CUDA(launch_ahead(kern, pl.grid_f, pl.threads_f, pl.smem_f, st, p));
     if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
@@ -1289,16 +1313,7 @@ int launch_spine_bwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const u
     cudaEvent_t ev0 = g_pass_events[2], ev1 = g_pass_events[3];
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
     const bool extra = ES || LS || slack_sum || n_critical;
-    void (*kern)(SpineParams) = nullptr;
-    const bool wide = g->sflow.spine.bundle > 2;
-#define EMO_PICK_S(VW, VS, NB, MAXT) kern = extra ? emo_spine_bwd<VW, VS, NB, MAXT, true> : emo_spine_bwd<VW, VS, NB, MAXT, false>
-    if (pl.vw == 1 && wide) EMO_PICK_S(1, 4, 4, 512);
-    else if (pl.vw == 1) EMO_PICK_S(1, 2, 2, 512);
-    else if (pl.vw == 2 && wide) EMO_PICK_S(2, 4, 4, 512);
-    else if (pl.vw == 2) EMO_PICK_S(2, 2, 2, 512);
-    else if (wide) EMO_PICK_S(4, 4, 4, 640);
-    else EMO_PICK_S(4, 4, 2, 640);
-#undef EMO_PICK_S
+    void (*kern)(SpineParams) = extra ? pl.k->bwd_extra : pl.k->bwd;
     if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
     EMO_CUDA(launch_ahead(kern, pl.grid_b, pl.threads_b, pl.smem_b, st, p));
     if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
@@ -1486,7 +1501,6 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
     const int64_t m = row_ptr[n];
     if (m > 0 && !col) return EMO_E_INVALID_ARG;
     int32_t max_span = 0;
-    SpineImage image_s, image_l;
     for (int32_t v = 0; v < n; ++v)
         for (int64_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
             if (col[e] < 0 || col[e] >= n) return EMO_E_INVALID_ARG;
@@ -1603,7 +1617,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             auto compile_spine = [&](int k, Flow &out, DevSpine &d, SpineImage &im, int &rc_k, std::string &err_k) {
                 try {
                     rc_k = compile_flow(h, lat, energy, lanes, look, k, k, out, err_k, true);
-                    if (rc_k == EMO_OK && !(flags & EMO_F_HOST_ONLY)) rc_k = lay_out_spine(out, d, im);
+                    if (rc_k == EMO_OK) rc_k = lay_out_spine(out, d, im);
                 } catch (const std::bad_alloc &) {
                     rc_k = EMO_E_OOM;
                 }
@@ -1615,13 +1629,13 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 // 16, 17.2 with 12; 1 013 x 65 536 0.36 with 16, 0.48 with 20 and 0.43 with 8.
                 int sk = code == 1 ? 8 : (code == 3 ? 32 : (code == 2 || flanes <= 8 ? 16 : 4));
                 while (sk > 8 && flanes * sk > 32 * kFlowRowRegs) sk /= 2;
-                spine_thread = std::thread([&, sk]() { compile_spine(sk, g->sflow, g->dspine, image_s, rc_s, err_s); });
+                spine_thread = std::thread([&, sk]() { compile_spine(sk, g->sflow, g->dspine, g->simage, rc_s, err_s); });
                 // the long stages: as many positions as keep a stage at about a hundred entries (25 000 nodes, 5 lanes x 2 000
                 // policies: 20 positions 0.78 ms, 16 0.83; 10 000, 3 lanes x 4 096: 32 0.60, 24 0.66; 51 000, 18 lanes x 1 000: 7 1.82,
                 // 6 1.90, 5 1.96)
                 const int lk = std::min(32, (flanes > 8 ? 126 : 100) / flanes);
-                if (code == 0 && lk > sk && !(flags & EMO_F_HOST_ONLY))
-                    long_thread = std::thread([&, lk]() { compile_spine(lk, g->lflow, g->dlong, image_l, rc_l, err_l); });
+                if (code == 0 && lk > sk)
+                    long_thread = std::thread([&, lk]() { compile_spine(lk, g->lflow, g->dlong, g->limage, rc_l, err_l); });
             }
             try {
                 rc = compile_flow(h, lat, energy, lanes, look, fk, fs, g->flow, err);
@@ -1669,7 +1683,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
         return EMO_E_OOM;
     }
     g->host_only = (flags & EMO_F_HOST_ONLY) != 0;
-    if (!g->host_only) {
+    if (g->host_only) {
+        g->dspine.ready = g->sflow.spine.ok && !g->simage.host.empty();
+        g->dlong.ready = g->lflow.spine.ok && !g->limage.host.empty();
+    } else {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); delete g; return EMO_E_CUDA; }
         cudaDeviceProp prop;
@@ -1727,8 +1744,9 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 if (rc == EMO_OK) rc = upload_flow(g->flow, g->dflow, (flags & EMO_F_INTERVALS) != 0);
             }
         }
-        if (rc == EMO_OK && g->sflow.spine.ok) rc = upload_spine(image_s, g->dspine);
-        if (rc == EMO_OK && g->lflow.spine.ok) rc = upload_spine(image_l, g->dlong);
+        if (rc == EMO_OK && g->sflow.spine.ok) rc = upload_spine(g->simage, g->dspine);
+        if (rc == EMO_OK && g->lflow.spine.ok) rc = upload_spine(g->limage, g->dlong);
+        g->simage = g->limage = SpineImage();
         }
         } catch (const std::bad_alloc &) {
             rc = EMO_E_OOM;
@@ -1831,6 +1849,19 @@ int emo_graph_spine(const emo_graph *g, int64_t out[12])
     for (uint32_t c : f.spine.b.n_ops) nb += c;
     const int64_t v[12] = {1, f.lanes, f.K, f.stages, f.spine.segments, nf, nb, f.spine.f.slots, f.spine.b.slots,
                            f.spine.max_segs, f.spine.acc_words, f.spine.pushes};
+    for (int i = 0; i < 12; ++i) out[i] = v[i];
+    return EMO_OK;
+}
+
+int emo_graph_spine_plan(const emo_graph *g, int64_t B, int need_slack, int want_base, int32_t sm_count, int64_t smem_bytes, int64_t out[12])
+{
+    if (!g || !out || B < 0 || sm_count < 1 || smem_bytes < 0) return EMO_E_INVALID_ARG;
+    for (int i = 0; i < 12; ++i) out[i] = 0;
+    SpinePlan pl;
+    if (!spine_plan_on(g, SpineChip{sm_count, (size_t)smem_bytes}, B, want_base != 0, need_slack != 0, pl)) return EMO_OK;
+    const Flow &f = pl.is_long ? g->lflow : g->sflow;
+    const int64_t v[12] = {1, pl.is_long ? 1 : 0, f.lanes, f.K, f.stages, f.spine.bundle, pl.k->nb, pl.k->max_threads, pl.groups, pl.vw, pl.vs,
+                           std::max(pl.threads_f, pl.threads_b)};
     for (int i = 0; i < 12; ++i) out[i] = v[i];
     return EMO_OK;
 }

@@ -33,7 +33,7 @@ EXPORTS = [
     "emo_strerror", "emo_graph_load", "emo_graph_free", "emo_graph_info", "emo_workspace_bytes",
     "emo_eval_policies", "emo_slack_batch", "emo_slack", "emo_baseline", "emo_target_from_delta",
     "emo_select", "emo_transpose_policies", "emo_slack_batch_host", "emo_graph_program",
-    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_set_wait_limit", "emo_call_path", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
+    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_graph_spine_plan", "emo_set_wait_limit", "emo_call_path", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
 ]
 
 
@@ -116,6 +116,7 @@ def lib():
         L.emo_graph_flow.argtypes = [p, ctypes.POINTER(emo_flow_view)]
         L.emo_graph_spine.argtypes = [p, ctypes.POINTER(ctypes.c_int64)]
         L.emo_graph_spine_view.argtypes = [p, ctypes.POINTER(emo_spine_view)]
+        L.emo_graph_spine_plan.argtypes = [p, i64, ctypes.c_int, ctypes.c_int, i32, i64, ctypes.POINTER(ctypes.c_int64)]
         L.emo_set_wait_limit.argtypes = [i64]
         L.emo_set_flow_counters.argtypes = [p]
         L.emo_measure_int_issue.argtypes = [p, p, p]
@@ -332,6 +333,15 @@ def emo_graph_spine(g: Graph) -> dict:
     out = (ctypes.c_int64 * 12)()
     _check(lib().emo_graph_spine(g.handle, out), "emo_graph_spine")
     keys = ("ok", "lanes", "K", "stages", "segments", "ops_fwd", "ops_bwd", "slots_fwd", "slots_bwd", "max_segs", "acc_words", "pushes")
+    return dict(zip(keys, [int(x) for x in out]))
+
+
+def emo_graph_spine_plan(g: Graph, B, need_slack: bool, want_base: bool, sm_count: int = 148, smem_bytes: int = 227 * 1024) -> dict:
+    """Launch of the spine kernels for B policies (see emo.h)."""
+    out = (ctypes.c_int64 * 12)()
+    _check(lib().emo_graph_spine_plan(g.handle, int(B), int(bool(need_slack)), int(bool(want_base)), int(sm_count), int(smem_bytes), out),
+           "emo_graph_spine_plan")
+    keys = ("ok", "long", "lanes", "K", "stages", "bundle", "kernel_bundle", "kernel_threads", "groups", "vw", "vs", "threads")
     return dict(zip(keys, [int(x) for x in out]))
 
 

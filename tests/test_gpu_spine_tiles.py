@@ -42,3 +42,28 @@ def test_tiles(torch_cuda, emo, oracle_mod, name, scale, groups, off):
         r = gpu_slack_batch(torch, emo, h, lv, B, g.n, flags=emo.EMO_F_SPINE_KERNEL, ldo=ldo)
         assert_matches(r, r_or, B)
     h.free()
+
+
+@pytest.mark.parametrize("name,scale", [("cfg3-8dev", 0.002), ("cfg3-8dev", 0.003), ("random", 38), ("random", 39)])
+def test_programs_with_different_bundles(torch_cuda, emo, oracle_mod, name, scale):
+    """Graphs whose program of long stages (batches of up to two groups per SM) has bundles of another size than the short one:
+    default flags, every output, batches on both sides of the line."""
+    torch = torch_cuda
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = W.make_graph(name, scale) if name != "random" else W.random_dag(*{38: (38, 253, 0.04348380468633499), 39: (39, 305, 0.03172406145819659)}[scale])
+    h = emo.load_workload(g)
+    bundles = set()
+    for B in (1, 64, 4096, sms * 64 + 33):
+        bundles.add(emo.emo_graph_spine_plan(h, B, True, True, sms)["bundle"])
+        host = np.full((g.n, (B + 15) // 16 * 16), 0xFF, dtype=np.uint8)
+        host[:, :B] = np.random.RandomState(B).randint(0, g.L, size=(g.n, B))
+        lv = torch.as_tensor(host, device="cuda")
+        r_or = oracle_mod.batch(g, host, B=B, want_arrays=True, threads=os.cpu_count() or 1)
+        base = oracle_mod.batch(g, np.full((g.n, 1), g.L - 1, dtype=np.uint8))
+        r = gpu_slack_batch(torch, emo, h, lv, B, g.n, want=("slack",), sums=False, base=True)
+        assert np.array_equal(r["makespan"], r_or["makespan"]) and r["T0"] == base["makespan"][0]
+        np.testing.assert_allclose(r["energy"], r_or["energy"], rtol=E_RTOL, atol=0)
+        assert np.array_equal(r["slack"][:, :B], r_or["slack"])
+        assert_matches(gpu_slack_batch(torch, emo, h, lv, B, g.n), r_or, B)
+    assert bundles == {2, 4}
+    h.free()

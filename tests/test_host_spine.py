@@ -75,3 +75,37 @@ def test_spine_program_on_random_dags(emo, oracle_mod, seed):
     lv[:, 1] = 0
     for lanes, k in ((0, 8), (3, 16)):
         compare(emo, oracle_mod, g, lv, emo.EMO_F_LANES(lanes) | emo.EMO_F_SPINE_STAGE(k))
+
+
+def plan_graphs():
+    """Small graphs whose two spine programs are scheduled apart: wide workloads scaled down, sparse random DAGs."""
+    for scale in (0.002, 0.003, 0.004, 0.006, 0.01):
+        yield W.make_graph("cfg3-8dev", scale)
+    yield W.random_dag(38, 253, 0.04348380468633499)
+    yield W.random_dag(39, 305, 0.03172406145819659)
+    for seed in range(40):
+        rs = np.random.RandomState(seed)
+        n = int(rs.randint(60, 600))
+        yield W.random_dag(seed, n, float(rs.uniform(5, 12)) / n)
+
+
+def test_launched_kernels_fit_the_program(emo):
+    """A launch takes the kernels made for the bundles of the program it walks, at every batch size, whichever of the
+    graph's two programs that is; some of the graphs have programs with bundles of different sizes."""
+    launches = longs = mixed = 0
+    for g in plan_graphs():
+        h = emo.load_workload(g, emo.EMO_F_HOST_ONLY)
+        bundles = set()
+        for B in (1, 64, 4096, 4736, 4737, 9472, 9473, 30000, 100000):
+            for need_slack in (False, True):
+                p = emo.emo_graph_spine_plan(h, B, need_slack, True)
+                if not p["ok"]:
+                    continue
+                assert p["kernel_bundle"] == p["bundle"] == (2 if p["lanes"] <= 8 else 4), (g.n, B, p)
+                assert p["threads"] <= p["kernel_threads"] and p["groups"] % p["vw"] == 0
+                launches += 1
+                longs += p["long"]
+                bundles.add(p["bundle"])
+        mixed += len(bundles) == 2
+        h.free()
+    assert launches > 100 and longs > 20 and mixed >= 4
