@@ -56,8 +56,11 @@ __host__ __device__ inline int64_t emo_budget(int64_t T0, int64_t ppm)
     return T0 + q * ppm + (r * ppm) / M;
 }
 
-// Kernels of one call that follow each other are launched ahead of their predecessor's end: its blocks allow that when they have
-// started, and what depends on its results waits here for all of it.
+// Kernels of one call that follow each other are launched ahead of their predecessor's end: its blocks allow that, and what
+// depends on its results waits here for all of it.  A kernel that is itself launched ahead and allows its successor before its
+// own wait lets the successor start while what lies in front of both still runs; a successor that reads anything before
+// its wait then has no order behind whoever wrote that.  So a kernel whose successor does (the forward spine kernel: the backward
+// one fetches level rows early) allows it only after its own wait; the others may at once, their successors wait first.
 __device__ __forceinline__ void emo_grid_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void emo_grid_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

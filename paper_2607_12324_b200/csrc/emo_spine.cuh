@@ -545,9 +545,9 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_fwd(SpineParams p)
     const unsigned smem0 = emo_smem_addr(emo_smem), bar0 = smem0 + p.off_bar;
     volatile int *abort_word = reinterpret_cast<volatile int *>(emo_smem + p.off_bar + kBarKinds * kSpRing * 8);
     const long long limit = p.wait_cycles;
-    emo_grid_allow_next();               // the backward kernel's blocks may take SMs that are free
     emo_spine_init(p, emo_smem, bar0, spines, subs, false);
     emo_grid_wait_previous();            // (who wrote the levels; nothing in memory was touched so far)
+    emo_grid_allow_next();               // the backward kernel's blocks may take SMs that are free: they read levels at once, and these are complete now
 
     long long T[VS];
     double ea[VW];
@@ -857,7 +857,8 @@ __global__ void __launch_bounds__(MAXT, 1) emo_spine_bwd(SpineParams p)
     const long long limit = p.wait_cycles;
     emo_grid_allow_next();
     emo_spine_init(p, emo_smem, bar0, spines, subs, true);
-    // everything but the first loads of level rows and tables waits for the forward kernel
+    // everything but the first loads of level rows and tables waits for the forward kernel (which has waited for the levels when
+    // this one starts)
     if (!(role.prod && role.idx == 0)) emo_grid_wait_previous();
 
     bool failed = false;
