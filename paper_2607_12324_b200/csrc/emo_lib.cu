@@ -2340,12 +2340,13 @@ int emo_pack_model(int32_t n_packs, int32_t n_metrics, int32_t m, int32_t L, con
     if (n_packs == 0) return EMO_OK;
     if (!Bmat || !feat || !Tb || !Eb || !x || !T_out || !E_out) return EMO_E_INVALID_ARG;
     const size_t smem = ((size_t)n_metrics * m + 2 * (size_t)m * L) * sizeof(double);
-    if (smem + (size_t)m * m * sizeof(double) > 48 * 1024) return EMO_E_UNSUPPORTED;
+    if (smem + (size_t)m * m * sizeof(double) > kModelMaxSmem) return EMO_E_UNSUPPORTED;
     int dev = 0, sms = 0;
     EMO_CUDA(cudaGetDevice(&dev));
     EMO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // with its own arrays the kernel passes what a launch has without asking
-    if (smem > 40 * 1024) EMO_CUDA(cudaFuncSetAttribute(emo_pack_model_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // with its own arrays the kernel passes what a launch has without asking (the same size in every call: concurrent callers
+    // with tables of different sizes would otherwise race on the attribute)
+    if (smem > 40 * 1024) EMO_CUDA(cudaFuncSetAttribute(emo_pack_model_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kModelMaxSmem));
     ModelParams p;
     p.n_packs = n_packs;
     p.n = n_metrics;

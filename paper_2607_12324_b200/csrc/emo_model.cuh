@@ -7,6 +7,7 @@
 #include <cstdint>
 
 constexpr int kModelMaxM = 16;       // micro-benchmarks (the paper uses 12)
+constexpr size_t kModelMaxSmem = 48 * 1024;      // most bytes of metrics, tables and Gram matrix that a call may bring
 
 struct ModelParams {
     int n_packs, n, m, L;

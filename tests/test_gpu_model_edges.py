@@ -23,3 +23,34 @@ def test_edges(torch_cuda, emo, oracle_mod, n, m, L, P):  # noqa: F811
     assert (np.abs(x - xo) <= tol * scale).all()
     for got, want, tab in ((T, To, Tb), (E, Eo, Eb)):
         assert (np.abs(got - want) <= tol * scale * m * np.abs(tab).max()).all()
+
+
+def test_two_threads_with_tables_of_different_sizes(torch_cuda, emo):  # noqa: F811
+    """Concurrent callers whose tables take 41 and 45 KB of shared memory: every call launches, with the results it has alone."""
+    import threading
+    n, m, P = 16, 12, 64
+    jobs, errors = [], []
+    for L in (212, 230):
+        B, Tb, Eb = W.microbench_model(31, n, m, L)
+        dev = [torch_cuda.as_tensor(np.ascontiguousarray(a), device="cuda") for a in (B, W.pack_features(32, B, P), Tb, Eb)]
+        out = [torch_cuda.zeros(s, dtype=torch_cuda.float64, device="cuda") for s in ((P, m), (P, L), (P, L))]
+        emo.emo_pack_model(P, n, m, L, *dev, *out)
+        jobs.append((L, dev, out, [o.clone() for o in out], torch_cuda.cuda.Stream()))
+    torch_cuda.cuda.synchronize()
+
+    def call(L, dev, out, want, stream):
+        try:
+            for _ in range(2000):
+                emo.emo_pack_model(P, n, m, L, *dev, *out, stream=stream)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=call, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch_cuda.cuda.synchronize()
+    assert not errors, errors[0]
+    for _, _, out, want, _ in jobs:
+        assert all(torch_cuda.equal(a, b) for a, b in zip(out, want))
