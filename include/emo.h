@@ -57,6 +57,8 @@ extern "C" {
                                       the device); without it that call runs its step-program kernel */
 #define EMO_F_GENERIC 0x4u         /* skip the schedule compilers: the generic kernels evaluate the graph (they also take every
                                       graph whose simultaneously live values exceed the on-chip exchange slots) */
+#define EMO_F_TEST_LONG_OOM 0x8u   /* test hook: there is no memory for the spine program with the longer stages (host-only handles: on the
+                                      host; else on the device); the load goes on without it */
 /* flags of the evaluation calls */
 #define EMO_F_VALIDATE 0x1u        /* check every level < L first; EMO_E_RANGE goes to *status */
 #define EMO_F_NO_STAGING 0x2u      /* use the plain-load kernels instead of the staged ones */

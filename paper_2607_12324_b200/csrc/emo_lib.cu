@@ -892,6 +892,35 @@ int lay_out_spine(const Flow &f, DevSpine &d, SpineImage &im)
     return EMO_OK;
 }
 
+// What launches take from a program: its sizes.  The tables are the compiler's and the layout's.
+void keep_sizes(Flow &f)
+{
+    Flow k;
+    k.ok32 = f.ok32;
+    k.lanes = f.lanes;
+    k.K = f.K;
+    k.sync = f.sync;
+    k.stages = f.stages;
+    k.steps = f.steps;
+    k.Lp = f.Lp;
+    k.entries = f.entries;
+    k.pushes = f.pushes;
+    const Spine &s = f.spine;
+    k.spine.ok = s.ok;
+    k.spine.max_segs = s.max_segs;
+    k.spine.max_pool = s.max_pool;
+    k.spine.bundle = s.bundle;
+    k.spine.acc_words = s.acc_words;
+    k.spine.pushes = s.pushes;
+    k.spine.segments = s.segments;
+    k.spine.unread_slot = s.unread_slot;
+    k.spine.f.slots = s.f.slots;
+    k.spine.f.max_ops = s.f.max_ops;
+    k.spine.b.slots = s.b.slots;
+    k.spine.b.max_ops = s.b.max_ops;
+    f = std::move(k);
+}
+
 int upload_spine(const SpineImage &im, DevSpine &d)
 {
     if (im.host.empty()) return EMO_OK;
@@ -1614,8 +1643,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             int rc_s = EMO_OK, rc_l = EMO_E_UNSUPPORTED;
             std::string err_s, err_l;
             std::thread spine_thread, long_thread;
+            const bool no_long = (flags & EMO_F_TEST_LONG_OOM) != 0 && (flags & EMO_F_HOST_ONLY) != 0;
             auto compile_spine = [&](int k, Flow &out, DevSpine &d, SpineImage &im, int &rc_k, std::string &err_k) {
                 try {
+                    if (no_long && &out == &g->lflow) throw std::bad_alloc();
                     rc_k = compile_flow(h, lat, energy, lanes, look, k, k, out, err_k, true);
                     if (rc_k == EMO_OK) rc_k = lay_out_spine(out, d, im);
                 } catch (const std::bad_alloc &) {
@@ -1649,7 +1680,6 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 rc = EMO_OK;
             }
             if (rc == EMO_OK && rc_s != EMO_OK && rc_s != EMO_E_UNSUPPORTED) rc = rc_s;
-            if (rc == EMO_OK && rc_l == EMO_E_OOM) rc = rc_l;
             if (rc != EMO_OK) { delete g; return rc; }
             if (!want_spine || rc_s != EMO_OK || !g->flow.ok32 || !g->sflow.spine.ok) g->sflow = Flow();
             else {
@@ -1665,6 +1695,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 for (uint32_t k : s2.b.n_ops) c += k;
                 return c;
             };
+            // (nor is it there when memory did not suffice for it: every call has the short one)
             if (rc_l != EMO_OK || !g->sflow.spine.ok || !g->lflow.spine.ok || operations(g->lflow.spine) > operations(g->sflow.spine) * 5 / 4) g->lflow = Flow();
             g->lflow.f = FlowDir();
             g->lflow.b = FlowDir();
@@ -1745,7 +1776,12 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             }
         }
         if (rc == EMO_OK && g->sflow.spine.ok) rc = upload_spine(g->simage, g->dspine);
-        if (rc == EMO_OK && g->lflow.spine.ok) rc = upload_spine(g->limage, g->dlong);
+        if (rc == EMO_OK && g->lflow.spine.ok) {
+            const int rc_l = (flags & EMO_F_TEST_LONG_OOM) ? EMO_E_OOM : upload_spine(g->limage, g->dlong);
+            if (rc_l == EMO_OK) keep_sizes(g->lflow);
+            else if (rc_l == EMO_E_OOM) g->lflow = Flow();      // the short program serves every call
+            else rc = rc_l;
+        }
         g->simage = g->limage = SpineImage();
         }
         } catch (const std::bad_alloc &) {

@@ -28,6 +28,7 @@ EMO_F_SPINE_KERNEL = 0x20
 EMO_F_GENERIC = 0x4        # load flag (shares its value with the call flag EMO_F_PAIR_KERNEL)
 EMO_F_INTERVALS = 0x2      # load flag (shares its value with the call flag EMO_F_NO_STAGING)
 EMO_F_TEST_STALL = 0x100
+EMO_F_TEST_LONG_OOM = 0x8  # load flag
 
 EXPORTS = [
     "emo_strerror", "emo_graph_load", "emo_graph_free", "emo_graph_info", "emo_workspace_bytes",

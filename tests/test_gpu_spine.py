@@ -170,3 +170,17 @@ def test_forward_spine_feeds_lane_stream_backward(torch_cuda, emo, oracle_mod):
     np.testing.assert_allclose(r_pair["energy"][cols], r_or["energy"], rtol=E_RTOL)
     assert np.array_equal(r_pair["slack"][:, cols], r_or["slack"])
     h.free()
+
+
+def test_load_without_device_memory_for_the_long_program(torch_cuda, emo, oracle_mod):
+    """Without device memory for the program with the longer stages the load succeeds; small batches take the short one."""
+    torch = torch_cuda
+    g = W.make_graph("cfg1-train", 0.05)
+    B = 200
+    lv_dev = W.policies_for(g, B=B, device="cuda")
+    r_or = oracle_mod.batch(g, lv_dev.cpu().numpy(), B=B, want_arrays=True)
+    for flags, long_program in ((0, 1), (emo.EMO_F_TEST_LONG_OOM, 0)):
+        h = emo.load_workload(g, flags)
+        assert emo.emo_graph_spine_plan(h, B, True, True)["long"] == long_program
+        check(torch, emo, oracle_mod, g, h, lv_dev, B, r_or)
+        h.free()

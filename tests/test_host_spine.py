@@ -109,3 +109,15 @@ def test_launched_kernels_fit_the_program(emo):
         mixed += len(bundles) == 2
         h.free()
     assert launches > 100 and longs > 20 and mixed >= 4
+
+
+def test_load_without_memory_for_the_long_program(emo):
+    """The program with the longer stages is optional: without memory for it the load succeeds and small batches take the other."""
+    g = W.make_graph("cfg1-train", 0.05)
+    h = emo.load_workload(g, emo.EMO_F_HOST_ONLY)
+    assert emo.emo_graph_spine_plan(h, 64, True, True)["long"] == 1
+    h.free()
+    h = emo.load_workload(g, emo.EMO_F_HOST_ONLY | emo.EMO_F_TEST_LONG_OOM)
+    p = emo.emo_graph_spine_plan(h, 64, True, True)
+    assert p["ok"] == 1 and p["long"] == 0
+    h.free()
