@@ -1642,7 +1642,19 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             const bool want_spine = !(flags & EMO_F_INTERVALS);
             int rc_s = EMO_OK, rc_l = EMO_E_UNSUPPORTED;
             std::string err_s, err_l;
-            std::thread spine_thread, long_thread;
+            // (what ends the block early, an exception among it, waits for them)
+            struct Helper {
+                std::thread t;
+                void wait() { if (t.joinable()) t.join(); }
+                ~Helper() { wait(); }
+            } spine_thread, long_thread;
+            auto start = [](Helper &helper, auto work) {
+                try {
+                    helper.t = std::thread(work);
+                } catch (const std::exception &) {      // no more threads: here, one after the other
+                    work();
+                }
+            };
             const bool no_long = (flags & EMO_F_TEST_LONG_OOM) != 0 && (flags & EMO_F_HOST_ONLY) != 0;
             auto compile_spine = [&](int k, Flow &out, DevSpine &d, SpineImage &im, int &rc_k, std::string &err_k) {
                 try {
@@ -1651,6 +1663,8 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                     if (rc_k == EMO_OK) rc_k = lay_out_spine(out, d, im);
                 } catch (const std::bad_alloc &) {
                     rc_k = EMO_E_OOM;
+                } catch (const std::exception &) {
+                    rc_k = EMO_E_UNSUPPORTED;
                 }
             };
             if (want_spine) {
@@ -1660,21 +1674,21 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 // 16, 17.2 with 12; 1 013 x 65 536 0.36 with 16, 0.48 with 20 and 0.43 with 8.
                 int sk = code == 1 ? 8 : (code == 3 ? 32 : (code == 2 || flanes <= 8 ? 16 : 4));
                 while (sk > 8 && flanes * sk > 32 * kFlowRowRegs) sk /= 2;
-                spine_thread = std::thread([&, sk]() { compile_spine(sk, g->sflow, g->dspine, g->simage, rc_s, err_s); });
+                start(spine_thread, [&, sk]() { compile_spine(sk, g->sflow, g->dspine, g->simage, rc_s, err_s); });
                 // the long stages: as many positions as keep a stage at about a hundred entries (25 000 nodes, 5 lanes x 2 000
                 // policies: 20 positions 0.78 ms, 16 0.83; 10 000, 3 lanes x 4 096: 32 0.60, 24 0.66; 51 000, 18 lanes x 1 000: 7 1.82,
                 // 6 1.90, 5 1.96)
                 const int lk = std::min(32, (flanes > 8 ? 126 : 100) / flanes);
                 if (code == 0 && lk > sk)
-                    long_thread = std::thread([&, lk]() { compile_spine(lk, g->lflow, g->dlong, g->limage, rc_l, err_l); });
+                    start(long_thread, [&, lk]() { compile_spine(lk, g->lflow, g->dlong, g->limage, rc_l, err_l); });
             }
             try {
                 rc = compile_flow(h, lat, energy, lanes, look, fk, fs, g->flow, err);
             } catch (const std::bad_alloc &) {
                 rc = EMO_E_OOM;
             }
-            if (spine_thread.joinable()) spine_thread.join();
-            if (long_thread.joinable()) long_thread.join();
+            spine_thread.wait();
+            long_thread.wait();
             if (rc == EMO_E_UNSUPPORTED) {      // the 64-bit programs exist: they serve
                 g->flow = Flow();
                 rc = EMO_OK;

@@ -121,3 +121,38 @@ def test_load_without_memory_for_the_long_program(emo):
     p = emo.emo_graph_spine_plan(h, 64, True, True)
     assert p["ok"] == 1 and p["long"] == 0
     h.free()
+
+
+def test_load_without_threads(emo):
+    """Where the system has no more threads the programs are compiled one after the other: same handle, nothing aborts.  In a
+    process of its own, whose default thread stack is made larger than the address space."""
+    import os
+    import subprocess
+    import sys
+    code = r"""
+import ctypes, sys
+import numpy as np
+from paper_2607_12324_b200 import emo, workloads as W
+g = W.make_graph("cfg1-train", 0.05)
+emo.lib()
+shape = lambda h: (emo.emo_graph_spine(h), [emo.emo_graph_spine_plan(h, B, True, True) for B in (1, 4096, 40000)])
+h = emo.load_workload(g, emo.EMO_F_HOST_ONLY)
+want = shape(h)
+libc = ctypes.CDLL("libc.so.6")
+attr = (ctypes.c_char * 256)()
+assert libc.pthread_attr_init(attr) == 0
+assert libc.pthread_attr_setstacksize(attr, ctypes.c_size_t(1 << 47)) == 0
+assert libc.pthread_setattr_default_np(attr) == 0
+import threading
+try:
+    threading.Thread(target=print).start()
+    sys.exit("threads can still be made")
+except RuntimeError:
+    pass
+h = emo.load_workload(g, emo.EMO_F_HOST_ONLY)
+assert shape(h) == want and want[1][0]["long"] == 1
+print("loaded")
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, env=dict(os.environ, PYTHONPATH=root), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "loaded", (r.returncode, r.stderr)
