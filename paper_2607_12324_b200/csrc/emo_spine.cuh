@@ -343,14 +343,14 @@ __device__ __forceinline__ void emo_spine_produce(const SpineParams &p, unsigned
         pr[1] = t_issue;
         pr[2] = EMO_SCLK() - t_begin;
     }
-    if (gave_up) {
-        // do not leave the block while copies into its shared memory may still be in flight
-        for (int c = max(0, issued - nbuf); c < issued; ++c)
-            (void)emo_spine_wait(emo_spine_bar(bar0, full_k, c % nbuf), (c / nbuf) & 1, abort_word + 1, p.wait_cycles);
-        if (which == 0)
-            for (int c = issued; c < min(rows_issued, stages); ++c)
-                (void)emo_spine_wait(emo_spine_bar(bar0, kBarRows, c % kSpRowRing), (c / kSpRowRing) & 1, abort_word + 1, p.wait_cycles);
-    }
+    // Do not leave the block while copies into its shared memory may still be in flight: other warps may have given up, also after
+    // the last stage was issued.  The copies land whatever the other warps do, so the limit here is the caller's or 10 ms.
+    const long long drain = max(p.wait_cycles, 20000000LL);
+    for (int c = max(0, issued - nbuf); c < issued; ++c)
+        (void)emo_spine_wait(emo_spine_bar(bar0, full_k, c % nbuf), (c / nbuf) & 1, abort_word + 1, drain);
+    if (which == 0)
+        for (int c = issued; c < min(rows_issued, stages); ++c)
+            (void)emo_spine_wait(emo_spine_bar(bar0, kBarRows, c % kSpRowRing), (c / kSpRowRing) & 1, abort_word + 1, drain);
 }
 
 // The level bytes of an entry for this thread's V consecutive policies, as table addresses: one load, then one dp4a per

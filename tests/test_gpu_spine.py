@@ -184,3 +184,31 @@ def test_load_without_device_memory_for_the_long_program(torch_cuda, emo, oracle
         assert emo.emo_graph_spine_plan(h, B, True, True)["long"] == long_program
         check(torch, emo, oracle_mod, g, h, lv_dev, B, r_or)
         h.free()
+
+
+@pytest.mark.parametrize("name,scale", [("cfg0-tiny", 1.0), ("cfg2-packed", 0.05), ("cfg3-8dev", 0.003)])
+def test_bounded_waits_on_short_graphs(torch_cuda, emo, oracle_mod, name, scale):
+    """The same where the program has hardly more stages than the rings have buffers: what was issued lands before the block ends,
+    whoever gave up, and the next call is right."""
+    torch = torch_cuda
+    g = W.make_graph(name, scale)
+    B = 70
+    lv_dev = W.policies_for(g, B=B, device="cuda")
+    r_or = oracle_mod.batch(g, lv_dev.cpu().numpy(), B=B, want_arrays=True)
+    h = emo.load_workload(g)
+    slack = torch.zeros((g.n, B), dtype=torch.int64, device="cuda")
+    T = torch.zeros(B, dtype=torch.int64, device="cuda")
+    E = torch.zeros(B, dtype=torch.float64, device="cuda")
+    fl = emo.EMO_F_SPINE_KERNEL | emo.EMO_F_TEST_STALL
+    ws = torch.empty(emo.emo_workspace_bytes(h, B, 1, fl), dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        emo.emo_set_wait_limit(1_000_000)
+        try:
+            status = torch.zeros(1, dtype=torch.int32, device="cuda")
+            emo.emo_slack_batch(h, B, lv_dev, lv_dev.stride(0), None, None, slack, B, T, E, None, None, ws, status, fl)
+            torch.cuda.synchronize()
+            assert int(status.item()) == emo.EMO_E_TIMEOUT
+        finally:
+            emo.emo_set_wait_limit(4_000_000_000)
+        check(torch, emo, oracle_mod, g, h, lv_dev, B, r_or)
+    h.free()
