@@ -555,6 +555,28 @@ typedef struct emo_spine_view {
 } emo_spine_view;
 int emo_graph_spine_view(const emo_graph *g, emo_spine_view *out);
 
+/* The spine programs as the kernels read them (long_program = 1: the one with the longer stages; ok = 0 if there is none, or
+ * on a handle with a device, whose layout lies there).  Host-only handles; pointers into the handle's memory, for the host-side tests
+ * of the layout, which interpret it.  Index 0 = forward, 1 = backward.  w [stages][w_bytes], the workers' part: chunk table
+ * (first entry | entries << 16; behind most_chunks words the storing workers', bit 31 = some entry is folded), at off_pos a
+ * word per look-up entry (bit 0 first, bit 1 last of its segment, bits 16.. word of the sum), at off_mem (backward) 32
+ * bytes per member as in emo_spine_view.mem but with the segment's word, at off_first (backward) a bit per entry: first of its
+ * segment, at off_tab the table rows.  s [stages][s_bytes], the spine's part: words {bundles, (forward) terminal nodes,
+ * records, spare}, forward 16 bytes per terminal node {slot, spare, lbC}, at off_ops 48 bytes per operation {operand slots
+ * 0, 1, word of the sum, slot to clear, corrections 0, 1, the lane's slot, published slot, word to write, spare}, at off_rec
+ * forward {word, restore row}, backward per round and stream {the lane's slot, word of the sum, word of the segment, flags |
+ * restore row in the stage << 8}.  words: words per policy and stage of a buffer of sums (backward: the second half holds the
+ * completion offsets); zero: the one that stays zero, the next one nobody reads.  rows [stages][nlook] policy rows. */
+typedef struct emo_spine_layout {
+    int32_t ok, lanes, stages, Lp, bundle, nlook, chunks, most_chunks, max_segs, unread_slot, slots_fwd, slots_bwd;
+    int32_t w_bytes[2], s_bytes[2], off_pos[2], off_tab[2], off_ops[2], off_rec[2], words[2], zero[2];
+    int32_t off_mem, off_first;
+    int64_t pushes;
+    const uint8_t *w[2], *s[2];
+    const uint32_t *rows[2], *push_base;
+} emo_spine_layout;
+int emo_graph_spine_layout(const emo_graph *g, int long_program, emo_spine_layout *out);
+
 #ifdef __cplusplus
 }
 #endif

@@ -1949,6 +1949,47 @@ int emo_graph_spine_view(const emo_graph *g, emo_spine_view *v)
     return EMO_OK;
 }
 
+int emo_graph_spine_layout(const emo_graph *g, int long_program, emo_spine_layout *v)
+{
+    if (!g || !v || (long_program != 0 && long_program != 1)) return EMO_E_INVALID_ARG;
+    std::memset(v, 0, sizeof *v);
+    const Flow &f = long_program ? g->lflow : g->sflow;
+    const DevSpine &d = long_program ? g->dlong : g->dspine;
+    const SpineImage &im = long_program ? g->limage : g->simage;
+    if (!f.ok32 || !f.spine.ok || im.host.empty()) return EMO_OK;
+    v->ok = 1;
+    v->lanes = f.lanes;
+    v->stages = f.stages;
+    v->Lp = f.Lp;
+    v->bundle = f.spine.bundle;
+    v->nlook = d.nlook;
+    v->chunks = d.chunks;
+    v->most_chunks = kSpChunks;
+    v->max_segs = f.spine.max_segs;
+    v->unread_slot = (int32_t)f.spine.unread_slot;
+    v->slots_fwd = f.spine.f.slots;
+    v->slots_bwd = f.spine.b.slots;
+    v->pushes = f.spine.pushes;
+    const DevSpineDir *dir[2] = {&d.f, &d.b};
+    for (int k = 0; k < 2; ++k) {
+        v->w_bytes[k] = (int32_t)dir[k]->w_bytes;
+        v->s_bytes[k] = (int32_t)dir[k]->s_bytes;
+        v->off_pos[k] = (int32_t)dir[k]->off_pos;
+        v->off_tab[k] = (int32_t)dir[k]->off_tab;
+        v->off_ops[k] = (int32_t)dir[k]->off_ops;
+        v->off_rec[k] = (int32_t)dir[k]->off_rec;
+        v->words[k] = dir[k]->words;
+        v->zero[k] = dir[k]->zero;
+        v->w[k] = im.host.data() + (k ? im.at_bW : im.at_fW);
+        v->s[k] = im.host.data() + (k ? im.at_bS : im.at_fS);
+        v->rows[k] = (const uint32_t *)(im.host.data() + (k ? im.at_rowsB : im.at_rowsF));
+    }
+    v->off_mem = (int32_t)d.b.off_mem;
+    v->off_first = (int32_t)d.b.off_first;
+    v->push_base = (const uint32_t *)(im.host.data() + im.at_pb);
+    return EMO_OK;
+}
+
 int emo_graph_program(const emo_graph *g, int dir, int32_t *lanes, int32_t *steps, int32_t *slots,
                       int32_t *Lp, const uint32_t **entries, const uint32_t **rows, const uint32_t **lat)
 {

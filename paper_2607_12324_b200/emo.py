@@ -34,7 +34,7 @@ EXPORTS = [
     "emo_strerror", "emo_graph_load", "emo_graph_free", "emo_graph_info", "emo_workspace_bytes",
     "emo_eval_policies", "emo_slack_batch", "emo_slack", "emo_baseline", "emo_target_from_delta",
     "emo_select", "emo_transpose_policies", "emo_slack_batch_host", "emo_graph_program",
-    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_graph_spine_plan", "emo_set_wait_limit", "emo_call_path", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
+    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_graph_spine_plan", "emo_graph_spine_layout", "emo_set_wait_limit", "emo_call_path", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
 ]
 
 
@@ -118,6 +118,7 @@ def lib():
         L.emo_graph_spine.argtypes = [p, ctypes.POINTER(ctypes.c_int64)]
         L.emo_graph_spine_view.argtypes = [p, ctypes.POINTER(emo_spine_view)]
         L.emo_graph_spine_plan.argtypes = [p, i64, ctypes.c_int, ctypes.c_int, i32, i64, ctypes.POINTER(ctypes.c_int64)]
+        L.emo_graph_spine_layout.argtypes = [p, ctypes.c_int, ctypes.POINTER(emo_spine_layout)]
         L.emo_set_wait_limit.argtypes = [i64]
         L.emo_set_flow_counters.argtypes = [p]
         L.emo_measure_int_issue.argtypes = [p, p, p]
@@ -344,6 +345,28 @@ def emo_graph_spine_plan(g: Graph, B, need_slack: bool, want_base: bool, sm_coun
            "emo_graph_spine_plan")
     keys = ("ok", "long", "lanes", "K", "stages", "bundle", "kernel_bundle", "kernel_threads", "groups", "vw", "vs", "threads")
     return dict(zip(keys, [int(x) for x in out]))
+
+
+class emo_spine_layout(ctypes.Structure):
+    _fields_ = ([(k, ctypes.c_int32) for k in ("ok", "lanes", "stages", "Lp", "bundle", "nlook", "chunks", "most_chunks", "max_segs",
+                                               "unread_slot", "slots_fwd", "slots_bwd")]
+                + [(k, ctypes.c_int32 * 2) for k in ("w_bytes", "s_bytes", "off_pos", "off_tab", "off_ops", "off_rec", "words", "zero")]
+                + [("off_mem", ctypes.c_int32), ("off_first", ctypes.c_int32), ("pushes", ctypes.c_int64)]
+                + [(k, ctypes.c_void_p * 2) for k in ("w", "s", "rows")] + [("push_base", ctypes.c_void_p)])
+
+
+def emo_graph_spine_layout(g: Graph, long_program: bool) -> dict:
+    """A spine program as the kernels read it, as numpy copies: w, s [2][stages][bytes], rows [2][stages][nlook] (see emo.h)."""
+    v = emo_spine_layout()
+    _check(lib().emo_graph_spine_layout(g.handle, int(bool(long_program)), ctypes.byref(v)), "emo_graph_spine_layout")
+    out = {k: (list(x) if isinstance(x, ctypes.Array) else x) for k, x in ((k, getattr(v, k)) for k, _ in v._fields_)}
+    if v.ok:
+        copy = lambda ptr, shape, ctype: np.ctypeslib.as_array(ctypes.cast(ptr, ctypes.POINTER(ctype)), shape=shape).copy()
+        out["w"] = [copy(v.w[k], (v.stages, v.w_bytes[k]), ctypes.c_uint8) for k in range(2)]
+        out["s"] = [copy(v.s[k], (v.stages, v.s_bytes[k]), ctypes.c_uint8) for k in range(2)]
+        out["rows"] = [copy(v.rows[k], (v.stages, v.nlook), ctypes.c_uint32) for k in range(2)]
+        out["push_base"] = copy(v.push_base, (v.stages + 1,), ctypes.c_uint32)
+    return out
 
 
 class emo_spine_view(ctypes.Structure):
