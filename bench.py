@@ -161,7 +161,7 @@ def other_workloads_leg(sm_mhz, hbm_gbs):
     import numpy as np
     import torch
     from paper_2607_12324_b200 import emo, workloads as W
-    names = {5: "32-bit spine, several policies per thread", 4: "32-bit spine", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}
+    names = {5: "32-bit spine, several policies per thread", 4: "32-bit spine, one policy per thread", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}
     out = []
     for name in ("cfg0-tiny", "cfg1-train", "cfg2-packed", "cfg3-8dev"):
         g = W.make_graph(name)
@@ -405,16 +405,22 @@ def main():
               "frac_of_binding": max(t_hbm, t_issue) / ms_per_step,
               "warp_costs_cycles": {k: round(v, 2) for k, v in costs.items()}}
     path = emo.emo_call_path(h, B, lv, ldb, B, True, args.call_flags)
-    if path in (2, 5) and fl["steps"]:
-        bounds["cycles_per_schedule_step"] = {"forward": fwd * 1e-3 * sm_mhz * 1e6 / fl["steps"], "backward": bwd * 1e-3 * sm_mhz * 1e6 / fl["steps"]}
+    # the schedule of the kernels that ran
+    sched = {"lanes": info.lanes, "steps": info.steps_fwd}
+    if path == 2:
+        sched = {"lanes": fl["lanes"], "steps": fl["steps"], "stage_steps": fl["K"], "barrier_steps": fl["sync"], "restore_rows": fl["pushes"]}
+    elif path in (4, 5):
+        props = torch.cuda.get_device_properties(torch.cuda.current_device())
+        pl = emo.emo_graph_spine_plan(h, B, True, True, props.multi_processor_count, props.shared_memory_per_block_optin)
+        sched = {"lanes": pl["lanes"], "steps": pl["stages"] * pl["K"], "stage_steps": pl["K"], "spine_launch": pl}
+    if path in (2, 4, 5) and sched["steps"]:
+        bounds["cycles_per_schedule_step"] = {"forward": fwd * 1e-3 * sm_mhz * 1e6 / sched["steps"], "backward": bwd * 1e-3 * sm_mhz * 1e6 / sched["steps"]}
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "int64", "data": "synthetic",
             "config": workload_config(args.workload, args.scale, g, B, ppm),
-            "details": {"kernels": {5: "32-bit spine, several policies per thread", 4: "32-bit spine", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}[path],
-                        "slack_sums": bool(args.sums), "lanes": fl["lanes"] if path in (2, 5) else info.lanes,
-                        "steps": fl["steps"] if path in (2, 5) else info.steps_fwd, "stage_steps": fl["K"], "barrier_steps": fl["sync"],
-                        "restore_rows": fl["pushes"], "depth": info.depth, "graph_load_s": t_load,
+            "details": {"kernels": {5: "32-bit spine, several policies per thread", 4: "32-bit spine, one policy per thread", 3: "generic", 2: "32-bit lane-stream", 1: "staged 64-bit", 0: "plain 64-bit"}[path],
+                        "slack_sums": bool(args.sums), **sched, "depth": info.depth, "graph_load_s": t_load,
                         "workspace_gb": ws.numel() / 1e9,
                         "parallelism": "replicas" if world > 1 else "single"},
             "policies_per_s": world * B / (ms_per_step * 1e-3),

@@ -66,8 +66,8 @@ extern "C" {
 #define EMO_F_LANE_KERNEL 0x8u     /* staged pass kernel with one policy per thread (the default otherwise) */
 #define EMO_F_FLOW_KERNEL 0x10u    /* the 32-bit lane-stream kernels (the default for n * B >= 2^31, or more than three policy groups of
                                     * 32 per SM on a graph of at most eight lanes, where there is no spine program) */
-#define EMO_F_SPINE_KERNEL 0x20u   /* the spine kernels (the default on graphs of at most eight lanes, and on wider ones from two policy
-                                    * groups of 32 per SM on) */
+#define EMO_F_SPINE_KERNEL 0x20u   /* the spine kernels (the default wherever there is a spine program, but on graphs of more than eight lanes
+                                    * without a program of longer stages only from two policy groups of 32 per SM on) */
 #define EMO_F_TEST_STALL 0x100u    /* test hook of the 32-bit kernels: the producer warps stop half way, so that the
                                       consumers' bounded waits run out and EMO_E_TIMEOUT is reported */
 
@@ -435,8 +435,8 @@ int emo_set_pass_events(void *fwd_start, void *fwd_stop, void *bwd_start, void *
 
 /*
  * emo_call_path - which kernels emo_eval_policies (need_slack = 0) or emo_slack_batch (need_slack = 1)
- * would run for these arguments: 4 = the spine kernels (one policy per worker thread, or asked for with
- * EMO_F_SPINE_KERNEL), 5 = the spine kernels with several policies per worker thread, 2 = the 32-bit lane-stream kernels,
+ * would run for these arguments: 4 = the spine kernels with one policy per worker thread, 5 = the
+ * spine kernels with several, 2 = the 32-bit lane-stream kernels,
  * 1 = the staged 64-bit kernels,
  * 0 = the plain-load 64-bit kernels, 3 = the generic kernels (a graph beyond the on-chip schedules' limits, or
  * loaded with EMO_F_GENERIC); negative = an EMO_E_* code.  lvl may be any pointer with the

@@ -1437,7 +1437,7 @@ int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
     if (g->generic) return 3;
     if (spine_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
         SpinePlan sp;
-        if (spine_plan(g, B, true, need_slack != 0, sp)) return (sp.vw == 1 || (flags & EMO_F_SPINE_KERNEL)) ? 4 : 5;
+        if (spine_plan(g, B, true, need_slack != 0, sp)) return sp.vw == 1 ? 4 : 5;
     }
     if (flow_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
         FlowPlan fp;

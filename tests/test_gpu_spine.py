@@ -70,8 +70,8 @@ def test_config_graphs(torch_cuda, emo, oracle_mod, name, scale, B, k):
     sp = emo.emo_graph_spine(h)
     assert sp["ok"] == 1 and sp["ops_bwd"] >= sp["segments"] > 0 and sp["ops_fwd"] > 0
     check(torch, emo, oracle_mod, g, h, lv_dev, B, r_or, ldo=B + 1)
-    # the default: narrow graphs below the large-batch rule take the spine kernels for slack-only calls, every other
-    # call (per-node ES / LS, sums) the kernels that produce those outputs
+    # the default: narrow graphs take the spine kernels for every call (here one policy per worker thread); wide ones with a forced
+    # stage length, and so without a program of longer stages, do not at these batch sizes
     path = emo.emo_call_path(h, B, lv_dev, lv_dev.stride(0), B, 1, 0)
     assert (path == 4) == (sp["lanes"] <= 8)
     if path == 4:
@@ -145,19 +145,17 @@ def test_random_dags(torch_cuda, emo, oracle_mod):
     assert done >= 8
 
 
-def test_forward_spine_feeds_lane_stream_backward(torch_cuda, emo, oracle_mod):
-    """Four policy groups per SM on a narrow graph: the forward spine kernel writes the restore list in the lane-stream
-    program's numbering and the lane-stream backward kernel reads it.  Same slack matrix as the lane-stream pair alone,
-    and the oracle's on sampled policies."""
+def test_spine_pair_against_lane_stream_pair(torch_cuda, emo, oracle_mod):
+    """Four policy groups per SM on a narrow graph: the default there are the spine kernels with several policies per worker
+    thread.  Same slack matrix as the lane-stream kernels, and the oracle's on sampled policies."""
     torch = torch_cuda
     g = W.make_graph("cfg4-llm", 0.1)
     B = 16384
     lv_dev = W.policies_for(g, B=B, device="cuda")
     h = emo.load_workload(g)
-    path = emo.emo_call_path(h, B, lv_dev, lv_dev.stride(0), B, True, 0)
-    assert path in (2, 5)
-    if path != 5:
-        pytest.skip("this graph's lane-stream program does not share the spine program's schedule")
+    assert emo.emo_call_path(h, B, lv_dev, lv_dev.stride(0), B, True, 0) == 5
+    assert emo.emo_call_path(h, B, lv_dev, lv_dev.stride(0), B, True, emo.EMO_F_SPINE_KERNEL) == 5
+    assert emo.emo_call_path(h, 64, lv_dev, lv_dev.stride(0), 64, True, 0) == 4
     r_pair = gpu_slack_batch(torch, emo, h, lv_dev, B, g.n, want=("slack",), sums=False, base=True)
     r_flow = gpu_slack_batch(torch, emo, h, lv_dev, B, g.n, want=("slack",), sums=False, base=True, flags=emo.EMO_F_FLOW_KERNEL)
     assert np.array_equal(r_pair["makespan"], r_flow["makespan"]) and r_pair["T0"] == r_flow["T0"]
