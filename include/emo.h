@@ -436,7 +436,7 @@ int emo_set_pass_events(void *fwd_start, void *fwd_stop, void *bwd_start, void *
 /*
  * emo_call_path - which kernels emo_eval_policies (need_slack = 0) or emo_slack_batch (need_slack = 1)
  * would run for these arguments: 4 = the spine kernels with one policy per worker thread, 5 = the
- * spine kernels with several, 2 = the 32-bit lane-stream kernels,
+ * spine kernels with several (calls without ES, LS and the sums), 2 = the 32-bit lane-stream kernels,
  * 1 = the staged 64-bit kernels,
  * 0 = the plain-load 64-bit kernels, 3 = the generic kernels (a graph beyond the on-chip schedules' limits, or
  * loaded with EMO_F_GENERIC); negative = an EMO_E_* code.  lvl may be any pointer with the
@@ -527,7 +527,7 @@ int emo_graph_flow(const emo_graph *g, emo_flow_view *out);
 int emo_graph_spine(const emo_graph *g, int64_t out[12]);
 
 /* The launch of the spine kernels that B policies would get on a device of sm_count SMs with smem_bytes of shared memory per
- * block: out[0] = 1 if there is one (else the rest is 0), 1 for the program with the longer stages, its lanes, steps per
+ * block (need_slack = 0: makespan and energy; 1: slack; 2: ES, LS or the sums too): out[0] = 1 if there is one (else the rest is 0), 1 for the program with the longer stages, its lanes, steps per
  * stage, stages and operations per bundle, the bundle and most threads of the kernels that are launched, policy groups of 32
  * per block, policies per worker and per spine thread, threads per block (the larger of the two passes).  Host-only handles
  * answer too; it launches nothing. */

@@ -1135,9 +1135,8 @@ int launch_flow_bwd(const emo_graph *g, const FlowPlan &pl, int64_t B, const uin
     return EMO_OK;
 }
 
-// Launch shape of the spine kernels: the smallest tile of 32 * G policies (G a power of two) that covers the batch with
-// one block per SM; as many policies per worker thread (up to four) as the tile has groups; two policies per spine thread up
-// to two groups, else four (bundles of four, 8 threads per operation: always four, so that a row of 32 policies is one
+// Launch shape of the spine kernels: a tile of 32 * G policies (kSpineTiles); two policies per spine thread up
+// to three groups, else four (bundles of four, 8 threads per operation: always four, so that a row of 32 policies is one
 // conflict-free access of those threads).
 struct SpinePlan {
     bool ok = false, is_long = false;
@@ -1149,15 +1148,41 @@ struct SpinePlan {
 };
 
 // The kernels of one shape.  The operations of a program come in bundles of its own size (the two programs of a graph are
-// scheduled apart, so their lanes and with them their bundles may differ): a plan names the kernels of its program's.
+// scheduled apart, so their lanes and with them their bundles may differ): a plan names the kernels of its program's.  SLACK,
+// EXTRA: which backward kernels some tile below reaches.
 struct SpineKernels {
     int vw, vs, nb, max_threads;
     void (*fwd)(SpineParams), (*bwd)(SpineParams), (*bwd_extra)(SpineParams);
 };
-template <int VW, int VS, int NB, int MAXT>
-constexpr SpineKernels spine_kernels() { return {VW, VS, NB, MAXT, emo_spine_fwd<VW, VS, NB, MAXT>, emo_spine_bwd<VW, VS, NB, MAXT, false>, emo_spine_bwd<VW, VS, NB, MAXT, true>}; }
-const SpineKernels kSpineKernels[] = {spine_kernels<1, 2, 2, 512>(), spine_kernels<2, 2, 2, 512>(), spine_kernels<4, 4, 2, 640>(),
-                                      spine_kernels<1, 4, 4, 512>(), spine_kernels<2, 4, 4, 512>(), spine_kernels<4, 4, 4, 640>()};
+template <int VW, int VS, int NB, int MAXT, bool SLACK, bool EXTRA>
+constexpr SpineKernels spine_kernels()
+{
+    SpineKernels k = {VW, VS, NB, MAXT, emo_spine_fwd<VW, VS, NB, MAXT>, nullptr, nullptr};
+    if constexpr (SLACK) k.bwd = emo_spine_bwd<VW, VS, NB, MAXT, false>;
+    if constexpr (EXTRA) k.bwd_extra = emo_spine_bwd<VW, VS, NB, MAXT, true>;
+    return k;
+}
+const SpineKernels kSpineKernels[] = {spine_kernels<1, 2, 2, 512, true, true>(), spine_kernels<1, 2, 2, 640, false, true>(), spine_kernels<2, 2, 2, 512, true, true>(),
+                                      spine_kernels<2, 4, 2, 640, true, true>(), spine_kernels<4, 4, 2, 640, true, false>(), spine_kernels<1, 4, 4, 512, true, true>(),
+                                      spine_kernels<2, 4, 4, 512, true, true>(), spine_kernels<2, 4, 4, 640, false, true>(), spine_kernels<4, 4, 4, 640, true, false>()};
+
+// Tiles of policies: groups of 32 per block, policies per worker and (bundles of two) per spine thread, what a wave of blocks
+// costs (in units of a group); whether wide graphs have it, and calls without and with per-node ES / LS or sums.  A batch takes
+// the tile whose waves cost least.
+// Measured (both passes, ms).  All outputs: four policies per worker leave a storing warp one entry at a time, fewer are faster:
+// 10 000 nodes x 14 000 policies 1.15 with three groups, 1.79 with four at four per worker; x 18 900 1.33 with four at two per
+// worker, 1.82 at four; 500 nodes x 19 000 0.108 with six, 0.185 at four per worker; the one loss met is 25 000 nodes x
+// 37 000, 5.98 against 5.87.  Slack alone: six groups where eight would leave half of the SMs without a block, 1 013 nodes x 19 000 0.160 / 0.187;
+// but four rather than three, 25 000 x 9 600 1.54 / 1.73.  The cost of six: 500 nodes x 60 000 take 0.224 in four waves of four
+// and 0.238 in three of six.
+struct SpineTile {
+    int groups, vw, vs;
+    double cost;
+    bool wide, slack, extra;
+};
+constexpr SpineTile kSpineTiles[] = {{8, 4, 4, 10.0, false, true, false}, {8, 2, 4, 10.0, false, false, true}, {6, 2, 4, 8.1, false, true, true},
+                                     {4, 4, 4, 6.0, true, true, false}, {4, 2, 4, 6.0, true, false, true}, {3, 1, 2, 5.0, false, false, true},
+                                     {2, 2, 2, 4.0, true, true, true}, {1, 1, 2, 3.0, true, true, true}};
 
 // What a launch shape depends on beside the program and the batch.
 struct SpineChip {
@@ -1165,21 +1190,25 @@ struct SpineChip {
     size_t smem;
 };
 
-bool spine_plan_for(const emo_graph *g, const SpineChip &chip, const Flow &f, const DevSpine &d, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+bool spine_plan_for(const emo_graph *g, const SpineChip &chip, const Flow &f, const DevSpine &d, int64_t B, bool want_base, bool need_bwd, bool extra, SpinePlan &pl)
 {
     const Spine &sp = f.spine;
     pl.ok = false;
     if (!f.ok32 || !sp.ok || !d.ready || !chip.smem || f.stages == 0) return false;
     const int64_t NBf = B + (want_base ? 1 : 0);
     const int64_t n_groups = (NBf + 31) / 32;
-    const int64_t want = (n_groups + chip.sm_count - 1) / chip.sm_count;
     const size_t budget = chip.smem;
-    int G0 = 1;
-    const int gmax = sp.bundle > 2 ? 4 : 8;
-    while (G0 < gmax && G0 < want) G0 *= 2;
-    for (int G = G0; G >= 1; G /= 2) {
+    const bool wide = sp.bundle > 2;
+    double best = 0.0;
+    for (const SpineTile &tile : kSpineTiles) {
+        if ((wide && !tile.wide) || (extra ? !tile.extra : !tile.slack)) continue;
+        const int64_t blocks = (n_groups + tile.groups - 1) / tile.groups;
+        const double cost = (double)((blocks + chip.sm_count - 1) / chip.sm_count) * tile.cost;
+        if (pl.ok && cost >= best) continue;
+        SpinePlan cand;
+        const int G = tile.groups;
         const size_t P = 32 * (size_t)G;
-        const int VW = std::min(G, 4), VS = (G >= 4 || sp.bundle > 2) ? 4 : 2, spines = (int)P / (32 / sp.bundle * VS), subs = G / VW;
+        const int VW = tile.vw, VS = wide ? 4 : tile.vs, spines = (int)P / (32 / sp.bundle * VS), subs = G / VW;
         auto shape = [&](bool backward, SpineParams &p, size_t &smem, int &threads) {
             const SpineDir &dir = backward ? sp.b : sp.f;
             const DevSpineDir &dd = backward ? d.b : d.f;
@@ -1256,38 +1285,44 @@ bool spine_plan_for(const emo_graph *g, const SpineChip &chip, const Flow &f, co
             }
             return false;
         };
-        if (!shape(false, pl.pf, pl.smem_f, pl.threads_f)) continue;
-        if (need_bwd && !shape(true, pl.pb, pl.smem_b, pl.threads_b)) continue;
-        pl.k = nullptr;
+        if (!shape(false, cand.pf, cand.smem_f, cand.threads_f)) continue;
+        if (need_bwd && !shape(true, cand.pb, cand.smem_b, cand.threads_b)) continue;
         for (const SpineKernels &k : kSpineKernels)
-            if (k.vw == VW && k.vs == VS && k.nb == sp.bundle && pl.threads_f <= k.max_threads && (!need_bwd || pl.threads_b <= k.max_threads)) pl.k = &k;
-        if (!pl.k) continue;
-        pl.groups = G;
-        pl.vw = VW;
-        pl.vs = VS;
-        pl.grid_f = (int)((n_groups + G - 1) / G);
-        pl.grid_b = (int)(((B + 31) / 32 + G - 1) / G);
-        pl.restore_bytes = need_bwd ? round_up((size_t)pl.grid_f * (size_t)(sp.pushes + f.lanes) * P * 4, 256) : 0;
-        pl.ok = true;
-        return true;
+            if (!cand.k && k.vw == VW && k.vs == VS && k.nb == sp.bundle && cand.threads_f <= k.max_threads && (!need_bwd || cand.threads_b <= k.max_threads) &&
+                (extra ? k.bwd_extra : k.bwd))
+                cand.k = &k;
+        if (!cand.k) continue;
+        cand.groups = G;
+        cand.vw = VW;
+        cand.vs = VS;
+        cand.grid_f = (int)blocks;
+        cand.grid_b = (int)(((B + 31) / 32 + G - 1) / G);
+        cand.restore_bytes = need_bwd ? round_up((size_t)cand.grid_f * (size_t)(sp.pushes + f.lanes) * P * 4, 256) : 0;
+        cand.ok = true;
+        best = cost;
+        pl = cand;
     }
-    return false;
+    return pl.ok;
 }
 
 // Up to two policy groups per SM a block has shared memory to spare and its stages are bound by latency: the program with the
 // longer stages.  Measured (both passes, ms, long / short stages): 10 000 nodes x 4 096 policies 0.60 / 0.77, x 9 000 0.69 / 0.86;
 // 25 000 x 2 000 0.78 / 0.83, x 8 192 1.03 / 1.07; 1 013 x 4 096 0.085 / 0.096.  Above that the larger buffers cost tiles or stages in
 // flight: 1 013 x 65 536 0.50 / 0.36.  On wide graphs only up to one group: 18 lanes, 51 000 x 1 000 1.82 / 2.09, x 8 192 2.7 / 2.49.
-bool spine_plan_on(const emo_graph *g, const SpineChip &chip, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+bool spine_plan_on(const emo_graph *g, const SpineChip &chip, int64_t B, bool want_base, bool need_bwd, bool extra, SpinePlan &pl)
 {
     const int64_t n_groups = (B + (want_base ? 1 : 0) + 31) / 32;
-    pl.is_long = n_groups <= (g->lflow.lanes > 8 ? 1 : 2) * (int64_t)chip.sm_count && spine_plan_for(g, chip, g->lflow, g->dlong, B, want_base, need_bwd, pl);
-    return pl.is_long || spine_plan_for(g, chip, g->sflow, g->dspine, B, want_base, need_bwd, pl);
+    if (n_groups <= (g->lflow.lanes > 8 ? 1 : 2) * (int64_t)chip.sm_count && spine_plan_for(g, chip, g->lflow, g->dlong, B, want_base, need_bwd, extra, pl)) {
+        pl.is_long = true;
+        return true;
+    }
+    return spine_plan_for(g, chip, g->sflow, g->dspine, B, want_base, need_bwd, extra, pl);
 }
 
-bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, SpinePlan &pl)
+// extra: the call asks for ES, LS or the sums
+bool spine_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, bool extra, SpinePlan &pl)
 {
-    return spine_plan_on(g, SpineChip{g->sm_count, g->smem_optin}, B, want_base, need_bwd, pl);
+    return spine_plan_on(g, SpineChip{g->sm_count, g->smem_optin}, B, want_base, need_bwd, extra, pl);
 }
 
 int launch_spine_fwd(const emo_graph *g, const SpinePlan &pl, int64_t B, const uint8_t *lvl, int64_t ldb, uint32_t *restore,
@@ -1437,7 +1472,7 @@ int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
     if (g->generic) return 3;
     if (spine_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
         SpinePlan sp;
-        if (spine_plan(g, B, true, need_slack != 0, sp)) return sp.vw == 1 ? 4 : 5;
+        if (spine_plan(g, B, true, need_slack != 0, false, sp)) return sp.vw == 1 ? 4 : 5;
     }
     if (flow_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
         FlowPlan fp;
@@ -1908,7 +1943,7 @@ int emo_graph_spine_plan(const emo_graph *g, int64_t B, int need_slack, int want
     if (!g || !out || B < 0 || sm_count < 1 || smem_bytes < 0) return EMO_E_INVALID_ARG;
     for (int i = 0; i < 12; ++i) out[i] = 0;
     SpinePlan pl;
-    if (!spine_plan_on(g, SpineChip{sm_count, (size_t)smem_bytes}, B, want_base != 0, need_slack != 0, pl)) return EMO_OK;
+    if (!spine_plan_on(g, SpineChip{sm_count, (size_t)smem_bytes}, B, want_base != 0, need_slack != 0, need_slack > 1, pl)) return EMO_OK;
     const Flow &f = pl.is_long ? g->lflow : g->sflow;
     const int64_t v[12] = {1, pl.is_long ? 1 : 0, f.lanes, f.K, f.stages, f.spine.bundle, pl.k->nb, pl.k->max_threads, pl.groups, pl.vw, pl.vs,
                            std::max(pl.threads_f, pl.threads_b)};
@@ -2109,9 +2144,13 @@ int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint3
         else
             need = spill_need(g, B);
         SpinePlan sp;
-        if (!g->host_only && B > 0 && spine_allowed(g, B, fake, aligned ? 16 : 1, 0, flags) && spine_plan(g, B, true, true, sp))
-            // (rows of the larger of the two programs: a smaller batch may take the other one)
-            need = std::max(need, sp.restore_bytes / (size_t)sp.pf.restore_rows * (size_t)std::max(sp.pf.restore_rows, g->lflow.spine.pushes + g->lflow.lanes) + 256);
+        if (!g->host_only && B > 0 && spine_allowed(g, B, fake, aligned ? 16 : 1, 0, flags) && spine_plan(g, B, true, true, false, sp))
+        {
+            // (rows of the larger of the two programs and, where tiles are larger than two groups, up to seven groups more: a smaller
+            // batch, or a call with other outputs, may take the other program or a larger tile)
+            const size_t cover = (size_t)sp.grid_f * (size_t)sp.groups, groups = cover + (cover > 2 * (size_t)g->sm_count ? 7 : 0);
+            need = std::max(need, groups * 128 * (size_t)std::max(sp.pf.restore_rows, g->lflow.spine.pushes + g->lflow.lanes) + 256);
+        }
         bytes += need;
     }
     if (need_slack == 2) bytes += 4 * round_up((size_t)B * 8, 256) + 256;
@@ -2145,7 +2184,7 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
                               ws_bytes, st);
     if (spine_allowed(g, B, lvl, ldb, 0, flags)) {
         SpinePlan fp;
-        if (spine_plan(g, B, T0 || E0, false, fp))
+        if (spine_plan(g, B, T0 || E0, false, false, fp))
             return launch_spine_fwd(g, fp, B, lvl, ldb, nullptr, makespan, energy, T0, E0, status, flags, st);
     }
     if (flow_allowed(g, B, lvl, ldb, 0, flags)) {
@@ -2482,7 +2521,7 @@ int emo_slack_batch(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t l
                               st);
     if (spine_allowed(g, B, lvl, ldb, ldo, flags)) {
         SpinePlan fp;
-        if (spine_plan(g, B, T0 || E0, true, fp)) {
+        if (spine_plan(g, B, T0 || E0, true, ES || LS || slack_sum || n_critical, fp)) {
             const size_t head = kSmallWs + lvl_area(g);
             if (!ws || ws_bytes < head + fp.restore_bytes) return EMO_E_OOM;
             uint32_t *restore = (uint32_t *)((char *)ws + head);

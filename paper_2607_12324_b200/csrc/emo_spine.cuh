@@ -254,10 +254,12 @@ __device__ __forceinline__ void emo_spine_produce(const SpineParams &p, unsigned
     const int64_t b0 = (int64_t)blockIdx.x * p.ptile;
     const int64_t left = p.lvl ? p.ldb - b0 : 0;
     const unsigned lvl_bytes = left > 0 ? (unsigned)min((int64_t)p.ptile, left) : 0u, P = (unsigned)p.ptile, ldb = (unsigned)p.ldb;
-    // pieces of a full row (2 .. 32, a power of two); this lane's piece, and its row among those of one instruction
-    const int pshift = 31 - __clz(p.ptile >> 4);
+    // pieces of a full row (2 .. 16) by lanes, rounded up to a power of two (tiles of 96 and 192 policies leave a quarter of the
+    // lanes without one; dividing the lanes by the pieces made the forward pass 1.5 % slower); this lane's piece, and its row among
+    // those of one instruction
+    const int pshift = 32 - __clz((p.ptile >> 4) - 1);
     const unsigned pc16 = ((unsigned)lane & ((1u << pshift) - 1u)) * 16u, sub_row = (unsigned)lane >> pshift, step = 32u >> pshift;
-    // rows of this lane: none where its piece lies beyond the matrix
+    // rows of this lane: none where its piece lies beyond the tile or the matrix
     const unsigned n_rows = pc16 < lvl_bytes ? (unsigned)p.nlook : 0u;
     const uint8_t *const lvl0 = p.lvl + b0 + pc16;
     const unsigned row_bytes = (unsigned)p.nlook * 4u;

@@ -338,10 +338,10 @@ def emo_graph_spine(g: Graph) -> dict:
     return dict(zip(keys, [int(x) for x in out]))
 
 
-def emo_graph_spine_plan(g: Graph, B, need_slack: bool, want_base: bool, sm_count: int = 148, smem_bytes: int = 227 * 1024) -> dict:
+def emo_graph_spine_plan(g: Graph, B, need_slack: int, want_base: bool, sm_count: int = 148, smem_bytes: int = 227 * 1024) -> dict:
     """Launch of the spine kernels for B policies (see emo.h)."""
     out = (ctypes.c_int64 * 12)()
-    _check(lib().emo_graph_spine_plan(g.handle, int(B), int(bool(need_slack)), int(bool(want_base)), int(sm_count), int(smem_bytes), out),
+    _check(lib().emo_graph_spine_plan(g.handle, int(B), int(need_slack), int(bool(want_base)), int(sm_count), int(smem_bytes), out),
            "emo_graph_spine_plan")
     keys = ("ok", "long", "lanes", "K", "stages", "bundle", "kernel_bundle", "kernel_threads", "groups", "vw", "vs", "threads")
     return dict(zip(keys, [int(x) for x in out]))

@@ -20,6 +20,10 @@ CASES = [("cfg1-train", 0.02, g, d) for g in (1, 2, 4, 8) for d in (-1, 0)] + \
         [("cfg3-8dev", 0.004, g, d) for g in (1, 2) for d in (-31, 0)]
 
 
+# three groups for calls with ES, LS or the sums (one policy per worker thread), six (two)
+CASES += [("cfg1-train", 0.02, g, d) for g in (3, 6) for d in (-1, 0, -33)] + [("cfg2-packed", 0.5, 6, -1), ("cfg4-llm", 0.002, 3, -1)]
+
+
 @pytest.mark.parametrize("name,scale,groups,off", CASES)
 def test_tiles(torch_cuda, emo, oracle_mod, name, scale, groups, off):
     torch = torch_cuda
@@ -66,4 +70,29 @@ def test_programs_with_different_bundles(torch_cuda, emo, oracle_mod, name, scal
         assert np.array_equal(r["slack"][:, :B], r_or["slack"])
         assert_matches(gpu_slack_batch(torch, emo, h, lv, B, g.n), r_or, B)
     assert bundles == {2, 4}
+    h.free()
+
+
+@pytest.mark.parametrize("name,scale", [("cfg1-train", 0.02), ("cfg3-8dev", 0.003)])
+def test_one_workspace_for_smaller_batches_and_other_outputs(torch_cuda, emo, name, scale):
+    """The workspace of a batch serves every smaller one, whichever tile and program that takes, and calls with more outputs."""
+    torch = torch_cuda
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = W.make_graph(name, scale)
+    h = emo.load_workload(g)
+    most = 7 * 32 * sms + 1
+    lv = W.policies_for(g, B=most, device="cuda")
+    X = torch.zeros((3, g.n, most), dtype=torch.int64, device="cuda")
+    T, E = torch.zeros(most, dtype=torch.int64, device="cuda"), torch.zeros(most, dtype=torch.float64, device="cuda")
+    want = None
+    for top in (most, 6 * 32 * sms, 4 * 32 * sms + 1, 3 * 32 * sms - 1, 2 * 32 * sms - 1, 32 * sms):
+        ws = torch.empty(emo.emo_workspace_bytes(h, top, 1), dtype=torch.uint8, device="cuda")
+        for B in sorted({top, top - 31, 5 * 32 * sms, 3 * 32 * sms, 2 * 32 * sms - 1, 32 * sms + 1, 32 * sms - 1, 7}, reverse=True):
+            if B > top:
+                continue
+            T.zero_()
+            emo.emo_slack_batch(h, B, lv, lv.stride(0), X[0], X[1], X[2], most, T, E, None, None, ws=ws)
+            if want is None:
+                want = T.clone()
+            assert torch.equal(T[:B], want[:B])
     h.free()
