@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(kModelThreads, 3) emo_pack_model_kernel(ModelP
     // variable is above 2
     if (threadIdx.x < kModelMaxM) {
         const double g = G[threadIdx.x * (kModelMaxM + 1)];
-        unit[threadIdx.x] = (g > 0.0 && g < 1e300) ? ldexp(1.0, -(ilogb(g) / 2)) : 1.0;
+        // (half the exponent, odd ones rounded up: a shift, a division would round towards zero and leave [2, 4) as it is)
+        unit[threadIdx.x] = (g > 0.0 && g < 1e300) ? ldexp(1.0, -((ilogb(g) + 1) >> 1)) : 1.0;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < kModelMaxM * kModelMaxM; i += blockDim.x) G[i] *= unit[i / kModelMaxM] * unit[i % kModelMaxM];

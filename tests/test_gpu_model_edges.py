@@ -54,3 +54,19 @@ def test_two_threads_with_tables_of_different_sizes(torch_cuda, emo):  # noqa: F
     assert not errors, errors[0]
     for _, _, out, want, _ in jobs:
         assert all(torch_cuda.equal(a, b) for a, b in zip(out, want))
+
+
+@pytest.mark.parametrize("scale", [1.5, 2.0, 3.0, 6.5, 2.0 ** -3.3, 2.0 ** 40.5, 2.0 ** -61.4])
+def test_gram_diagonals_with_odd_exponents(torch_cuda, emo, oracle_mod, scale):  # noqa: F811
+    """Metric matrices whose Gram diagonal has odd exponents (columns of length `scale` and multiples of it): the unknowns' units
+    are powers of two, so twice the metrics and features give the same weights bit for bit, whatever the exponent."""
+    n, m, L, P = 12, 6, 5, 40
+    B, Tb, Eb = W.microbench_model(41, n, m, L)
+    B = B / np.linalg.norm(B, axis=0) * scale * np.array([1.0, 1.5, 1.0, 3.0, 1.0, 0.75])
+    feat = W.pack_features(42, B, P, noise=0.1)
+    xo, _, _ = oracle_mod.pack_model(B, feat, Tb, Eb)
+    x, _, _ = run(torch_cuda, emo, B, feat, Tb, Eb)
+    tol = 4e-13 * np.linalg.cond(B) ** 2
+    assert (np.abs(x - xo) <= tol * (np.abs(xo).max(axis=1, keepdims=True) + 1e-300)).all()
+    x2, _, _ = run(torch_cuda, emo, 2.0 * B, 2.0 * feat, Tb, Eb)
+    assert np.array_equal(x2, x)
