@@ -599,11 +599,54 @@ __device__ __forceinline__ void emo_flow_fwd_run_intv_slow(const FlowParams &p, 
     }
 }
 
+// DENSE: where hardly any entry stays in the interval of the one before it, every entry looks its own up and none is kept at hand.
+// No branch on anything loaded here: a node outside every policy reads the last row and any level (its table row holds one
+// value); busy time is collected in a register while the (row, interval) stays the same.
+__device__ __forceinline__ void emo_flow_intv_own(const FlowParams &p, FlowIntv &iv, const uint4 &meta, unsigned eo, unsigned ta0, unsigned lmask,
+                                                  unsigned tok, unsigned &dd, double &e)
+{
+    const long long start = (long long)((unsigned long long)meta.x | ((unsigned long long)meta.y << 32)) + (long long)eo;
+    const unsigned row = min(meta.z, (unsigned)p.rowsF - 1u);
+    long long iend;
+    const int i = emo_interval_index<true>(start, p.I, p.delta, p.inv_mean, iv.brk, iend);
+    const unsigned key = row * (unsigned)p.I + (unsigned)i;
+    const unsigned ta = ta0 + (emo_vld_u8(iv.Fs + key * (unsigned)p.ptile) & lmask) * 12u;
+    dd = emo_tld_u32(ta, tok);
+    e = emo_flow_intv_energy(ta, tok);
+    const long long dur = (long long)meta.w + (long long)dd;
+    const bool on = meta.z != emo::kNone && iv.count;
+    if (on && key != iv.key) {           // rare within an interval
+        if (iv.sum) atomicAdd(p.busy + (size_t)iv.key * p.ldw + iv.b, iv.sum);
+        iv.key = key;
+        iv.sum = 0;
+    }
+    const bool single = start + dur <= iend;
+    iv.sum += (on && single) ? (unsigned long long)dur : 0ull;
+    if (on && !single) emo_interval_busy(p.busy, p.ldw, iv.b, row, p.I, i, iend, start, start + dur, iv.brk);
+}
+// A run of such entries, the next one's constants requested ahead.
+__device__ __forceinline__ void emo_flow_fwd_run_intv_each(const FlowParams &p, FlowIntv &iv, unsigned r, unsigned meta_a, unsigned ta0,
+                                                           unsigned tab_row, unsigned lmask, unsigned tok, unsigned &h, double &ea)
+{
+    uint4 meta = emo_tld_128(meta_a, tok);
+#pragma unroll 1
+    for (unsigned i = 0; i < r; ++i, ta0 += tab_row) {
+        const uint4 cur = meta;
+        meta_a += 32u;
+        meta = emo_tld_128(meta_a, tok);      // (one entry more than a stage has is there)
+        unsigned dd;
+        double e;
+        emo_flow_intv_own(p, iv, cur, h, ta0, lmask, tok, dd, e);
+        h += dd;
+        ea += e;
+    }
+}
+
 // The consumers read the clock only in the instantiations that fill the cycle counters (PROF): the reads sit
 // between the entries of the lanes' chains and cost the backward pass 6 % when they are always there.
 #define EMO_CLK() (PROF ? clock64() : 0LL)
 
-template <int MAXT, bool INTV, bool PROF>
+template <int MAXT, bool INTV, bool PROF, bool DENSE = false>
 __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
 {
     extern __shared__ __align__(128) unsigned char emo_smem[];
@@ -713,7 +756,9 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                     unsigned dd = 0;
                     double ee = 0.0;
                     uint4 meta = make_uint4(0, 0, 0, 0);
-                    if (INTV) {
+                    if (INTV && DENSE) {
+                        meta = emo_tld_128(meta_a, tok);
+                    } else if (INTV) {
                         // the level of the interval at hand
                         meta = emo_tld_128(meta_a + 16u, tok);
                         dd = emo_tld_u32(tab_a + iv.at, tok);
@@ -756,7 +801,9 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                         }
                     }
                     v = max(v, emo_floor_sub(x0, r1.z));
-                    if (INTV && meta.z != emo::kNone) {
+                    if (INTV && DENSE) {
+                        emo_flow_intv_own(p, iv, meta, v, tab_a, lmask, tok, dd, ee);
+                    } else if (INTV && meta.z != emo::kNone) {
                         const bool out = emo_flow_intv_leaves(iv, meta, v + dd);
                         if (__any_sync(0xFFFFFFFFu, out)) emo_flow_intv_cross(p, iv, emo_tld_128(meta_a, tok), v, out, tab_a, lmask, tok, dd, ee);
                         else iv.sum += (unsigned long long)meta.w + dd;
@@ -780,7 +827,9 @@ __global__ void __launch_bounds__(MAXT, 1) emo_flow_fwd(FlowParams p)
                     lvl_a += 32u;
                 }
                 // the run: every entry continues from the lane's previous value
-                if (INTV) {
+                if (INTV && DENSE) {
+                    emo_flow_fwd_run_intv_each(p, iv, (unsigned)r, meta_a, tab_a, tab_row, lmask, tok, h, ea);
+                } else if (INTV) {
                     const uint4 run = emo_tld_128(meta_a + 16u, tok);      // (an empty run's is not looked at; it lies inside the stage buffer)
                     bool ok = true;
                     switch (r) {

@@ -47,6 +47,7 @@ struct DevFlow {
     unsigned char *blobFI = nullptr;      // the forward blob followed by 32 bytes per entry: time-interval policies
     uint32_t *rows = nullptr, *push_base = nullptr;
     unsigned blobF_bytes = 0, blobB_bytes = 0, blobFI_bytes = 0, f_off_meta = 0;
+    int64_t packs = 0, switches = 0;      // time-interval policies: entries with a policy, and those whose predecessor on the lane is another device's
     unsigned off_seg = 0;
     unsigned f_off_rec = 0, f_off_pool = 0, f_off_tab = 0;
     unsigned b_off_rec = 0, b_off_pool = 0, b_off_lbes = 0, b_off_tab = 0;
@@ -614,6 +615,17 @@ int upload_flow(const Flow &f, DevFlow &d, bool intervals)
                     e += sg & kSegRunMask;
                 }
             }
+        }
+        for (int ln = 0; ln < f.lanes; ++ln) {
+            uint32_t last = kNone;
+            for (int st = 0; st < f.stages; ++st)
+                for (int k = 0; k < f.K; ++k) {
+                    const uint32_t grp = f.grp[((size_t)st * f.lanes + ln) * f.K + k];
+                    if (grp == kNone) continue;
+                    d.packs++;
+                    if (last != kNone && grp != last) d.switches++;
+                    last = grp;
+                }
         }
         rc = upload(&d.blobFI, bi.data(), bi.size());
     }
@@ -2261,7 +2273,16 @@ int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t 
             q.breaks = (const long long *)d_breaks;
             q.busy = busy;
             q.ldw = ldw;
-            void (*kern)(FlowParams) = fp.threads <= 512 ? emo_flow_fwd<512, true, false> : (fp.threads <= 768 ? emo_flow_fwd<768, true, false> : emo_flow_fwd<1024, true, false>);
+            // Where the lanes often change the device, or an interval holds less than an entry of a lane, keeping the interval at hand costs
+            // more than it saves: every entry looks its interval up.  Measured (ms, at hand / looked up): 8 devices on 18 lanes, 20 % of a lane's
+            // packs on another device than the one before, 38 000 nodes x 8 192 policies 3.06 / 2.83 with 2 intervals, 5.27 / 4.69 with 200;
+            // one device, 3 lanes, 2 500 packs x 16 384: 800 intervals 1.99 / 2.04, 1 600 4.46 / 4.35; 2 lanes, 250 packs: 200 0.310 /
+            // 0.282 (100: 0.237 / 0.223 would pay, the line is where 5 000 nodes turn); 25 000 nodes, 100 intervals 1.43 / 2.43.
+            const DevFlow &df = g->dflow;
+            const bool dense = df.switches * 20 > df.packs * 3 || (int64_t)g->flow.lanes * I > df.packs;
+            void (*kern)(FlowParams) = nullptr;
+            if (dense) kern = fp.threads <= 512 ? emo_flow_fwd<512, true, false, true> : (fp.threads <= 768 ? emo_flow_fwd<768, true, false, true> : emo_flow_fwd<1024, true, false, true>);
+            else kern = fp.threads <= 512 ? emo_flow_fwd<512, true, false> : (fp.threads <= 768 ? emo_flow_fwd<768, true, false> : emo_flow_fwd<1024, true, false>);
             if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
             kern<<<fp.grid_f, fp.threads, fp.smem_f, st>>>(q);
             EMO_CUDA(cudaGetLastError());
