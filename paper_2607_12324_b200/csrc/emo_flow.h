@@ -121,7 +121,6 @@ struct Spine {
     int max_segs = 0, max_pool = 0;
     int bundle = 2;                   // operations per bundle (n_ops is a multiple of it)
     int acc_words = 0;                // 4-byte words per policy that the sums / results of one stage take
-    int acc_words_all = 0;            // the same when every segment's head tail is kept (one more word per segment, behind the others)
     int64_t pushes = 0;
     int64_t segments = 0;
     std::vector<uint32_t> n_segs;     // [stages]

@@ -1722,9 +1722,9 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 int sk = code == 1 ? 8 : (code == 3 ? 32 : (code == 2 || flanes <= 8 ? 16 : 4));
                 while (sk > 8 && flanes * sk > 32 * kFlowRowRegs) sk /= 2;
                 start(spine_thread, [&, sk]() { compile_spine(sk, g->sflow, g->dspine, g->simage, rc_s, err_s); });
-                // the long stages: as many positions as keep a stage at about a hundred entries (25 000 nodes, 5 lanes x 2 000
-                // policies: 20 positions 0.78 ms, 16 0.83; 10 000, 3 lanes x 4 096: 32 0.60, 24 0.66; 51 000, 18 lanes x 1 000: 7 1.82,
-                // 6 1.90, 5 1.96)
+                // the long stages: as many positions as make about a hundred entries (ms, both passes: 25 000 nodes, 5 lanes x 2 000
+                // policies: 20 positions 0.78, 16 0.83; 10 000, 3 lanes x 4 096: 32 0.60, 24 0.66); more than eight lanes about 126, the
+                // seven positions that were best on the one wide graph measured (51 000, 18 lanes x 1 000: 7 1.82, 6 1.90, 5 1.96)
                 const int lk = std::min(32, (flanes > 8 ? 126 : 100) / flanes);
                 if (code == 0 && lk > sk)
                     start(long_thread, [&, lk]() { compile_spine(lk, g->lflow, g->dlong, g->limage, rc_l, err_l); });

@@ -214,7 +214,6 @@ int build_spine(const SpineIn &in, Spine &out, std::string &err)
     }
     out.max_segs = max_segs;
     out.acc_words = acc_words + 2;      // two scratch words behind the stage's sums (merge operations write there)
-    out.acc_words_all = out.acc_words + max_segs;      // with the heads' tails of all segments behind them (calls that want ES / LS / sums)
     const uint32_t scratch_acc = (uint32_t)acc_words;
 
     // ---- segment and member lists ---------------------------------------------------------------------
