@@ -68,6 +68,7 @@ extern "C" {
                                     * 32 per SM on a graph of at most eight lanes, where there is no spine program) */
 #define EMO_F_SPINE_KERNEL 0x20u   /* the spine kernels (the default wherever there is a spine program, but on graphs of more than eight lanes
                                     * without a program of longer stages only from two policy groups of 32 per SM on) */
+#define EMO_F_SLICE_KERNEL 0x40u   /* the slice kernels (the default for few policies) */
 #define EMO_F_TEST_STALL 0x100u    /* test hook of the 32-bit kernels: the producer warps stop half way, so that the
                                       consumers' bounded waits run out and EMO_E_TIMEOUT is reported */
 
@@ -434,8 +435,8 @@ int emo_slack_batch_prefetched(const emo_graph *g, int64_t B, int bits, const ui
 int emo_set_pass_events(void *fwd_start, void *fwd_stop, void *bwd_start, void *bwd_stop);
 
 /*
- * emo_call_path - which kernels emo_eval_policies (need_slack = 0) or emo_slack_batch (need_slack = 1)
- * would run for these arguments: 4 = the spine kernels with one policy per worker thread, 5 = the
+ * emo_call_path - which pass kernels emo_eval_policies (need_slack = 0) or emo_slack_batch (need_slack = 1)
+ * would run for these arguments, where the slice kernels do not take the call (emo_call_slices): 4 = the spine kernels with one policy per worker thread, 5 = the
  * spine kernels with several (calls without ES, LS and the sums), 2 = the 32-bit lane-stream kernels,
  * 1 = the staged 64-bit kernels,
  * 0 = the plain-load 64-bit kernels, 3 = the generic kernels (a graph beyond the on-chip schedules' limits, or
@@ -444,6 +445,13 @@ int emo_set_pass_events(void *fwd_start, void *fwd_stop, void *bwd_start, void *
  */
 int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb, int64_t ldo,
                   int need_slack, uint32_t flags);
+
+/*
+ * emo_call_slices - whether a call (as for emo_call_path, with a baseline column) is taken by the slice kernels: the number of
+ * slices that the graph is cut into, 0 when the kernels that emo_call_path names run.  The slice kernels take levels of any
+ * alignment and pitch; a workspace that is too small for them (but not for the others) also sends the call to the others.
+ */
+int emo_call_slices(const emo_graph *g, int64_t B, int need_slack, uint32_t flags);
 
 /*
  * emo_measure_int_issue - measurement helper (no counterpart in the method): the rate at which this GPU

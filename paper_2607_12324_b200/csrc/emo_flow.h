@@ -177,9 +177,20 @@ struct SpineIn {
 };
 int build_spine(const SpineIn &in, Spine &out, std::string &err);
 
+// What the compilers know about a graph before they schedule it: deduplicated edges both ways, static bounds of completion times
+// and tails (the recurrences above with the smallest / largest entry of every duration row) and the edges that can decide a maximum.
+struct GraphBounds {
+    std::vector<int64_t> pp, sp;                  // predecessor / successor CSR
+    std::vector<int32_t> pc, sc;
+    std::vector<int64_t> dmin, dmax, lbES, lbC, ubC, lbQin, lbQ, ubQ;
+    std::vector<char> constant;                   // node's tables do not depend on the level
+    std::vector<char> liveF, liveB;               // per predecessor-CSR edge
+};
+void graph_bounds(const HostGraph &g, const int64_t *lat, const double *energy, GraphBounds &b);
+
 // Compiles g into a lane-stream program.  Returns EMO_OK with out.ok32 = false when the 32-bit
 // representation does not apply (spread too large, too many lanes); other codes are errors.
-int compile_flow(const HostGraph &g, const int64_t *lat, const double *energy, int lanes, int lookahead,
+int compile_flow(const HostGraph &g, const int64_t *lat, const double *energy, const GraphBounds &gb, int lanes, int lookahead,
                  int K, int sync, Flow &out, std::string &err, bool spine = false);
 
 }  // namespace emo

@@ -63,7 +63,94 @@ void assign_slots(std::vector<SlotObj> &objs, int &n_tag, int &n_set)   // n_set
 
 }  // namespace
 
-int compile_flow(const HostGraph &g, const int64_t *lat, const double *energy, int lanes, int lookahead, int K, int sync,
+void graph_bounds(const HostGraph &g, const int64_t *lat, const double *energy, GraphBounds &b)
+{
+    const int32_t n = g.n;
+    const int L = g.L;
+    auto &pp = b.pp, &sp = b.sp;
+    auto &pc = b.pc, &sc = b.sc;
+    // ---- deduplicated predecessor and successor lists -------------------------------------------
+    pp.assign((size_t)n + 1, 0);
+    pc.clear();
+    pc.reserve((size_t)g.m);
+    for (int32_t v = 0; v < n; ++v) {
+        pc.insert(pc.end(), g.col.begin() + g.row_ptr[v], g.col.begin() + g.row_ptr[v + 1]);
+        std::sort(pc.begin() + pp[v], pc.end());
+        pc.erase(std::unique(pc.begin() + pp[v], pc.end()), pc.end());
+        pp[v + 1] = (int64_t)pc.size();
+    }
+    const int64_t m = (int64_t)pc.size();
+    sp.assign((size_t)n + 1, 0);
+    for (int64_t e = 0; e < m; ++e) sp[pc[e] + 1]++;
+    for (int32_t v = 0; v < n; ++v) sp[v + 1] += sp[v];
+    sc.assign((size_t)std::max<int64_t>(m, 1), 0);
+    {
+        std::vector<int64_t> fill(sp.begin(), sp.end() - 1);
+        for (int32_t v = 0; v < n; ++v)
+            for (int64_t e = pp[v]; e < pp[v + 1]; ++e) sc[fill[pc[e]]++] = v;
+    }
+
+    // ---- static bounds --------------------------------------------------------------------------
+    auto &dmin = b.dmin, &dmax = b.dmax;
+    dmin.assign((size_t)n, 0);
+    dmax.assign((size_t)n, 0);
+    b.constant.assign((size_t)n, 1);
+    for (int32_t v = 0; v < n; ++v) {
+        int64_t lo = lat[(size_t)v * L], hi = lo;
+        if (g.group[v] >= 0) {
+            for (int l = 1; l < L; ++l) {
+                lo = std::min(lo, lat[(size_t)v * L + l]);
+                hi = std::max(hi, lat[(size_t)v * L + l]);
+                if (lat[(size_t)v * L + l] != lat[(size_t)v * L] || energy[(size_t)v * L + l] != energy[(size_t)v * L]) b.constant[v] = 0;
+            }
+        }
+        dmin[v] = lo;
+        dmax[v] = hi;
+    }
+    auto &lbES = b.lbES, &lbC = b.lbC, &ubC = b.ubC, &lbQin = b.lbQin, &lbQ = b.lbQ, &ubQ = b.ubQ;
+    lbES.assign((size_t)n, 0);
+    lbC.assign((size_t)n, 0);
+    ubC.assign((size_t)n, 0);
+    std::vector<int64_t> ubES((size_t)n, 0), ubQin((size_t)n, 0);
+    std::vector<int32_t> bestF((size_t)n, -1), bestB((size_t)n, -1);
+    for (int32_t v = 0; v < n; ++v) {
+        for (int64_t e = pp[v]; e < pp[v + 1]; ++e) {
+            const int32_t k = pc[e];
+            ubES[v] = std::max(ubES[v], ubC[k]);
+            if (bestF[v] < 0 || lbC[k] > lbC[bestF[v]]) bestF[v] = k;
+        }
+        if (bestF[v] >= 0) lbES[v] = lbC[bestF[v]];
+        lbC[v] = lbES[v] + dmin[v];
+        ubC[v] = ubES[v] + dmax[v];
+    }
+    lbQin.assign((size_t)n, 0);
+    lbQ.assign((size_t)n, 0);
+    ubQ.assign((size_t)n, 0);
+    for (int32_t v = n - 1; v >= 0; --v) {
+        for (int64_t e = sp[v]; e < sp[v + 1]; ++e) {
+            const int32_t u = sc[e];
+            ubQin[v] = std::max(ubQin[v], ubQ[u]);
+            if (bestB[v] < 0 || lbQ[u] > lbQ[bestB[v]]) bestB[v] = u;
+        }
+        if (bestB[v] >= 0) lbQin[v] = lbQ[bestB[v]];
+        lbQ[v] = lbQin[v] + dmin[v];
+        ubQ[v] = ubQin[v] + dmax[v];
+    }
+
+    // ---- live edges -------------------------------------------------------------------------------
+    // edge e (k = pc[e] -> v): live forward unless C_k can never exceed the start every policy gives v
+    // through its strongest predecessor; live backward under the mirrored test on the tails
+    b.liveF.assign((size_t)std::max<int64_t>(m, 1), 0);
+    b.liveB.assign((size_t)std::max<int64_t>(m, 1), 0);
+    for (int32_t v = 0; v < n; ++v)
+        for (int64_t e = pp[v]; e < pp[v + 1]; ++e) {
+            const int32_t k = pc[e];
+            b.liveF[e] = (k == bestF[v]) || ubC[k] > lbES[v];
+            b.liveB[e] = (v == bestB[k]) || ubQ[v] > lbQin[k];
+        }
+}
+
+int compile_flow(const HostGraph &g, const int64_t *lat, const double *energy, const GraphBounds &gb, int lanes, int lookahead, int K, int sync,
                  Flow &out, std::string &err, bool spine)
 {
     out = Flow();
@@ -79,74 +166,15 @@ int compile_flow(const HostGraph &g, const int64_t *lat, const double *energy, i
     out.sync = sync;
     if (n == 0) return EMO_OK;
 
-    // ---- deduplicated predecessor and successor lists -------------------------------------------
-    std::vector<int64_t> pp((size_t)n + 1, 0);
-    std::vector<int32_t> pc;
-    pc.reserve((size_t)g.m);
-    for (int32_t v = 0; v < n; ++v) {
-        std::vector<int32_t> p(g.col.begin() + g.row_ptr[v], g.col.begin() + g.row_ptr[v + 1]);
-        std::sort(p.begin(), p.end());
-        p.erase(std::unique(p.begin(), p.end()), p.end());
-        pc.insert(pc.end(), p.begin(), p.end());
-        pp[v + 1] = (int64_t)pc.size();
-    }
-    const int64_t m = (int64_t)pc.size();
-    std::vector<int64_t> sp((size_t)n + 1, 0);
-    for (int64_t e = 0; e < m; ++e) sp[pc[e] + 1]++;
-    for (int32_t v = 0; v < n; ++v) sp[v + 1] += sp[v];
-    std::vector<int32_t> sc((size_t)std::max<int64_t>(m, 1));
-    {
-        std::vector<int64_t> fill(sp.begin(), sp.end() - 1);
-        for (int32_t v = 0; v < n; ++v)
-            for (int64_t e = pp[v]; e < pp[v + 1]; ++e) sc[fill[pc[e]]++] = v;
-    }
-
-    // ---- static bounds --------------------------------------------------------------------------
-    std::vector<int64_t> dmin((size_t)n), dmax((size_t)n);
-    std::vector<char> constant((size_t)n, 1);
-    for (int32_t v = 0; v < n; ++v) {
-        int64_t lo = lat[(size_t)v * L], hi = lo;
-        if (g.group[v] >= 0) {
-            for (int l = 1; l < L; ++l) {
-                lo = std::min(lo, lat[(size_t)v * L + l]);
-                hi = std::max(hi, lat[(size_t)v * L + l]);
-                if (lat[(size_t)v * L + l] != lat[(size_t)v * L] || energy[(size_t)v * L + l] != energy[(size_t)v * L]) constant[v] = 0;
-            }
-        }
-        dmin[v] = lo;
-        dmax[v] = hi;
-    }
-    std::vector<int64_t> lbES((size_t)n, 0), ubES((size_t)n, 0), lbC((size_t)n), ubC((size_t)n);
-    std::vector<int32_t> bestF((size_t)n, -1), bestB((size_t)n, -1);
-    for (int32_t v = 0; v < n; ++v) {
-        for (int64_t e = pp[v]; e < pp[v + 1]; ++e) {
-            const int32_t k = pc[e];
-            ubES[v] = std::max(ubES[v], ubC[k]);
-            if (bestF[v] < 0 || lbC[k] > lbC[bestF[v]]) bestF[v] = k;
-        }
-        if (bestF[v] >= 0) lbES[v] = lbC[bestF[v]];
-        lbC[v] = lbES[v] + dmin[v];
-        ubC[v] = ubES[v] + dmax[v];
-    }
-    std::vector<int64_t> lbQin((size_t)n, 0), ubQin((size_t)n, 0), lbQ((size_t)n), ubQ((size_t)n);
-    for (int32_t v = n - 1; v >= 0; --v) {
-        for (int64_t e = sp[v]; e < sp[v + 1]; ++e) {
-            const int32_t u = sc[e];
-            ubQin[v] = std::max(ubQin[v], ubQ[u]);
-            if (bestB[v] < 0 || lbQ[u] > lbQ[bestB[v]]) bestB[v] = u;
-        }
-        if (bestB[v] >= 0) lbQin[v] = lbQ[bestB[v]];
-        lbQ[v] = lbQin[v] + dmin[v];
-        ubQ[v] = ubQin[v] + dmax[v];
-    }
+    const auto &pp = gb.pp, &sp = gb.sp;
+    const auto &pc = gb.pc, &sc = gb.sc;
+    const auto &dmin = gb.dmin, &lbES = gb.lbES, &lbC = gb.lbC, &ubC = gb.ubC, &lbQin = gb.lbQin, &lbQ = gb.lbQ, &ubQ = gb.ubQ;
+    const auto &constant = gb.constant, &liveF = gb.liveF, &liveB = gb.liveB;
     const int64_t kMax32 = 0xFFFFFFFFLL;
     for (int32_t v = 0; v < n; ++v)
         if (ubC[v] - lbC[v] > kMax32 || ubQ[v] - lbQ[v] > kMax32) return EMO_OK;   // ok32 stays false
 
-    // ---- live edges and the schedule ------------------------------------------------------------
-    // edge e (k = pc[e] -> v): live forward unless C_k can never exceed the start every policy gives v
-    // through its strongest predecessor; live backward under the mirrored test on the tails
-    std::vector<char> liveF((size_t)std::max<int64_t>(m, 1), 0), liveB((size_t)std::max<int64_t>(m, 1), 0);
+    // ---- the schedule ----------------------------------------------------------------------------
     // An edge that is live in one direction only keeps its two nodes a period apart in the schedule:
     // its reader (in that direction) then finds the value settled behind a barrier instead of polling
     // for it, and nothing waits for the reader in the other direction.  (Typical: a launch node and
@@ -157,8 +185,6 @@ int compile_flow(const HostGraph &g, const int64_t *lat, const double *energy, i
     for (int32_t v = 0; v < n; ++v)
         for (int64_t e = pp[v]; e < pp[v + 1]; ++e) {
             const int32_t k = pc[e];
-            liveF[e] = (k == bestF[v]) || ubC[k] > lbES[v];
-            liveB[e] = (v == bestB[k]) || ubQ[v] > lbQin[k];
             if (!liveF[e]) out.f.pruned++;
             if (!liveB[e]) out.b.pruned++;
             if (liveF[e] || liveB[e]) {

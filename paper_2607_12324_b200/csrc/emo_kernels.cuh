@@ -318,6 +318,31 @@ __global__ void emo_select_stage2(int nparts, const SelectPartial *part, const i
     }
 }
 
+// Where the first stage is one block it finishes by itself, in the same order.
+__global__ void emo_select_one(int64_t B, const int64_t *makespan, const double *energy, int64_t target, const int64_t *target_dev, int64_t delta_ppm,
+                               int64_t *out_index, int64_t *out_T, double *out_E)
+{
+    __shared__ SelectPartial sh[32];
+    emo_grid_wait_previous();
+    if (target_dev) target = emo_budget(target_dev[0], delta_ppm);
+    double e = 0.0;
+    long long idx = -1;
+    for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
+        const int64_t t = makespan[b];
+        const double x = energy[b];
+        if (t <= target && emo_better(x, b, e, idx)) {
+            e = x;
+            idx = b;
+        }
+    }
+    emo_select_reduce(e, idx, sh);
+    if (threadIdx.x == 0) {
+        *out_index = idx;
+        if (out_T) *out_T = idx >= 0 ? makespan[idx] : 0;
+        if (out_E) *out_E = idx >= 0 ? e : 0.0;
+    }
+}
+
 // src [B][lds] -> dst [rows][ldb], 32x32 byte tiles through shared memory.
 __global__ void emo_transpose_u8(int64_t B, int64_t rows, const uint8_t *src, int64_t lds, uint8_t *dst, int64_t ldb)
 {

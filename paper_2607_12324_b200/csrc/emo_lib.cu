@@ -22,6 +22,7 @@
 #include "emo_intervals.cuh"
 #include "emo_model.cuh"
 #include "emo_generic.cuh"
+#include "emo_slice.cuh"
 
 using namespace emo;
 
@@ -73,6 +74,23 @@ struct DevSpine {
     bool ready = false;             // on the device (host-only handles: laid out)
 };
 
+// Blocks of the slice kernels: policies, slices.
+constexpr int kSliceShapes = 3;
+constexpr int kSliceP[kSliceShapes] = {1, 8, 16}, kSliceS[kSliceShapes] = {4, 1, 1};
+
+// The slice program on the device (emo_slice.cuh), and what its launches need to know.
+struct DevSlice {
+    unsigned char *mem = nullptr;   // the allocation that holds all of it
+    uint32_t *blob = nullptr;
+    uint4 *index = nullptr, *rec = nullptr;
+    uint32_t *tabT = nullptr;
+    double *tabE = nullptr;
+    int count = 0, cols = 0, Lp = 0, group = 0, groups = 0;
+    unsigned head = 0, words = 0, steps[2] = {0, 0}, nodes = 0, len[2] = {0, 0};      // most of one slice
+    unsigned slots1[2] = {0, 0}, slots2[2] = {0, 0};
+    bool ready = false;
+};
+
 // The spine program as the device gets it: one allocation, one copy.
 struct SpineImage {
     std::vector<unsigned char> host;
@@ -90,6 +108,7 @@ struct emo_graph {
     DevSpine dspine;
     Flow lflow;                      // ... and once more with longer stages, for calls of at most two policy groups per SM
     DevSpine dlong;
+    DevSlice dslice;                 // slices of the graph, for calls with few policies
     SpineImage simage, limage;       // both as laid out for the device (kept by host-only handles, else until they are copied)
     bool host_only = false;
     // graphs beyond the schedule compilers' limits (or loaded with EMO_F_GENERIC): evaluated by the generic kernels
@@ -1056,10 +1075,10 @@ bool flow_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, Flo
 // Launches a kernel that may start before its predecessor in the stream ends (it waits for it where it needs it).  Measured:
 // 400 nodes x 64, forward, backward and selection, 41 us one after the other, 31 ahead.
 template <typename... A>
-cudaError_t launch_ahead(void (*kern)(A...), int grid, int threads, size_t smem, cudaStream_t st, A... args)
+cudaError_t launch_ahead_grid(void (*kern)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t c = {};
-    c.gridDim = dim3((unsigned)grid);
+    c.gridDim = grid;
     c.blockDim = dim3((unsigned)threads);
     c.dynamicSmemBytes = smem;
     c.stream = st;
@@ -1069,6 +1088,12 @@ cudaError_t launch_ahead(void (*kern)(A...), int grid, int threads, size_t smem,
     c.attrs = attr;
     c.numAttrs = 1;
     return cudaLaunchKernelEx(&c, kern, args...);
+}
+
+template <typename... A>
+cudaError_t launch_ahead(void (*kern)(A...), int grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    return launch_ahead_grid(kern, dim3((unsigned)grid), threads, smem, st, args...);
 }
 
 // The opt-in shared-memory size is set once per kernel (not per launch: concurrent callers with
@@ -1436,6 +1461,310 @@ bool flow_allowed(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
     return ldb % 16 == 0 && aligned16(lvl) && ldb < big && ldo < big;
 }
 
+// ---- slices -------------------------------------------------------------------------------------------------
+int upload_slices(const Slices &s, DevSlice &d)
+{
+    d = DevSlice();
+    if (!s.ok) return EMO_OK;
+    std::vector<uint4> index((size_t)s.count);
+    for (int k = 0; k < s.count; ++k) {
+        SliceHdr h;
+        std::memcpy(&h, s.blob.data() + s.off[(size_t)k], sizeof(h));
+        index[(size_t)k] = make_uint4(s.off[(size_t)k], h.nodes, h.node0, std::min(h.head, 0xFFFFu) | std::min(h.words, 0xFFFFu) << 16);
+        d.words = std::max(d.words, h.words);
+        d.head = std::max(d.head, h.head);
+        d.nodes = std::max(d.nodes, h.nodes);
+        for (int i = 0; i < 2; ++i) {
+            d.len[i] = std::max(d.len[i], h.dir[i].len);
+            d.steps[i] = std::max(d.steps[i], h.dir[i].steps);
+            d.slots1[i] = std::max(d.slots1[i], h.dir[i].slots1);
+            d.slots2[i] = std::max(d.slots2[i], h.dir[i].slots2);
+        }
+    }
+    const void *src[5] = {s.blob.data(), index.data(), s.rec.data(), s.tabT.data(), s.tabE.data()};
+    const size_t bytes[5] = {s.blob.size() * 4, index.size() * sizeof(uint4), s.rec.size() * 4, s.tabT.size() * 4, s.tabE.size() * 8};
+    size_t at[5], total = 0;
+    for (int i = 0; i < 5; ++i) {
+        at[i] = total;
+        total += round_up(bytes[i], 256);
+    }
+    std::vector<unsigned char> image(total);
+    for (int i = 0; i < 5; ++i) std::memcpy(image.data() + at[i], src[i], bytes[i]);
+    unsigned char *mem = nullptr;
+    const cudaError_t rc = cudaMalloc(&mem, total);
+    if (rc != cudaSuccess || cudaMemcpy(mem, image.data(), total, cudaMemcpyHostToDevice) != cudaSuccess) {
+        (void)cudaGetLastError();
+        if (mem) cudaFree(mem);
+        return rc == cudaErrorMemoryAllocation ? EMO_E_OOM : EMO_E_CUDA;
+    }
+    d.mem = mem;
+    d.blob = (uint32_t *)(d.mem + at[0]);
+    d.index = (uint4 *)(d.mem + at[1]);
+    d.rec = (uint4 *)(d.mem + at[2]);
+    d.tabT = (uint32_t *)(d.mem + at[3]);
+    d.tabE = (double *)(d.mem + at[4]);
+    d.count = s.count;
+    d.cols = s.cols;
+    d.Lp = s.Lp;
+    d.group = s.group;
+    d.groups = s.groups;
+    d.ready = true;
+    return EMO_OK;
+}
+
+// How a call takes the slice kernels.
+struct SlicePlan {
+    int shape = 0;                  // index into kSliceP
+    SliceParams p, pv;              // of the matrices' kernel and the chaining, of the values' kernel; workspace pointers as offsets
+    size_t smem_m = 0, smem_v = 0, smem_g = 0, smem_s = 0, ws = 0;
+    int whole = -1;                 // index into kSliceWhole: one block per policy does everything (p, smem_m)
+};
+struct SliceKernels {
+    void (*matrix)(SliceParams), (*values)(SliceParams), (*single)(SliceParams);
+    int threads;
+};
+template <int SHAPE, int NT>
+constexpr SliceKernels slice_kernels()
+{
+    return {emo_slice_matrix<kSliceP[SHAPE], kSliceS[SHAPE], NT>, emo_slice_values<kSliceP[SHAPE], kSliceS[SHAPE], NT, false>, emo_slice_values<kSliceP[SHAPE], 1, NT, true>, NT};
+}
+const SliceKernels kSliceKernels[kSliceShapes] = {slice_kernels<0, 256>(), slice_kernels<1, 256>(), slice_kernels<2, 256>()};
+
+// The kernels that chain matrices: threads per unit and block, buffers of the ring.  Matrices of more than 16 columns are not
+// multiplied (the product of two costs as many additions as a chaining of all slices), their slices are chained one by one.
+struct SliceChain {
+    int cols, lanes, threads, ring;
+    void (*group)(SliceParams), (*scan)(SliceParams);
+};
+template <int LPP, int D, int CW>
+constexpr SliceChain slice_chain_of()
+{
+    return {CW, LPP, 32, D, emo_slice_group<LPP, D, CW>, emo_slice_scan<LPP, D, CW>};
+}
+const SliceChain kSliceChains[] = {slice_chain_of<8, 16, 4>(), slice_chain_of<8, 16, 8>(), slice_chain_of<16, 8, 12>(), slice_chain_of<16, 8, 16>(),
+                                   {emo::kSliceMaxCols, 256, 256, 6, nullptr, emo_slice_scan_wide<6>}};
+const SliceChain &slice_chain(int cols)
+{
+    int i = 0;
+    while (kSliceChains[i].cols < cols) ++i;
+    return kSliceChains[i];
+}
+
+// One block per policy: most slices, threads.
+struct SliceWhole {
+    int slices, threads;
+    void (*kern)(SliceParams);
+};
+const SliceWhole kSliceWhole[] = {{4, 512, emo_slice_whole<4, 512>}, {8, 512, emo_slice_whole<8, 512>}};
+
+bool slice_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, int shape, SlicePlan &pl)
+{
+    const DevSlice &d = g->dslice;
+    if (!d.ready) return false;
+    if (d.head > 0xFFFF) return false;
+    const int64_t nb = B + (want_base ? 1 : 0), P = kSliceP[shape];
+    const int64_t tiles = (nb + P - 1) / P;
+    pl.shape = shape;
+    SliceParams &p = pl.p;
+    p = SliceParams();
+    p.blob = d.blob;
+    p.index = d.index;
+    p.rec = d.rec;
+    p.tabT = d.tabT;
+    p.tabE = d.tabE;
+    p.count = d.count;
+    p.cols = d.cols;
+    p.Lp = d.Lp;
+    p.L = g->h.L;
+    p.dirs = need_bwd ? 2 : 1;
+    const SliceChain &ch = slice_chain(d.cols);
+    const bool grouped = d.groups > 1 && ch.group;
+    p.group = grouped ? d.group : d.count;
+    p.groups = grouped ? d.groups : 1;
+    p.B = B;
+    p.nb = nb;
+    p.nbp = tiles * P;
+    if (tiles * d.count > 0x7FFFFFFF || (int64_t)p.groups * p.nbp > 0x7FFFFFFF) return false;
+    p.tiles = (int)tiles;
+    // workspace: matrices, groups' matrices, values that enter, energies
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        const size_t here = at;
+        at += round_up(bytes, 256);
+        return (unsigned char *)nullptr + here;
+    };
+    const size_t size = (size_t)d.cols * d.cols;
+    if (d.count > 1) {
+        for (int i = 0; i < p.dirs; ++i) {
+            p.mat[i] = (int32_t *)take((size_t)d.count * p.nbp * size * 4);
+            p.gmat[i] = (int32_t *)take(p.groups > 1 ? (size_t)p.groups * p.nbp * size * 4 : 0);
+            p.state[i] = (long long *)take((size_t)d.count * p.nbp * d.cols * 8);
+        }
+        p.epart = (double *)take((size_t)d.count * p.nbp * 8);
+        p.gepart = (double *)take((size_t)p.groups * p.nbp * 8);
+    }
+    pl.ws = at;
+    // shared memory
+    pl.pv = p;
+    const int NT = kSliceKernels[shape].threads, S = d.count > 1 ? kSliceS[shape] : 1;
+    auto layout = [&](SliceParams &q, const unsigned (&slots)[2], unsigned slot_bytes) {
+        size_t o = round_up((size_t)d.head * 4, 128);
+        q.at_rec = (unsigned)o;
+        o += (size_t)d.nodes * 16;
+        for (int i = 0; i < q.dirs; ++i) {
+            q.at_ops[i] = (unsigned)o;
+            o += (size_t)(d.steps[i] + 1) * 32;
+        }
+        for (int i = 0; i < q.dirs; ++i) {
+            o = round_up(o, 128);
+            q.at_inc[i] = (unsigned)o;
+            o += (size_t)d.len[i] * P * 4;
+        }
+        for (int i = 0; i < q.dirs; ++i) {
+            o = round_up(o, 128);
+            q.at_slot[i] = (unsigned)o;
+            o += (size_t)slots[i] * slot_bytes;
+        }
+        o = round_up(o, 128) + (S > 1 ? 32 : 0);      // (slices side by side in a warp: not on the same banks)
+        q.slice_bytes = (unsigned)o;
+        q.at_red = (unsigned)(o * S);
+        return o * S + (size_t)NT * 8 + (size_t)P * 8;
+    };
+    pl.smem_m = layout(pl.p, d.slots1, 4u * (unsigned)P * (unsigned)d.cols);
+    pl.smem_v = layout(pl.pv, d.slots2, 8u * (unsigned)P);
+    pl.whole = -1;
+    if (shape == 0 && d.count > 1 && d.cols <= 32 && d.words <= 0xFFFF && nb <= 0x7FFFFFFF) {
+        for (int w = 0; w < 2 && pl.whole < 0; ++w) {
+            const SliceWhole &k = kSliceWhole[w];
+            if (d.count > k.slices) continue;
+            SliceParams q = p;
+            size_t o = (size_t)d.words * 4;
+            q.at_rec = (unsigned)o;
+            o += (size_t)d.nodes * 16;
+            for (int i = 0; i < q.dirs; ++i) {
+                q.at_inc[i] = (unsigned)o;
+                o += round_up((size_t)d.len[i] * 4, 16);
+            }
+            for (int i = 0; i < q.dirs; ++i) {
+                q.at_slot[i] = (unsigned)o;
+                o += round_up(std::max((size_t)d.slots1[i] * d.cols * 4, (size_t)d.slots2[i] * 8), 16);
+            }
+            o = round_up(o, 128) + 32;      // (slices side by side in a warp: not on the same banks)
+            q.slice_bytes = (unsigned)o;
+            q.at_red = (unsigned)(o * d.count);
+            const size_t total = o * d.count + (size_t)k.threads * 8 + 16 + (size_t)2 * k.slices * d.cols * 8 + (size_t)2 * k.slices * size * 4;
+            if (total > g->smem_optin) continue;
+            pl.p = q;
+            pl.smem_m = total;
+            pl.ws = 0;
+            pl.whole = w;
+        }
+    }
+    if (pl.whole >= 0) return true;
+    pl.smem_g = (size_t)(ch.threads / ch.lanes) * size * 4 * ch.ring;
+    pl.smem_s = pl.smem_g + (size_t)(ch.threads / ch.lanes) * d.cols * 16;
+    const size_t budget = g->smem_optin;
+    return (d.count == 1 || pl.smem_m <= budget) && pl.smem_v <= budget && pl.smem_g <= budget && pl.smem_s <= budget;
+}
+
+// Most policies (the all-max one included) of a call that the slice kernels take.  Their time grows with the policies, that of the
+// spine kernels not before they fill the SMs.  Measured (us, slices / the others):
+//   slack       10 000 nodes x 257 105 / 593, x 1 025 348 / 596; 25 000 x 1 025 676 / 770, x 1 501 964 / 768; 1 013 x 1 025 55 / 76, x 1 501 71 / 76
+//   all outputs 10 000 x 1 501 532 / 689; 25 000 x 1 025 712 / 911, x 1 501 1 013 / 911
+//   forward     10 000 x 1 025 98 / 263; 25 000 x 1 501 250 / 249; 400 x 1 501 16 / 14
+//   one slice   213 x 4 097 20.7 / 23.3 (forward 12.0 / 12.9, both the call)
+//   40 columns (12 839 nodes, 18 lanes): slack x 17 192 / 447, x 65 438 / 447; forward x 17 109 / 123, x 65 207 / 123
+int64_t slice_limit(const emo_graph *g, bool need_bwd, bool extra)
+{
+    const DevSlice &d = g->dslice;
+    if (d.count == 1) return 4352;
+    if (d.cols <= 8) return need_bwd ? (extra ? 1300 : 1100) : 1400;
+    return 65536 / ((int64_t)d.cols * d.cols) / (need_bwd ? 1 : 2);
+}
+
+// Whether a call takes the slice kernels, and with which blocks.  Measured (us): one block per policy where all are there at once, 400
+// nodes x 64 16.6 / 21.5, 1 013 x 64 23.7 / 26.3 in three kernels.  Else one policy per block (four slices) for up to four, and for wide
+// matrices, which fill a warp's lanes with one policy (12 839 nodes x 16, 40 columns 192 / 293); 16 policies instead of 8 where a
+// block's columns are the work, forward (250 000 x 256 440 / 603), or where three large blocks still fit an SM and there are plenty
+// (250 000 x 256 1 749 / 2 002; but 10 000 x 257 115 / 105, two blocks and a half).
+bool slice_allowed(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, bool extra, uint32_t flags, SlicePlan &pl)
+{
+    const DevSlice &d = g->dslice;
+    if (!d.ready) return false;
+    if (flags & (EMO_F_NO_STAGING | EMO_F_PAIR_KERNEL | EMO_F_LANE_KERNEL | EMO_F_FLOW_KERNEL | EMO_F_SPINE_KERNEL | EMO_F_TEST_STALL)) return false;
+    const int64_t nb = B + (want_base ? 1 : 0);
+    if (nb == 0) return false;
+    if (!(flags & EMO_F_SLICE_KERNEL) && nb > slice_limit(g, need_bwd, extra)) return false;
+    const bool one = slice_plan(g, B, want_base, need_bwd, 0, pl);
+    const int64_t at_once = one ? (int64_t)g->sm_count * std::min<int64_t>(4, (int64_t)g->smem_optin / (int64_t)std::max<size_t>(pl.whole >= 0 ? pl.smem_m : pl.smem_v, 1)) : 0;
+    if (one && (d.count == 1 ? nb <= at_once : (pl.whole >= 0 ? nb <= at_once : nb <= 4 || d.cols > 16))) return true;
+    if (d.count > 1 && nb > 32 && slice_plan(g, B, want_base, need_bwd, 2, pl) &&
+        (!need_bwd || (3 * pl.smem_v <= (size_t)200 * 1024 && (int64_t)d.count * pl.p.tiles >= 9 * (int64_t)g->sm_count)))
+        return true;
+    return slice_plan(g, B, want_base, need_bwd, 1, pl);
+}
+
+int launch_slices(const emo_graph *g, SlicePlan &pl, const uint8_t *lvl, int64_t ldb, int64_t *ES, int64_t *LS, int64_t *slack, int64_t ldo, int64_t *makespan,
+                  double *energy, int64_t *slack_sum, int32_t *n_critical, int64_t *base_T, double *base_E, unsigned char *ws, cudaStream_t st)
+{
+    const SliceKernels &k = kSliceKernels[pl.shape];
+    for (SliceParams *p : {&pl.p, &pl.pv}) {
+        p->lvl = lvl;
+        p->ldb = ldb;
+        p->ES = ES;
+        p->LS = LS;
+        p->slack = slack;
+        p->ldo = ldo;
+        p->makespan = makespan;
+        p->energy = energy;
+        p->slack_sum = slack_sum;
+        p->n_critical = n_critical;
+        p->base_T = base_T;
+        p->base_E = base_E;
+        for (int i = 0; i < p->dirs; ++i) {
+            p->mat[i] = (int32_t *)(ws + (size_t)p->mat[i]);
+            p->gmat[i] = (int32_t *)(ws + (size_t)p->gmat[i]);
+            p->state[i] = (long long *)(ws + (size_t)p->state[i]);
+        }
+        p->epart = (double *)(ws + (size_t)p->epart);
+        p->gepart = (double *)(ws + (size_t)p->gepart);
+    }
+    const SliceParams &p = pl.p;
+    const int slices = p.count > 1 ? kSliceS[pl.shape] : 1, blocks = (p.count + slices - 1) / slices * p.tiles;
+    cudaEvent_t ev0 = g_pass_events[0], ev1 = g_pass_events[1], ev2 = g_pass_events[2], ev3 = g_pass_events[3];
+    if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
+    if (pl.whole >= 0) {
+        const SliceWhole &w = kSliceWhole[pl.whole];
+        if (flow_optin(w.kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+        EMO_CUDA(launch_ahead(w.kern, (int)p.nb, w.threads, pl.smem_m, st, p));
+        for (cudaEvent_t ev : {ev1, ev2, ev3})
+            if (ev) EMO_CUDA(cudaEventRecord(ev, st));
+        return EMO_OK;
+    }
+    if (p.count > 1) {
+        if (flow_optin(k.matrix, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+        EMO_CUDA(launch_ahead(k.matrix, blocks, k.threads, pl.smem_m, st, p));
+        const SliceChain &ch = slice_chain(p.cols);
+        const int64_t units = (int64_t)p.groups * p.nbp, per = ch.threads / ch.lanes;
+        const dim3 grid((unsigned)((units + per - 1) / per), (unsigned)p.dirs);
+        if (p.groups > 1) {
+            if (flow_optin(ch.group, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+            EMO_CUDA(launch_ahead_grid(ch.group, grid, ch.threads, pl.smem_g, st, p));
+        }
+        if (flow_optin(ch.scan, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+        EMO_CUDA(launch_ahead_grid(ch.scan, grid, ch.threads, pl.smem_s, st, p));
+    }
+    if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
+    if (ev2) EMO_CUDA(cudaEventRecord(ev2, st));
+    if (p.count == 1 || p.dirs > 1) {
+        void (*values)(SliceParams) = p.count == 1 ? k.single : k.values;
+        if (flow_optin(values, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+        EMO_CUDA(launch_ahead(values, blocks, k.threads, pl.smem_v, st, pl.pv));
+    }
+    if (ev3) EMO_CUDA(cudaEventRecord(ev3, st));
+    return EMO_OK;
+}
+
 int launch_validate(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb, int32_t *status, cudaStream_t st)
 {
     if (!status) return EMO_E_INVALID_ARG;
@@ -1495,6 +1824,14 @@ int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
     int rc = make_plan(g, B, true, need_slack != 0, lvl, ldb, ld_ws, ldo, flags, pl);
     if (rc) return rc;
     return pl.staged ? 1 : 0;
+}
+
+int emo_call_slices(const emo_graph *g, int64_t B, int need_slack, uint32_t flags)
+{
+    if (!g || B < 0) return EMO_E_INVALID_ARG;
+    if (g->host_only) return EMO_E_CUDA;
+    SlicePlan cp;
+    return slice_allowed(g, B, true, need_slack != 0, false, flags, cp) ? g->dslice.count : 0;
 }
 
 int emo_measure_int_issue(double *ops_per_s, void *scratch_dev, void *stream)
@@ -1614,6 +1951,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
 
     emo_graph *g = new (std::nothrow) emo_graph();
     if (!g) return EMO_E_OOM;
+    Slices slices;
     try {
         HostGraph &h = g->h;
         h.n = n;
@@ -1687,6 +2025,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             // says otherwise; compiled on a thread of its own beside the lane-stream program (they share nothing but
             // their inputs)
             const bool want_spine = !(flags & EMO_F_INTERVALS);
+            // the slice program, for calls with few policies: another thread (not where the caller shapes the spine program)
+            const bool want_slices = want_spine && !(flags & (EMO_F_HOST_ONLY | 0xC0000000u));
+            GraphBounds bounds;
+            graph_bounds(h, lat, energy, bounds);
             int rc_s = EMO_OK, rc_l = EMO_E_UNSUPPORTED;
             std::string err_s, err_l;
             // (what ends the block early, an exception among it, waits for them)
@@ -1694,7 +2036,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 std::thread t;
                 void wait() { if (t.joinable()) t.join(); }
                 ~Helper() { wait(); }
-            } spine_thread, long_thread;
+            } spine_thread, long_thread, slice_thread;
             auto start = [](Helper &helper, auto work) {
                 try {
                     helper.t = std::thread(work);
@@ -1706,7 +2048,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             auto compile_spine = [&](int k, Flow &out, DevSpine &d, SpineImage &im, int &rc_k, std::string &err_k) {
                 try {
                     if (no_long && &out == &g->lflow) throw std::bad_alloc();
-                    rc_k = compile_flow(h, lat, energy, lanes, look, k, k, out, err_k, true);
+                    rc_k = compile_flow(h, lat, energy, bounds, lanes, look, k, k, out, err_k, true);
                     if (rc_k == EMO_OK) rc_k = lay_out_spine(out, d, im);
                 } catch (const std::bad_alloc &) {
                     rc_k = EMO_E_OOM;
@@ -1714,6 +2056,14 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                     rc_k = EMO_E_UNSUPPORTED;
                 }
             };
+            if (want_slices)
+                start(slice_thread, [&]() {
+                    try {
+                        compile_slices(h, lat, energy, bounds, slices);
+                    } catch (const std::exception &) {      // no memory for it: the others serve
+                        slices = Slices();
+                    }
+                });
             if (want_spine) {
                 const int code = (int)((flags >> 30) & 3u);
                 // Measured (forward + backward, ms): 18 lanes, 128 039 nodes x 8 192 policies 6.2 with 4 positions, 6.6 with 5
@@ -1730,12 +2080,13 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                     start(long_thread, [&, lk]() { compile_spine(lk, g->lflow, g->dlong, g->limage, rc_l, err_l); });
             }
             try {
-                rc = compile_flow(h, lat, energy, lanes, look, fk, fs, g->flow, err);
+                rc = compile_flow(h, lat, energy, bounds, lanes, look, fk, fs, g->flow, err);
             } catch (const std::bad_alloc &) {
                 rc = EMO_E_OOM;
             }
             spine_thread.wait();
             long_thread.wait();
+            slice_thread.wait();
             if (rc == EMO_E_UNSUPPORTED) {      // the 64-bit programs exist: they serve
                 g->flow = Flow();
                 rc = EMO_OK;
@@ -1828,7 +2179,9 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                 int lanes = (int)((flags >> 8) & 0xFF);
                 std::string err;
                 free_flow(g->dflow);
-                rc = compile_flow(g->h, lat, energy, lanes, look, fk, 16, g->flow, err);
+                GraphBounds bounds;
+                graph_bounds(g->h, lat, energy, bounds);
+                rc = compile_flow(g->h, lat, energy, bounds, lanes, look, fk, 16, g->flow, err);
                 if (rc == EMO_E_UNSUPPORTED) {
                     g->flow = Flow();
                     rc = EMO_OK;
@@ -1844,6 +2197,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             else rc = rc_l;
         }
         g->simage = g->limage = SpineImage();
+        if (rc == EMO_OK && slices.ok) {
+            const int rc_c = upload_slices(slices, g->dslice);
+            if (rc_c != EMO_OK && rc_c != EMO_E_OOM) rc = rc_c;      // (no memory for it: the others serve)
+        }
         }
         } catch (const std::bad_alloc &) {
             rc = EMO_E_OOM;
@@ -1865,6 +2222,7 @@ int emo_graph_free(emo_graph *g)
         free_flow(g->dflow);
         free_spine(g->dspine);
         free_spine(g->dlong);
+        if (g->dslice.mem) cudaFree(g->dslice.mem);
         void *gen[] = {g->gen_row_ptr, g->gen_col, g->gen_srow_ptr, g->gen_scol, g->gen_group, g->gen_lat, g->gen_energy};
         for (void *q : gen)
             if (q) cudaFree(q);
@@ -2135,15 +2493,13 @@ static int launch_generic(const emo_graph *g, int64_t B, const uint8_t *lvl, int
     return EMO_OK;
 }
 
-int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint32_t flags, int aligned, size_t *out)
+// Workspace of the pass kernels (a call with less than that is refused; the slice kernels' share is only for their use).
+static size_t pass_ws_bytes(const emo_graph *g, int64_t B, int need_slack, uint32_t flags, int aligned)
 {
-    if (!g || !out || B < 0) return EMO_E_INVALID_ARG;
     size_t bytes = kSmallWs + lvl_area(g);
     if (g->generic) {
         bytes += generic_need(g, B, need_slack != 0);
-        if (need_slack == 2) bytes += 4 * round_up((size_t)B * 8, 256) + 256;
-        *out = bytes;
-        return EMO_OK;
+        return bytes;
     }
     if (need_slack) {
         // what the call with these flags will run: the 32-bit kernels keep a restore list between the
@@ -2165,6 +2521,15 @@ int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint3
         }
         bytes += need;
     }
+    return bytes;
+}
+
+int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint32_t flags, int aligned, size_t *out)
+{
+    if (!g || !out || B < 0) return EMO_E_INVALID_ARG;
+    size_t bytes = pass_ws_bytes(g, B, need_slack, flags, aligned);
+    SlicePlan cp;
+    if (!g->host_only && !g->generic && slice_allowed(g, B, true, need_slack != 0, true, flags, cp)) bytes = std::max(bytes, kSmallWs + lvl_area(g) + cp.ws);
     if (need_slack == 2) bytes += 4 * round_up((size_t)B * 8, 256) + 256;
     *out = bytes;
     return EMO_OK;
@@ -2183,8 +2548,6 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
     if (g->host_only) return EMO_E_CUDA;
     if (B == 0 && !T0 && !E0) return EMO_OK;
     if (B > 0 && (!lvl || !makespan || !energy || ldb < B)) return EMO_E_INVALID_ARG;
-    (void)ws;
-    (void)ws_bytes;
     cudaStream_t st = (cudaStream_t)stream;
     if ((flags & EMO_F_VALIDATE) && B > 0) {
         int rc = launch_validate(g, B, lvl, ldb, status, st);
@@ -2194,6 +2557,12 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
     if (g->generic)
         return launch_generic(g, B, lvl, ldb, false, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, ws,
                               ws_bytes, st);
+    {
+        SlicePlan cp;
+        const size_t head = kSmallWs + lvl_area(g);
+        if (slice_allowed(g, B, T0 || E0, false, false, flags, cp) && (cp.ws == 0 || (ws && ws_bytes >= head + cp.ws)))
+            return launch_slices(g, cp, lvl, ldb, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, (unsigned char *)ws + head, st);
+    }
     if (spine_allowed(g, B, lvl, ldb, 0, flags)) {
         SpinePlan fp;
         if (spine_plan(g, B, T0 || E0, false, false, fp))
@@ -2540,6 +2909,12 @@ int emo_slack_batch(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t l
     if (g->generic)
         return launch_generic(g, B, lvl, ldb, true, ES, LS, slack, ldo, makespan, energy, slack_sum, n_critical, T0, E0, ws, ws_bytes,
                               st);
+    {
+        SlicePlan cp;
+        const size_t head = kSmallWs + lvl_area(g);
+        if (slice_allowed(g, B, T0 || E0, true, ES || LS || slack_sum || n_critical, flags, cp) && (cp.ws == 0 || (ws && ws_bytes >= head + cp.ws)))
+            return launch_slices(g, cp, lvl, ldb, ES, LS, slack, ldo, makespan, energy, slack_sum, n_critical, T0, E0, (unsigned char *)ws + head, st);
+    }
     if (spine_allowed(g, B, lvl, ldb, ldo, flags)) {
         SpinePlan fp;
         if (spine_plan(g, B, T0 || E0, true, ES || LS || slack_sum || n_critical, fp)) {
@@ -2590,18 +2965,22 @@ int emo_slack(const emo_graph *g, const uint8_t *lvl_one, int64_t *ES, int64_t *
 {
     if (!g || !makespan || !lvl_one) return EMO_E_INVALID_ARG;
     if (g->host_only) return EMO_E_CUDA;
-    size_t need = 0;
-    emo_workspace_bytes(g, 1, 1, &need);
-    if (!ws || ws_bytes < need) return EMO_E_OOM;
+    if (!ws || ws_bytes < pass_ws_bytes(g, 1, 1, 0, 1)) return EMO_E_OOM;
     cudaStream_t st = (cudaStream_t)stream;
+    double *const e1 = energy ? energy : (double *)((char *)ws + 1024);
+    {
+        SlicePlan cp;
+        const size_t head = kSmallWs + lvl_area(g);
+        if (slice_allowed(g, 1, false, true, true, 0, cp) && ws_bytes >= head + cp.ws)
+            return launch_slices(g, cp, lvl_one, 1, ES, LS, slack, 1, makespan, e1, nullptr, nullptr, nullptr, nullptr, (unsigned char *)ws + head, st);
+    }
     // re-pitch the level vector to [rows][16] so that the staged kernels can be used; the
     // per-node outputs are written at pitch 1 directly
     uint8_t *lv = (uint8_t *)ws + kSmallWs;
     const size_t rows = (size_t)std::max(g->h.rows, 1);
     emo_spread_levels<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(lvl_one, lv, (int64_t)rows);
     EMO_CUDA(cudaGetLastError());
-    double *e = energy ? energy : (double *)((char *)ws + 1024);
-    return emo_slack_batch(g, 1, lv, 16, ES, LS, slack, 1, makespan, e, nullptr, nullptr, nullptr, nullptr, ws, ws_bytes,
+    return emo_slack_batch(g, 1, lv, 16, ES, LS, slack, 1, makespan, e1, nullptr, nullptr, nullptr, nullptr, ws, ws_bytes,
                            status, 0, stream);
 }
 
@@ -2626,6 +3005,10 @@ int emo_select(int64_t B, const int64_t *makespan, const double *energy, int64_t
     if (!ws || ws_bytes < kSmallWs) return EMO_E_OOM;
     cudaStream_t st = (cudaStream_t)stream;
     int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((B + 1023) / 1024, kSelectMaxBlocks));
+    if (blocks == 1) {
+        EMO_CUDA(launch_ahead(emo_select_one, 1, 256, 0, st, B, makespan, energy, target, target_dev, delta_ppm, out_index, out_T, out_E));
+        return EMO_OK;
+    }
     SelectPartial *part = (SelectPartial *)ws;
     EMO_CUDA(launch_ahead(emo_select_stage1, blocks, 256, 0, st, B, makespan, energy, target, target_dev, delta_ppm, part));
     EMO_CUDA(launch_ahead(emo_select_stage2, 1, 256, 0, st, blocks, (const SelectPartial *)part, makespan, out_index, out_T, out_E));

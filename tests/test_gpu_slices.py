@@ -1,0 +1,69 @@
+"""The slice kernels (calls with few policies: the graph cut into slices that are evaluated at the same time) against the oracle:
+graphs of one, two and many slices (chained one by one and by groups), tiles with remainders, every output."""
+import os
+
+import numpy as np
+import pytest
+
+from paper_2607_12324_b200 import workloads as W
+from tests.test_gpu_parity import assert_matches, emo, gpu_slack_batch, torch_cuda  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+def levels(torch, rows, L, B, seed, pitch=0):
+    """[rows][ldb] with bytes that no policy owns behind the batch."""
+    ldb = pitch or (B + 15) // 16 * 16
+    lv = np.full((rows, ldb), 0xFF, dtype=np.uint8)
+    lv[:, :B] = np.random.RandomState(seed).randint(0, L, size=(rows, B))
+    return lv[:, :B].copy(), torch.as_tensor(lv, device="cuda")
+
+
+@pytest.mark.parametrize("name, scale, B", [("cfg0-tiny", 1.0, 64), ("cfg1-train", 0.02, 1), ("cfg1-train", 0.026, 9), ("cfg1-train", 0.3, 8), ("cfg1-train", 0.6, 31),
+                                            ("cfg2-packed", 0.25, 33), ("cfg2-packed", 1.0, 257), ("cfg3-8dev", 0.02, 17), ("cfg3-8dev", 0.1, 7), ("cfg4-llm", 0.05, 40)])
+def test_against_oracle(torch_cuda, emo, oracle_mod, name, scale, B):
+    torch = torch_cuda
+    g = W.make_graph(name, scale)
+    lv, lv_dev = levels(torch, g.n, g.L, B, 5, pitch=B + 3 if B % 2 else 0)
+    r_or = oracle_mod.batch(g, lv, want_arrays=True, threads=os.cpu_count() or 1)
+    h = emo.load_workload(g)
+    assert emo.emo_call_slices(h, B, True, emo.EMO_F_SLICE_KERNEL) > 0
+    r = gpu_slack_batch(torch, emo, h, lv_dev, B, g.n, ldo=B + 2, base=True, flags=emo.EMO_F_SLICE_KERNEL)
+    assert_matches(r, r_or, B)
+    for k in ("ES", "LS", "slack"):
+        assert (r[k][:, B:] == -7).all(), "padding columns of the outputs were written"
+    base = oracle_mod.batch(g, np.full((g.n, 1), g.L - 1, dtype=np.uint8))
+    assert r["T0"] == base["makespan"][0] and np.isclose(r["E0"], base["energy"][0], rtol=1e-12, atol=0)
+    # forward only, and one policy alone
+    T, E = torch.zeros(B, dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.float64, device="cuda")
+    ws = torch.empty(emo.emo_workspace_bytes(h, B, 0, emo.EMO_F_SLICE_KERNEL), dtype=torch.uint8, device="cuda")
+    emo.emo_eval_policies(h, B, lv_dev, lv_dev.stride(0), T, E, ws, flags=emo.EMO_F_SLICE_KERNEL)
+    assert np.array_equal(T.cpu().numpy(), r_or["makespan"]) and np.allclose(E.cpu().numpy(), r_or["energy"], rtol=1e-12, atol=0)
+    X = torch.zeros((3, g.n), dtype=torch.int64, device="cuda")
+    ws = torch.empty(emo.emo_workspace_bytes(h, 1, 1), dtype=torch.uint8, device="cuda")
+    emo.emo_slack(h, lv_dev[:, B - 1].contiguous(), X[0], X[1], X[2], T[:1], E[:1], ws)
+    for k, x in zip(("ES", "LS", "slack"), X.cpu().numpy()):
+        assert np.array_equal(x, r_or[k][:, B - 1]), k
+    assert int(T[0]) == r_or["makespan"][B - 1]
+    h.free()
+
+
+def test_random_dags(torch_cuda, emo, oracle_mod):
+    """Random graphs (ties, zero durations, several sources and terminal nodes, nodes outside every policy) of one to six slices."""
+    torch = torch_cuda
+    done = 0
+    for seed in range(24):
+        rs = np.random.RandomState(900 + seed)
+        n, L, B = int(rs.choice([1, 40, 255, 256, 257, 400, 900])), int(rs.randint(1, 9)), int(rs.choice([1, 7, 8, 9, 40]))
+        g = W.random_dag(40 + seed, n, float(rs.choice([1.0, 2.0, 4.0])) / n, L=L, max_dur=int(rs.choice([2, 40, 100000])))
+        group = rs.randint(-1, 6, size=g.n).astype(np.int32) if seed % 3 == 0 else None
+        rows = g.n if group is None else 6
+        lv, lv_dev = levels(torch, rows, L, B, seed)
+        r_or = oracle_mod.batch(g, lv, want_arrays=True, group_of=group)
+        h = emo.load_workload(g, group_of=group)
+        if emo.emo_call_slices(h, B, True, emo.EMO_F_SLICE_KERNEL) > 0:      # (not where too many values cross every cut)
+            r = gpu_slack_batch(torch, emo, h, lv_dev, B, g.n, flags=emo.EMO_F_SLICE_KERNEL)
+            assert_matches(r, r_or, B)
+            done += 1
+        h.free()
+    assert done >= 12
