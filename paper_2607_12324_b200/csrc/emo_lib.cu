@@ -13,6 +13,7 @@
 
 #include "../../include/emo.h"
 #include "emo_compile.h"
+#include "emo_contract.h"
 #include "emo_flow.h"
 #include "emo_kernels.cuh"
 #include "emo_pass_lane.cuh"
@@ -110,6 +111,7 @@ struct emo_graph {
     DevSpine dlong;
     DevSlice dslice;                 // slices of the graph, for calls with few policies
     SpineImage simage, limage;       // both as laid out for the device (kept by host-only handles, else until they are copied)
+    emo_graph *joined = nullptr;     // the contracted graph (emo_contract.h) that emo_eval_policies evaluates; null where it saves little
     bool host_only = false;
     // graphs beyond the schedule compilers' limits (or loaded with EMO_F_GENERIC): evaluated by the generic kernels
     bool generic = false;
@@ -1440,6 +1442,12 @@ bool spine_allowed(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ld
     return ldb % 16 == 0 && aligned16(lvl) && ldb < big && ldo < big;
 }
 
+// The contracted graph for a call without outputs per node, unless the caller names its kernels.
+const emo_graph *joined_for(const emo_graph *g, uint32_t flags)
+{
+    return flags & (EMO_F_NO_STAGING | EMO_F_PAIR_KERNEL | EMO_F_LANE_KERNEL | EMO_F_FLOW_KERNEL | EMO_F_SPINE_KERNEL | EMO_F_TEST_STALL) ? nullptr : g->joined;
+}
+
 // Whether a call takes the 32-bit lane-stream kernels: the program exists, the level matrix can be
 // fetched in 16-byte pieces, and either the caller asks for them (EMO_F_FLOW_KERNEL) or the batch is
 // large (for the graph or for the SMs).  Measured on the five workloads: on the 250 000-node graph with 16 384 policies they are
@@ -1488,11 +1496,10 @@ int upload_slices(const Slices &s, DevSlice &d)
         at[i] = total;
         total += round_up(bytes[i], 256);
     }
-    std::vector<unsigned char> image(total);
-    for (int i = 0; i < 5; ++i) std::memcpy(image.data() + at[i], src[i], bytes[i]);
     unsigned char *mem = nullptr;
-    const cudaError_t rc = cudaMalloc(&mem, total);
-    if (rc != cudaSuccess || cudaMemcpy(mem, image.data(), total, cudaMemcpyHostToDevice) != cudaSuccess) {
+    cudaError_t rc = cudaMalloc(&mem, total);
+    for (int i = 0; i < 5 && rc == cudaSuccess; ++i) rc = cudaMemcpy(mem + at[i], src[i], bytes[i], cudaMemcpyHostToDevice);
+    if (rc != cudaSuccess) {
         (void)cudaGetLastError();
         if (mem) cudaFree(mem);
         return rc == cudaErrorMemoryAllocation ? EMO_E_OOM : EMO_E_CUDA;
@@ -1831,7 +1838,12 @@ int emo_call_slices(const emo_graph *g, int64_t B, int need_slack, uint32_t flag
     if (!g || B < 0) return EMO_E_INVALID_ARG;
     if (g->host_only) return EMO_E_CUDA;
     SlicePlan cp;
-    return slice_allowed(g, B, true, need_slack != 0, false, flags, cp) ? g->dslice.count : 0;
+    for (const emo_graph *e : {need_slack ? nullptr : joined_for(g, flags), g}) {
+        if (!e) continue;
+        if (slice_allowed(e, B, true, need_slack != 0, false, flags, cp)) return e->dslice.count;
+        if (e != g && e->dspine.ready) return 0;
+    }
+    return 0;
 }
 
 int emo_measure_int_issue(double *ops_per_s, void *scratch_dev, void *stream)
@@ -1899,9 +1911,23 @@ int emo_set_wait_limit(int64_t cycles)
     return EMO_OK;
 }
 
-int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const int32_t *level_ptr,
-                   int32_t n_levels, int32_t L, const int64_t *lat, const double *energy,
-                   const int32_t *group_of, uint32_t flags, emo_graph **out)
+static int32_t hop_depth(const HostGraph &h)
+{
+    std::vector<int32_t> hop((size_t)std::max(h.n, 1), 0);
+    int32_t depth = 0;
+    for (int32_t v = 0; v < h.n; ++v) {
+        int32_t a = 0;
+        for (int64_t e = h.row_ptr[v]; e < h.row_ptr[v + 1]; ++e) a = std::max(a, hop[h.col[e]] + 1);
+        hop[v] = a;
+        depth = std::max(depth, a + 1);
+    }
+    return depth;
+}
+
+// inner: this is a contracted graph; only what its calls read is compiled (the spine and slice programs).
+static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, const int32_t *level_ptr,
+                      int32_t n_levels, int32_t L, const int64_t *lat, const double *energy,
+                      const int32_t *group_of, uint32_t flags, bool inner, emo_graph **out)
 {
     if (!out) return EMO_E_INVALID_ARG;
     *out = nullptr;
@@ -1952,6 +1978,10 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
     emo_graph *g = new (std::nothrow) emo_graph();
     if (!g) return EMO_E_OOM;
     Slices slices;
+    struct Joined {
+        emo_graph *g = nullptr;
+        ~Joined() { if (g) emo_graph_free(g); }
+    } joined;
     try {
         HostGraph &h = g->h;
         h.n = n;
@@ -1999,8 +2029,39 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             }
             return rc;
         };
-        int rc = (flags & EMO_F_GENERIC) ? EMO_E_UNSUPPORTED : compile_dir(true, nullptr, g->bwd);
-        if (rc == EMO_OK) rc = compile_dir(false, &g->bwd.pos_of_node, g->fwd);
+        // (what ends the block early, an exception among it, waits for them: they come behind what their threads use)
+        struct Helper {
+            std::thread t;
+            void wait() { if (t.joinable()) t.join(); }
+            ~Helper() { wait(); }
+        };
+        auto start = [](Helper &helper, auto work) {
+            try {
+                helper.t = std::thread(work);
+            } catch (const std::exception &) {      // no more threads: here, one after the other
+                work();
+            }
+        };
+        GraphBounds bounds;
+        if (!(flags & EMO_F_GENERIC)) graph_bounds(h, lat, energy, bounds);
+        // the contracted graph, beside everything else (not where the caller shapes the programs)
+        int device = 0;
+        Helper joined_thread;
+        if (!inner && n >= 2000 && flags == 0 && cudaGetDevice(&device) == cudaSuccess)
+            start(joined_thread, [&, device]() {
+                try {
+                    Contracted c;
+                    contract_forward(h, lat, energy, bounds, false, c);
+                    // where it leaves three nodes of five (measured, forward, us: 75 000 nodes to 11 088 x 10 001 policies 520 / 1 271; with
+                    // four of five left a call gains 7 % and a load pays the second set of programs)
+                    if ((int64_t)c.n * 5 > (int64_t)n * 3 || cudaSetDevice(device) != cudaSuccess) return;
+                    if (load_graph(c.n, c.row_ptr.data(), c.col.data(), nullptr, 0, L, c.lat.data(), c.energy.data(), c.group.data(), flags, true, &joined.g) != EMO_OK)
+                        joined.g = nullptr;
+                } catch (const std::exception &) {      // no memory for it: the graph itself serves
+                }
+            });
+        int rc = (flags & EMO_F_GENERIC) ? EMO_E_UNSUPPORTED : (inner ? EMO_OK : compile_dir(true, nullptr, g->bwd));
+        if (rc == EMO_OK && !inner) rc = compile_dir(false, &g->bwd.pos_of_node, g->fwd);
         if (rc == EMO_E_UNSUPPORTED) {
             // more live exchanged values than the on-chip schedules can hold: the generic kernels take the graph
             g->generic = true;
@@ -2017,7 +2078,8 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             // 250 000-node workload with 16 384 policies: 8 / 16 / 32 steps between barriers gave 24.8 / 22.3 / 21.3 ms for
             // both passes)
             int fk = (int)((flags >> 24) & 0x3F), fs = (int)((flags >> 4) & 0xF) * 8;
-            const int flanes = g->fwd.lanes > 0 ? std::max(g->fwd.lanes, g->bwd.lanes) : 1;
+            int flanes = g->fwd.lanes > 0 ? std::max(g->fwd.lanes, g->bwd.lanes) : 1;
+            if (inner) flanes = pick_lanes(n, hop_depth(h));
             if (fk == 0) fk = flanes * 32 <= 32 * kFlowRowRegs ? 32 : (flanes * 16 <= 32 * kFlowRowRegs ? 16 : 8);
             if (fs == 0) fs = fk;
             if (fs > fk) fs = fk;
@@ -2027,23 +2089,9 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             const bool want_spine = !(flags & EMO_F_INTERVALS);
             // the slice program, for calls with few policies: another thread (not where the caller shapes the spine program)
             const bool want_slices = want_spine && !(flags & (EMO_F_HOST_ONLY | 0xC0000000u));
-            GraphBounds bounds;
-            graph_bounds(h, lat, energy, bounds);
             int rc_s = EMO_OK, rc_l = EMO_E_UNSUPPORTED;
             std::string err_s, err_l;
-            // (what ends the block early, an exception among it, waits for them)
-            struct Helper {
-                std::thread t;
-                void wait() { if (t.joinable()) t.join(); }
-                ~Helper() { wait(); }
-            } spine_thread, long_thread, slice_thread;
-            auto start = [](Helper &helper, auto work) {
-                try {
-                    helper.t = std::thread(work);
-                } catch (const std::exception &) {      // no more threads: here, one after the other
-                    work();
-                }
-            };
+            Helper spine_thread, long_thread, slice_thread;
             const bool no_long = (flags & EMO_F_TEST_LONG_OOM) != 0 && (flags & EMO_F_HOST_ONLY) != 0;
             auto compile_spine = [&](int k, Flow &out, DevSpine &d, SpineImage &im, int &rc_k, std::string &err_k) {
                 try {
@@ -2080,7 +2128,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
                     start(long_thread, [&, lk]() { compile_spine(lk, g->lflow, g->dlong, g->limage, rc_l, err_l); });
             }
             try {
-                rc = compile_flow(h, lat, energy, bounds, lanes, look, fk, fs, g->flow, err);
+                if (!inner) rc = compile_flow(h, lat, energy, bounds, lanes, look, fk, fs, g->flow, err);
             } catch (const std::bad_alloc &) {
                 rc = EMO_E_OOM;
             }
@@ -2093,7 +2141,7 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             }
             if (rc == EMO_OK && rc_s != EMO_OK && rc_s != EMO_E_UNSUPPORTED) rc = rc_s;
             if (rc != EMO_OK) { delete g; return rc; }
-            if (!want_spine || rc_s != EMO_OK || !g->flow.ok32 || !g->sflow.spine.ok) g->sflow = Flow();
+            if (!want_spine || rc_s != EMO_OK || !(g->flow.ok32 || inner) || !g->sflow.spine.ok) g->sflow = Flow();
             else {
                 // only the spine's parts are kept
                 g->sflow.f = FlowDir();
@@ -2112,15 +2160,9 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             g->lflow.f = FlowDir();
             g->lflow.b = FlowDir();
         }
-        std::vector<int32_t> hop((size_t)std::max(n, 1), 0);
-        int32_t depth = 0;
-        for (int32_t v = 0; v < n; ++v) {
-            int32_t a = 0;
-            for (int64_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) a = std::max(a, hop[col[e]] + 1);
-            hop[v] = a;
-            depth = std::max(depth, a + 1);
-        }
-        h.depth = depth;
+        h.depth = hop_depth(h);
+        joined_thread.wait();
+        if (!g->generic) std::swap(g->joined, joined.g);
     } catch (const std::bad_alloc &) {
         delete g;
         return EMO_E_OOM;
@@ -2131,9 +2173,9 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
         g->dlong.ready = g->lflow.spine.ok && !g->limage.host.empty();
     } else {
         int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); delete g; return EMO_E_CUDA; }
+        if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); emo_graph_free(g); return EMO_E_CUDA; }
         cudaDeviceProp prop;
-        if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { (void)cudaGetLastError(); delete g; return EMO_E_CUDA; }
+        if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { (void)cudaGetLastError(); emo_graph_free(g); return EMO_E_CUDA; }
         g->device = dev;
         g->sm_count = prop.multiProcessorCount;
         g->smem_optin = prop.sharedMemPerBlockOptin;
@@ -2159,13 +2201,13 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
             g->host_lat = std::vector<int64_t>();
             g->host_energy = std::vector<double>();
         } else {
-        rc = upload_program(g->fwd, g->dfwd);
-        if (rc == EMO_OK) rc = upload_program(g->bwd, g->dbwd);
-        if (rc == EMO_OK && g->fwd.lanes <= 32 - kProducerWarps && g->bwd.lanes <= 32 - kProducerWarps) {
+        if (!inner) rc = upload_program(g->fwd, g->dfwd);
+        if (rc == EMO_OK && !inner) rc = upload_program(g->bwd, g->dbwd);
+        if (rc == EMO_OK && !inner && g->fwd.lanes <= 32 - kProducerWarps && g->bwd.lanes <= 32 - kProducerWarps) {
             rc = upload_program_lane(g->fwd, g->lfwd);
             if (rc == EMO_OK) rc = upload_program_lane(g->bwd, g->lbwd);
         }
-        if (rc == EMO_OK) rc = upload_flow(g->flow, g->dflow, (flags & EMO_F_INTERVALS) != 0);
+        if (rc == EMO_OK && !inner) rc = upload_flow(g->flow, g->dflow, (flags & EMO_F_INTERVALS) != 0);
         // One barrier per stage needs more exchange slots than one every 16 steps (on the 250 000-node graph 20.9 KB
         // against 13.8 KB per policy group, at 0.3 scale 29.8 KB against 17.9 KB).  Where four groups then no longer fit a
         // block, the grid doubles and the gain turns into a loss (11.7 ms against 6.8 ms at 0.3 scale): take the shorter
@@ -2211,9 +2253,17 @@ int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const 
     return EMO_OK;
 }
 
+int emo_graph_load(int32_t n, const int64_t *row_ptr, const int32_t *col, const int32_t *level_ptr,
+                   int32_t n_levels, int32_t L, const int64_t *lat, const double *energy,
+                   const int32_t *group_of, uint32_t flags, emo_graph **out)
+{
+    return load_graph(n, row_ptr, col, level_ptr, n_levels, L, lat, energy, group_of, flags, false, out);
+}
+
 int emo_graph_free(emo_graph *g)
 {
     if (!g) return EMO_OK;
+    emo_graph_free(g->joined);
     if (!g->host_only) {
         free_program(g->dfwd);
         free_program(g->dbwd);
@@ -2529,7 +2579,8 @@ int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint3
     if (!g || !out || B < 0) return EMO_E_INVALID_ARG;
     size_t bytes = pass_ws_bytes(g, B, need_slack, flags, aligned);
     SlicePlan cp;
-    if (!g->host_only && !g->generic && slice_allowed(g, B, true, need_slack != 0, true, flags, cp)) bytes = std::max(bytes, kSmallWs + lvl_area(g) + cp.ws);
+    for (const emo_graph *e : {need_slack ? nullptr : joined_for(g, flags), g})
+        if (e && !g->host_only && !g->generic && slice_allowed(e, B, true, need_slack != 0, true, flags, cp)) bytes = std::max(bytes, kSmallWs + lvl_area(g) + cp.ws);
     if (need_slack == 2) bytes += 4 * round_up((size_t)B * 8, 256) + 256;
     *out = bytes;
     return EMO_OK;
@@ -2557,16 +2608,15 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
     if (g->generic)
         return launch_generic(g, B, lvl, ldb, false, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, ws,
                               ws_bytes, st);
-    {
+    const size_t head = kSmallWs + lvl_area(g);
+    for (const emo_graph *e : {joined_for(g, flags), g}) {
+        if (!e) continue;
         SlicePlan cp;
-        const size_t head = kSmallWs + lvl_area(g);
-        if (slice_allowed(g, B, T0 || E0, false, false, flags, cp) && (cp.ws == 0 || (ws && ws_bytes >= head + cp.ws)))
-            return launch_slices(g, cp, lvl, ldb, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, (unsigned char *)ws + head, st);
-    }
-    if (spine_allowed(g, B, lvl, ldb, 0, flags)) {
+        if (slice_allowed(e, B, T0 || E0, false, false, flags, cp) && (cp.ws == 0 || (ws && ws_bytes >= head + cp.ws)))
+            return launch_slices(e, cp, lvl, ldb, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, (unsigned char *)ws + head, st);
         SpinePlan fp;
-        if (spine_plan(g, B, T0 || E0, false, false, fp))
-            return launch_spine_fwd(g, fp, B, lvl, ldb, nullptr, makespan, energy, T0, E0, status, flags, st);
+        if (spine_allowed(e, B, lvl, ldb, 0, flags) && spine_plan(e, B, T0 || E0, false, false, fp))
+            return launch_spine_fwd(e, fp, B, lvl, ldb, nullptr, makespan, energy, T0, E0, status, flags, st);
     }
     if (flow_allowed(g, B, lvl, ldb, 0, flags)) {
         FlowPlan fp;
