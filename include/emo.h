@@ -68,7 +68,8 @@ extern "C" {
                                     * 32 per SM on a graph of at most eight lanes, where there is no spine program) */
 #define EMO_F_SPINE_KERNEL 0x20u   /* the spine kernels (the default wherever there is a spine program, but on graphs of more than eight lanes
                                     * without a program of longer stages only from two policy groups of 32 per SM on) */
-#define EMO_F_SLICE_KERNEL 0x40u   /* the slice kernels (the default for few policies) */
+#define EMO_F_SLICE_KERNEL 0x40u   /* the slice kernels, whatever the number of policies (the default for about a thousand and fewer, fewer
+                                      still on graphs with many streams: emo_call_slices) */
 #define EMO_F_TEST_STALL 0x100u    /* test hook of the 32-bit kernels: the producer warps stop half way, so that the
                                       consumers' bounded waits run out and EMO_E_TIMEOUT is reported */
 
@@ -186,8 +187,9 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
  * (exact when the packs of a device do not overlap in time, as packs of one device timeline do not; the paper
  * does not define idle_time further).
  * Kernels: a graph loaded with EMO_F_INTERVALS runs the 32-bit lane-stream kernel when the change points are a
- * uniform grid and the columns of F fit shared memory; otherwise, or with EMO_F_NO_STAGING in flags, the
- * step-program kernel runs.  Both give the same results.
+ * uniform grid and the columns of F fit shared memory (on graphs of at most three lanes, and where its blocks would come in several
+ * waves, a kernel that gives every policy a thread; EMO_F_FLOW_KERNEL in flags keeps to the former); otherwise, or with
+ * EMO_F_NO_STAGING in flags, the step-program kernel runs.  All give the same results.
  * Errors: EMO_E_INVALID_ARG (sizes, breaks not increasing from 0, energy_idle without p_idle), EMO_E_OOM
  * (workspace too small), EMO_E_UNSUPPORTED (change points and exchange slots do not fit shared memory).
  * Asynchronous on `stream` after the change points are copied.

@@ -24,6 +24,7 @@
 #include "emo_model.cuh"
 #include "emo_generic.cuh"
 #include "emo_slice.cuh"
+#include "emo_walk.cuh"
 
 using namespace emo;
 
@@ -111,6 +112,8 @@ struct emo_graph {
     DevSpine dlong;
     DevSlice dslice;                 // slices of the graph, for calls with few policies
     SpineImage simage, limage;       // both as laid out for the device (kept by host-only handles, else until they are copied)
+    Walk walk;                       // time-interval policies (EMO_F_INTERVALS), a thread per policy; its blob is kept on the device
+    unsigned char *dwalk = nullptr;
     emo_graph *joined = nullptr;     // the contracted graph (emo_contract.h) that emo_eval_policies evaluates; null where it saves little
     bool host_only = false;
     // graphs beyond the schedule compilers' limits (or loaded with EMO_F_GENERIC): evaluated by the generic kernels
@@ -120,6 +123,7 @@ struct emo_graph {
     double *gen_energy = nullptr;
     std::vector<int64_t> host_lat;      // kept only for the generic path's upload
     std::vector<double> host_energy;
+    size_t one_bytes = 0;            // workspace that emo_slack asks for
     int device = 0;
     int sm_count = 148;
     size_t smem_optin = 0;
@@ -1911,6 +1915,8 @@ int emo_set_wait_limit(int64_t cycles)
     return EMO_OK;
 }
 
+static size_t pass_ws_bytes(const emo_graph *g, int64_t B, int need_slack, uint32_t flags, int aligned);
+
 static int32_t hop_depth(const HostGraph &h)
 {
     std::vector<int32_t> hop((size_t)std::max(h.n, 1), 0);
@@ -2091,7 +2097,7 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
             const bool want_slices = want_spine && !(flags & (EMO_F_HOST_ONLY | 0xC0000000u));
             int rc_s = EMO_OK, rc_l = EMO_E_UNSUPPORTED;
             std::string err_s, err_l;
-            Helper spine_thread, long_thread, slice_thread;
+            Helper spine_thread, long_thread, slice_thread, walk_thread;
             const bool no_long = (flags & EMO_F_TEST_LONG_OOM) != 0 && (flags & EMO_F_HOST_ONLY) != 0;
             auto compile_spine = [&](int k, Flow &out, DevSpine &d, SpineImage &im, int &rc_k, std::string &err_k) {
                 try {
@@ -2104,6 +2110,14 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
                     rc_k = EMO_E_UNSUPPORTED;
                 }
             };
+            if ((flags & EMO_F_INTERVALS) && !(flags & EMO_F_HOST_ONLY))
+                start(walk_thread, [&]() {
+                    try {
+                        compile_walk(h, lat, energy, bounds, g->walk);
+                    } catch (const std::exception &) {      // no memory for it: the others serve
+                        g->walk = Walk();
+                    }
+                });
             if (want_slices)
                 start(slice_thread, [&]() {
                     try {
@@ -2135,6 +2149,7 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
             spine_thread.wait();
             long_thread.wait();
             slice_thread.wait();
+            walk_thread.wait();
             if (rc == EMO_E_UNSUPPORTED) {      // the 64-bit programs exist: they serve
                 g->flow = Flow();
                 rc = EMO_OK;
@@ -2239,6 +2254,12 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
             else rc = rc_l;
         }
         g->simage = g->limage = SpineImage();
+        if (rc == EMO_OK && g->walk.ok) {
+            const int rc_w = upload(&g->dwalk, g->walk.blob.data(), g->walk.blob.size());
+            if (rc_w != EMO_OK && rc_w != EMO_E_OOM) rc = rc_w;
+            g->walk.ok = rc_w == EMO_OK;
+            g->walk.blob = std::vector<unsigned char>();
+        }
         if (rc == EMO_OK && slices.ok) {
             const int rc_c = upload_slices(slices, g->dslice);
             if (rc_c != EMO_OK && rc_c != EMO_E_OOM) rc = rc_c;      // (no memory for it: the others serve)
@@ -2248,6 +2269,7 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
             rc = EMO_E_OOM;
         }
         if (rc != EMO_OK) { emo_graph_free(g); return rc; }
+        if (!inner) g->one_bytes = pass_ws_bytes(g, 1, 1, 0, 1);
     }
     *out = g;
     return EMO_OK;
@@ -2273,6 +2295,7 @@ int emo_graph_free(emo_graph *g)
         free_spine(g->dspine);
         free_spine(g->dlong);
         if (g->dslice.mem) cudaFree(g->dslice.mem);
+        if (g->dwalk) cudaFree(g->dwalk);
         void *gen[] = {g->gen_row_ptr, g->gen_col, g->gen_srow_ptr, g->gen_scol, g->gen_group, g->gen_lat, g->gen_energy};
         for (void *q : gen)
             if (q) cudaFree(q);
@@ -2639,6 +2662,65 @@ int emo_workspace_bytes_intervals(const emo_graph *g, int64_t B, int32_t I, int 
     return EMO_OK;
 }
 
+// The shape of a call that the walk kernel takes: a uniform grid, the columns of F in shared memory.
+static bool walk_plan(const emo_graph *g, int64_t B, int rows, int32_t I, int64_t delta, WalkParams &p, int &grid, size_t &smem)
+{
+    const Walk &w = g->walk;
+    if (!w.ok || delta <= 0 || delta >= kWalkMaxDur) return false;
+    p = WalkParams();
+    p.blob = g->dwalk;
+    p.chunks = w.chunks;
+    p.Lp = w.Lp;
+    p.L = g->h.L;
+    p.chunk_bytes = w.chunk_bytes;
+    p.off_dur = w.off_dur;
+    p.off_en = w.off_en;
+    p.rows = rows;
+    p.I = I;
+    p.B = B;
+    p.delta = (int)delta;
+    p.inv = 1.0f / (float)delta;
+    p.energy0 = w.energy0;
+    // fewer policies per warp as long as every warp has a scheduler of its own (fewer of them leave an interval inside an item); then
+    // as many warps per block as bring all in at once
+    int64_t pl = 4;
+    while (pl < 32 && (B + pl - 1) / pl > (int64_t)g->sm_count * 4) pl *= 2;
+    const int64_t warps = (B + pl - 1) / pl;
+    int groups = (int)std::min<int64_t>(kWalkMaxGroups, (warps + g->sm_count - 1) / g->sm_count);
+    for (; groups >= 1; --groups) {
+        p.groups = groups;
+        p.pl = (int)pl;
+        p.P = groups * (int)pl;
+        p.off_F = 2 * kWalkMaxBuffers * 8 + 16;
+        const size_t f_bytes = (size_t)rows * (size_t)I * (size_t)p.P, off_slots = round_up(p.off_F + f_bytes, 128);
+        const size_t off_buf = round_up(off_slots + (size_t)w.slots * groups * 256, 128);
+        for (p.buffers = kWalkMaxBuffers; p.buffers >= 2; --p.buffers) {
+            smem = off_buf + (size_t)p.buffers * w.chunk_bytes;
+            if (smem > g->smem_optin) continue;
+            p.off_slots = (unsigned)off_slots;
+            p.off_buf = (unsigned)off_buf;
+            grid = (int)((B + p.P - 1) / p.P);
+            return true;
+        }
+    }
+    return false;
+}
+
+// Whether the walk kernel is the faster one.  Measured (us, it / the lane-stream kernel): up to three lanes, 500 nodes x 4 096 policies, 26
+// intervals 63 / 170, 10 000 x 16 384 1 921 / 2 422; more lanes in one wave of blocks against two or more, 18 lanes, 38 000 nodes x
+// 16 384 2 248 / 6 158, 5 lanes, 25 000 x 40 000 2 387 / 3 167; not in one against one, 75 000 x 16 384 5 462 / 3 795, 38 000 x 4 096
+// 2 014 / 1 645.  Where F does not fit the lane-stream kernel's blocks it seldom suits these (8 rows, 400 intervals, 6 439 nodes x 16
+// 2 065 / 1 522 by the step program).
+static bool walk_pays(const emo_graph *g, int64_t B, int rows, int32_t I, int walk_grid)
+{
+    const int64_t sms = std::max(g->sm_count, 1), walk_waves = (walk_grid + sms - 1) / sms;
+    FlowPlan fp;
+    const size_t brk_b = round_up((size_t)I * 8, 16), f_per_group = (size_t)rows * (size_t)I * 32;
+    if (!g->dflow.blobFI || !flow_plan(g, B, false, false, fp, true, brk_b, f_per_group)) return false;
+    const int64_t flow_waves = (fp.grid_f + sms - 1) / sms;
+    return g->flow.lanes <= 3 ? walk_waves <= flow_waves : walk_waves * 2 <= flow_waves;
+}
+
 int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t ldb, int32_t I, const int64_t *breaks,
                        const double *p_idle, int64_t *makespan, double *energy, double *energy_idle, void *ws,
                        size_t ws_bytes, int32_t *status, uint32_t flags, void *stream)
@@ -2670,7 +2752,26 @@ int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t 
     cudaEvent_t ev0 = g_pass_events[0], ev1 = g_pass_events[1];
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
     bool done = false;
-    if (!(flags & EMO_F_NO_STAGING) && g->dflow.blobFI && delta > 0) {
+    {
+        WalkParams q;
+        int grid = 0;
+        size_t smem = 0;
+        if (!(flags & (EMO_F_NO_STAGING | EMO_F_FLOW_KERNEL)) && walk_plan(g, B, rows, I, delta, q, grid, smem) && walk_pays(g, B, rows, I, grid)) {
+            q.F = F;
+            q.ldF = ldb;
+            q.makespan = makespan;
+            q.energy = energy;
+            q.busy = busy;
+            q.ldw = ldw;
+            q.status = status;
+            q.wait_cycles = g_wait_cycles;
+            if (flow_optin(emo_walk, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+            emo_walk<<<grid, (q.groups + 1) * 32, smem, st>>>(q);
+            EMO_CUDA(cudaGetLastError());
+            done = true;
+        }
+    }
+    if (!done && !(flags & EMO_F_NO_STAGING) && g->dflow.blobFI && delta > 0) {
         // the lane-stream forward kernel with the look-up inside the chain: uniform grids, F's columns in shared memory
         FlowPlan fp;
         const size_t brk_b = round_up((size_t)I * 8, 16), f_per_group = (size_t)rows * (size_t)I * 32;
@@ -3015,7 +3116,7 @@ int emo_slack(const emo_graph *g, const uint8_t *lvl_one, int64_t *ES, int64_t *
 {
     if (!g || !makespan || !lvl_one) return EMO_E_INVALID_ARG;
     if (g->host_only) return EMO_E_CUDA;
-    if (!ws || ws_bytes < pass_ws_bytes(g, 1, 1, 0, 1)) return EMO_E_OOM;
+    if (!ws || ws_bytes < g->one_bytes) return EMO_E_OOM;
     cudaStream_t st = (cudaStream_t)stream;
     double *const e1 = energy ? energy : (double *)((char *)ws + 1024);
     {
@@ -3140,6 +3241,14 @@ int emo_unpack_levels(int bits, int64_t rows, int64_t B, const uint8_t *packed, 
 
 // The passes, the selection and the copies of the per-policy results to the host, once the levels are on the device:
 // packed in dev_packed (bits < 8: spread to dev_lvl first) or as bytes in dev_lvl (bits = 8).
+// Workspace of the passes inside a host-buffer call: with the slice kernels' share where the caller's has room for it.
+static size_t host_call_bytes(const emo_graph *g, int64_t B, uint32_t flags, int aligned, size_t ws_bytes)
+{
+    size_t need = 0;
+    emo_workspace_bytes_for(g, B, 1, flags, aligned, &need);
+    return ws_bytes >= need + 4 * round_up((size_t)B * 8, 256) + 256 ? need : pass_ws_bytes(g, B, 1, flags, aligned);
+}
+
 static int host_batch_tail(const emo_graph *g, int64_t B, int bits, const uint8_t *dev_packed, int64_t ld_packed, uint8_t *dev_lvl,
                            int64_t ldb, int64_t *slack_dev, int64_t ldo, int64_t delta_ppm, int64_t *makespan_host,
                            double *energy_host, int64_t *slack_sum_host, int32_t *n_critical_host, int64_t *sel_host, void *ws,
@@ -3192,8 +3301,8 @@ int emo_slack_batch_host_packed(const emo_graph *g, int64_t B, int bits, const u
     if (g->host_only) return EMO_E_CUDA;
     size_t need = 0, total = 0;
     const int aligned = (ldb % 16 == 0 && aligned16(dev_lvl)) ? 1 : 0;
-    emo_workspace_bytes_for(g, B, 1, flags, aligned, &need);
-    emo_workspace_bytes_for(g, B, 2, flags, aligned, &total);
+    need = host_call_bytes(g, B, flags, aligned, ws_bytes);
+    total = need + 4 * round_up((size_t)B * 8, 256) + 256;
     // per-policy result arrays live behind the slack workspace
     if (!ws || ws_bytes < total) return EMO_E_OOM;
     cudaStream_t st = (cudaStream_t)stream;
@@ -3231,8 +3340,8 @@ int emo_slack_batch_prefetched(const emo_graph *g, int64_t B, int bits, const ui
     if (g->host_only) return EMO_E_CUDA;
     size_t need = 0, total = 0;
     const int aligned = (ldb % 16 == 0 && aligned16(dev_lvl)) ? 1 : 0;
-    emo_workspace_bytes_for(g, B, 1, flags, aligned, &need);
-    emo_workspace_bytes_for(g, B, 2, flags, aligned, &total);
+    need = host_call_bytes(g, B, flags, aligned, ws_bytes);
+    total = need + 4 * round_up((size_t)B * 8, 256) + 256;
     if (!ws || ws_bytes < total) return EMO_E_OOM;
     cudaStream_t st = (cudaStream_t)stream;
     if (ready) EMO_CUDA(cudaStreamWaitEvent(st, (cudaEvent_t)ready, 0));

@@ -54,6 +54,9 @@ struct Slices {
     std::vector<double> tabE;                    // [n][Lp]
 };
 
+// A topological order in which few values are alive at a time.
+std::vector<int32_t> narrow_order(int32_t n, const GraphBounds &b);
+
 // Builds the slice program; ok stays false where it does not apply (too many values cross every cut, or a path too long).
 void compile_slices(const HostGraph &g, const int64_t *lat, const double *energy, const GraphBounds &b, Slices &out);
 

@@ -9,8 +9,6 @@
 
 namespace emo {
 
-namespace {
-
 // A topological order in which few values are alive at a time: from the last node to the first, always the node that adds least
 // to the set of nodes that placed ones still wait for, the highest-numbered among equals.  (Values alive at the best cut of every
 // 64 nodes, mean / most: 250 000-node graph 5.1 / 7; in the given order, level by level, its launch nodes wait for up to 600.)
@@ -58,6 +56,8 @@ std::vector<int32_t> narrow_order(int32_t n, const GraphBounds &b)
     }
     return order;
 }
+
+namespace {
 
 struct Operand {
     int32_t slot;      // virtual slot: 0 time zero, 1 .. W the values that cross, then operations

@@ -1,0 +1,52 @@
+"""Time intervals, a thread per policy (graphs of few lanes): the oracle's times, busy times and energies and
+those of the step-program kernel, at batches around a warp's and a block's policies, short and long intervals, nodes that outlast them."""
+import numpy as np
+import pytest
+
+from paper_2607_12324_b200 import workloads as W
+from tests.test_gpu_parity import emo, torch_cuda  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+def weave(seed, n, rows):
+    """Every node waits for the last one of its stream and, half of the time, for one of the streams beside it."""
+    rs = np.random.RandomState(seed)
+    last, edges = [-1] * 2, []
+    for v in range(n):
+        k = rs.randint(2)
+        for u in {last[k], last[rs.randint(2)] if rs.rand() < 0.5 else -1}:
+            if u >= 0:
+                edges.append((u, v))
+        last[k] = v
+    lat = rs.randint(0, 1000, size=(n, 5)).astype(np.int64)
+    lat[rs.rand(n) < 0.02] *= 60                      # outlasts an interval
+    group = np.where(rs.rand(n) < 0.2, -1, rs.randint(0, rows, size=n)).astype(np.int32)
+    return W.tiny_graph(n, sorted(set(edges)), lat, rs.rand(n, 5), name=f"weave{seed}"), group
+
+
+@pytest.mark.parametrize("seed, n, rows, I, B", [(0, 40, 1, 2, 1), (1, 300, 1, 7, 5), (2, 700, 3, 40, 33), (3, 700, 2, 400, 129), (4, 1500, 1, 3, 2500), (5, 1500, 4, 26, 20000)])
+def test_against_oracle_and_step_program(torch_cuda, emo, oracle_mod, seed, n, rows, I, B):
+    torch = torch_cuda
+    g, group = weave(seed, n, rows)
+    rows = int(group.max()) + 1
+    h = emo.load_workload(g, emo.EMO_F_INTERVALS, group_of=group)
+    assert emo.emo_graph_flow(h, arrays=False)["lanes"] <= 3      # (the call takes a thread per policy)
+    # a grid that ends before the schedule does, and one that outlasts it
+    for span in (0.6, 1.5):
+        breaks = np.arange(I, dtype=np.int64) * max(1, int(h.info.T_best * span / I))
+        F = np.random.RandomState(seed).randint(0, g.L, size=(rows, I, (B + 15) // 16 * 16)).astype(np.uint8)
+        Fd, idle = torch.from_numpy(F).cuda(), torch.from_numpy(W.idle_power(g.L)).cuda()
+        out = []
+        for flags in (0, emo.EMO_F_NO_STAGING):
+            T, E, Ei = (torch.zeros(B, dtype=d, device="cuda") for d in (torch.int64, torch.float64, torch.float64))
+            ws = torch.empty(emo.emo_workspace_bytes_intervals(h, B, I, True), dtype=torch.uint8, device="cuda")
+            emo.emo_eval_intervals(h, B, Fd, F.shape[2], I, breaks, idle, T, E, Ei, ws, flags=flags)
+            out.append([x.cpu().numpy() for x in (T, E, Ei)])
+        # busy times are whole numbers: the idle energies are the same sums; energies of at most 1 500 non-negative terms, in another order
+        assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][2], out[1][2])
+        assert np.allclose(out[0][1], out[1][1], rtol=1e-12, atol=0)
+        some = np.unique(np.r_[0, B // 2, B - 1])
+        want = oracle_mod.intervals(g, group, breaks, np.ascontiguousarray(F[:, :, some]), W.idle_power(g.L))
+        assert np.array_equal(out[0][0][some], want["makespan"]) and np.allclose(out[0][1][some], want["energy"], rtol=1e-12, atol=0)
+    h.free()
