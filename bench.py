@@ -188,7 +188,7 @@ def other_workloads_leg(sm_mhz, hbm_gbs):
                 bw.append(ev[2].elapsed_time(ev[3]))
         assert int(status.item()) == 0
         out.append({"workload": name, "n": int(g.n), "policies": int(B),
-                    "kernels": names[emo.emo_call_path(h, B, lv, lv.stride(0), B, True, 0)],
+                    "kernels": "slices" if emo.emo_call_slices(h, B, True) else names[emo.emo_call_path(h, B, lv, lv.stride(0), B, True, 0)],
                     "fwd_ms": float(np.median(fw)), "bwd_ms": float(np.median(bw)),
                     "depth_floor_ms": 2 * info.depth * 30.0 / (sm_mhz * 1e6) * 1e3,
                     "t_hbm_ms": 9.0 * g.n * B / (hbm_gbs * 1e9) * 1e3})
