@@ -58,7 +58,8 @@ extern "C" {
 #define EMO_F_GENERIC 0x4u         /* skip the schedule compilers: the generic kernels evaluate the graph (they also take every
                                       graph whose simultaneously live values exceed the on-chip exchange slots) */
 #define EMO_F_TEST_LONG_OOM 0x8u   /* test hook: there is no memory for the spine program with the longer stages (host-only handles: on the
-                                      host; else on the device); the load goes on without it */
+                                      host; else on the device); the load goes on without it.  With EMO_F_HOST_ONLY | EMO_F_GENERIC: the load
+                                      finds no memory for its programs while a thread of its own still reads the graph (EMO_E_OOM) */
 /* flags of the evaluation calls */
 #define EMO_F_VALIDATE 0x1u        /* check every level < L first; EMO_E_RANGE goes to *status */
 #define EMO_F_NO_STAGING 0x2u      /* use the plain-load kernels instead of the staged ones */

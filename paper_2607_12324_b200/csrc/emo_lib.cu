@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <map>
@@ -1983,13 +1984,15 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
         }
     }
 
-    emo_graph *g = new (std::nothrow) emo_graph();
-    if (!g) return EMO_E_OOM;
-    Slices slices;
-    struct Joined {
+    // (declared before the threads below, so that however the load ends it waits for them before the graph goes)
+    struct Owned {
         emo_graph *g = nullptr;
-        ~Joined() { if (g) emo_graph_free(g); }
-    } joined;
+        ~Owned() { emo_graph_free(g); }
+    } owned, joined;
+    emo_graph *const g = owned.g = new (std::nothrow) emo_graph();
+    if (!g) return EMO_E_OOM;
+    g->host_only = (flags & EMO_F_HOST_ONLY) != 0;
+    Slices slices;
     try {
         HostGraph &h = g->h;
         h.n = n;
@@ -2011,7 +2014,7 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
             for (int l = 1; l < L; ++l) x = std::min(x, lat[(size_t)v * L + l]);
             return (__int128)x;
         });
-        if (tw >= ((__int128)1 << 62)) { delete g; return EMO_E_OVERFLOW; }
+        if (tw >= ((__int128)1 << 62)) return EMO_E_OVERFLOW;
         h.T_worst = (int64_t)tw;
         h.T_best = (int64_t)tb;
         int lanes = (int)((flags >> 8) & 0xFF);
@@ -2050,14 +2053,17 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
                 work();
             }
         };
+        constexpr uint32_t kTestOom = EMO_F_HOST_ONLY | EMO_F_GENERIC | EMO_F_TEST_LONG_OOM;
+        const bool test_oom = flags == kTestOom;
         GraphBounds bounds;
-        if (!(flags & EMO_F_GENERIC)) graph_bounds(h, lat, energy, bounds);
+        if (!(flags & EMO_F_GENERIC) || test_oom) graph_bounds(h, lat, energy, bounds);
         // the contracted graph, beside everything else (not where the caller shapes the programs)
         int device = 0;
         Helper joined_thread;
-        if (!inner && n >= 2000 && flags == 0 && cudaGetDevice(&device) == cudaSuccess)
+        if (!inner && n >= 2000 && (test_oom || (flags == 0 && cudaGetDevice(&device) == cudaSuccess)))
             start(joined_thread, [&, device]() {
                 try {
+                    if (test_oom) std::this_thread::sleep_for(std::chrono::milliseconds(100));
                     Contracted c;
                     contract_forward(h, lat, energy, bounds, false, c);
                     // where it leaves three nodes of five (measured, forward, us: 75 000 nodes to 11 088 x 10 001 policies 520 / 1 271; with
@@ -2068,7 +2074,7 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
                 } catch (const std::exception &) {      // no memory for it: the graph itself serves
                 }
             });
-        int rc = (flags & EMO_F_GENERIC) ? EMO_E_UNSUPPORTED : (inner ? EMO_OK : compile_dir(true, nullptr, g->bwd));
+        int rc = test_oom ? EMO_E_OOM : (flags & EMO_F_GENERIC) ? EMO_E_UNSUPPORTED : (inner ? EMO_OK : compile_dir(true, nullptr, g->bwd));
         if (rc == EMO_OK && !inner) rc = compile_dir(false, &g->bwd.pos_of_node, g->fwd);
         if (rc == EMO_E_UNSUPPORTED) {
             // more live exchanged values than the on-chip schedules can hold: the generic kernels take the graph
@@ -2079,7 +2085,7 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
             g->host_energy.assign(energy, energy + (size_t)n * L);
             rc = EMO_OK;
         }
-        if (rc != EMO_OK) { delete g; return rc; }
+        if (rc != EMO_OK) return rc;
         if (!g->generic) {
             // stage length: the longest of 32, 16, 8 steps whose entries the producers can index
             // (32 * kFlowRowRegs per stage); one barrier per stage unless the caller says otherwise (measured on the
@@ -2157,7 +2163,7 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
                 rc = EMO_OK;
             }
             if (rc == EMO_OK && rc_s != EMO_OK && rc_s != EMO_E_UNSUPPORTED) rc = rc_s;
-            if (rc != EMO_OK) { delete g; return rc; }
+            if (rc != EMO_OK) return rc;
             if (!want_spine || rc_s != EMO_OK || !(g->flow.ok32 || inner) || !g->sflow.spine.ok) g->sflow = Flow();
             else {
                 // only the spine's parts are kept
@@ -2181,18 +2187,16 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
         joined_thread.wait();
         if (!g->generic) std::swap(g->joined, joined.g);
     } catch (const std::bad_alloc &) {
-        delete g;
         return EMO_E_OOM;
     }
-    g->host_only = (flags & EMO_F_HOST_ONLY) != 0;
     if (g->host_only) {
         g->dspine.ready = g->sflow.spine.ok && !g->simage.host.empty();
         g->dlong.ready = g->lflow.spine.ok && !g->limage.host.empty();
     } else {
         int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); emo_graph_free(g); return EMO_E_CUDA; }
+        if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return EMO_E_CUDA; }
         cudaDeviceProp prop;
-        if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { (void)cudaGetLastError(); emo_graph_free(g); return EMO_E_CUDA; }
+        if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { (void)cudaGetLastError(); return EMO_E_CUDA; }
         g->device = dev;
         g->sm_count = prop.multiProcessorCount;
         g->smem_optin = prop.sharedMemPerBlockOptin;
@@ -2270,9 +2274,10 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
         } catch (const std::bad_alloc &) {
             rc = EMO_E_OOM;
         }
-        if (rc != EMO_OK) { emo_graph_free(g); return rc; }
+        if (rc != EMO_OK) return rc;
         if (!inner) g->one_bytes = pass_ws_bytes(g, 1, 1, 0, 1);
     }
+    owned.g = nullptr;
     *out = g;
     return EMO_OK;
 }
