@@ -182,6 +182,7 @@ int build_spine(const SpineIn &in, Spine &out, std::string &err);
 struct GraphBounds {
     std::vector<int64_t> pp, sp;                  // predecessor / successor CSR
     std::vector<int32_t> pc, sc;
+    std::vector<int64_t> se;                      // per successor-CSR edge its place in the predecessor CSR
     std::vector<int64_t> dmin, dmax, lbES, lbC, ubC, lbQin, lbQ, ubQ;
     std::vector<char> constant;                   // node's tables do not depend on the level
     std::vector<char> liveF, liveB;               // per predecessor-CSR edge

@@ -84,10 +84,14 @@ void graph_bounds(const HostGraph &g, const int64_t *lat, const double *energy, 
     for (int64_t e = 0; e < m; ++e) sp[pc[e] + 1]++;
     for (int32_t v = 0; v < n; ++v) sp[v + 1] += sp[v];
     sc.assign((size_t)std::max<int64_t>(m, 1), 0);
+    b.se.assign((size_t)std::max<int64_t>(m, 1), 0);
     {
         std::vector<int64_t> fill(sp.begin(), sp.end() - 1);
         for (int32_t v = 0; v < n; ++v)
-            for (int64_t e = pp[v]; e < pp[v + 1]; ++e) sc[fill[pc[e]]++] = v;
+            for (int64_t e = pp[v]; e < pp[v + 1]; ++e) {
+                b.se[fill[pc[e]]] = e;
+                sc[fill[pc[e]]++] = v;
+            }
     }
 
     // ---- static bounds --------------------------------------------------------------------------

@@ -18,21 +18,17 @@ std::vector<int32_t> narrow_order(int32_t n, const GraphBounds &b)
     std::vector<char> ready((size_t)n, 0), live((size_t)n, 0), done((size_t)n, 0);
     using Key = std::pair<int32_t, int32_t>;      // (growth, -node)
     std::priority_queue<Key, std::vector<Key>, std::greater<Key>> heap;
-    auto growth = [&](int32_t v) {
-        int32_t k = live[v] ? -1 : 0;
-        for (int64_t e = b.pp[v]; e < b.pp[v + 1]; ++e) k += live[b.pc[e]] ? 0 : 1;
-        return k;
-    };
+    // (counted once, when the node can be placed; from then on it falls by one with every operand that begins to be waited for: nodes with
+    // tens of thousands of operands are common, a host sync behind every kernel)
     auto offer = [&](int32_t v) {
-        cur[v] = growth(v);
+        ready[v] = 1;
+        cur[v] = live[v] ? -1 : 0;
+        for (int64_t e = b.pp[v]; e < b.pp[v + 1]; ++e) cur[v] += live[b.pc[e]] ? 0 : 1;
         heap.push({cur[v], -v});
     };
     for (int32_t v = 0; v < n; ++v) {
         left[v] = (int32_t)(b.sp[v + 1] - b.sp[v]);
-        if (left[v] == 0) {
-            ready[v] = 1;
-            offer(v);
-        }
+        if (left[v] == 0) offer(v);
     }
     int32_t at = n;
     while (!heap.empty()) {
@@ -46,12 +42,9 @@ std::vector<int32_t> narrow_order(int32_t n, const GraphBounds &b)
             if (!live[u]) {
                 live[u] = 1;
                 for (int64_t f = b.sp[u]; f < b.sp[u + 1]; ++f)
-                    if (ready[b.sc[f]] && !done[b.sc[f]]) offer(b.sc[f]);
+                    if (ready[b.sc[f]] && !done[b.sc[f]]) heap.push({--cur[b.sc[f]], -b.sc[f]});
             }
-            if (--left[u] == 0) {
-                ready[u] = 1;
-                offer(u);
-            }
+            if (--left[u] == 0) offer(u);
         }
     }
     return order;
@@ -327,11 +320,8 @@ void compile_slices(const HostGraph &g, const int64_t *lat, const double *energy
                   [&](int32_t v) { return b.sp[v + 1] == b.sp[v]; }, h.dir[0], lists[0]);
         build_dir(back, cross_b[c + 1], cross_b[c], local, cross, false,
                   [&](int32_t v, auto f) {
-                      for (int64_t s = b.sp[v]; s < b.sp[v + 1]; ++s) {
-                          const int32_t u = b.sc[s];
-                          for (int64_t e = b.pp[u]; e < b.pp[u + 1]; ++e)
-                              if (b.pc[e] == v && b.liveB[e]) f(u);
-                      }
+                      for (int64_t s = b.sp[v]; s < b.sp[v + 1]; ++s)
+                          if (b.liveB[b.se[s]]) f(b.sc[s]);
                   },
                   [](int32_t) { return false; }, h.dir[1], lists[1]);
         // the words of the slice
