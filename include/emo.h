@@ -135,8 +135,9 @@ int emo_graph_info(const emo_graph *g, emo_info *info);
  * emo_workspace_bytes - device scratch a call on B policies needs.  need_slack = 0 gives the size
  * for emo_eval_policies, emo_baseline and emo_select; 1 the size emo_slack_batch needs when the
  * caller passes no ES array (the earliest start times are then kept in the workspace between the
- * two passes); 2 the size emo_slack_batch_host needs.  The caller allocates; no call allocates
- * device memory per invocation.
+ * two passes); 2 the size emo_slack_batch_host needs.  The caller allocates, aligned as cudaMalloc aligns (16 bytes
+ * suffice; a forward-only call that finds less does without the workspace); no call allocates device memory per
+ * invocation.
  */
 int emo_workspace_bytes(const emo_graph *g, int64_t B, int need_slack, size_t *out);
 

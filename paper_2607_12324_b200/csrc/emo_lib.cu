@@ -1718,6 +1718,13 @@ bool slice_allowed(const emo_graph *g, int64_t B, bool want_base, bool need_bwd,
     return slice_plan(g, B, want_base, need_bwd, 1, pl);
 }
 
+// Bytes that the slice kernels may use of a caller's workspace, behind its head.  They move it 16 bytes at a time: none where it is not
+// aligned to that (forward calls do not touch it otherwise, so there it may lie anywhere).
+size_t slice_room(const void *ws, size_t ws_bytes, size_t head)
+{
+    return ws && aligned16(ws) && ws_bytes > head ? ws_bytes - head : 0;
+}
+
 int launch_slices(const emo_graph *g, SlicePlan &pl, const uint8_t *lvl, int64_t ldb, int64_t *ES, int64_t *LS, int64_t *slack, int64_t ldo, int64_t *makespan,
                   double *energy, int64_t *slack_sum, int32_t *n_critical, int64_t *base_T, double *base_E, unsigned char *ws, cudaStream_t st)
 {
@@ -2642,7 +2649,7 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
     for (const emo_graph *e : {joined_for(g, flags), g}) {
         if (!e) continue;
         SlicePlan cp;
-        if (slice_allowed(e, B, T0 || E0, false, false, flags, cp) && (cp.ws == 0 || (ws && ws_bytes >= head + cp.ws)))
+        if (slice_allowed(e, B, T0 || E0, false, false, flags, cp) && cp.ws <= slice_room(ws, ws_bytes, head))
             return launch_slices(e, cp, lvl, ldb, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, (unsigned char *)ws + head, st);
         SpinePlan fp;
         if (spine_allowed(e, B, lvl, ldb, 0, flags) && spine_plan(e, B, T0 || E0, false, false, fp))
@@ -3070,7 +3077,7 @@ int emo_slack_batch(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t l
     {
         SlicePlan cp;
         const size_t head = kSmallWs + lvl_area(g);
-        if (slice_allowed(g, B, T0 || E0, true, ES || LS || slack_sum || n_critical, flags, cp) && (cp.ws == 0 || (ws && ws_bytes >= head + cp.ws)))
+        if (slice_allowed(g, B, T0 || E0, true, ES || LS || slack_sum || n_critical, flags, cp) && cp.ws <= slice_room(ws, ws_bytes, head))
             return launch_slices(g, cp, lvl, ldb, ES, LS, slack, ldo, makespan, energy, slack_sum, n_critical, T0, E0, (unsigned char *)ws + head, st);
     }
     if (spine_allowed(g, B, lvl, ldb, ldo, flags)) {
@@ -3129,7 +3136,7 @@ int emo_slack(const emo_graph *g, const uint8_t *lvl_one, int64_t *ES, int64_t *
     {
         SlicePlan cp;
         const size_t head = kSmallWs + lvl_area(g);
-        if (slice_allowed(g, 1, false, true, true, 0, cp) && ws_bytes >= head + cp.ws)
+        if (slice_allowed(g, 1, false, true, true, 0, cp) && cp.ws <= slice_room(ws, ws_bytes, head))
             return launch_slices(g, cp, lvl_one, 1, ES, LS, slack, 1, makespan, e1, nullptr, nullptr, nullptr, nullptr, (unsigned char *)ws + head, st);
     }
     // re-pitch the level vector to [rows][16] so that the staged kernels can be used; the

@@ -67,3 +67,21 @@ def test_random_dags(torch_cuda, emo, oracle_mod):
             done += 1
         h.free()
     assert done >= 12
+
+
+def test_forward_calls_take_a_workspace_anywhere(torch_cuda, emo, oracle_mod):
+    """A workspace at any address (a forward-only call needs none): the slice kernels, which move it in 16-byte pieces, leave the call to others."""
+    torch = torch_cuda
+    g, B = W.make_graph("cfg1-train", 0.3), 40
+    lv, lv_dev = levels(torch, g.n, g.L, B, 7)
+    want = oracle_mod.batch(g, lv)
+    h = emo.load_workload(g)
+    assert emo.emo_call_slices(h, B, False) > 8      # (fewer need no workspace either)
+    buf = torch.zeros(emo.emo_workspace_bytes(h, B, 0) + 64, dtype=torch.uint8, device="cuda")
+    for offset in (0, 1, 4, 8, 16):
+        T, E = torch.zeros(B, dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.float64, device="cuda")
+        buf.fill_(0xEE)
+        emo.emo_eval_policies(h, B, lv_dev, lv_dev.stride(0), T, E, buf[offset:])
+        assert np.array_equal(T.cpu().numpy(), want["makespan"]) and np.allclose(E.cpu().numpy(), want["energy"], rtol=1e-12, atol=0), offset
+        assert bool((buf == 0xEE).all()) == (offset % 16 != 0), offset
+    h.free()
