@@ -153,7 +153,7 @@ struct WalkState {
             const int over = leaves ? (int)sum - left : 0;
             const int step = i + 1 >= p.I - 1 ? kWalkBig : p.delta;
             if (__any_sync(0xFFFFFFFFu, over >= step)) {
-                one_by_one(p, n, da, ea);
+                one_by_one<K>(p, n, da, ea);
                 return;
             }
             if (leaves) {
@@ -174,20 +174,38 @@ struct WalkState {
             for (int j = 0; j + w < K; j += 2 * w) e[j] += e[j + w];
         E += e[0];
     }
+    // The same node after node, where some policy of the warp has a node that outlasts an interval.  The energies are added pair by pair as
+    // above: a policy's energy does not depend on the policies beside it.
+    template <int K>
     __device__ __forceinline__ void one_by_one(const WalkParams &p, int n, unsigned da, unsigned ea)
     {
-        for (int j = 0; j < n; ++j) {
-            const unsigned o = (unsigned)j * (unsigned)p.Lp * 4u + la;
-            const int d = (int)emo_lds_u32(da + o);
-            E += emo_walk_ldf(ea + 2u * o);
-            bacc += d;
-            left -= d;
-            while (left <= 0) {
-                flush(p, bacc + left);
-                bacc = -left;
-                advance(p, -left);
+        double one = 0.0, two = 0.0, four = 0.0, sum = 0.0;      // first halves of the pairs, of the fours, of the eight
+#pragma unroll 1
+        for (int j = 0; j < K; ++j) {
+            double e = 0.0;
+            if (j < n) {
+                const unsigned o = (unsigned)j * (unsigned)p.Lp * 4u + la;
+                const int d = (int)emo_lds_u32(da + o);
+                e = emo_walk_ldf(ea + 2u * o);
+                bacc += d;
+                left -= d;
+                while (left <= 0) {
+                    flush(p, bacc + left);
+                    bacc = -left;
+                    advance(p, -left);
+                }
+            }
+            if (!(j & 1)) {
+                one = e;
+            } else if (!(j & 2)) {
+                two = one + e;
+            } else if (!(j & 4)) {
+                sum = four = two + (one + e);
+            } else {
+                sum = four + (two + (one + e));
             }
         }
+        E += sum;
     }
 };
 

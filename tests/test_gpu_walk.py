@@ -50,3 +50,31 @@ def test_against_oracle_and_step_program(torch_cuda, emo, oracle_mod, seed, n, r
         want = oracle_mod.intervals(g, group, breaks, np.ascontiguousarray(F[:, :, some]), W.idle_power(g.L))
         assert np.array_equal(out[0][0][some], want["makespan"]) and np.allclose(out[0][1][some], want["energy"], rtol=1e-12, atol=0)
     h.free()
+
+
+def test_energy_does_not_depend_on_the_policies_beside_it(torch_cuda, emo):
+    """The same policy alone, among copies of itself and among policies whose nodes outlast whole intervals: the same energy, bit for bit (a
+    search keeps the first of equal candidates)."""
+    torch = torch_cuda
+    n, rs = 400, np.random.RandomState(11)            # one chain: items of as many nodes as there can be, and some of four and fewer
+    lat = rs.randint(1, 100, size=(n, 5)).astype(np.int64)
+    lat[:, 0] *= 20                                   # level 0: an item of eight nodes outlasts the intervals below, elsewhere none does
+    g = W.tiny_graph(n, [(v - 1, v) for v in range(1, n)], lat, rs.rand(n, 5))
+    h = emo.load_workload(g, emo.EMO_F_INTERVALS, group_of=np.where(np.arange(n) < 300, 0, np.arange(n) // 4 % 2).astype(np.int32))
+    I, rs = 600, np.random.RandomState(13)
+    breaks = np.arange(I, dtype=np.int64) * 1500      # (and none is in the last one before the end)
+    mine = rs.randint(1, 5, size=(2, I))
+
+    def energies(F):
+        B = F.shape[2]
+        Fd = torch.from_numpy(np.ascontiguousarray(F.astype(np.uint8))).cuda()
+        T, E = torch.zeros(B, dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.float64, device="cuda")
+        ws = torch.empty(emo.emo_workspace_bytes_intervals(h, B, I, False), dtype=torch.uint8, device="cuda")
+        emo.emo_eval_intervals(h, B, Fd, B, I, breaks, None, T, E, None, ws)
+        return E.cpu().numpy()
+    alone = energies(mine[:, :, None])[0]
+    for B in (4, 16, 3000):
+        assert (energies(np.repeat(mine[:, :, None], B, axis=2)) == alone).all()
+        F = np.where(np.arange(B) % 3 == 0, mine[:, :, None], 0)
+        assert (energies(F)[::3] == alone).all(), B
+    h.free()
