@@ -203,6 +203,12 @@ int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t 
 int emo_workspace_bytes_intervals(const emo_graph *g, int64_t B, int32_t I, int with_idle, size_t *out);
 
 /*
+ * emo_call_intervals - which kernel emo_eval_intervals runs for these arguments: 2 = a thread per policy, 1 = the lane-stream kernel,
+ * 0 = the step-program kernel.  Launches nothing.
+ */
+int emo_call_intervals(const emo_graph *g, int64_t B, int32_t I, const int64_t *breaks, uint32_t flags);
+
+/*
  * emo_pack_greedy - kernel packing (Sec. 4.4): the critical predecessor of every node at the default frequency
  * (Eq. 5: k*_v = argmax over predecessors of C_k; among equals the lowest index, the one Alg. 1's update meets
  * first) and the dependency-aware greedy packing of GPU kernels.  The kernels of every stream are walked in

@@ -2735,12 +2735,38 @@ static bool walk_pays(const emo_graph *g, int64_t B, int rows, int32_t I, int wa
     return g->flow.lanes <= 3 ? walk_waves <= flow_waves : walk_waves * 2 <= flow_waves;
 }
 
-int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t ldb, int32_t I, const int64_t *breaks,
-                       const double *p_idle, int64_t *makespan, double *energy, double *energy_idle, void *ws,
-                       size_t ws_bytes, int32_t *status, uint32_t flags, void *stream)
+// Length of the intervals of a uniform grid, else 0.
+static long long interval_length(int32_t I, const int64_t *breaks)
 {
-    (void)flags;
-    (void)status;
+    const long long delta = I > 1 ? breaks[1] : 0;
+    for (int32_t i = 1; i < I && delta > 0; ++i)
+        if (breaks[i] != (int64_t)i * delta) return 0;
+    return delta;
+}
+
+// Which kernel evaluates a call with time intervals, and how it is launched.
+enum { kIntervalSteps, kIntervalFlow, kIntervalWalk };
+struct IntervalPlan {
+    WalkParams walk;
+    FlowPlan flow;
+    int walk_grid = 0;
+    size_t walk_smem = 0;
+};
+// walk: whether the walk kernel may take it (1), must where it can (2), or does not (0)
+static int interval_kernel(const emo_graph *g, int64_t B, int32_t I, long long delta, uint32_t flags, int walk, IntervalPlan &pl)
+{
+    const int rows = std::max(g->h.rows, 1);
+    if ((flags & EMO_F_NO_STAGING) || delta <= 0) return kIntervalSteps;
+    if (walk && !(flags & EMO_F_FLOW_KERNEL) && walk_plan(g, B, rows, I, delta, pl.walk, pl.walk_grid, pl.walk_smem) &&
+        (walk == 2 || walk_pays(g, B, rows, I, pl.walk_grid)))
+        return kIntervalWalk;
+    return g->dflow.blobFI && flow_plan(g, B, false, false, pl.flow, true, round_up((size_t)I * 8, 16), (size_t)rows * (size_t)I * 32) ? kIntervalFlow : kIntervalSteps;
+}
+
+static int eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t ldb, int32_t I, const int64_t *breaks,
+                          const double *p_idle, int64_t *makespan, double *energy, double *energy_idle, void *ws,
+                          size_t ws_bytes, int32_t *status, uint32_t flags, int walk, void *stream)
+{
     if (!g || B < 0 || I < 1 || I > 4096 || !breaks || breaks[0] != 0) return EMO_E_INVALID_ARG;
     for (int32_t i = 1; i < I; ++i)
         if (breaks[i] <= breaks[i - 1]) return EMO_E_INVALID_ARG;
@@ -2760,70 +2786,58 @@ int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t 
     EMO_CUDA(cudaMemcpyAsync(d_breaks, breaks, (size_t)I * 8, cudaMemcpyHostToDevice, st));
     if (busy) EMO_CUDA(cudaMemsetAsync(busy, 0, (size_t)rows * (size_t)I * (size_t)ldw * 8, st));
     const float inv_mean = (I > 1) ? (float)((double)(I - 1) / (double)breaks[I - 1]) : 0.0f;
-    long long delta = (I > 1) ? breaks[1] : 0;
-    for (int32_t i = 1; i < I && delta > 0; ++i)
-        if (breaks[i] != (int64_t)i * delta) delta = 0;
+    const long long delta = interval_length(I, breaks);
     cudaEvent_t ev0 = g_pass_events[0], ev1 = g_pass_events[1];
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
-    bool done = false;
-    {
-        WalkParams q;
-        int grid = 0;
-        size_t smem = 0;
-        if (!(flags & (EMO_F_NO_STAGING | EMO_F_FLOW_KERNEL)) && walk_plan(g, B, rows, I, delta, q, grid, smem) && walk_pays(g, B, rows, I, grid)) {
-            q.F = F;
-            q.ldF = ldb;
-            q.makespan = makespan;
-            q.energy = energy;
-            q.busy = busy;
-            q.ldw = ldw;
-            q.status = status;
-            q.wait_cycles = g_wait_cycles;
-            if (flow_optin(emo_walk, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
-            emo_walk<<<grid, (q.groups + 1) * 32, smem, st>>>(q);
-            EMO_CUDA(cudaGetLastError());
-            done = true;
-        }
-    }
-    if (!done && !(flags & EMO_F_NO_STAGING) && g->dflow.blobFI && delta > 0) {
+    IntervalPlan plan;
+    const int which = interval_kernel(g, B, I, delta, flags, walk, plan);
+    if (which == kIntervalWalk) {
+        WalkParams &q = plan.walk;
+        q.F = F;
+        q.ldF = ldb;
+        q.makespan = makespan;
+        q.energy = energy;
+        q.busy = busy;
+        q.ldw = ldw;
+        q.status = status;
+        q.wait_cycles = g_wait_cycles;
+        if (flow_optin(emo_walk, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+        emo_walk<<<plan.walk_grid, (q.groups + 1) * 32, plan.walk_smem, st>>>(q);
+        EMO_CUDA(cudaGetLastError());
+    } else if (which == kIntervalFlow) {
         // the lane-stream forward kernel with the look-up inside the chain: uniform grids, F's columns in shared memory
-        FlowPlan fp;
-        const size_t brk_b = round_up((size_t)I * 8, 16), f_per_group = (size_t)rows * (size_t)I * 32;
-        if (flow_plan(g, B, false, false, fp, true, brk_b, f_per_group)) {
-            FlowParams q = fp.pf;
-            q.B = B;
-            q.lvl = nullptr;
-            q.ldb = 0;
-            q.restore = nullptr;
-            q.makespan = makespan;
-            q.energy = energy;
-            q.status = status;
-            q.F = F;
-            q.ldF = ldb;
-            q.I = I;
-            q.rowsF = rows;
-            q.delta = delta;
-            q.inv_mean = inv_mean;
-            q.breaks = (const long long *)d_breaks;
-            q.busy = busy;
-            q.ldw = ldw;
-            // Where the lanes often change the device, or an interval holds less than an entry of a lane, keeping the interval at hand costs
-            // more than it saves: every entry looks its interval up.  Measured (ms, at hand / looked up): 8 devices on 18 lanes, 20 % of a lane's
-            // packs on another device than the one before, 38 000 nodes x 8 192 policies 3.06 / 2.83 with 2 intervals, 5.27 / 4.69 with 200;
-            // one device, 3 lanes, 2 500 packs x 16 384: 800 intervals 1.99 / 2.04, 1 600 4.46 / 4.35; 2 lanes, 250 packs: 200 0.310 /
-            // 0.282 (100: 0.237 / 0.223 would pay, the line is where 5 000 nodes turn); 25 000 nodes, 100 intervals 1.43 / 2.43.
-            const DevFlow &df = g->dflow;
-            const bool dense = df.switches * 20 > df.packs * 3 || (int64_t)g->flow.lanes * I > df.packs;
-            void (*kern)(FlowParams) = nullptr;
-            if (dense) kern = fp.threads <= 512 ? emo_flow_fwd<512, true, false, true> : (fp.threads <= 768 ? emo_flow_fwd<768, true, false, true> : emo_flow_fwd<1024, true, false, true>);
-            else kern = fp.threads <= 512 ? emo_flow_fwd<512, true, false> : (fp.threads <= 768 ? emo_flow_fwd<768, true, false> : emo_flow_fwd<1024, true, false>);
-            if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
-            kern<<<fp.grid_f, fp.threads, fp.smem_f, st>>>(q);
-            EMO_CUDA(cudaGetLastError());
-            done = true;
-        }
-    }
-    if (!done) {
+        const FlowPlan &fp = plan.flow;
+        FlowParams q = fp.pf;
+        q.B = B;
+        q.lvl = nullptr;
+        q.ldb = 0;
+        q.restore = nullptr;
+        q.makespan = makespan;
+        q.energy = energy;
+        q.status = status;
+        q.F = F;
+        q.ldF = ldb;
+        q.I = I;
+        q.rowsF = rows;
+        q.delta = delta;
+        q.inv_mean = inv_mean;
+        q.breaks = (const long long *)d_breaks;
+        q.busy = busy;
+        q.ldw = ldw;
+        // Where the lanes often change the device, or an interval holds less than an entry of a lane, keeping the interval at hand costs
+        // more than it saves: every entry looks its interval up.  Measured (ms, at hand / looked up): 8 devices on 18 lanes, 20 % of a lane's
+        // packs on another device than the one before, 38 000 nodes x 8 192 policies 3.06 / 2.83 with 2 intervals, 5.27 / 4.69 with 200;
+        // one device, 3 lanes, 2 500 packs x 16 384: 800 intervals 1.99 / 2.04, 1 600 4.46 / 4.35; 2 lanes, 250 packs: 200 0.310 /
+        // 0.282 (100: 0.237 / 0.223 would pay, the line is where 5 000 nodes turn); 25 000 nodes, 100 intervals 1.43 / 2.43.
+        const DevFlow &df = g->dflow;
+        const bool dense = df.switches * 20 > df.packs * 3 || (int64_t)g->flow.lanes * I > df.packs;
+        void (*kern)(FlowParams) = nullptr;
+        if (dense) kern = fp.threads <= 512 ? emo_flow_fwd<512, true, false, true> : (fp.threads <= 768 ? emo_flow_fwd<768, true, false, true> : emo_flow_fwd<1024, true, false, true>);
+        else kern = fp.threads <= 512 ? emo_flow_fwd<512, true, false> : (fp.threads <= 768 ? emo_flow_fwd<768, true, false> : emo_flow_fwd<1024, true, false>);
+        if (flow_optin(kern, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+        kern<<<fp.grid_f, fp.threads, fp.smem_f, st>>>(q);
+        EMO_CUDA(cudaGetLastError());
+    } else {
     const Program &p = g->fwd;
     const DevProgram &d = g->dfwd;
     if (p.steps == 0) return EMO_E_UNSUPPORTED;
@@ -2885,6 +2899,22 @@ int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t 
     return EMO_OK;
 }
 
+int emo_eval_intervals(const emo_graph *g, int64_t B, const uint8_t *F, int64_t ldb, int32_t I, const int64_t *breaks,
+                       const double *p_idle, int64_t *makespan, double *energy, double *energy_idle, void *ws,
+                       size_t ws_bytes, int32_t *status, uint32_t flags, void *stream)
+{
+    return eval_intervals(g, B, F, ldb, I, breaks, p_idle, makespan, energy, energy_idle, ws, ws_bytes, status, flags, 1, stream);
+}
+
+int emo_call_intervals(const emo_graph *g, int64_t B, int32_t I, const int64_t *breaks, uint32_t flags)
+{
+    if (!g || B < 0 || I < 1 || I > 4096 || !breaks) return EMO_E_INVALID_ARG;
+    if (g->host_only) return EMO_E_CUDA;
+    if (g->generic) return EMO_E_UNSUPPORTED;
+    IntervalPlan plan;
+    return interval_kernel(g, B, I, interval_length(I, breaks), flags, 1, plan);
+}
+
 // Workspace of emo_search_dp: the candidates' levels, their times and energies, and what the evaluation needs.
 static void search_layout(const emo_graph *g, int32_t I, int64_t batch, int with_idle, size_t &off_T, size_t &off_E, size_t &off_ws,
                           size_t &total, int64_t &ldb)
@@ -2935,6 +2965,13 @@ int emo_search_dp(const emo_graph *g, int32_t I, const int64_t *breaks, const do
     };
     int64_t calls = 0;
     *found = 0;
+    // One kernel for all of a search: it compares the energies of one batch with those of another, and two kernels add them in different
+    // orders.  The walk kernel where the rule takes it for the smallest batch and for the largest (what fits it with many policies
+    // fits with fewer).
+    IntervalPlan probe;
+    const long long delta = interval_length(I, breaks);
+    const bool walk = !g->generic && interval_kernel(g, std::min<int64_t>(L, max_batch), I, delta, 0, 1, probe) == kIntervalWalk &&
+                      interval_kernel(g, max_batch, I, delta, 0, 1, probe) == kIntervalWalk;
     try {
         std::vector<uint8_t> hF((size_t)rows * I * ldb);
         std::vector<int64_t> hT((size_t)max_batch);
@@ -2949,7 +2986,7 @@ int emo_search_dp(const emo_graph *g, int32_t I, const int64_t *breaks, const do
                     for (int64_t c = 0; c < nb; ++c) dst[c] = (patch[c].first == i) ? patch[c].second : cand[c][i];
                 }
             if (cudaMemcpyAsync(dF, hF.data(), (size_t)rows * I * ld, cudaMemcpyHostToDevice, st) != cudaSuccess) return EMO_E_CUDA;
-            int rc = emo_eval_intervals(g, nb, dF, ld, I, breaks, p_idle, dT, dE, nullptr, iws, iws_bytes, nullptr, 0, stream);
+            int rc = eval_intervals(g, nb, dF, ld, I, breaks, p_idle, dT, dE, nullptr, iws, iws_bytes, nullptr, 0, walk ? 2 : 0, stream);
             if (rc) return rc;
             if (cudaMemcpyAsync(hT.data(), dT, (size_t)nb * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) return EMO_E_CUDA;
             if (cudaMemcpyAsync(hE.data(), dE, (size_t)nb * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) return EMO_E_CUDA;

@@ -35,7 +35,7 @@ EXPORTS = [
     "emo_strerror", "emo_graph_load", "emo_graph_free", "emo_graph_info", "emo_workspace_bytes",
     "emo_eval_policies", "emo_slack_batch", "emo_slack", "emo_baseline", "emo_target_from_delta",
     "emo_select", "emo_transpose_policies", "emo_slack_batch_host", "emo_graph_program",
-    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_graph_spine_plan", "emo_graph_spine_layout", "emo_set_wait_limit", "emo_call_path", "emo_call_slices", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
+    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_graph_spine_plan", "emo_graph_spine_layout", "emo_set_wait_limit", "emo_call_path", "emo_call_slices", "emo_call_intervals", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
 ]
 
 
@@ -139,6 +139,7 @@ def lib():
         L.emo_slack_batch_prefetched.argtypes = [p, i64, ctypes.c_int, p, i64, p, p, i64, p, i64, i64, p, p, p, p, p, p, sz, u32, p]
         L.emo_call_path.argtypes = [p, i64, p, i64, i64, ctypes.c_int, u32]
         L.emo_call_slices.argtypes = [p, i64, ctypes.c_int, u32]
+        L.emo_call_intervals.argtypes = [p, i64, i32, p, u32]
         L.emo_select_static.argtypes = [i64, p, p, i64, p, i64, p, p, p, p]
         for name in EXPORTS:
             if name not in ("emo_strerror", "emo_target_from_delta"):
@@ -497,6 +498,15 @@ def emo_eval_intervals(g, B, F, ldb, I, breaks, p_idle, makespan, energy, energy
     return _check(lib().emo_eval_intervals(g.handle, int(B), _addr(F), int(ldb), int(I), brk.ctypes.data_as(ctypes.c_void_p),
                                            _addr(p_idle), _addr(makespan), _addr(energy), _addr(energy_idle), _addr(ws),
                                            _nbytes(ws), _addr(status), int(flags), _stream(stream)), "emo_eval_intervals")
+
+
+def emo_call_intervals(g: Graph, B, breaks, flags: int = 0) -> int:
+    """Which kernel emo_eval_intervals would run (inspection): 2 a thread per policy, 1 lane streams, 0 step program."""
+    brk = np.ascontiguousarray(breaks, dtype=np.int64)
+    rc = lib().emo_call_intervals(g.handle, int(B), len(brk), brk.ctypes.data_as(ctypes.c_void_p), int(flags))
+    if rc < 0:
+        raise EmoError(rc, "emo_call_intervals")
+    return rc
 
 
 def emo_workspace_bytes_search(g, I, max_batch=0, with_idle=True) -> int:

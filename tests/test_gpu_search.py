@@ -25,8 +25,10 @@ def emo():
     return E
 
 
-def run_search(torch, emo, g, dev_of, breaks, p_idle, T_max, bin_ns, max_batch=0):
-    h = emo.load_workload(g, group_of=np.asarray(dev_of, np.int32))
+def run_search(torch, emo, g, dev_of, breaks, p_idle, T_max, bin_ns, max_batch=0, flags=0, kernels=None):
+    """kernels: those that one policy and a full batch outside a search run (emo_call_intervals)."""
+    h = emo.load_workload(g, flags, group_of=np.asarray(dev_of, np.int32))
+    assert kernels is None or kernels == (emo.emo_call_intervals(h, 1, breaks), emo.emo_call_intervals(h, max_batch or 16384, breaks))
     pi = torch.from_numpy(np.asarray(p_idle, np.float64)).cuda() if p_idle is not None else None
     ws = torch.empty(emo.emo_workspace_bytes_search(h, len(breaks), max_batch, p_idle is not None), dtype=torch.uint8, device="cuda")
     r = emo.emo_search_dp(h, breaks, pi, T_max, bin_ns, ws, max_batch=max_batch)
@@ -68,3 +70,39 @@ def test_config_graph(torch_cuda, emo, oracle_mod):
     b = oracle_mod.search_dp(g, dev_of, breaks, p_idle, T_max, 1000)
     compare(a, b)
     assert a["found"] and a["T"] <= T_max
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_a_thread_per_policy(torch_cuda, emo, oracle_mod, seed):
+    """The kernel that gives every policy a thread, with nodes that outlast intervals (a level that no node starts at makes candidates
+    equal: the first stays) and batches that split a round."""
+    from tests.test_gpu_walk import weave
+    g, dev_of = weave(70 + seed, 60, 2)
+    dev_of[:2] = 0, 1
+    t0 = int(oracle_mod.intervals(g, dev_of, np.zeros(1, np.int64), np.full((2, 1, 1), g.L - 1, np.uint8), None)["makespan"][0])
+    breaks = np.arange(6, dtype=np.int64) * (t0 // 5)
+    for p_idle in (W.idle_power(g.L), None):
+        for slack, bin_ns, mb in ((0.1, 1, 0), (0.3, 5, 0), (0.3, t0 // 50, 7), (1.0, t0 // 20, 33)):
+            T_max = int(t0 * (1 + slack))
+            compare(run_search(torch_cuda, emo, g, dev_of, breaks, p_idle, T_max, bin_ns, mb, emo.EMO_F_INTERVALS, (2, 2)),
+                    oracle_mod.search_dp(g, dev_of, breaks, p_idle, T_max, bin_ns))
+
+
+def test_one_kernel_for_all_of_a_search(torch_cuda, emo, oracle_mod):
+    """Many lanes, rounds of several batches: a full batch by itself would run another kernel than the small ones.  The search compares the
+    energies of all of them, so they come from one kernel: that of the policy it chose is, bit for bit, what the call for one policy gives."""
+    torch = torch_cuda
+    g = W.make_graph("cfg3-8dev", 0.01)
+    dev_of = W.device_of(g)
+    t0 = int(oracle_mod.batch(g, np.full((g.n, 1), g.L - 1, np.uint8))["makespan"][0])
+    breaks, p_idle, T_max = np.arange(3, dtype=np.int64) * (t0 // 3), W.idle_power(g.L), t0 + t0 // 4
+    a = run_search(torch, emo, g, dev_of, breaks, p_idle, T_max, 1, 6000, emo.EMO_F_INTERVALS, (1, 2))
+    assert a["n_pred"] > 6000      # (a round of more than one batch)
+    compare(a, oracle_mod.search_dp(g, dev_of, breaks, p_idle, T_max, 1))
+    h = emo.load_workload(g, emo.EMO_F_INTERVALS, group_of=dev_of)
+    F = torch.from_numpy(np.repeat(np.asarray(a["F"], np.uint8)[None, :, None], int(dev_of.max()) + 1, axis=0).copy()).cuda()
+    T, E = torch.zeros(1, dtype=torch.int64, device="cuda"), torch.zeros(1, dtype=torch.float64, device="cuda")
+    ws = torch.empty(emo.emo_workspace_bytes_intervals(h, 1, 3, True), dtype=torch.uint8, device="cuda")
+    emo.emo_eval_intervals(h, 1, F, 1, 3, breaks, torch.from_numpy(p_idle).cuda(), T, E, None, ws)
+    assert float(E[0]) == a["E"] and int(T[0]) == a["T"]
+    h.free()

@@ -35,6 +35,7 @@ def test_against_oracle_and_step_program(torch_cuda, emo, oracle_mod, seed, n, r
     # a grid that ends before the schedule does, and one that outlasts it
     for span in (0.6, 1.5):
         breaks = np.arange(I, dtype=np.int64) * max(1, int(h.info.T_best * span / I))
+        assert emo.emo_call_intervals(h, B, breaks) == 2 and emo.emo_call_intervals(h, B, breaks, emo.EMO_F_NO_STAGING) == 0
         F = np.random.RandomState(seed).randint(0, g.L, size=(rows, I, (B + 15) // 16 * 16)).astype(np.uint8)
         Fd, idle = torch.from_numpy(F).cuda(), torch.from_numpy(W.idle_power(g.L)).cuda()
         out = []
@@ -64,6 +65,7 @@ def test_energy_does_not_depend_on_the_policies_beside_it(torch_cuda, emo):
     I, rs = 600, np.random.RandomState(13)
     breaks = np.arange(I, dtype=np.int64) * 1500      # (and none is in the last one before the end)
     mine = rs.randint(1, 5, size=(2, I))
+    assert emo.emo_call_intervals(h, 4, breaks) == 2
 
     def energies(F):
         B = F.shape[2]
@@ -77,4 +79,31 @@ def test_energy_does_not_depend_on_the_policies_beside_it(torch_cuda, emo):
         assert (energies(np.repeat(mine[:, :, None], B, axis=2)) == alone).all()
         F = np.where(np.arange(B) % 3 == 0, mine[:, :, None], 0)
         assert (energies(F)[::3] == alone).all(), B
+    h.free()
+
+
+def test_many_lanes_in_several_waves(torch_cuda, emo, oracle_mod):
+    """More than three lanes: the walk from the batch on whose lane-stream blocks come in two waves."""
+    torch = torch_cuda
+    g = W.make_graph("cfg3-8dev", 0.01)
+    group = W.device_of(g)
+    h = emo.load_workload(g, emo.EMO_F_INTERVALS, group_of=group)
+    I, rows = 6, int(group.max()) + 1
+    breaks = np.arange(I, dtype=np.int64) * max(1, int(h.info.T_worst // I))
+    assert emo.emo_graph_flow(h, arrays=False)["lanes"] > 8
+    idle = W.idle_power(g.L)
+    for B, kernel in ((1000, 1), (4737, 2), (6000, 2)):
+        assert emo.emo_call_intervals(h, B, breaks) == kernel
+        F = W.interval_policies(3, rows, I, g.L, B, device="cuda")
+        out = []
+        for flags in (0, emo.EMO_F_FLOW_KERNEL):
+            T, E, Ei = (torch.zeros(B, dtype=d, device="cuda") for d in (torch.int64, torch.float64, torch.float64))
+            ws = torch.empty(emo.emo_workspace_bytes_intervals(h, B, I, True), dtype=torch.uint8, device="cuda")
+            emo.emo_eval_intervals(h, B, F, F.shape[2], I, breaks, torch.from_numpy(idle).cuda(), T, E, Ei, ws, flags=flags)
+            out.append([x.cpu().numpy() for x in (T, E, Ei)])
+        # (busy times are whole numbers; energies are 1 300 terms in another order)
+        assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][2], out[1][2]) and np.allclose(out[0][1], out[1][1], rtol=1e-12, atol=0)
+        some = np.unique(np.r_[0, 31, 32, B // 2, B - 1])
+        want = oracle_mod.intervals(g, group, breaks, np.ascontiguousarray(F.cpu().numpy()[:, :, some]), idle)
+        assert np.array_equal(out[0][0][some], want["makespan"]) and np.allclose(out[0][1][some], want["energy"], rtol=1e-12, atol=0)
     h.free()
