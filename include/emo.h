@@ -138,6 +138,10 @@ int emo_graph_info(const emo_graph *g, emo_info *info);
  * two passes); 2 the size emo_slack_batch_host needs.  The caller allocates, aligned as cudaMalloc aligns (16 bytes
  * suffice; a forward-only call that finds less does without the workspace); no call allocates device memory per
  * invocation.
+ * The size for forward-only calls covers every smaller batch.  It is kilobytes and the slice kernels' share, which is
+ * bounded (256 MB; 80 policies' worth on graphs of millions of nodes): larger calls run in tiles of policies.  With
+ * less, or with no workspace at all, a forward-only call takes smaller tiles or other kernels.  A slack call needs
+ * what this function gives for its own B; what larger batches need may be less.
  */
 int emo_workspace_bytes(const emo_graph *g, int64_t B, int need_slack, size_t *out);
 
@@ -146,7 +150,8 @@ int emo_workspace_bytes(const emo_graph *g, int64_t B, int need_slack, size_t *o
  * they choose the kernels, and the kernels differ in what they keep between the two passes) and a
  * level matrix that is (aligned = 1) or is not (aligned = 0) fetchable in 16-byte pieces: pointer
  * 16-byte aligned and ldb a multiple of 16.  emo_workspace_bytes assumes no flags and an aligned
- * matrix.  A workspace that is too small for what the call ends up running gives EMO_E_OOM.
+ * matrix.  A slack call whose workspace is too small for the slice kernels (where they would take it) goes to the
+ * others; one that is too small for those gives EMO_E_OOM.
  */
 int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint32_t flags, int aligned,
                             size_t *out);

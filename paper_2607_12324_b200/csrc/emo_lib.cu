@@ -1694,19 +1694,18 @@ int64_t slice_limit(const emo_graph *g, bool need_bwd, bool extra)
     return 65536 / ((int64_t)d.cols * d.cols) / (need_bwd ? 1 : 2);
 }
 
-// Whether a call takes the slice kernels, and with which blocks.  Measured (us): one block per policy where all are there at once, 400
-// nodes x 64 16.6 / 21.5, 1 013 x 64 23.7 / 26.3 in three kernels.  Else one policy per block (four slices) for up to four, and for wide
-// matrices, which fill a warp's lanes with one policy (12 839 nodes x 16, 40 columns 192 / 293); 16 policies instead of 8 where a
-// block's columns are the work, forward (250 000 x 256 440 / 603), or where three large blocks still fit an SM and there are plenty
-// (250 000 x 256 1 749 / 2 002; but 10 000 x 257 115 / 105, two blocks and a half).
-bool slice_allowed(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, bool extra, uint32_t flags, SlicePlan &pl)
+// Call flags that name other kernels.
+constexpr uint32_t kNotSlices = EMO_F_NO_STAGING | EMO_F_PAIR_KERNEL | EMO_F_LANE_KERNEL | EMO_F_FLOW_KERNEL | EMO_F_SPINE_KERNEL | EMO_F_TEST_STALL;
+
+// Blocks of a call on the slice kernels.  Measured (us): one block per policy where all are there at once, 400 nodes x 64 16.6 / 21.5,
+// 1 013 x 64 23.7 / 26.3 in three kernels.  Else one policy per block (four slices) for up to four, and for wide matrices, which fill
+// a warp's lanes with one policy (12 839 nodes x 16, 40 columns 192 / 293); 16 policies instead of 8 where a block's columns are the
+// work, forward (250 000 x 256 440 / 603), or where three large blocks still fit an SM and there are plenty (250 000 x 256 1 749 /
+// 2 002; but 10 000 x 257 115 / 105, two blocks and a half).
+bool slice_shape(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, uint32_t flags, SlicePlan &pl)
 {
     const DevSlice &d = g->dslice;
-    if (!d.ready) return false;
-    if (flags & (EMO_F_NO_STAGING | EMO_F_PAIR_KERNEL | EMO_F_LANE_KERNEL | EMO_F_FLOW_KERNEL | EMO_F_SPINE_KERNEL | EMO_F_TEST_STALL)) return false;
     const int64_t nb = B + (want_base ? 1 : 0);
-    if (nb == 0) return false;
-    if (!(flags & EMO_F_SLICE_KERNEL) && nb > slice_limit(g, need_bwd, extra)) return false;
     const bool one = slice_plan(g, B, want_base, need_bwd, 0, pl);
     // forward on two to four slices: one block per policy and SM, else the spine kernel's one launch (400 nodes x 1 025 14.2 against 18.8)
     if (!need_bwd && d.count > 1 && d.count <= 4 && !(flags & EMO_F_SLICE_KERNEL) && !(one && pl.whole >= 0 && nb <= g->sm_count)) return false;
@@ -1718,6 +1717,49 @@ bool slice_allowed(const emo_graph *g, int64_t B, bool want_base, bool need_bwd,
     return slice_plan(g, B, want_base, need_bwd, 1, pl);
 }
 
+// Whether a call takes the slice kernels, and with which blocks (a workspace for all policies at once provided).
+bool slice_allowed(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, bool extra, uint32_t flags, SlicePlan &pl)
+{
+    if (!g->dslice.ready || (flags & kNotSlices)) return false;
+    const int64_t nb = B + (want_base ? 1 : 0);
+    if (nb == 0) return false;
+    if (!(flags & EMO_F_SLICE_KERNEL) && nb > slice_limit(g, need_bwd, extra)) return false;
+    return slice_shape(g, B, want_base, need_bwd, flags, pl);
+}
+
+// ---- workspace of the slice kernels
+// Matrices and entering values of every slice take 0.5 MB a policy and direction on 250 000 nodes.  Forward calls need next to
+// nothing otherwise, so they would ask for 0.76 GB there with 1 399 policies: beyond kSliceWs a call runs in tiles of policies, one
+// after the other.  Measured (us, 250 000 nodes x 1 024, one tile / 512 / 256 / 128 / 64 a tile): forward 1 605 / 1 666 / 1 783 / 1 973 /
+// 2 406, slack 6 498 / 6 657 / 6 861 / 7 144 / 7 688 (slack calls have room for one tile: the other kernels' restore lists need more).
+constexpr size_t kSliceWs = (size_t)256 << 20;
+constexpr int64_t kSliceLeastTile = 64;          // fewer policies a tile (unless the call has no more) are left to the other kernels
+
+size_t slice_policy_bytes(const emo_graph *g, bool need_bwd)
+{
+    const DevSlice &d = g->dslice;
+    if (d.count <= 1) return 0;
+    const size_t size = (size_t)d.cols * d.cols * 4, groups = d.groups > 1 ? (size_t)d.groups : 0;
+    return (need_bwd ? 2 : 1) * (((size_t)d.count + groups) * size + (size_t)d.count * d.cols * 8) + ((size_t)d.count + std::max<size_t>(groups, 1)) * 8;
+}
+
+// ... of nb policies; no plan of as many needs more (blocks of up to 16 policies, eight arrays in pieces of 256 bytes).
+size_t slice_ws(const emo_graph *g, int64_t nb, bool need_bwd)
+{
+    return slice_policy_bytes(g, need_bwd) * round_up((size_t)nb, 16) + 8 * 256;
+}
+
+// What a call on B policies asks for; it suffices for every smaller call too.
+size_t slice_call_ws(const emo_graph *g, int64_t B, bool need_bwd, uint32_t flags)
+{
+    const DevSlice &d = g->dslice;
+    if (!d.ready || d.count <= 1 || (flags & kNotSlices)) return 0;
+    const int64_t nb = flags & EMO_F_SLICE_KERNEL ? B + 1 : std::min(B + 1, slice_limit(g, need_bwd, true));
+    SlicePlan pl;
+    if (nb <= 0 || !slice_plan(g, 1, false, need_bwd, 1, pl)) return 0;
+    return std::min(slice_ws(g, nb, need_bwd), std::max(kSliceWs, slice_ws(g, kSliceLeastTile + 16, need_bwd)));
+}
+
 // Bytes that the slice kernels may use of a caller's workspace, behind its head.  They move it 16 bytes at a time: none where it is not
 // aligned to that (forward calls do not touch it otherwise, so there it may lie anywhere).
 size_t slice_room(const void *ws, size_t ws_bytes, size_t head)
@@ -1725,23 +1767,38 @@ size_t slice_room(const void *ws, size_t ws_bytes, size_t head)
     return ws && aligned16(ws) && ws_bytes > head ? ws_bytes - head : 0;
 }
 
-int launch_slices(const emo_graph *g, SlicePlan &pl, const uint8_t *lvl, int64_t ldb, int64_t *ES, int64_t *LS, int64_t *slack, int64_t ldo, int64_t *makespan,
-                  double *energy, int64_t *slack_sum, int32_t *n_critical, int64_t *base_T, double *base_E, unsigned char *ws, cudaStream_t st)
+// What a call reads and writes.
+struct SliceCall {
+    const uint8_t *lvl;
+    int64_t ldb;
+    int64_t *ES, *LS, *slack;
+    int64_t ldo;
+    int64_t *makespan;
+    double *energy;
+    int64_t *slack_sum;
+    int32_t *n_critical;
+    int64_t *base_T;
+    double *base_E;
+};
+
+// One tile of a call: policies b0 and following.  first, last: of the call (its events).
+int launch_slices(const emo_graph *g, SlicePlan pl, const SliceCall &c, int64_t b0, bool first, bool last, unsigned char *ws, cudaStream_t st)
 {
     const SliceKernels &k = kSliceKernels[pl.shape];
+    auto from = [&](auto *x) { return x ? x + b0 : x; };
     for (SliceParams *p : {&pl.p, &pl.pv}) {
-        p->lvl = lvl;
-        p->ldb = ldb;
-        p->ES = ES;
-        p->LS = LS;
-        p->slack = slack;
-        p->ldo = ldo;
-        p->makespan = makespan;
-        p->energy = energy;
-        p->slack_sum = slack_sum;
-        p->n_critical = n_critical;
-        p->base_T = base_T;
-        p->base_E = base_E;
+        p->lvl = from(c.lvl);
+        p->ldb = c.ldb;
+        p->ES = from(c.ES);
+        p->LS = from(c.LS);
+        p->slack = from(c.slack);
+        p->ldo = c.ldo;
+        p->makespan = from(c.makespan);
+        p->energy = from(c.energy);
+        p->slack_sum = from(c.slack_sum);
+        p->n_critical = from(c.n_critical);
+        p->base_T = c.base_T;
+        p->base_E = c.base_E;
         for (int i = 0; i < p->dirs; ++i) {
             p->mat[i] = (int32_t *)(ws + (size_t)p->mat[i]);
             p->gmat[i] = (int32_t *)(ws + (size_t)p->gmat[i]);
@@ -1752,7 +1809,7 @@ int launch_slices(const emo_graph *g, SlicePlan &pl, const uint8_t *lvl, int64_t
     }
     const SliceParams &p = pl.p;
     const int slices = p.count > 1 ? kSliceS[pl.shape] : 1, blocks = (p.count + slices - 1) / slices * p.tiles;
-    cudaEvent_t ev0 = g_pass_events[0], ev1 = g_pass_events[1], ev2 = g_pass_events[2], ev3 = g_pass_events[3];
+    cudaEvent_t ev0 = first ? g_pass_events[0] : nullptr, ev1 = last ? g_pass_events[1] : nullptr, ev2 = last ? g_pass_events[2] : nullptr, ev3 = last ? g_pass_events[3] : nullptr;
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
     if (pl.whole >= 0) {
         const SliceWhole &w = kSliceWhole[pl.whole];
@@ -1784,6 +1841,29 @@ int launch_slices(const emo_graph *g, SlicePlan &pl, const uint8_t *lvl, int64_t
     }
     if (ev3) EMO_CUDA(cudaEventRecord(ev3, st));
     return EMO_OK;
+}
+
+// Runs a call on the slice kernels, in tiles of as many policies as the workspace holds; false where it does not take them.
+bool slice_call(const emo_graph *g, int64_t B, bool need_bwd, uint32_t flags, const SliceCall &c, void *ws, size_t ws_bytes, size_t head, cudaStream_t st, int &rc)
+{
+    const bool base = c.base_T || c.base_E;
+    SlicePlan pl, end;
+    if (!slice_allowed(g, B, base, need_bwd, c.ES || c.LS || c.slack_sum || c.n_critical, flags, pl)) return false;
+    const size_t room = slice_room(ws, ws_bytes, head);
+    unsigned char *const area = room ? (unsigned char *)ws + head : nullptr;
+    if (pl.ws <= room) {
+        rc = launch_slices(g, pl, c, 0, true, true, area, st);
+        return true;
+    }
+    // (the last tile has the all-max policy too)
+    int64_t tile = std::min<int64_t>(B, (int64_t)(room / std::max<size_t>(slice_policy_bytes(g, need_bwd), 1))) / 16 * 16 - 16;
+    while (tile >= kSliceLeastTile && slice_ws(g, tile + 1, need_bwd) > room) tile -= 16;
+    if (tile < kSliceLeastTile) return false;
+    const int64_t tiles = (B + tile - 1) / tile, rest = B - (tiles - 1) * tile;
+    if (!slice_shape(g, tile, false, need_bwd, flags, pl) || !slice_shape(g, rest, base, need_bwd, flags, end) || pl.ws > room || end.ws > room) return false;
+    rc = EMO_OK;
+    for (int64_t k = 0; k < tiles && rc == EMO_OK; ++k) rc = launch_slices(g, k + 1 < tiles ? pl : end, c, k * tile, k == 0, k + 1 == tiles, area, st);
+    return true;
 }
 
 int launch_validate(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb, int32_t *status, cudaStream_t st)
@@ -2615,9 +2695,8 @@ int emo_workspace_bytes_for(const emo_graph *g, int64_t B, int need_slack, uint3
 {
     if (!g || !out || B < 0) return EMO_E_INVALID_ARG;
     size_t bytes = pass_ws_bytes(g, B, need_slack, flags, aligned);
-    SlicePlan cp;
-    for (const emo_graph *e : {need_slack ? nullptr : joined_for(g, flags), g})
-        if (e && !g->host_only && !g->generic && slice_allowed(e, B, true, need_slack != 0, true, flags, cp)) bytes = std::max(bytes, kSmallWs + lvl_area(g) + cp.ws);
+    const emo_graph *const joined = need_slack ? nullptr : joined_for(g, flags);
+    bytes = std::max(bytes, kSmallWs + lvl_area(g) + slice_call_ws(joined ? joined : g, B, need_slack != 0, flags));
     if (need_slack == 2) bytes += 4 * round_up((size_t)B * 8, 256) + 256;
     *out = bytes;
     return EMO_OK;
@@ -2648,9 +2727,8 @@ int emo_eval_policies(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t
     const size_t head = kSmallWs + lvl_area(g);
     for (const emo_graph *e : {joined_for(g, flags), g}) {
         if (!e) continue;
-        SlicePlan cp;
-        if (slice_allowed(e, B, T0 || E0, false, false, flags, cp) && cp.ws <= slice_room(ws, ws_bytes, head))
-            return launch_slices(e, cp, lvl, ldb, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0, (unsigned char *)ws + head, st);
+        int rc = EMO_OK;
+        if (slice_call(e, B, false, flags, {lvl, ldb, nullptr, nullptr, nullptr, 0, makespan, energy, nullptr, nullptr, T0, E0}, ws, ws_bytes, head, st, rc)) return rc;
         SpinePlan fp;
         if (spine_allowed(e, B, lvl, ldb, 0, flags) && spine_plan(e, B, T0 || E0, false, false, fp))
             return launch_spine_fwd(e, fp, B, lvl, ldb, nullptr, makespan, energy, T0, E0, status, flags, st);
@@ -3112,10 +3190,9 @@ int emo_slack_batch(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t l
         return launch_generic(g, B, lvl, ldb, true, ES, LS, slack, ldo, makespan, energy, slack_sum, n_critical, T0, E0, ws, ws_bytes,
                               st);
     {
-        SlicePlan cp;
-        const size_t head = kSmallWs + lvl_area(g);
-        if (slice_allowed(g, B, T0 || E0, true, ES || LS || slack_sum || n_critical, flags, cp) && cp.ws <= slice_room(ws, ws_bytes, head))
-            return launch_slices(g, cp, lvl, ldb, ES, LS, slack, ldo, makespan, energy, slack_sum, n_critical, T0, E0, (unsigned char *)ws + head, st);
+        int rc = EMO_OK;
+        if (slice_call(g, B, true, flags, {lvl, ldb, ES, LS, slack, ldo, makespan, energy, slack_sum, n_critical, T0, E0}, ws, ws_bytes, kSmallWs + lvl_area(g), st, rc))
+            return rc;
     }
     if (spine_allowed(g, B, lvl, ldb, ldo, flags)) {
         SpinePlan fp;
@@ -3171,10 +3248,8 @@ int emo_slack(const emo_graph *g, const uint8_t *lvl_one, int64_t *ES, int64_t *
     cudaStream_t st = (cudaStream_t)stream;
     double *const e1 = energy ? energy : (double *)((char *)ws + 1024);
     {
-        SlicePlan cp;
-        const size_t head = kSmallWs + lvl_area(g);
-        if (slice_allowed(g, 1, false, true, true, 0, cp) && cp.ws <= slice_room(ws, ws_bytes, head))
-            return launch_slices(g, cp, lvl_one, 1, ES, LS, slack, 1, makespan, e1, nullptr, nullptr, nullptr, nullptr, (unsigned char *)ws + head, st);
+        int rc = EMO_OK;
+        if (slice_call(g, 1, true, 0, {lvl_one, 1, ES, LS, slack, 1, makespan, e1, nullptr, nullptr, nullptr, nullptr}, ws, ws_bytes, kSmallWs + lvl_area(g), st, rc)) return rc;
     }
     // re-pitch the level vector to [rows][16] so that the staged kernels can be used; the
     // per-node outputs are written at pitch 1 directly

@@ -85,3 +85,50 @@ def test_forward_calls_take_a_workspace_anywhere(torch_cuda, emo, oracle_mod):
         assert np.array_equal(T.cpu().numpy(), want["makespan"]) and np.allclose(E.cpu().numpy(), want["energy"], rtol=1e-12, atol=0), offset
         assert bool((buf == 0xEE).all()) == (offset % 16 != 0), offset
     h.free()
+
+
+def test_tiles_of_policies(torch_cuda, emo, oracle_mod):
+    """A workspace that does not hold all policies at once: tiles of at least 64, with remainders, the baseline in the last one; less goes to the
+    other kernels.  (A forward call touches its workspace on the slice kernels only.)"""
+    torch = torch_cuda
+    g, B = W.make_graph("cfg1-train", 0.4), 301
+    lv, lv_dev = levels(torch, g.n, g.L, B, 8)
+    want, base = oracle_mod.batch(g, lv, want_arrays=True), oracle_mod.batch(g, np.full((g.n, 1), g.L - 1, dtype=np.uint8))
+    h = emo.load_workload(g)
+    head = emo.emo_workspace_bytes(h, B, 0, emo.EMO_F_SPINE_KERNEL)
+    per = (emo.emo_workspace_bytes(h, 160, 0) - emo.emo_workspace_bytes(h, 80, 0)) / 80.0
+    assert emo.emo_call_slices(h, B, False) > 8 and per > 0
+    for policies, takes in ((40, False), (81, True), (100, True), (200, True), (320, True)):
+        ws = torch.full((head + int(per * policies) + 4096,), 0xEE, dtype=torch.uint8, device="cuda")
+        T, E, T0, E0 = (torch.full((k,), -1, dtype=d, device="cuda") for k, d in ((B + 1, torch.int64), (B + 1, torch.float64), (1, torch.int64), (1, torch.float64)))
+        emo.emo_eval_policies(h, B, lv_dev, lv_dev.stride(0), T, E, ws, T0=T0, E0=E0)
+        assert np.array_equal(T.cpu().numpy(), np.r_[want["makespan"], -1]) and np.allclose(E.cpu().numpy(), np.r_[want["energy"], -1.0], rtol=1e-12, atol=0), policies
+        assert int(T0) == base["makespan"][0] and np.isclose(float(E0), base["energy"][0], rtol=1e-12, atol=0)
+        assert bool((ws != 0xEE).any()) == takes, policies
+        if takes:
+            ws = torch.zeros(head + int(2.1 * per * policies) + 8192, dtype=torch.uint8, device="cuda")
+            X = torch.full((3, g.n, B + 1), -7, dtype=torch.int64, device="cuda")
+            ss, nc = torch.full((B,), -1, dtype=torch.int64, device="cuda"), torch.full((B,), -1, dtype=torch.int32, device="cuda")
+            emo.emo_slack_batch(h, B, lv_dev, lv_dev.stride(0), X[0], X[1], X[2], B + 1, T, E, ss, nc, ws, flags=emo.EMO_F_SLICE_KERNEL, T0=T0, E0=E0)
+            for k, x in zip(("ES", "LS", "slack"), X.cpu().numpy()):
+                assert np.array_equal(x[:, :B], want[k]) and (x[:, B:] == -7).all(), (k, policies)
+            assert np.array_equal(ss.cpu().numpy(), want["slack"].sum(0)) and np.array_equal(nc.cpu().numpy(), (want["slack"] == 0).sum(0)) and int(T0) == base["makespan"][0]
+    h.free()
+
+
+def test_workspace_of_forward_calls(torch_cuda, emo):
+    """One size for all batches up to the largest, bounded: 250 000 nodes, where all of 1 399 policies would take 0.76 GB."""
+    torch = torch_cuda
+    g, B = W.make_graph("cfg4-llm", 1.0), 700
+    h = emo.load_workload(g)
+    head = emo.emo_workspace_bytes(h, 1, 0, emo.EMO_F_SPINE_KERNEL)
+    sizes = [emo.emo_workspace_bytes(h, b, 0) for b in (0, 1, 5, 16, 100, 700, 1399, 1400, 1401, 5000, 65536)]
+    assert sizes == sorted(sizes) and sizes[-1] <= head + (1 << 28)
+    lv = torch.randint(0, g.L, (g.n, 704), dtype=torch.uint8, device="cuda")
+    out = []
+    for ws in (None, torch.empty(sizes[-1], dtype=torch.uint8, device="cuda")):
+        T, E = torch.zeros(B, dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.float64, device="cuda")
+        emo.emo_eval_policies(h, B, lv, 704, T, E, ws)
+        out.append((T, E))
+    assert torch.equal(out[0][0], out[1][0]) and torch.allclose(out[0][1], out[1][1], rtol=1e-11, atol=0)
+    h.free()
