@@ -18,6 +18,8 @@ constexpr int kWalkNodes = 96;                   // nodes per chunk
 constexpr int64_t kWalkMaxDur = 1 << 30;         // duration of a node, and of the nodes of an item together, below this: what is left of an interval
                                                  // is a signed 32-bit number
 
+constexpr size_t kWalkShared = 227 * 1024;       // shared memory of a block
+
 // item: word 0 nodes (bits 0..3) | flags | published slot << 16; word 1 two slots (16 bits each); word 2 fixed duration, or the nodes'
 // policy row; word 3 the first node's place in the chunk's tables
 constexpr uint32_t kWalkStart = 16u;             // the path begins: the later of two slots
@@ -35,7 +37,8 @@ struct Walk {
     double energy0 = 0.0;                        // of the nodes outside every policy
 };
 
-// Builds the walk program; ok stays false where it does not apply (a duration too long, too many slots).
+// Builds the walk program; ok stays false, and nothing is kept, where it does not apply (a duration too long, too many slots, chunks too long for
+// a block).
 void compile_walk(const HostGraph &g, const int64_t *lat, const double *energy, const GraphBounds &b, Walk &out);
 
 }  // namespace emo

@@ -36,6 +36,7 @@ void compile_walk(const HostGraph &g0, const int64_t *lat0, const double *energy
     struct Item {
         uint32_t flags = 0, fixed = 0, first = 0;
         int32_t nodes = 0, from[2] = {-1, -1}, publish = -1, row = -1;
+        uint32_t slot[2] = {0, 0}, publish_slot = 0;
     };
     struct Chunk {
         std::vector<Item> items;
@@ -136,27 +137,13 @@ void compile_walk(const HostGraph &g0, const int64_t *lat0, const double *energy
     std::priority_queue<int32_t, std::vector<int32_t>, std::greater<int32_t>> free_ids;
     std::vector<int32_t> slot((size_t)n, 0);
     int32_t slots = 1;
-    int Lp = 4;
-    while (Lp < L) Lp <<= 1;
-    out.Lp = Lp;
-    out.chunks = (int)chunks.size();
-    out.off_dur = (uint32_t)((1 + most_items + 1) * 16);
-    out.off_en = out.off_dur + (uint32_t)kWalkRows * (uint32_t)Lp * 4u;
-    out.chunk_bytes = out.off_en + (uint32_t)kWalkRows * (uint32_t)Lp * 8u;
-    out.blob.assign((size_t)out.chunks * out.chunk_bytes, 0);
     at = 0;
-    for (size_t k = 0; k < chunks.size(); ++k) {
-        unsigned char *const p = out.blob.data() + k * out.chunk_bytes;
-        uint32_t *w = reinterpret_cast<uint32_t *>(p);
-        w[0] = (uint32_t)chunks[k].items.size();
-        for (const Item &it : chunks[k].items) {
-            w += 4;
-            uint32_t s[2] = {0, 0};
+    for (Chunk &ch : chunks)
+        for (Item &it : ch.items) {
             for (int i = 0; i < 2; ++i)
-                if (it.from[i] >= 0) s[i] = (uint32_t)slot[it.from[i]];
+                if (it.from[i] >= 0) it.slot[i] = (uint32_t)slot[it.from[i]];
             for (int i = 0; i < 2; ++i)
                 if (it.from[i] >= 0 && last_read[it.from[i]] == at) free_ids.push(slot[it.from[i]]);
-            uint32_t pub = 0;
             if (it.publish >= 0) {
                 int32_t id;
                 if (!free_ids.empty()) {
@@ -166,13 +153,33 @@ void compile_walk(const HostGraph &g0, const int64_t *lat0, const double *energy
                     id = slots++;
                 }
                 slot[it.publish] = id;
-                pub = kWalkPub | (uint32_t)id << 16;
+                it.publish_slot = (uint32_t)id;
             }
-            w[0] = (uint32_t)it.nodes | it.flags | pub;
-            w[1] = s[0] | s[1] << 16;
+            ++at;
+        }
+    int Lp = 4;
+    while (Lp < L) Lp <<= 1;
+    // a block holds two chunks and a warp's slots, or no call takes the program: a node with thousands of operands makes its chunk long
+    // (and all are as long), more than 128 levels make the tables of a chunk 192 KB
+    const size_t off_dur = (1 + most_items + 1) * 16, off_en = off_dur + (size_t)kWalkRows * Lp * 4, bytes = off_en + (size_t)kWalkRows * Lp * 8;
+    if (slots > 0xFFFF || 2 * bytes + (size_t)slots * 256 > kWalkShared) return;
+    out.Lp = Lp;
+    out.slots = slots;
+    out.chunks = (int)chunks.size();
+    out.off_dur = (uint32_t)off_dur;
+    out.off_en = (uint32_t)off_en;
+    out.chunk_bytes = (uint32_t)bytes;
+    out.blob.assign((size_t)out.chunks * out.chunk_bytes, 0);
+    for (size_t k = 0; k < chunks.size(); ++k) {
+        unsigned char *const p = out.blob.data() + k * out.chunk_bytes;
+        uint32_t *w = reinterpret_cast<uint32_t *>(p);
+        w[0] = (uint32_t)chunks[k].items.size();
+        for (const Item &it : chunks[k].items) {
+            w += 4;
+            w[0] = (uint32_t)it.nodes | it.flags | (it.publish >= 0 ? kWalkPub | it.publish_slot << 16 : 0u);
+            w[1] = it.slot[0] | it.slot[1] << 16;
             w[2] = it.nodes ? (uint32_t)it.row : it.fixed;
             w[3] = it.first;
-            ++at;
         }
         for (size_t r = 0; r < chunks[k].rows.size(); ++r) {
             const int32_t v = chunks[k].rows[r];
@@ -184,8 +191,6 @@ void compile_walk(const HostGraph &g0, const int64_t *lat0, const double *energy
             }
         }
     }
-    if (slots > 0xFFFF) return;
-    out.slots = slots;
     for (int32_t v = 0; v < n; ++v)
         if (g.group[v] < 0) out.energy0 += c.energy[(size_t)v * L];
     out.ok = true;

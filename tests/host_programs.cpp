@@ -423,7 +423,7 @@ int program_check(int kind, int32_t n, const int64_t *rp, const int32_t *col, co
     }
 }
 
-// Compiles only (bounds included).
+// Compiles only (bounds included).  Walk: -1 where a program that is refused is kept all the same.
 int program_compile(int kind, int32_t n, const int64_t *rp, const int32_t *col, const int32_t *group, int32_t rows, int32_t L, const int64_t *lat, const double *energy)
 {
     const Input in = take(n, rp, col, group, rows, L, lat, energy);
@@ -439,7 +439,7 @@ int program_compile(int kind, int32_t n, const int64_t *rp, const int32_t *col, 
     }
     Walk w;
     compile_walk(in.g, lat, energy, in.b, w);
-    return w.ok;
+    return w.ok ? 1 : (w.blob.empty() ? 0 : -1);
 }
 
 }  // extern "C"

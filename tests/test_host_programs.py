@@ -73,7 +73,7 @@ def test_slices(programs):
     assert kinds["one"] > 20 and kinds["several"] > 20 and kinds["groups"] == 4
 
 
-def streams(seed, n, k, dur=1000):
+def streams(seed, n, k, dur=1000, L=4):
     """k streams in program order with a cross edge now and then."""
     rs = np.random.RandomState(seed)
     last, edges = [-1] * k, []
@@ -83,7 +83,7 @@ def streams(seed, n, k, dur=1000):
             if u >= 0:
                 edges.append((u, v))
         last[s] = v
-    return W.tiny_graph(n, edges, rs.randint(0, dur, size=(n, 4)).astype(np.int64), rs.rand(n, 4), name=f"streams{seed}"), None
+    return W.tiny_graph(n, edges, rs.randint(0, dur, size=(n, L)).astype(np.int64), rs.rand(n, L), name=f"streams{seed}"), None
 
 
 def test_slices_of_long_paths(programs):
@@ -115,22 +115,37 @@ def test_workloads(programs, name, scale):
     assert check(programs, SLICES, g) and check(programs, CONTRACT, g) and check(programs, WALK, g, W.device_of(g))
 
 
-@pytest.mark.parametrize("ends", [False, True])
-def test_slices_of_a_wide_join(programs, ends):
-    """A chain whose every node one last node waits for (a host sync), and the same with an end of its own behind every node: the slices'
-    compiler looks at every edge a bounded number of times.  (Every operand looked up among its reader's, or a reader's operands counted
-    again with each of them, is 4e9 steps here, more than two seconds.)"""
-    n = 90_000
+def wide_join(n, L, ends=False):
+    """Arguments of program_compile: a chain whose every node one last node waits for, with an end behind every node or not."""
     chain = n // 2 if ends else n - 1
     edges = np.r_[np.c_[np.arange(chain - 1), np.arange(1, chain)], np.c_[np.arange(chain), np.full(chain, n - 1)]]
     if ends:
         edges = np.r_[edges, np.c_[np.arange(chain - 1), np.arange(chain, n - 1)]]
     edges = edges[np.lexsort((edges[:, 0], edges[:, 1]))]
     rp = np.r_[0, np.cumsum(np.bincount(edges[:, 1], minlength=n))].astype(np.int64)
-    col, group = np.ascontiguousarray(edges[:, 0], np.int32), np.full(n, -1, np.int32)
-    lat, energy = np.full((n, 1), 10, np.int64), np.ones((n, 1))
-    args = [a.ctypes.data_as(ctypes.c_void_p) for a in (rp, col, group)] + [ctypes.c_int32(0), ctypes.c_int32(1)] + [a.ctypes.data_as(ctypes.c_void_p) for a in (lat, energy)]
+    # (with several levels every operand can decide the last node's start: short nodes at one level, long ones at another)
+    lat = np.repeat([[10 if L == 1 else 1000 * n] + [10] * (L - 1)], n, axis=0).astype(np.int64)
+    lat[n - 1] = 10
+    keep = [rp, np.ascontiguousarray(edges[:, 0], np.int32), np.arange(n, dtype=np.int32) % 2 if L > 1 else np.full(n, -1, np.int32), lat, np.ones((n, L))]
+    a = [x.ctypes.data_as(ctypes.c_void_p) for x in keep]
+    return keep, [ctypes.c_int32(n), a[0], a[1], a[2], ctypes.c_int32(2 if L > 1 else 0), ctypes.c_int32(L), a[3], a[4]]
+
+
+@pytest.mark.parametrize("ends", [False, True])
+def test_slices_of_a_wide_join(programs, ends):
+    """A chain whose every node one last node waits for (a host sync), and the same with an end of its own behind every node: the slices'
+    compiler looks at every edge a bounded number of times.  (Every operand looked up among its reader's, or a reader's operands counted
+    again with each of them, is 4e9 steps here, more than two seconds.)"""
+    keep, args = wide_join(180_000 if ends else 90_000, 1, ends)
     t = time.process_time()
-    sliced = programs.program_compile(SLICES, ctypes.c_int32(n), *args)
+    sliced = programs.program_compile(SLICES, *args)
     t = time.process_time() - t
     assert (ends or sliced == 1) and t < 1.0, t      # (with the ends every chain node is waited for across every cut: left to others)
+
+
+@pytest.mark.parametrize("n, L", [(20_000, 4), (160_000, 4), (20_000, 200)])
+def test_walk_programs_that_no_block_can_hold(programs, n, L):
+    """A node with tens of thousands of operands, and more than 128 levels: refused, and nothing of the program is kept (0.9 GB for 160 000
+    nodes, 61 MB for 200 levels)."""
+    keep, args = wide_join(n, L) if L == 4 else arguments(streams(3, n, 2, L=L)[0], np.zeros(n, np.int32))
+    assert programs.program_compile(WALK, *args) == 0
