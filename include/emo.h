@@ -450,8 +450,9 @@ int emo_slack_batch_prefetched(const emo_graph *g, int64_t B, int bits, const ui
 int emo_set_pass_events(void *fwd_start, void *fwd_stop, void *bwd_start, void *bwd_stop);
 
 /*
- * emo_call_path - which pass kernels emo_eval_policies (need_slack = 0) or emo_slack_batch (need_slack = 1)
- * would run for these arguments, where the slice kernels do not take the call (emo_call_slices): 4 = the spine kernels with one policy per worker thread, 5 = the
+ * emo_call_path - which pass kernels emo_eval_policies (need_slack = 0; on the contracted graph where the handle has
+ * one, emo_graph_contracted) or emo_slack_batch (need_slack = 1) would run for these arguments where the slice kernels
+ * do not take the call (emo_call_slices): 4 = the spine kernels with one policy per worker thread, 5 = the
  * spine kernels with several (calls without ES, LS and the sums), 2 = the 32-bit lane-stream kernels,
  * 1 = the staged 64-bit kernels,
  * 0 = the plain-load 64-bit kernels, 3 = the generic kernels (a graph beyond the on-chip schedules' limits, or
@@ -460,6 +461,12 @@ int emo_set_pass_events(void *fwd_start, void *fwd_stop, void *bwd_start, void *
  */
 int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb, int64_t ldo,
                   int need_slack, uint32_t flags);
+
+/*
+ * emo_graph_contracted - nodes of the contracted graph that calls without outputs per node evaluate (nodes that only
+ * ever follow one other node of the same policy row are one with it); 0 where the graph itself is evaluated.
+ */
+int emo_graph_contracted(const emo_graph *g, int32_t *nodes);
 
 /*
  * emo_call_slices - whether a call (as for emo_call_path, with a baseline column) is taken by the slice kernels: the number of

@@ -1912,9 +1912,9 @@ int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
     if (!g || B < 0) return EMO_E_INVALID_ARG;
     if (g->host_only) return EMO_E_CUDA;
     if (g->generic) return 3;
-    if (spine_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
+    for (const emo_graph *e : {need_slack ? nullptr : joined_for(g, flags), g}) {
         SpinePlan sp;
-        if (spine_plan(g, B, true, need_slack != 0, false, sp)) return sp.vw == 1 ? 4 : 5;
+        if (e && spine_allowed(e, B, lvl, ldb, need_slack ? ldo : 0, flags) && spine_plan(e, B, true, need_slack != 0, false, sp)) return sp.vw == 1 ? 4 : 5;
     }
     if (flow_allowed(g, B, lvl, ldb, need_slack ? ldo : 0, flags)) {
         FlowPlan fp;
@@ -1925,6 +1925,13 @@ int emo_call_path(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
     int rc = make_plan(g, B, true, need_slack != 0, lvl, ldb, ld_ws, ldo, flags, pl);
     if (rc) return rc;
     return pl.staged ? 1 : 0;
+}
+
+int emo_graph_contracted(const emo_graph *g, int32_t *nodes)
+{
+    if (!g || !nodes) return EMO_E_INVALID_ARG;
+    *nodes = g->joined ? g->joined->h.n : 0;
+    return EMO_OK;
 }
 
 int emo_call_slices(const emo_graph *g, int64_t B, int need_slack, uint32_t flags)

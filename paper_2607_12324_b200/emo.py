@@ -35,7 +35,7 @@ EXPORTS = [
     "emo_strerror", "emo_graph_load", "emo_graph_free", "emo_graph_info", "emo_workspace_bytes",
     "emo_eval_policies", "emo_slack_batch", "emo_slack", "emo_baseline", "emo_target_from_delta",
     "emo_select", "emo_transpose_policies", "emo_slack_batch_host", "emo_graph_program",
-    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_graph_spine_plan", "emo_graph_spine_layout", "emo_set_wait_limit", "emo_call_path", "emo_call_slices", "emo_call_intervals", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
+    "emo_set_pass_events", "emo_select_static", "emo_graph_flow", "emo_graph_spine", "emo_graph_spine_view", "emo_graph_spine_plan", "emo_graph_spine_layout", "emo_set_wait_limit", "emo_call_path", "emo_call_slices", "emo_call_intervals", "emo_graph_contracted", "emo_set_flow_counters", "emo_workspace_bytes_for", "emo_measure_int_issue", "emo_measure_warp_costs", "emo_eval_intervals", "emo_workspace_bytes_intervals", "emo_search_dp", "emo_workspace_bytes_search", "emo_pack_greedy", "emo_pack_tables", "emo_pack_model", "emo_pack_classes", "emo_pack_levels", "emo_unpack_levels", "emo_slack_batch_host_packed", "emo_levels_prefetch", "emo_slack_batch_prefetched",
 ]
 
 
@@ -139,6 +139,7 @@ def lib():
         L.emo_slack_batch_prefetched.argtypes = [p, i64, ctypes.c_int, p, i64, p, p, i64, p, i64, i64, p, p, p, p, p, p, sz, u32, p]
         L.emo_call_path.argtypes = [p, i64, p, i64, i64, ctypes.c_int, u32]
         L.emo_call_slices.argtypes = [p, i64, ctypes.c_int, u32]
+        L.emo_graph_contracted.argtypes = [p, p]
         L.emo_call_intervals.argtypes = [p, i64, i32, p, u32]
         L.emo_select_static.argtypes = [i64, p, p, i64, p, i64, p, p, p, p]
         for name in EXPORTS:
@@ -451,6 +452,13 @@ def emo_call_path(g: Graph, B, lvl, ldb, ldo, need_slack: bool, flags: int = 0) 
     if rc < 0:
         raise EmoError(rc, "emo_call_path")
     return rc
+
+
+def emo_graph_contracted(g: Graph) -> int:
+    """Nodes of the contracted graph that calls without outputs per node evaluate, 0 without one."""
+    out = ctypes.c_int32()
+    _check(lib().emo_graph_contracted(g.handle, ctypes.byref(out)), "emo_graph_contracted")
+    return int(out.value)
 
 
 def emo_call_slices(g: Graph, B, need_slack: bool, flags: int = 0) -> int:

@@ -46,6 +46,7 @@ def test_random_chains(torch_cuda, emo, oracle_mod, seed, B):
     lv = np.random.RandomState(seed).randint(0, g.L, size=(rows, (B + 15) // 16 * 16)).astype(np.uint8)
     lv_dev = torch.from_numpy(lv).cuda()
     h = emo.load_workload(g, group_of=group)
+    assert 0 < emo.emo_graph_contracted(h) <= g.n * 3 // 5
     want = oracle_mod.batch(g, lv[:, :B].copy(), group_of=group)
     base = oracle_mod.batch(g, np.full((rows, 1), g.L - 1, np.uint8), group_of=group)
     for flags in (0, emo.EMO_F_SLICE_KERNEL, emo.EMO_F_NO_STAGING):
@@ -68,6 +69,7 @@ def test_workloads(torch_cuda, emo, oracle_mod, name, scale, B):
     for group, rows in ((None, g.n), (packs, n_packs)):
         lv = torch.randint(0, g.L, (rows, (B + 15) // 16 * 16), dtype=torch.uint8, device="cuda")
         h = emo.load_workload(g, group_of=group)
+        assert (emo.emo_graph_contracted(h) > 0) == (g.n >= 2000 and (group is not None or name == "cfg3-8dev"))
         T, E, _, _ = evaluate(torch, emo, h, lv, B)
         T2, E2, _, _ = evaluate(torch, emo, h, lv, B, emo.EMO_F_FLOW_KERNEL)
         assert np.array_equal(T, T2) and np.allclose(E, E2, rtol=1e-12, atol=0)
