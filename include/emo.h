@@ -445,7 +445,9 @@ int emo_slack_batch_prefetched(const emo_graph *g, int64_t B, int bits, const ui
  * emo_set_pass_events - measurement hook (no counterpart in the method): four cudaEvent_t handles
  * (as void*, any may be NULL) that later emo_slack_batch / emo_eval_policies / emo_baseline calls
  * record on their stream immediately before and after the forward pass kernel and before and after
- * the backward pass kernel.  Pass four NULLs to switch it off.  Process-wide, not thread-safe.
+ * the backward pass kernel.  The slice kernels run both passes side by side: there the forward events enclose them and
+ * the backward events the kernel that writes the per-node outputs, or nothing where one kernel does all.
+ * Forward-only calls record the first two.  Pass four NULLs to switch it off.  Process-wide, not thread-safe.
  */
 int emo_set_pass_events(void *fwd_start, void *fwd_stop, void *bwd_start, void *bwd_stop);
 

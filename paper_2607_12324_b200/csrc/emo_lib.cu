@@ -1809,7 +1809,9 @@ int launch_slices(const emo_graph *g, SlicePlan pl, const SliceCall &c, int64_t 
     }
     const SliceParams &p = pl.p;
     const int slices = p.count > 1 ? kSliceS[pl.shape] : 1, blocks = (p.count + slices - 1) / slices * p.tiles;
-    cudaEvent_t ev0 = first ? g_pass_events[0] : nullptr, ev1 = last ? g_pass_events[1] : nullptr, ev2 = last ? g_pass_events[2] : nullptr, ev3 = last ? g_pass_events[3] : nullptr;
+    // both passes run side by side: the backward events enclose the kernel that writes the outputs where it is one of its own
+    const bool back = last && pl.p.dirs > 1;
+    cudaEvent_t ev0 = first ? g_pass_events[0] : nullptr, ev1 = last ? g_pass_events[1] : nullptr, ev2 = back ? g_pass_events[2] : nullptr, ev3 = back ? g_pass_events[3] : nullptr;
     if (ev0) EMO_CUDA(cudaEventRecord(ev0, st));
     if (pl.whole >= 0) {
         const SliceWhole &w = kSliceWhole[pl.whole];
@@ -1832,14 +1834,16 @@ int launch_slices(const emo_graph *g, SlicePlan pl, const SliceCall &c, int64_t 
         if (flow_optin(ch.scan, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
         EMO_CUDA(launch_ahead_grid(ch.scan, grid, ch.threads, pl.smem_s, st, p));
     }
-    if (ev1) EMO_CUDA(cudaEventRecord(ev1, st));
-    if (ev2) EMO_CUDA(cudaEventRecord(ev2, st));
+    if (p.count > 1)
+        for (cudaEvent_t ev : {ev1, ev2})
+            if (ev) EMO_CUDA(cudaEventRecord(ev, st));
     if (p.count == 1 || p.dirs > 1) {
         void (*values)(SliceParams) = p.count == 1 ? k.single : k.values;
         if (flow_optin(values, g) != EMO_OK) { (void)cudaGetLastError(); return EMO_E_CUDA; }
         EMO_CUDA(launch_ahead(values, blocks, k.threads, pl.smem_v, st, pl.pv));
     }
-    if (ev3) EMO_CUDA(cudaEventRecord(ev3, st));
+    for (cudaEvent_t ev : {p.count == 1 ? ev1 : nullptr, p.count == 1 ? ev2 : nullptr, ev3})
+        if (ev) EMO_CUDA(cudaEventRecord(ev, st));
     return EMO_OK;
 }
 

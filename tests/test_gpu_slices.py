@@ -132,3 +132,33 @@ def test_workspace_of_forward_calls(torch_cuda, emo):
         out.append((T, E))
     assert torch.equal(out[0][0], out[1][0]) and torch.allclose(out[0][1], out[1][1], rtol=1e-11, atol=0)
     h.free()
+
+
+@pytest.mark.parametrize("name, scale, B", [("cfg2-packed", 0.2, 40), ("cfg0-tiny", 1.0, 40), ("cfg1-train", 0.3, 40)])
+def test_pass_events(torch_cuda, emo, name, scale, B):
+    """The forward events enclose the kernels of one slice, of a block per policy, of many slices; a forward call leaves the backward ones."""
+    torch = torch_cuda
+    g = W.make_graph(name, scale)
+    h = emo.load_workload(g)
+    assert emo.emo_call_slices(h, B, True) > 0
+    lv, lv_dev = levels(torch, g.n, g.L, B, 9)
+    ws = torch.empty(emo.emo_workspace_bytes(h, B, 1), dtype=torch.uint8, device="cuda")
+    X, T, E = torch.zeros((g.n, B), dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.float64, device="cuda")
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(5)]
+    for e in ev:
+        e.record()
+    busy = torch.zeros(1 << 28, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    emo.emo_set_pass_events(*ev[:4])
+    try:
+        emo.emo_slack_batch(h, B, lv_dev, lv_dev.stride(0), None, None, X, B, T, E, None, None, ws)
+        torch.cuda.synchronize()
+        forward, between, backward = (a.elapsed_time(b) for a, b in zip(ev, ev[1:4]))
+        assert forward > 0.004 and between >= 0 and backward >= 0      # (no kernel of these takes less than 5 us)
+        busy.fill_(1)
+        emo.emo_eval_policies(h, B, lv_dev, lv_dev.stride(0), T, E, ws)
+        torch.cuda.synchronize()
+        assert ev[0].elapsed_time(ev[1]) > 0.004 and ev[3].elapsed_time(ev[0]) > 0
+    finally:
+        emo.emo_set_pass_events(None, None, None, None)
+    h.free()
