@@ -2293,11 +2293,16 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
     } else {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return EMO_E_CUDA; }
-        cudaDeviceProp prop;
-        if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { (void)cudaGetLastError(); return EMO_E_CUDA; }
+        // (two attributes; all of a device's properties take 3 to 10 ms, more than everything else for a small graph)
+        int sms = 0, shared = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&shared, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return EMO_E_CUDA;
+        }
         g->device = dev;
-        g->sm_count = prop.multiProcessorCount;
-        g->smem_optin = prop.sharedMemPerBlockOptin;
+        g->sm_count = sms;
+        g->smem_optin = (size_t)shared;
         int rc = EMO_OK;
         try {
         if (g->generic) {
