@@ -1685,12 +1685,18 @@ bool slice_plan(const emo_graph *g, int64_t B, bool want_base, bool need_bwd, in
 //   all outputs 10 000 x 1 501 532 / 689; 25 000 x 1 025 712 / 911, x 1 501 1 013 / 911
 //   forward     10 000 x 1 025 98 / 263; 25 000 x 1 501 250 / 249; 400 x 1 501 16 / 14
 //   one slice   213 x 4 097 20.7 / 23.3 (forward 12.0 / 12.9, both the call)
-//   40 columns (12 839 nodes, 18 lanes): slack x 17 192 / 447, x 65 438 / 447; forward x 17 109 / 123, x 65 207 / 123
+//   12 columns  10 000 x 769 slack 209 / 290, all outputs 229 / 361, forward 84 / 117, x 1 025 271 / 291, 293 / 362, 105 / 118; 50 000 x 769 961 / 1 380
+//   16 columns  10 000 x 513 slack 201 / 283, all outputs 218 / 362, forward 84 / 102, x 769 286 / 282, 303 / 362, 113 / 103
+//   20 columns  50 000 x 65 slack 500 / 1 355, forward 318 / 476, x 129 793 / 1 356, 540 / 476; 12 014 x 129 slack 293 / 477
+//   36 columns  24 014 x 33 slack 423 / 793, x 65 616 / 791
+//   40 columns  12 839 (18 lanes): slack x 17 192 / 447, x 65 438 / 447; forward x 17 109 / 123, x 65 207 / 123
+// (Up to 16 columns slices are chained in groups; wider ones one by one, and a policy's matrices go with the columns' square.)
 int64_t slice_limit(const emo_graph *g, bool need_bwd, bool extra)
 {
     const DevSlice &d = g->dslice;
     if (d.count == 1) return 4352;
     if (d.cols <= 8) return need_bwd ? (extra ? 1300 : 1100) : 1400;
+    if (d.cols <= 16) return d.cols <= 12 ? 900 : 600;
     return 65536 / ((int64_t)d.cols * d.cols) / (need_bwd ? 1 : 2);
 }
 

@@ -162,3 +162,23 @@ def test_pass_events(torch_cuda, emo, name, scale, B):
     finally:
         emo.emo_set_pass_events(None, None, None, None)
     h.free()
+
+
+@pytest.mark.parametrize("streams, limit", [(8, 900), (12, 600)])
+def test_matrices_of_12_and_16_columns(torch_cuda, emo, oracle_mod, streams, limit):
+    """On both sides of the rule's line, every output."""
+    from tests.test_host_programs import streams as graph
+    torch = torch_cuda
+    g, _ = graph(1, 2500, streams)
+    h = emo.load_workload(g)
+    for B in (limit - 1, limit):
+        assert (emo.emo_call_slices(h, B, True) > 0) == (emo.emo_call_slices(h, B, False) > 0) == (B < limit)
+        lv, lv_dev = levels(torch, g.n, g.L, B, 10)
+        want = oracle_mod.batch(g, lv, want_arrays=True, threads=os.cpu_count() or 1)
+        r = gpu_slack_batch(torch, emo, h, lv_dev, B, g.n, ldo=B + 1, base=True)
+        assert_matches(r, want, B)
+        T, E = torch.zeros(B, dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.float64, device="cuda")
+        ws = torch.empty(emo.emo_workspace_bytes(h, B, 0), dtype=torch.uint8, device="cuda")
+        emo.emo_eval_policies(h, B, lv_dev, lv_dev.stride(0), T, E, ws)
+        assert np.array_equal(T.cpu().numpy(), want["makespan"]) and np.allclose(E.cpu().numpy(), want["energy"], rtol=1e-12, atol=0)
+    h.free()
