@@ -66,3 +66,38 @@ def test_levels_rewritten_between_calls(torch_cuda, emo, oracle_mod, late_copy, 
             assert np.array_equal(got.cpu().numpy(), want[k if i < 3 else 1 - k][("ES", "LS", "slack")[i % 3]][:, 0])
         assert int(T1.item()) == want[1 - k]["makespan"][0]
     h.free()
+
+
+@pytest.mark.parametrize("name,scale,B", [("cfg2-packed", 0.2, 40), ("cfg0-tiny", 1.0, 64), ("cfg1-train", 0.3, 200), ("cfg1-train", 0.6, 1000)])
+def test_selection_behind_rewritten_levels(torch_cuda, emo, oracle_mod, late_copy, name, scale, B):  # noqa: F811
+    """Slice kernels of one slice, of a block per policy, of chained slices and of groups of them, then the one-block selection under the
+    baseline's budget, levels rewritten before every call: each sees what its predecessor wrote."""
+    torch = torch_cuda
+    g = W.make_graph(name, scale)
+    ldb = (B + 15) // 16 * 16
+    rs = np.random.RandomState(B)
+    host = [rs.randint(0, g.L, size=(g.n, ldb)).astype(np.uint8) for _ in range(2)]
+    for x in host:
+        x[:, 3::4] = g.L - 1 - (x[:, 3::4] == 0)      # (policies near the default one, inside the budget)
+    want = [oracle_mod.batch(g, x, B=B, threads=os.cpu_count() or 1) for x in host]
+    T0 = int(oracle_mod.batch(g, np.full((g.n, 1), g.L - 1, np.uint8))["makespan"][0])
+    pick = [oracle_mod.select(r["makespan"], r["energy"], oracle_mod.target_from_delta(T0, 50_000)) for r in want]
+    assert pick[0] != pick[1] and min(pick) >= 0
+    src = [torch.as_tensor(x, device="cuda") for x in host]
+    lvl = torch.zeros_like(src[0])
+    h = emo.load_workload(g)
+    assert emo.emo_call_slices(h, B, True) > 0
+    ws = torch.empty(emo.emo_workspace_bytes(h, B, 1), dtype=torch.uint8, device="cuda")
+    X = torch.zeros((g.n, B), dtype=torch.int64, device="cuda")
+    T, E, base, base_E = (torch.zeros(k, dtype=d, device="cuda") for k, d in ((B, torch.int64), (B, torch.float64), (1, torch.int64), (1, torch.float64)))
+    got = torch.full((12,), -7, dtype=torch.int64, device="cuda")
+    for turn in range(12):
+        late_copy(lvl, src[turn // 2 % 2])
+        if turn % 2:
+            emo.emo_eval_policies(h, B, lvl, ldb, T, E, ws, T0=base, E0=base_E)
+        else:
+            emo.emo_slack_batch(h, B, lvl, ldb, None, None, X, B, T, E, None, None, ws, T0=base, E0=base_E)
+        emo.emo_select(B, T, E, 0, got[turn:turn + 1], None, None, ws=ws, target_dev=base, delta_ppm=50_000)
+    torch.cuda.synchronize()
+    assert got.cpu().tolist() == [pick[turn // 2 % 2] for turn in range(12)]
+    h.free()

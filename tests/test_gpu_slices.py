@@ -182,3 +182,51 @@ def test_matrices_of_12_and_16_columns(torch_cuda, emo, oracle_mod, streams, lim
         emo.emo_eval_policies(h, B, lv_dev, lv_dev.stride(0), T, E, ws)
         assert np.array_equal(T.cpu().numpy(), want["makespan"]) and np.allclose(E.cpu().numpy(), want["energy"], rtol=1e-12, atol=0)
     h.free()
+
+
+def test_sixteen_policies_a_block(torch_cuda, emo, oracle_mod):
+    """Slack calls with plenty of blocks (nine and more per SM) of 16 policies each, the last one partly filled; every output."""
+    torch = torch_cuda
+    g, B = W.make_graph("cfg1-train", 1.0), 397
+    h = emo.load_workload(g)
+    assert emo.emo_call_slices(h, B, True) * ((B + 1 + 15) // 16) >= 9 * torch.cuda.get_device_properties(0).multi_processor_count
+    lv, lv_dev = levels(torch, g.n, g.L, B, 11)
+    want = oracle_mod.batch(g, lv, want_arrays=True, threads=os.cpu_count() or 1)
+    r = gpu_slack_batch(torch, emo, h, lv_dev, B, g.n, ldo=B + 1, base=True)
+    assert_matches(r, want, B)
+    for k in ("ES", "LS", "slack"):
+        assert (r[k][:, B:] == -7).all(), "padding columns of the outputs were written"
+    h.free()
+
+
+def test_long_paths(torch_cuda, emo, oracle_mod):
+    """Slices of up to 2^30 ns: groups of fewer of them, so that their products stay 32-bit; times beyond 2^34."""
+    from tests.test_host_programs import streams as graph
+    torch = torch_cuda
+    g, _ = graph(5, 7000, 3, dur=30_000_000)
+    B = 21
+    lv, lv_dev = levels(torch, g.n, g.L, B, 12)
+    want = oracle_mod.batch(g, lv, want_arrays=True, threads=os.cpu_count() or 1)
+    assert int(want["makespan"].max()) > 1 << 34
+    h = emo.load_workload(g)
+    assert emo.emo_call_slices(h, B, True) > 32
+    assert_matches(gpu_slack_batch(torch, emo, h, lv_dev, B, g.n, base=True), want, B)
+    h.free()
+
+
+def test_slack_in_the_other_kernels_workspace(torch_cuda, emo, oracle_mod):
+    """Wide matrices take more workspace than the kernels beside them: with what those need the call goes to them."""
+    torch = torch_cuda
+    g, B = W.make_graph("cfg3-8dev", 0.05), 16
+    lv, lv_dev = levels(torch, g.n, g.L, B, 13)
+    want = oracle_mod.batch(g, lv, want_arrays=True, threads=os.cpu_count() or 1)
+    h = emo.load_workload(g)
+    small = emo.emo_workspace_bytes(h, B, 1, emo.EMO_F_LANE_KERNEL)
+    assert emo.emo_call_slices(h, B, True) > 0 and small < emo.emo_workspace_bytes(h, B, 1)
+    X, T, E = torch.zeros((g.n, B), dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.int64, device="cuda"), torch.zeros(B, dtype=torch.float64, device="cuda")
+    for size in (max(small, emo.emo_workspace_bytes(h, B, 1, emo.EMO_F_SPINE_KERNEL)), emo.emo_workspace_bytes(h, B, 1)):
+        ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+        X.zero_()
+        emo.emo_slack_batch(h, B, lv_dev, lv_dev.stride(0), None, None, X, B, T, E, None, None, ws)
+        assert np.array_equal(X.cpu().numpy(), want["slack"]) and np.array_equal(T.cpu().numpy(), want["makespan"]), size
+    h.free()
