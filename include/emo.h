@@ -67,10 +67,11 @@ extern "C" {
 #define EMO_F_LANE_KERNEL 0x8u     /* staged pass kernel with one policy per thread (the default otherwise) */
 #define EMO_F_FLOW_KERNEL 0x10u    /* the 32-bit lane-stream kernels (the default for n * B >= 2^31, or more than three policy groups of
                                     * 32 per SM on a graph of at most eight lanes, where there is no spine program) */
-#define EMO_F_SPINE_KERNEL 0x20u   /* the spine kernels (the default wherever there is a spine program, but on graphs of more than eight lanes
-                                    * without a program of longer stages only from two policy groups of 32 per SM on) */
+#define EMO_F_SPINE_KERNEL 0x20u   /* the spine kernels (the default for more policies than the slice kernels take wherever there is a spine
+                                    * program, but on graphs of more than eight lanes without a program of longer stages only from two
+                                    * policy groups of 32 per SM on) */
 #define EMO_F_SLICE_KERNEL 0x40u   /* the slice kernels, whatever the number of policies (the default for about a thousand and fewer, fewer
-                                      still on graphs with many streams: emo_call_slices) */
+                                    * still on graphs with many streams: emo_call_slices) */
 #define EMO_F_TEST_STALL 0x100u    /* test hook of the 32-bit kernels: the producer warps stop half way, so that the
                                       consumers' bounded waits run out and EMO_E_TIMEOUT is reported */
 

@@ -2820,11 +2820,11 @@ static bool walk_plan(const emo_graph *g, int64_t B, int rows, int32_t I, int64_
     return false;
 }
 
-// Whether the walk kernel is the faster one.  Measured (us, it / the lane-stream kernel): up to three lanes, 500 nodes x 4 096 policies, 26
-// intervals 63 / 170, 10 000 x 16 384 1 921 / 2 422; more lanes in one wave of blocks against two or more, 18 lanes, 38 000 nodes x
-// 16 384 2 248 / 6 158, 5 lanes, 25 000 x 40 000 2 387 / 3 167; not in one against one, 75 000 x 16 384 5 462 / 3 795, 38 000 x 4 096
-// 2 014 / 1 645.  Where F does not fit the lane-stream kernel's blocks it seldom suits these (8 rows, 400 intervals, 6 439 nodes x 16
-// 2 065 / 1 522 by the step program).
+// Whether the walk kernel is the faster one.  Measured (us, it / the lane-stream kernel, 26 intervals): up to three lanes, 500 nodes x 4 096
+// policies 67 / 173, 10 000 x 16 384 1 899 / 2 408; more lanes in one wave of blocks against two or more, 18 lanes, 38 000 nodes x
+// 16 384 2 212 / 6 161, 5 lanes, 25 000 x 40 000 2 184 / 2 834; not in one against one, 75 000 x 16 384 (80 intervals) 5 462 / 3 795, 38 000 x
+// 4 096 2 014 / 1 645.  Where F does not fit the lane-stream kernel's blocks it seldom suits these (8 rows, 400 intervals, 6 439 nodes x
+// 16 2 065 / 1 522 by the step program).
 static bool walk_pays(const emo_graph *g, int64_t B, int rows, int32_t I, int walk_grid)
 {
     const int64_t sms = std::max(g->sm_count, 1), walk_waves = (walk_grid + sms - 1) / sms;
