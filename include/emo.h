@@ -141,7 +141,8 @@ int emo_graph_info(const emo_graph *g, emo_info *info);
  * invocation.
  * The size for forward-only calls covers every smaller batch.  It is kilobytes and the slice kernels' share, which is
  * bounded (256 MB; 80 policies' worth on graphs of millions of nodes): larger calls run in tiles of policies.  With
- * less, or with no workspace at all, a forward-only call takes smaller tiles or other kernels.  A slack call needs
+ * less, or with no workspace at all, a forward-only call takes smaller tiles or other kernels (a graph that only the
+ * generic kernels can take needs what is asked for: completion times of every node and policy).  A slack call needs
  * what this function gives for its own B; what larger batches need may be less.
  */
 int emo_workspace_bytes(const emo_graph *g, int64_t B, int need_slack, size_t *out);

@@ -1475,15 +1475,13 @@ bool flow_allowed(const emo_graph *g, int64_t B, const uint8_t *lvl, int64_t ldb
 }
 
 // ---- slices -------------------------------------------------------------------------------------------------
-int upload_slices(const Slices &s, DevSlice &d)
+// What a launch needs to know of a slice program.
+void size_slices(const Slices &s, DevSlice &d)
 {
     d = DevSlice();
-    if (!s.ok) return EMO_OK;
-    std::vector<uint4> index((size_t)s.count);
     for (int k = 0; k < s.count; ++k) {
         SliceHdr h;
         std::memcpy(&h, s.blob.data() + s.off[(size_t)k], sizeof(h));
-        index[(size_t)k] = make_uint4(s.off[(size_t)k], h.nodes, h.node0, std::min(h.head, 0xFFFFu) | std::min(h.words, 0xFFFFu) << 16);
         d.words = std::max(d.words, h.words);
         d.head = std::max(d.head, h.head);
         d.nodes = std::max(d.nodes, h.nodes);
@@ -1493,6 +1491,22 @@ int upload_slices(const Slices &s, DevSlice &d)
             d.slots1[i] = std::max(d.slots1[i], h.dir[i].slots1);
             d.slots2[i] = std::max(d.slots2[i], h.dir[i].slots2);
         }
+    }
+    d.count = s.count;
+    d.cols = s.cols;
+    d.Lp = s.Lp;
+    d.group = s.group;
+    d.groups = s.groups;
+    d.ready = s.ok;
+}
+
+int upload_slices(const Slices &s, DevSlice &d)
+{
+    std::vector<uint4> index((size_t)s.count);
+    for (int k = 0; k < s.count; ++k) {
+        SliceHdr h;
+        std::memcpy(&h, s.blob.data() + s.off[(size_t)k], sizeof(h));
+        index[(size_t)k] = make_uint4(s.off[(size_t)k], h.nodes, h.node0, std::min(h.head, 0xFFFFu) | std::min(h.words, 0xFFFFu) << 16);
     }
     const void *src[5] = {s.blob.data(), index.data(), s.rec.data(), s.tabT.data(), s.tabE.data()};
     const size_t bytes[5] = {s.blob.size() * 4, index.size() * sizeof(uint4), s.rec.size() * 4, s.tabT.size() * 4, s.tabE.size() * 8};
@@ -1507,6 +1521,7 @@ int upload_slices(const Slices &s, DevSlice &d)
     if (rc != cudaSuccess) {
         (void)cudaGetLastError();
         if (mem) cudaFree(mem);
+        d = DevSlice();
         return rc == cudaErrorMemoryAllocation ? EMO_E_OOM : EMO_E_CUDA;
     }
     d.mem = mem;
@@ -1515,12 +1530,6 @@ int upload_slices(const Slices &s, DevSlice &d)
     d.rec = (uint4 *)(d.mem + at[2]);
     d.tabT = (uint32_t *)(d.mem + at[3]);
     d.tabE = (double *)(d.mem + at[4]);
-    d.count = s.count;
-    d.cols = s.cols;
-    d.Lp = s.Lp;
-    d.group = s.group;
-    d.groups = s.groups;
-    d.ready = true;
     return EMO_OK;
 }
 
@@ -2376,7 +2385,12 @@ static int load_graph(int32_t n, const int64_t *row_ptr, const int32_t *col, con
             g->walk.blob = std::vector<unsigned char>();
         }
         if (rc == EMO_OK && slices.ok) {
-            const int rc_c = upload_slices(slices, g->dslice);
+            // (nodes with very many operands: a slice's steps, or its matrices, that no block's shared memory holds)
+            size_slices(slices, g->dslice);
+            SlicePlan probe;
+            const bool fits = slice_plan(g, 1, false, false, 0, probe) || slice_plan(g, 1, false, false, 1, probe);
+            if (!fits) g->dslice = DevSlice();
+            const int rc_c = fits ? upload_slices(slices, g->dslice) : EMO_OK;
             if (rc_c != EMO_OK && rc_c != EMO_E_OOM) rc = rc_c;      // (no memory for it: the others serve)
         }
         }

@@ -230,3 +230,28 @@ def test_slack_in_the_other_kernels_workspace(torch_cuda, emo, oracle_mod):
         emo.emo_slack_batch(h, B, lv_dev, lv_dev.stride(0), None, None, X, B, T, E, None, None, ws)
         assert np.array_equal(X.cpu().numpy(), want["slack"]) and np.array_equal(T.cpu().numpy(), want["makespan"]), size
     h.free()
+
+
+def test_slices_that_no_block_can_hold(torch_cuda, emo, oracle_mod):
+    """Every node waits for the sixty before it: 150 KB of steps a slice and direction.  No call can use them, nothing of them stays on the
+    device (33 MB here); the other kernels take the calls."""
+    torch = torch_cuda
+    n, k, rs = 16_000, 60, np.random.RandomState(1)
+    rp = np.r_[0, np.cumsum(np.minimum(np.arange(n), k))].astype(np.int64)
+    col = np.concatenate([np.arange(max(0, v - k), v) for v in range(n)]).astype(np.int32)
+    lat, energy = np.stack([rs.randint(1, 100, n), rs.randint(10 ** 5, 10 ** 6, n)], 1).astype(np.int64), rs.rand(n, 2)
+    used = []
+    # (the same programs otherwise: a load that shapes the spine program compiles no slices, nor the program with the longer stages)
+    for flags in (emo.EMO_F_LANES(2) | emo.EMO_F_SPINE_STAGE(16), emo.EMO_F_LANES(2) | emo.EMO_F_TEST_LONG_OOM):
+        before = torch.cuda.mem_get_info()[0]
+        h = emo.emo_graph_load(n, rp, col, None, 2, lat, energy, None, flags)
+        used.append(before - torch.cuda.mem_get_info()[0])
+        assert emo.emo_call_slices(h, 1, True, emo.EMO_F_SLICE_KERNEL) == emo.emo_call_slices(h, 1, False, emo.EMO_F_SLICE_KERNEL) == 0
+        if len(used) == 2:
+            lv = rs.randint(0, 2, size=(n, 16)).astype(np.uint8)
+            T, E = torch.zeros(16, dtype=torch.int64, device="cuda"), torch.zeros(16, dtype=torch.float64, device="cuda")
+            emo.emo_eval_policies(h, 16, torch.from_numpy(lv).cuda(), 16, T, E, None)
+            g = W.Graph(n, rp, col, None, 2, lat, energy, None, "dense")
+            assert np.array_equal(T.cpu().numpy(), oracle_mod.batch(g, lv)["makespan"])
+        h.free()
+    assert used[1] < used[0] + (16 << 20), used
