@@ -3079,13 +3079,15 @@ int emo_search_dp(const emo_graph *g, int32_t I, const int64_t *breaks, const do
     };
     int64_t calls = 0;
     *found = 0;
-    // One kernel for all of a search: it compares the energies of one batch with those of another, and two kernels add them in different
-    // orders.  The walk kernel where the rule takes it for the smallest batch and for the largest (what fits it with many policies
-    // fits with fewer).
-    IntervalPlan probe;
+    // One kernel for all batches of a round: it compares their energies, and two kernels add them in different orders.  (Energies of
+    // different rounds are not compared.)  The walk kernel where the rule takes it for the round's first batch: what fits it with many
+    // policies fits with fewer.
     const long long delta = interval_length(I, breaks);
-    const bool walk = !g->generic && interval_kernel(g, std::min<int64_t>(L, max_batch), I, delta, 0, 1, probe) == kIntervalWalk &&
-                      interval_kernel(g, max_batch, I, delta, 0, 1, probe) == kIntervalWalk;
+    bool walk = false;
+    auto choose = [&](int64_t candidates) {
+        IntervalPlan plan;
+        walk = !g->generic && interval_kernel(g, std::min(candidates, max_batch), I, delta, 0, 1, plan) == kIntervalWalk;
+    };
     try {
         std::vector<uint8_t> hF((size_t)rows * I * ldb);
         std::vector<int64_t> hT((size_t)max_batch);
@@ -3112,12 +3114,14 @@ int emo_search_dp(const emo_graph *g, int32_t I, const int64_t *breaks, const do
         std::map<int64_t, State> cur, nxt;
         {
             std::vector<uint8_t> P0((size_t)I, (uint8_t)(L - 1));
+            choose(1);
             int rc = predict({P0.data()}, {{-1, 0}});
             if (rc) return rc;
             cur[hT[0] / bin_ns] = State{hT[0], hE[0], P0};
         }
         for (int32_t i = 0; i < I; ++i) {
             nxt.clear();
+            choose((int64_t)cur.size() * L);
             // candidates in the order of Alg. 2: states by ascending time, levels ascending; evaluated in chunks
             std::vector<const uint8_t *> cand;
             std::vector<std::pair<int32_t, uint8_t>> patch;

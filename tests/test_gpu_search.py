@@ -88,21 +88,24 @@ def test_a_thread_per_policy(torch_cuda, emo, oracle_mod, seed):
                     oracle_mod.search_dp(g, dev_of, breaks, p_idle, T_max, bin_ns))
 
 
-def test_one_kernel_for_all_of_a_search(torch_cuda, emo, oracle_mod):
-    """Many lanes, rounds of several batches: a full batch by itself would run another kernel than the small ones.  The search compares the
-    energies of all of them, so they come from one kernel: that of the policy it chose is, bit for bit, what the call for one policy gives."""
+@pytest.mark.parametrize("max_batch", [6000, 11000])
+def test_one_kernel_for_all_of_a_round(torch_cuda, emo, oracle_mod, max_batch):
+    """Many lanes, a last round of several batches: its full batches by themselves would run another kernel than the rest of it.  The search
+    compares the energies of all of them, so they come from one kernel: that of the chosen policy (in a full batch of 6 000, in the rest
+    of 2 824 behind a batch of 11 000) is, bit for bit, what a full batch gives."""
     torch = torch_cuda
     g = W.make_graph("cfg3-8dev", 0.01)
     dev_of = W.device_of(g)
     t0 = int(oracle_mod.batch(g, np.full((g.n, 1), g.L - 1, np.uint8))["makespan"][0])
     breaks, p_idle, T_max = np.arange(3, dtype=np.int64) * (t0 // 3), W.idle_power(g.L), t0 + t0 // 4
-    a = run_search(torch, emo, g, dev_of, breaks, p_idle, T_max, 1, 6000, emo.EMO_F_INTERVALS, (1, 2))
-    assert a["n_pred"] > 6000      # (a round of more than one batch)
+    a = run_search(torch, emo, g, dev_of, breaks, p_idle, T_max, 1, max_batch, emo.EMO_F_INTERVALS, (1, 2))
+    assert a["n_pred"] == 1 + 24 + 24 ** 2 + 24 ** 3
     compare(a, oracle_mod.search_dp(g, dev_of, breaks, p_idle, T_max, 1))
     h = emo.load_workload(g, emo.EMO_F_INTERVALS, group_of=dev_of)
-    F = torch.from_numpy(np.repeat(np.asarray(a["F"], np.uint8)[None, :, None], int(dev_of.max()) + 1, axis=0).copy()).cuda()
-    T, E = torch.zeros(1, dtype=torch.int64, device="cuda"), torch.zeros(1, dtype=torch.float64, device="cuda")
-    ws = torch.empty(emo.emo_workspace_bytes_intervals(h, 1, 3, True), dtype=torch.uint8, device="cuda")
-    emo.emo_eval_intervals(h, 1, F, 1, 3, breaks, torch.from_numpy(p_idle).cuda(), T, E, None, ws)
-    assert float(E[0]) == a["E"] and int(T[0]) == a["T"]
+    assert emo.emo_call_intervals(h, 24 ** 3 % 11000, breaks) == 1
+    F = torch.from_numpy(np.asarray(a["F"], np.uint8)).cuda()[None, :, None].repeat(int(dev_of.max()) + 1, 1, 6000).contiguous()
+    T, E = torch.zeros(6000, dtype=torch.int64, device="cuda"), torch.zeros(6000, dtype=torch.float64, device="cuda")
+    ws = torch.empty(emo.emo_workspace_bytes_intervals(h, 6000, 3, True), dtype=torch.uint8, device="cuda")
+    emo.emo_eval_intervals(h, 6000, F, 6000, 3, breaks, torch.from_numpy(p_idle).cuda(), T, E, None, ws)
+    assert bool((E == a["E"]).all()) and bool((T == a["T"]).all())
     h.free()
