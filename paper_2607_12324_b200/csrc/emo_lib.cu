@@ -1796,8 +1796,8 @@ struct SliceCall {
     double *base_E;
 };
 
-// One tile of a call: policies b0 and following.  first, last: of the call (its events).
-int launch_slices(const emo_graph *g, SlicePlan pl, const SliceCall &c, int64_t b0, bool first, bool last, unsigned char *ws, cudaStream_t st)
+// One tile of a call: policies b0 and following, on a plan of its own (its pointers are set here).  first, last: of the call (its events).
+int launch_slices(const emo_graph *g, SlicePlan &pl, const SliceCall &c, int64_t b0, bool first, bool last, unsigned char *ws, cudaStream_t st)
 {
     const SliceKernels &k = kSliceKernels[pl.shape];
     auto from = [&](auto *x) { return x ? x + b0 : x; };
@@ -1862,26 +1862,33 @@ int launch_slices(const emo_graph *g, SlicePlan pl, const SliceCall &c, int64_t 
     return EMO_OK;
 }
 
-// Runs a call on the slice kernels, in tiles of as many policies as the workspace holds; false where it does not take them.
-bool slice_call(const emo_graph *g, int64_t B, bool need_bwd, uint32_t flags, const SliceCall &c, void *ws, size_t ws_bytes, size_t head, cudaStream_t st, int &rc)
+// A call in tiles of as many policies as the workspace holds; false where too few of them fit.
+bool slice_tiles(const emo_graph *g, int64_t B, bool need_bwd, uint32_t flags, const SliceCall &c, unsigned char *area, size_t room, cudaStream_t st, int &rc)
 {
-    const bool base = c.base_T || c.base_E;
-    SlicePlan pl, end;
-    if (!slice_allowed(g, B, base, need_bwd, c.ES || c.LS || c.slack_sum || c.n_critical, flags, pl)) return false;
-    const size_t room = slice_room(ws, ws_bytes, head);
-    unsigned char *const area = room ? (unsigned char *)ws + head : nullptr;
-    if (pl.ws <= room) {
-        rc = launch_slices(g, pl, c, 0, true, true, area, st);
-        return true;
-    }
-    // (the last tile has the all-max policy too)
+    const bool base = c.base_T || c.base_E;      // (the last tile has the all-max policy too)
     int64_t tile = std::min<int64_t>(B, (int64_t)(room / std::max<size_t>(slice_policy_bytes(g, need_bwd), 1))) / 16 * 16 - 16;
     while (tile >= kSliceLeastTile && slice_ws(g, tile + 1, need_bwd) > room) tile -= 16;
     if (tile < kSliceLeastTile) return false;
     const int64_t tiles = (B + tile - 1) / tile, rest = B - (tiles - 1) * tile;
-    if (!slice_shape(g, tile, false, need_bwd, flags, pl) || !slice_shape(g, rest, base, need_bwd, flags, end) || pl.ws > room || end.ws > room) return false;
+    SlicePlan each, end;
+    if (!slice_shape(g, tile, false, need_bwd, flags, each) || !slice_shape(g, rest, base, need_bwd, flags, end) || each.ws > room || end.ws > room) return false;
     rc = EMO_OK;
-    for (int64_t k = 0; k < tiles && rc == EMO_OK; ++k) rc = launch_slices(g, k + 1 < tiles ? pl : end, c, k * tile, k == 0, k + 1 == tiles, area, st);
+    for (int64_t k = 0; k < tiles && rc == EMO_OK; ++k) {
+        SlicePlan pl = k + 1 < tiles ? each : end;
+        rc = launch_slices(g, pl, c, k * tile, k == 0, k + 1 == tiles, area, st);
+    }
+    return true;
+}
+
+// Runs a call on the slice kernels; false where it does not take them.
+bool slice_call(const emo_graph *g, int64_t B, bool need_bwd, uint32_t flags, const SliceCall &c, void *ws, size_t ws_bytes, size_t head, cudaStream_t st, int &rc)
+{
+    SlicePlan pl;
+    if (!slice_allowed(g, B, c.base_T || c.base_E, need_bwd, c.ES || c.LS || c.slack_sum || c.n_critical, flags, pl)) return false;
+    const size_t room = slice_room(ws, ws_bytes, head);
+    unsigned char *const area = room ? (unsigned char *)ws + head : nullptr;
+    if (pl.ws > room) return slice_tiles(g, B, need_bwd, flags, c, area, room, st, rc);
+    rc = launch_slices(g, pl, c, 0, true, true, area, st);
     return true;
 }
 
